@@ -231,7 +231,7 @@ template <typename T> struct Solver {
   void gemm(Op opA, const T* A, int64_t lda, Op opB, const T* B, int64_t ldb, int64_t M, int64_t N, int64_t K,
             const Epi& e, int mode, bool force_split = false) {
     if ((force_split && mode != CHASE_FP64_NATIVE && oz::available()) || use_split(mode, M, N, K))
-      oz::gemm<T>(st(), c->ozw, opA, A, lda, opB, B, ldb, M, N, K, e, CHASE_FP64);
+      oz::gemm<T>(st(), c->ozw, opA, A, lda, opB, B, ldb, M, N, K, e);
     else
       gemm_f64<T>(st(), opA, opB, M, N, K, A, lda, B, ldb, e, W(), c->work_elems);
   }
@@ -1156,12 +1156,16 @@ int64_t chase_workspace_bytes(int64_t n_max, int ne_max, chase_dtype dtype, cons
   int64_t esz = dtype == CHASE_C128 ? 16 : 8;
   int64_t b = 3 * n_max * ne_max * esz + 2 * (int64_t)ne_max * ne_max * esz + work_elems_for(n_max, ne_max, o) * esz;
   b += (3 * 32 * (int64_t)ne_max + ne_max + 1024) * esz;  // Householder QR scratch
-  b += oz::workspace_bytes(n_max, ne_max, dtype == CHASE_C128, o.oz_slices);
+  b += oz::workspace_bytes(n_max, ne_max, dtype == CHASE_C128, 0);
   return b;
 }
 
-chase_status chase_create(chase_ctx** out, int64_t n_max, int ne_max, chase_dtype dtype, const chase_opts* opts,
-                          void* stream) {
+}  // extern "C"
+
+// extra_bytes: device memory the context may take beyond chase_workspace_bytes to hold A's residue planes for more
+// moduli at a time (< 0: half of what is free after it).  All of them resident save a conversion of A per product.
+static chase_status create_ctx(chase_ctx** out, int64_t n_max, int ne_max, chase_dtype dtype, const chase_opts* opts,
+                               void* stream, int64_t extra_bytes) {
   if (!out) return CHASE_ERR_ARG;
   *out = nullptr;
   if (n_max < 1 || ne_max < 1 || ne_max > n_max || (dtype != CHASE_R64 && dtype != CHASE_C128)) return CHASE_ERR_ARG;
@@ -1220,7 +1224,11 @@ chase_status chase_create(chase_ctx** out, int64_t n_max, int ne_max, chase_dtyp
     CHASE_CUDA(cudaMalloc(&c->status_dev, 4 * sizeof(int)));
     CHASE_CUDA(cudaMalloc(&c->qr_dep, (size_t)(ne_max + 1) * sizeof(int)));
     CHASE_CUDA(cudaMalloc(&c->hh, (size_t)(3 * 32 * (size_t)ne_max + ne_max + 1024) * c->esz));
-    oz::create(c->ozw, n_max, ne_max, dtype == CHASE_C128, c->opts.oz_slices);
+    const bool cplx = dtype == CHASE_C128;
+    if (extra_bytes < 0) extra_bytes = ((int64_t)freeb - need - (64ll << 20)) / (2 * nctx);
+    const int fewest = oz::a_mods_within(n_max, cplx, 0);
+    oz::create(c->ozw, n_max, ne_max, cplx,
+               oz::a_mods_within(n_max, cplx, crt::plane_bytes(n_max, n_max, cplx, fewest) + extra_bytes));
     // workers of batched solves: same sizes and options, one non-blocking stream each
     chase_opts wo = c->opts;
     wo.batch_workers = 1;
@@ -1228,7 +1236,7 @@ chase_status chase_create(chase_ctx** out, int64_t n_max, int ne_max, chase_dtyp
       cudaStream_t ws = nullptr;
       CHASE_CUDA(cudaStreamCreateWithFlags(&ws, cudaStreamNonBlocking));
       chase_ctx* wc = nullptr;
-      chase_status st = chase_create(&wc, n_max, ne_max, dtype, &wo, ws);
+      chase_status st = create_ctx(&wc, n_max, ne_max, dtype, &wo, ws, extra_bytes);
       if (st != CHASE_OK) {
         cudaStreamDestroy(ws);
         throw chase::Error{(int)st, "creating a batch worker failed"};
@@ -1242,6 +1250,13 @@ chase_status chase_create(chase_ctx** out, int64_t n_max, int ne_max, chase_dtyp
   }
   *out = c;
   return CHASE_OK;
+}
+
+extern "C" {
+
+chase_status chase_create(chase_ctx** out, int64_t n_max, int ne_max, chase_dtype dtype, const chase_opts* opts,
+                          void* stream) {
+  return create_ctx(out, n_max, ne_max, dtype, opts, stream, -1);
 }
 
 void chase_destroy(chase_ctx* c) {
@@ -1572,6 +1587,8 @@ static void solve_batched_grouped(chase_ctx* c, int nprob, const void* const* A,
   so.batch_workers = 1;
   so.batch_grouped = 0;
   if ((int)c->slots.size() < nprob) c->slots.resize(nprob, nullptr);
+  int64_t need_new = 0;
+  double n2_new = 0.0;
   for (int p = 0; p < nprob; ++p) {
     chase_ctx*& sl = c->slots[p];
     const int ne = nev[p] + nex[p];
@@ -1580,9 +1597,25 @@ static void solve_batched_grouped(chase_ctx* c, int nprob, const void* const* A,
       sl = nullptr;
     }
     if (!sl) {
+      need_new += chase_workspace_bytes(n[p], ne, c->dtype, &so);
+      n2_new += (double)n[p] * (double)n[p];
+    }
+  }
+  // memory beyond the new slots' workspaces: half of it goes to their residue planes, in proportion to n^2
+  double extra = 0.0;
+  if (need_new > 0) {
+    size_t freeb = 0, totb = 0;
+    CHASE_CUDA(cudaMemGetInfo(&freeb, &totb));
+    extra = std::max(0.0, 0.5 * ((double)freeb - (double)need_new - (double)(64ll << 20)));
+  }
+  for (int p = 0; p < nprob; ++p) {
+    chase_ctx*& sl = c->slots[p];
+    const int ne = nev[p] + nex[p];
+    if (!sl) {
       cudaStream_t ws = nullptr;
       CHASE_CUDA(cudaStreamCreateWithFlags(&ws, cudaStreamNonBlocking));
-      chase_status st = chase_create(&sl, n[p], ne, c->dtype, &so, ws);
+      chase_status st = create_ctx(&sl, n[p], ne, c->dtype, &so, ws,
+                                   (int64_t)(extra * ((double)n[p] * (double)n[p] / n2_new)));
       if (st != CHASE_OK) {
         cudaStreamDestroy(ws);
         sl = nullptr;
@@ -1680,10 +1713,11 @@ static void solve_batched_grouped(chase_ctx* c, int nprob, const void* const* A,
       plans.push_back(std::move(fp));
     }
     CHASE_CUDA(cudaEventRecord(t0, fs));
-    // the digit planes of A: computed once per solve (cached in the problem's workspace)
-    for (FilterPlan& fp : plans) oz::prepare_A<T>(fs, c->slots[fp.p]->ozw, R[fp.p].A, R[fp.p].n, R[fp.p].lda,
-                                                  CHASE_FP64);
-    std::vector<oz::ProductOp> ops_hi, ops_lo;
+    // the planes of A: computed once per solve and arithmetic (cached in the problem's workspace)
+    for (FilterPlan& fp : plans)
+      oz::prepare_A<T>(fs, c->slots[fp.p]->ozw, R[fp.p].A, R[fp.p].n, R[fp.p].lda, R[fp.p].fmode());
+    std::vector<crt::Product> ops_hi;
+    std::vector<oz::ProductOp> ops_lo;
     for (int sstep = 1; sstep <= smax; ++sstep) {
       ops_hi.clear();
       ops_lo.clear();
@@ -1701,7 +1735,6 @@ static void solve_batched_grouped(chase_ctx* c, int nprob, const void* const* A,
         T* out = Bb[sstep & 1] + (int64_t)fp.f * r.n;
         const T* in = Bb[(sstep - 1) & 1] + (int64_t)fp.f * r.n;
         const int fmode = r.fmode();
-        oz::split_right<T>(fs, sc->ozw, fmode, in, r.n, cols, r.n);
         Epi e;
         e.C = out;
         e.ldc = r.n;
@@ -1714,12 +1747,18 @@ static void solve_batched_grouped(chase_ctx* c, int nprob, const void* const* A,
           e.ldz = r.n;
           e.beta = fp.be[sstep];
         }
-        oz::ProductOp op{sc->ozw.a_planes, sc->ozw.a_scale, sc->ozw.slices, sc->ozw.b_planes, sc->ozw.b_scale,
-                         r.n, cols, r.n, e, c->ozw.group_m};
-        (fmode == CHASE_FP64 ? ops_hi : ops_lo).push_back(op);
+        if (fmode != CHASE_FP64) {
+          oz::split_right<T>(fs, sc->ozw, fmode, in, r.n, cols, r.n);
+          ops_lo.push_back(oz::ProductOp{sc->ozw.a_planes, sc->ozw.a_scale, oz::MIXED_SLICES, sc->ozw.b_planes,
+                                         sc->ozw.b_scale, r.n, cols, r.n, e, c->ozw.group_m});
+        } else if (oz::groupable(sc->ozw, r.n, cols)) {
+          ops_hi.push_back(oz::group_product<T>(fs, sc->ozw, in, r.n, cols, r.n, e));
+        } else {
+          oz::hemm<T>(fs, sc->ozw, r.A, r.n, r.lda, in, r.n, cols, e, CHASE_FP64);  // A's planes in passes
+        }
         sc->stats.filter_launches++;
       }
-      if (!ops_hi.empty()) oz::launch_group<CPLX>(fs, c->ozw, CHASE_FP64, ops_hi.data(), (int)ops_hi.size());
+      if (!ops_hi.empty()) oz::multiply_group<CPLX>(fs, c->ozw, ops_hi.data(), (int)ops_hi.size());
       // the low-precision problems of one batch share its mode
       if (!ops_lo.empty()) oz::launch_group<CPLX>(fs, c->ozw, mode, ops_lo.data(), (int)ops_lo.size());
     }

@@ -1,0 +1,910 @@
+// FP64-class products C = L R on the bf16 tensor cores (tcgen05, TMEM, TMA, CTA pairs) through residues.
+//
+// Every left row / right column x is scaled by a power of two so that its 2-norm is below 2^62 and rounded to
+// integers X (at most half a unit each).  The integer product then satisfies |C_ij| <= ||X_i|| ||Y_j|| < 2^124
+// (Cauchy-Schwarz), and it is determined by its residues modulo NMOD = 14 pairwise coprime moduli m_i <= 512 whose
+// product is M = 2^125.25 (Chinese remainder theorem): 2^124 = 0.42 M < M / 2.  Each residue of X lies in
+// [-256, 256] and is exact in bf16, a product of two residues is at most 2^16, and 256 of them sum to at most 2^24,
+// so FP32 accumulators are exact over chunks of 256 along K.  Complex operands take three real products per modulus
+// instead of four, P1 = Xr Yr, P2 = Xi Yi, P3 = (Xr + Xi)(Yr + Yi): modulo m_i nothing is lost to the sums or to
+// Re = P1 - P2, Im = P3 - P1 - P2.
+//
+// Why residues and not digits: splitting FP64 operands into seven 8-bit digits takes 28 digit-pair products (112 for
+// complex operands) and one accumulator per digit level, which caps the MMA width at 80 columns (44 cycles per MMA,
+// the instruction's floor, for 40 cycles of math).  Residues take 14 (42 complex) products, each a plain bf16 GEMM
+// with the widest MMA (256 x 256 x 16 on a CTA pair), and round the operands no more coarsely: an entry keeps
+// 62 - log2(norm / |entry|) bits.
+#include <cuda.h>
+#include <cuda_bf16.h>
+
+#include <algorithm>
+#include <mutex>
+
+#include "common.cuh"
+#include "crt.h"
+#include "tcgen05.cuh"
+#include "tmap.h"
+
+namespace chase {
+namespace crt {
+
+using oz::fence_after;
+using oz::fence_before;
+using oz::globaltimer;
+using oz::mbar_expect_tx;
+using oz::mbar_init;
+using oz::mbar_try;
+using oz::smem_u32;
+
+// ---------------------------------------------------------------- moduli and reconstruction constants
+typedef unsigned __int128 u128;
+
+// The 14 pairwise coprime integers <= 512 with the largest product (exhaustive search from the top).
+#define CRT_MODULI {512, 511, 509, 505, 503, 501, 499, 493, 491, 487, 481, 479, 473, 467}
+
+struct Tables {
+  int m[NMOD];           // moduli
+  int inv[NMOD];         // round(2^39 / m): nearest-integer quotients of |t| < 2^31 by a multiply and a shift
+  int c1[NMOD], c2[NMOD];  // 2^21 and 2^42 modulo m, in [-256, 256]
+  uint32_t w[NMOD][4];   // (M / m_i) ((M / m_i)^-1 mod m_i): the CRT weights, 32-bit limbs
+  uint32_t off[4];       // -BIAS sum_i w_i mod M
+  uint64_t Mlo, Mhi;
+  float q;               // 2^112 / M
+};
+constexpr int BIAS = 1024;  // added to every residue (at most 3 * 256 + 2 in size) so that the limb products are unsigned
+
+constexpr int sym_mod(u128 x, int m) {
+  int r = (int)(x % (u128)m);
+  return r > m / 2 ? r - m : r;
+}
+
+constexpr Tables make_tables() {
+  Tables t{};
+  const int ms[NMOD] = CRT_MODULI;
+  u128 M = 1;
+  for (int i = 0; i < NMOD; ++i) M *= (u128)ms[i];
+  u128 wsum = 0;
+  for (int i = 0; i < NMOD; ++i) {
+    const int m = ms[i];
+    t.m[i] = m;
+    t.inv[i] = (int)((((uint64_t)1 << 39) + (uint64_t)m / 2) / (uint64_t)m);
+    t.c1[i] = sym_mod((u128)1 << 21, m);
+    t.c2[i] = sym_mod((u128)1 << 42, m);
+    const u128 Mi = M / (u128)m;
+    const int a = (int)(Mi % (u128)m);
+    int iv = 1;
+    while (a * iv % m != 1) ++iv;
+    const u128 w = Mi * (u128)iv;  // < M: iv < m
+    for (int l = 0; l < 4; ++l) t.w[i][l] = (uint32_t)(w >> (32 * l));
+    wsum = (wsum + w) % M;
+  }
+  u128 off = 0;
+  for (int i = 0; i < BIAS; ++i) off = (off + wsum) % M;
+  off = M - off;
+  for (int l = 0; l < 4; ++l) t.off[l] = (uint32_t)(off >> (32 * l));
+  t.Mlo = (uint64_t)M;
+  t.Mhi = (uint64_t)(M >> 64);
+  t.q = (float)(281474976710656.0 / (double)t.Mhi);  // 2^112 / M = 2^48 / (M / 2^64)
+  return t;
+}
+
+constexpr Tables kTables = make_tables();
+static_assert(kTables.Mhi >> 61 == 1, "M lies in [2^125, 2^126)");
+__constant__ const Tables cT = make_tables();
+
+// ---------------------------------------------------------------- scales
+// Exponent e with norm < 2^e from the sum of squares.
+__device__ __forceinline__ int norm_exponent(double ss) {
+  int e;
+  frexp(sqrt(ss) * (1.0 + 1e-9), &e);
+  return e;
+}
+
+// Column norms: one pass of plain squares; a sum outside the range where squares neither overflow nor lose
+// bits to underflow (or a non-finite one) takes a second, scaled pass.  HBM/L2-bound, one block per column.
+template <typename T>
+__global__ void __launch_bounds__(256) col_exponent_kernel(int64_t K, const T* __restrict__ X, int64_t ldx, int* ex) {
+  using s = S<T>;
+  const T* x = X + (int64_t)blockIdx.x * ldx;
+  __shared__ double red[8];
+  __shared__ double sum_sh;
+  auto block_sum = [&](double v) {
+    v = warp_sum(v);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double t = 0.0;
+      for (int w = 0; w < 8; ++w) t += red[w];
+      sum_sh = t;
+    }
+    __syncthreads();
+    return sum_sh;
+  };
+  double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
+  int64_t i = threadIdx.x;
+  for (; i + 768 < K; i += 1024) {
+    const T v0 = x[i], v1 = x[i + 256], v2 = x[i + 512], v3 = x[i + 768];
+    a0 += s::abs2(v0);
+    a1 += s::abs2(v1);
+    a2 += s::abs2(v2);
+    a3 += s::abs2(v3);
+  }
+  for (; i < K; i += 256) a0 += s::abs2(x[i]);
+  double ss = block_sum((a0 + a1) + (a2 + a3));
+  if (ss > 1e-250 && ss < 1e250) {
+    if (threadIdx.x == 0) ex[blockIdx.x] = norm_exponent(ss);
+    return;
+  }
+  // largest magnitude (through the bit pattern, so that NaN and infinity compare largest), then scaled squares
+  __shared__ unsigned long long mx;
+  if (threadIdx.x == 0) mx = 0ull;
+  __syncthreads();
+  unsigned long long m = 0ull;
+  for (int64_t j = threadIdx.x; j < K; j += 256) {
+    const T v = x[j];
+    const unsigned long long br = (unsigned long long)__double_as_longlong(fabs(s::re(v)));
+    const unsigned long long bi = (unsigned long long)__double_as_longlong(fabs(s::im(v)));
+    m = m > br ? m : br;
+    m = m > bi ? m : bi;
+  }
+  atomicMax(&mx, m);
+  __syncthreads();
+  if (mx >= 0x7ff0000000000000ull) {
+    if (threadIdx.x == 0) ex[blockIdx.x] = NONFINITE;
+    return;
+  }
+  if (mx == 0ull) {
+    if (threadIdx.x == 0) ex[blockIdx.x] = 0;
+    return;
+  }
+  int em;
+  frexp(__longlong_as_double((long long)mx), &em);
+  double b = 0.0;
+  for (int64_t j = threadIdx.x; j < K; j += 256) {
+    const T v = x[j];
+    const double r = ldexp(s::re(v), -em), q = ldexp(s::im(v), -em);
+    b += r * r + q * q;
+  }
+  ss = block_sum(b);
+  if (threadIdx.x == 0) ex[blockIdx.x] = em + norm_exponent(ss);
+}
+
+// Row norms of a column-major X (vector = row): 32 rows x 8 threads along K per block, so that a short and a long
+// K both fill the SMs; same two-pass rule as the columns.
+template <typename T>
+__global__ void __launch_bounds__(256) row_exponent_kernel(int64_t nvec, int64_t K, const T* __restrict__ X, int64_t ldx,
+                                                            int* ex) {
+  using s = S<T>;
+  const int r = threadIdx.x & 31, c = threadIdx.x >> 5;
+  const int64_t i = (int64_t)blockIdx.x * 32 + r;
+  __shared__ double red[8][33];
+  __shared__ unsigned long long redm[8][33];
+  double a = 0.0;
+  unsigned long long m = 0ull;
+  if (i < nvec) {
+#pragma unroll 4
+    for (int64_t k = c; k < K; k += 8) {
+      const T v = X[i + k * ldx];
+      a += s::abs2(v);
+      const unsigned long long br = (unsigned long long)__double_as_longlong(fabs(s::re(v)));
+      const unsigned long long bi = (unsigned long long)__double_as_longlong(fabs(s::im(v)));
+      m = m > br ? m : br;
+      m = m > bi ? m : bi;
+    }
+  }
+  red[c][r] = a;
+  redm[c][r] = m;
+  __syncthreads();
+  if (c != 0 || i >= nvec) return;
+  for (int w = 1; w < 8; ++w) {
+    a += red[w][r];
+    m = m > redm[w][r] ? m : redm[w][r];
+  }
+  int e;
+  if (m >= 0x7ff0000000000000ull) {
+    e = NONFINITE;
+  } else if (m == 0ull) {
+    e = 0;
+  } else if (a > 1e-250 && a < 1e250) {
+    e = norm_exponent(a);
+  } else {
+    int em;
+    frexp(__longlong_as_double((long long)m), &em);
+    double b = 0.0;
+    for (int64_t k = 0; k < K; ++k) {
+      const T v = X[i + k * ldx];
+      const double p = ldexp(s::re(v), -em), q = ldexp(s::im(v), -em);
+      b += p * p + q * q;
+    }
+    e = em + norm_exponent(b);
+  }
+  ex[i] = e;
+}
+
+// ---------------------------------------------------------------- residue planes
+// round(x 2^(62 - e)) by integer shifts of the mantissa (GB300's FP64 conversions run at 1/64 of the integer
+// rate); |result| <= 2^62 because |x| < 2^e.  Non-finite vectors give arbitrary in-range integers.
+__device__ __forceinline__ long long scaled_int(double x, int e) {
+  const long long b = __double_as_longlong(x);
+  const int be = (int)((b >> 52) & 0x7ff);
+  long long m = b & 0xfffffffffffffll;
+  if (be != 0) m |= 0x10000000000000ll;
+  const int sh = (be != 0 ? be : 1) - 1075 + 62 - e;  // x = m 2^(exponent - 1075)
+  long long r;
+  if (sh >= 0) {
+    r = m << (sh < 9 ? sh : 9);
+  } else {
+    const int rs = sh > -62 ? -sh : 62;
+    r = ((m >> (rs - 1)) + 1) >> 1;
+  }
+  return b < 0 ? -r : r;
+}
+
+struct Limbs {
+  int x0, x1, x2;
+};
+__device__ __forceinline__ Limbs limbs(long long x) {
+  return Limbs{(int)(x & 0x1fffff), (int)((x >> 21) & 0x1fffff), (int)(x >> 42)};
+}
+
+// x mod m_i in [-256, 256]: the limbs' residue sum t (|t| < 2^31), then t - m round(t / m).  The quotient's error is
+// below 2^-9 / 2, so |r| <= m / 2 + 1 / 2, which is 256 at most for odd m <= 511 and for m = 512.
+__device__ __forceinline__ int residue(const Limbs& x, int i) {
+  const int t = x.x0 + x.x1 * cT.c1[i] + x.x2 * cT.c2[i];
+  const int q = (int)(((long long)t * cT.inv[i] + (1ll << 38)) >> 39);
+  return t - q * cT.m[i];
+}
+// sum of two residues brought back to [-256, 256]
+__device__ __forceinline__ int residue_sum(int a, int b, int i) {
+  int r = a + b;
+  if (r > 256) r -= cT.m[i];
+  if (r < -256) r += cT.m[i];
+  return r;
+}
+// two integers |r| <= 256 as packed bf16 (exact: the upper halves of their FP32 images)
+__device__ __forceinline__ uint32_t pack_bf16(int a, int b) {
+  const float fa = __int_as_float(0x4b400000 + a) - 12582912.0f;
+  const float fb = __int_as_float(0x4b400000 + b) - 12582912.0f;
+  return __byte_perm(__float_as_uint(fa), __float_as_uint(fb), 0x7632);
+}
+
+// Four consecutive K elements of one vector: every modulus' planes, one 8-byte store per plane.
+template <typename T>
+__device__ __forceinline__ void write_residues(const T (&v)[4], int e, bool conj, int mod0, int nmod, int64_t plane,
+                                               __nv_bfloat16* out) {
+  using s = S<T>;
+  Limbs re[4], im[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) {
+    re[j] = limbs(scaled_int(s::re(v[j]), e));
+    if (s::cplx) {
+      const long long q = scaled_int(s::im(v[j]), e);
+      im[j] = limbs(conj ? -q : q);
+    }
+  }
+  for (int i = 0; i < nmod; ++i) {
+    int rr[4], ri[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) rr[j] = residue(re[j], mod0 + i);
+    *reinterpret_cast<uint2*>(out) = make_uint2(pack_bf16(rr[0], rr[1]), pack_bf16(rr[2], rr[3]));
+    out += plane;
+    if (s::cplx) {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) ri[j] = residue(im[j], mod0 + i);
+      *reinterpret_cast<uint2*>(out) = make_uint2(pack_bf16(ri[0], ri[1]), pack_bf16(ri[2], ri[3]));
+      out += plane;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) rr[j] = residue_sum(rr[j], ri[j], mod0 + i);
+      *reinterpret_cast<uint2*>(out) = make_uint2(pack_bf16(rr[0], rr[1]), pack_bf16(rr[2], rr[3]));
+      out += plane;
+    }
+  }
+}
+
+// vector = column of X
+template <typename T>
+__global__ void __launch_bounds__(128) residues_cols_kernel(int64_t K, int64_t Kp, int64_t nvec, const T* __restrict__ X,
+                                                             int64_t ldx, const int* __restrict__ ex, int conj, int mod0,
+                                                             int nmod, __nv_bfloat16* planes) {
+  const int64_t col = blockIdx.y;
+  const T* x = X + col * ldx;
+  int e = ex[col];
+  if (e == NONFINITE) e = 0;
+  for (int64_t i = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x); i < K; i += 4 * (int64_t)gridDim.x * blockDim.x) {
+    T v[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = i + j < K ? x[i + j] : S<T>::zero();
+    write_residues<T>(v, e, conj != 0, mod0, nmod, nvec * Kp, planes + col * Kp + i);
+  }
+}
+
+// vector = row of X: 32 x 32 tiles transposed through shared memory
+template <typename T>
+__global__ void __launch_bounds__(256) residues_rows_kernel(int64_t nvec, int64_t K, int64_t Kp, const T* __restrict__ X,
+                                                             int64_t ldx, const int* __restrict__ ex, int conj, int mod0,
+                                                             int nmod, __nv_bfloat16* planes) {
+  __shared__ T tile[32][33];
+  const int64_t i0 = (int64_t)blockIdx.x * 32, k0 = (int64_t)blockIdx.y * 32;
+  for (int r = threadIdx.x >> 5; r < 32; r += 8) {
+    const int64_t kk = k0 + r, i = i0 + (threadIdx.x & 31);
+    tile[r][threadIdx.x & 31] = (kk < K && i < nvec) ? X[i + kk * ldx] : S<T>::zero();
+  }
+  __syncthreads();
+  const int r = threadIdx.x >> 3, g = (threadIdx.x & 7) * 4;
+  const int64_t i = i0 + r;
+  if (i >= nvec || k0 + g >= K) return;
+  T v[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) v[j] = tile[g + j][r];
+  int e = ex[i];
+  if (e == NONFINITE) e = 0;
+  write_residues<T>(v, e, conj != 0, mod0, nmod, nvec * Kp, planes + i * Kp + k0 + g);
+}
+
+// ---------------------------------------------------------------- product kernel
+constexpr int TM = 256;           // rows of a tile: 128 per CTA of the pair
+constexpr int TN = 256;           // columns of a tile at most
+constexpr int TK = 64;            // K per stage: 128 bytes of bf16 (the 128-byte swizzle atom)
+constexpr int CHUNK = 4;          // stages per exact FP32 accumulation (256 along K)
+constexpr int STAGES = 6;
+constexpr int STAGE_BYTES = (128 + 128) * TK * 2;  // this CTA's 128 left rows and up to 128 right rows
+constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
+constexpr int NTHREADS = 384;     // warps 0-3: copies, MMA issue, TMEM; warps 4-11: accumulator reduction
+constexpr int EPI_WARPS = 8;
+constexpr int MAXG = 64;          // products per launch
+constexpr unsigned long long TIMEOUT_NS = 2000000000ull;
+
+template <int G> struct Params {
+  CUtensorMap tmA[G];
+  CUtensorMap tmB[G];
+  int16_t* R[G];
+  int M[G], N[G], nkb[G], mt[G], nt[G], ldr[G];
+  int nblk[G];                   // 32-column blocks of the product's columns
+  int box_b[G];                  // right rows per copy
+  int unit_begin[G + 1];
+  int nprob, mod0, np;           // np: planes per modulus
+};
+
+// column blocks of tile n: the nblk 32-column blocks spread evenly over nt tiles
+__device__ __forceinline__ void tile_cols(int nblk, int nt, int n, int& n0, int& width) {
+  const int base = nblk / nt, rem = nblk % nt;
+  n0 = 32 * (n * base + min(n, rem));
+  width = 32 * (base + (n < rem ? 1 : 0));
+}
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// shared::cluster address of this CTA-local address in CTA 0 (the leader) of the pair
+__device__ __forceinline__ uint32_t leader_addr(uint32_t a) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(a));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void arrive_cluster(uint32_t bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+// bounded wait: false on expiry (which sets the launch's error flag) or when another role set it
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* err) {
+  unsigned long long t0 = 0;
+  for (uint32_t it = 0;; ++it) {
+    if (mbar_try(bar, parity)) return true;
+    if ((it & 255) == 255) {
+      if (*(volatile int*)err != 0) return false;
+      const unsigned long long t = globaltimer();
+      if (t0 == 0) t0 = t;
+      else if (t - t0 > TIMEOUT_NS) {
+        atomicOr(err, 1);
+        return false;
+      }
+    }
+  }
+}
+__device__ __forceinline__ void tma_load_pair(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y, int z) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, "
+      "%5}], [%2];" ::"r"(dst),
+      "l"((unsigned long long)map), "r"(bar), "r"(x), "r"(y), "r"(z)
+      : "memory");
+}
+__device__ __forceinline__ void mma_pair(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
+      "l"(a), "l"(b), "r"(idesc), "r"(acc));
+}
+// arrives on the barrier at this offset in both CTAs when every MMA issued so far has completed
+__device__ __forceinline__ void commit_pair(uint32_t bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
+      "h"((uint16_t)3)
+      : "memory");
+}
+// K-major operand tile, 128-byte swizzle: 8-row groups 1024 bytes apart
+__device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr >> 4) & 0x3FFF);
+  d |= (uint64_t)1 << 16;
+  d |= (uint64_t)(1024 >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)2 << 61;
+  return d;
+}
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,%16,%17,%18,%19,"
+      "%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+
+// two FP32 lanes per instruction
+__device__ __forceinline__ uint64_t pack2(uint32_t a, uint32_t b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "r"(a), "r"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t both(float x) { return pack2(__float_as_uint(x), __float_as_uint(x)); }
+
+// v - m round(v / m) on both lanes, exact for integers |v| <= 2^24 (result at most m / 2 + 1 in size)
+struct Mod2 {
+  uint64_t inv, negm, magic, negmagic;
+  __device__ __forceinline__ explicit Mod2(int m)
+      : inv(both(1.0f / (float)m)), negm(both(-(float)m)), magic(both(12582912.0f)), negmagic(both(-12582912.0f)) {}
+  __device__ __forceinline__ uint64_t operator()(uint64_t v) const {
+    const uint64_t q = add2(fma2(v, inv, magic), negmagic);
+    return fma2(q, negm, v);
+  }
+};
+
+// One CTA pair per unit (tile of one residue plane's product), persistent over the launch's units.  Each CTA copies
+// its 128 left rows and half of the right rows of a stage; the leader issues the pair's MMAs into one of two
+// accumulator sets (2 x 256 TMEM columns) and the eight reduction warps of each CTA take a finished chunk modulo m
+// into FP32 registers while the next chunk accumulates in the other set.  At a unit's end they write residues
+// (16-bit); the copies and MMAs of the next unit run meanwhile.
+// Register split: 384 threads at 168 (64512 at launch); warps 0-3 give down to 40, warps 4-11 take 232.
+template <int G>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
+    crt_gemm_kernel(const __grid_constant__ Params<G> gp, int* err) {
+  extern __shared__ __align__(1024) unsigned char smem_raw[];
+  unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
+  uint64_t* full = (uint64_t*)(smem + STAGES * STAGE_BYTES);  // leader's: both CTAs' copies of a stage have landed
+  uint64_t* empty = full + STAGES;                            // each CTA's: the stage's MMAs are done
+  uint64_t* acc_full = empty + STAGES;                        // each CTA's: a chunk is complete in set b
+  uint64_t* acc_empty = acc_full + 2;                         // leader's: both CTAs have read set b
+  uint64_t* drain = acc_empty + 2;
+  uint32_t* tmem_slot = (uint32_t*)(drain + 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_rank();
+  const int cluster = blockIdx.x >> 1, nclusters = gridDim.x >> 1;
+  const int total = gp.unit_begin[gp.nprob];
+
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < STAGES; ++i) {
+      mbar_init(smem_u32(&full[i]), 1);
+      mbar_init(smem_u32(&empty[i]), 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(smem_u32(&acc_full[i]), 1);
+      mbar_init(smem_u32(&acc_empty[i]), 2 * EPI_WARPS);
+    }
+    mbar_init(smem_u32(drain), 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 2) {
+    asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(tmem_slot)));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;");
+  }
+  fence_before();
+  __syncthreads();
+  cluster_sync();
+  fence_after();
+  const uint32_t tmem = *tmem_slot;
+
+  if (warp < 4) {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
+    if (warp == 0 && lane == 0) {
+      // ---------------------------------------------------------- copies
+      int it = 0;
+      bool ok = true;
+      int prob = 0;
+      for (int unit = cluster; unit < total && ok; unit += nclusters) {
+        while (G > 1 && unit >= gp.unit_begin[prob + 1]) ++prob;
+        const int tiles = gp.mt[prob] * gp.nt[prob];
+        const int local = unit - gp.unit_begin[prob];
+        const int plane = local / tiles, t = local - plane * tiles;
+        const int m = t / gp.nt[prob], n = t - m * gp.nt[prob];
+        int n0, width;
+        tile_cols(gp.nblk[prob], gp.nt[prob], n, n0, width);
+        const int box = gp.box_b[prob];
+        const int y_a = m * TM + (int)rank * 128, y_b = n0 + (int)rank * (width >> 1);
+        const int z_b = gp.mod0 * gp.np + plane;
+        const uint32_t bytes = 2u * (uint32_t)(128 + box) * TK * 2;
+        const int nkb = gp.nkb[prob];
+        for (int kb = 0; kb < nkb; ++kb, ++it) {
+          const int s = it % STAGES;
+          if (!mbar_wait(smem_u32(&empty[s]), ((it / STAGES) & 1) ^ 1, err)) {
+            ok = false;
+            break;
+          }
+          if (rank == 0) mbar_expect_tx(smem_u32(&full[s]), bytes);
+          const uint32_t dst = smem_u32(smem + s * STAGE_BYTES), bar = leader_addr(smem_u32(&full[s]));
+          tma_load_pair(dst, &gp.tmA[prob], bar, kb * TK, y_a, plane);
+          tma_load_pair(dst + 128 * TK * 2, &gp.tmB[prob], bar, kb * TK, y_b, z_b);
+        }
+      }
+      if (ok) {
+        // every stage's release has arrived in this CTA before it may exit
+        for (int i = 0; i < STAGES && ok; ++i, ++it)
+          ok = mbar_wait(smem_u32(&empty[it % STAGES]), ((it / STAGES) & 1) ^ 1, err);
+      } else if (rank == 0) {
+        // aborted: the copies in flight (this CTA's and its peer's) land before the pair exits
+        for (int j = it > STAGES ? it - STAGES : 0; j < it; ++j) {
+          const unsigned long long t0 = globaltimer();
+          while (!mbar_try(smem_u32(&full[j % STAGES]), (j / STAGES) & 1) && globaltimer() - t0 < TIMEOUT_NS) {
+          }
+        }
+      }
+    } else if (warp == 1 && lane == 0 && rank == 0) {
+      // ---------------------------------------------------------- MMA issue
+      int it = 0, chunk = 0;
+      bool ok = true;
+      int prob = 0;
+      for (int unit = cluster; unit < total && ok; unit += nclusters) {
+        while (G > 1 && unit >= gp.unit_begin[prob + 1]) ++prob;
+        const int tiles = gp.mt[prob] * gp.nt[prob];
+        const int local = unit - gp.unit_begin[prob];
+        const int n = (local % tiles) % gp.nt[prob];
+        int n0, width;
+        tile_cols(gp.nblk[prob], gp.nt[prob], n, n0, width);
+        const uint32_t idesc = oz::idesc_bf16(TM, width);
+        const int nkb = gp.nkb[prob];
+        for (int kb = 0; kb < nkb; ++kb, ++it) {
+          const int b = chunk & 1;
+          if (kb % CHUNK == 0) {
+            if (!mbar_wait(smem_u32(&acc_empty[b]), ((chunk >> 1) & 1) ^ 1, err)) {
+              ok = false;
+              break;
+            }
+            fence_after();
+          }
+          const int s = it % STAGES;
+          if (!mbar_wait(smem_u32(&full[s]), (it / STAGES) & 1, err)) {
+            ok = false;
+            break;
+          }
+          fence_after();
+          const uint32_t base = smem_u32(smem + s * STAGE_BYTES);
+          const uint64_t ad = sw128_desc(base), bd = sw128_desc(base + 128 * TK * 2);
+          const uint32_t d = tmem + (uint32_t)(b * 256);
+#pragma unroll
+          for (int ks = 0; ks < TK / 16; ++ks)
+            mma_pair(d, ad + (uint64_t)(ks * 2), bd + (uint64_t)(ks * 2), idesc, (kb % CHUNK != 0 || ks != 0) ? 1u : 0u);
+          commit_pair(smem_u32(&empty[s]));
+          if (kb % CHUNK == CHUNK - 1 || kb == nkb - 1) {
+            commit_pair(smem_u32(&acc_full[b]));
+            ++chunk;
+          }
+        }
+      }
+      // every MMA is done before TMEM is freed
+      commit_pair(smem_u32(drain));
+      const unsigned long long t0 = globaltimer();
+      while (!mbar_try(smem_u32(drain), 0) && globaltimer() - t0 < TIMEOUT_NS) {
+      }
+    }
+    __syncwarp();
+  } else {
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 232;");
+    // ------------------------------------------------------------ chunk reduction
+    const int ew = warp - 4, q = ew & 3, half = ew >> 2;  // TMEM lane quadrant, column half
+    const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
+    const uint32_t rel0 = leader_addr(smem_u32(&acc_empty[0])), rel1 = leader_addr(smem_u32(&acc_empty[1]));
+    int chunk = 0;
+    bool ok = true;
+    int prob = 0;
+    for (int unit = cluster; unit < total && ok; unit += nclusters) {
+      while (G > 1 && unit >= gp.unit_begin[prob + 1]) ++prob;
+      const int nt = gp.nt[prob];
+      const int tiles = gp.mt[prob] * nt;
+      const int local = unit - gp.unit_begin[prob];
+      const int plane = local / tiles, t = local - plane * tiles;
+      const int m = t / nt, n = t - m * nt;
+      int n0, width;
+      tile_cols(gp.nblk[prob], nt, n, n0, width);
+      const int hc = width >> 1;  // this warp's columns: [half hc, half hc + hc)
+      const Mod2 mod(cT.m[gp.mod0 + plane / gp.np]);
+      const int nchunk = (gp.nkb[prob] + CHUNK - 1) / CHUNK;
+      uint64_t acc[64];
+#pragma unroll
+      for (int j = 0; j < 64; ++j) acc[j] = 0ull;
+      for (int c = 0; c < nchunk; ++c, ++chunk) {
+        const int b = chunk & 1;
+        // one verdict per warp: the loads below need every lane
+        ok = __all_sync(0xffffffffu, mbar_wait(smem_u32(&acc_full[b]), (chunk >> 1) & 1, err));
+        if (!ok) break;
+        fence_after();
+        const uint32_t src = lane_addr + (uint32_t)(b * 256 + half * hc);
+#pragma unroll
+        for (int g = 0; g < 4; ++g) {
+          if (g * 32 >= hc) continue;
+          uint32_t r[32];
+          tmem_ld32(src + (uint32_t)(g * 32), r);
+          tmem_wait_ld();
+          if (g * 32 + 32 >= hc) {  // the last read of this set: release it before the arithmetic
+            fence_before();
+            __syncwarp();
+            if (lane == 0) arrive_cluster(b ? rel1 : rel0);
+          }
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            const uint64_t v = pack2(r[2 * j], r[2 * j + 1]);
+            acc[g * 16 + j] = add2(acc[g * 16 + j], mod(v));
+          }
+        }
+      }
+      if (!ok) break;
+      const int row = m * TM + (int)rank * 128 + q * 32 + lane;
+      if (row < gp.M[prob]) {
+        const int N = gp.N[prob], ldr = gp.ldr[prob];
+        const int c0 = n0 + half * hc;
+        int16_t* out = gp.R[prob] + ((int64_t)(gp.mod0 * gp.np + plane) * N + c0) * ldr + row;
+#pragma unroll
+        for (int j = 0; j < 64; ++j) {
+          // integers of at most 2^24 / 257 chunks of 257: exact in FP32; residue at most 257 in size
+          const uint64_t v = mod(acc[j]);
+          const float lo = __uint_as_float((uint32_t)v), hi = __uint_as_float((uint32_t)(v >> 32));
+          if (2 * j < hc && c0 + 2 * j < N) out[(int64_t)(2 * j) * ldr] = (int16_t)(int)lo;
+          if (2 * j + 1 < hc && c0 + 2 * j + 1 < N) out[(int64_t)(2 * j + 1) * ldr] = (int16_t)(int)hi;
+        }
+      }
+    }
+  }
+  fence_before();
+  __syncthreads();
+  cluster_sync();
+  fence_after();
+  if (threadIdx.x == 0) {
+    // the leader's last commit has arrived in this CTA too
+    const unsigned long long t0 = globaltimer();
+    while (!mbar_try(smem_u32(drain), 0) && globaltimer() - t0 < TIMEOUT_NS) {
+    }
+  }
+  __syncthreads();
+  if (warp == 2) asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, 512;" ::"r"(tmem));
+  cluster_sync();
+}
+
+// ---------------------------------------------------------------- reconstruction
+// Double nearest to X 2^e for a signed 128-bit integer X (round to nearest even up to sticky bits below 2^-63 of the
+// leading one), by integer operations; exponents outside the normal range go through ldexp.
+__device__ __forceinline__ double to_double(__int128 x, int e) {
+  const bool neg = x < 0;
+  u128 u = neg ? (u128)(-x) : (u128)x;
+  uint64_t hi = (uint64_t)(u >> 64), lo = (uint64_t)u;
+  if ((hi | lo) == 0ull) return 0.0;
+  int sh;  // u = top 2^(64 - sh)
+  uint64_t top;
+  if (hi) {
+    sh = __clzll((long long)hi);
+    top = sh ? (hi << sh) | (lo >> (64 - sh)) : hi;
+  } else {
+    sh = 64 + __clzll((long long)lo);
+    top = lo << (sh - 64);
+  }
+  const uint64_t r = (top >> 11) + ((top >> 10) & 1ull & (uint64_t)(((top & 0x3ffull) != 0ull) | ((top >> 11) & 1ull)));
+  // value = r 2^(75 - sh + e); r in [2^52, 2^53]
+  const int ex = 75 - sh + e + 1075;  // biased exponent of r's leading bit at 2^52
+  double v;
+  if (ex >= 1 && ex <= 2045)
+    v = __longlong_as_double((long long)(r + ((uint64_t)(ex - 1) << 52)));
+  else
+    v = ldexp((double)r, ex - 1075);
+  return neg ? -v : v;
+}
+
+// The product entry (in units of 2^e) whose residues, each plus BIAS, have been summed against the weights' limbs.
+__device__ __forceinline__ double reconstruct(const uint64_t (&a)[4], int e) {
+  const uint64_t s0 = a[0] + cT.off[0];
+  const uint64_t s1 = a[1] + cT.off[1] + (s0 >> 32);
+  const uint64_t s2 = a[2] + cT.off[2] + (s1 >> 32);
+  const uint64_t s3 = a[3] + cT.off[3] + (s2 >> 32);
+  // T = s3 2^96 + ...; T / M < 2^15 lies within 0.42 of an integer; FP32 of its top 31 bits is off by 2^-9 at most
+  const uint32_t q = (uint32_t)__float2int_rn((float)(uint32_t)(s3 >> 16) * cT.q);
+  u128 t = ((u128)((s3 << 32) | (uint32_t)s2) << 64) | (u128)((s1 << 32) | (uint32_t)s0);
+  const u128 M = ((u128)cT.Mhi << 64) | cT.Mlo;
+  t -= M * (u128)q;
+  return to_double((__int128)t, e);
+}
+
+// Two rows per thread (one 4-byte load per plane).  HBM-bound on the residues (2 bytes per plane and entry); the
+// weights' limb products run on the integer pipe.
+template <bool CPLX>
+__global__ void __launch_bounds__(128) combine_kernel(int M, int N, int ldr, const int16_t* __restrict__ R,
+                                                       const int* __restrict__ lex, const int* __restrict__ rex, Epi ep) {
+  constexpr int NP = CPLX ? 3 : 1, NC = CPLX ? 2 : 1;
+  const int i0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x), j = blockIdx.y;
+  if (i0 >= M) return;
+  const int16_t* src = R + (int64_t)j * ldr + i0;
+  const int64_t plane = (int64_t)N * ldr;
+  uint64_t acc[2][NC][4];
+#pragma unroll
+  for (int r = 0; r < 2; ++r)
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+#pragma unroll
+      for (int l = 0; l < 4; ++l) acc[r][c][l] = 0ull;
+#pragma unroll
+  for (int i = 0; i < NMOD; ++i) {
+    short2 p[NP];
+#pragma unroll
+    for (int k = 0; k < NP; ++k) p[k] = *reinterpret_cast<const short2*>(src + (int64_t)(i * NP + k) * plane);
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const int p0 = r ? p[0].y : p[0].x;
+      uint32_t v[NC];
+      if (CPLX) {
+        const int p1 = r ? p[NP - 2].y : p[NP - 2].x, p2 = r ? p[NP - 1].y : p[NP - 1].x;
+        v[0] = (uint32_t)(p0 - p1 + BIAS);
+        v[NC - 1] = (uint32_t)(p2 - p0 - p1 + BIAS);
+      } else {
+        v[0] = (uint32_t)(p0 + BIAS);
+      }
+#pragma unroll
+      for (int c = 0; c < NC; ++c)
+#pragma unroll
+        for (int l = 0; l < 4; ++l) acc[r][c][l] += (uint64_t)v[c] * cT.w[i][l];
+    }
+  }
+  const int ej = rex[j];
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    const int i = i0 + r;
+    if (i >= M) return;
+    const int ei = lex[i];
+    const bool bad = ei == NONFINITE || ej == NONFINITE;
+    double* C = (double*)ep.C + (i + (int64_t)j * ep.ldc) * NC;
+    const double g = ep.Y ? ep.gamma * (ep.ycol ? ep.ycol[j] : 1.0) : 0.0;
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      double v = bad ? __longlong_as_double(0x7ff8000000000000ll) : reconstruct(acc[r][c], ei + ej - 124);
+      double out = ep.alpha * v;
+      if (ep.Y) out += g * ((const double*)ep.Y)[(i + (int64_t)j * ep.ldy) * NC + c];
+      if (ep.Z) out += ep.beta * ((const double*)ep.Z)[(i + (int64_t)j * ep.ldz) * NC + c];
+      C[c] = out;
+    }
+  }
+}
+
+// ---------------------------------------------------------------- host side
+template <typename T>
+void scales(cudaStream_t st, bool by_rows, int64_t nvec, int64_t K, const T* X, int64_t ldx, int* ex) {
+  if (by_rows)
+    row_exponent_kernel<T><<<ceil_div(nvec, 32), 256, 0, st>>>(nvec, K, X, ldx, ex);
+  else
+    col_exponent_kernel<T><<<(unsigned)nvec, 256, 0, st>>>(K, X, ldx, ex);
+  CHASE_CHECK_LAUNCH();
+}
+
+template <typename T>
+void residues(cudaStream_t st, bool by_rows, bool conj, int64_t nvec, int64_t K, const T* X, int64_t ldx, const int* ex,
+              int mod0, int nmod, void* planes) {
+  const int64_t kp = kpad(K);
+  if (by_rows) {
+    const dim3 grid(ceil_div(nvec, 32), ceil_div(K, 32));
+    CHASE_REQUIRE(grid.y <= 65535, 1, "residues: vectors too long");
+    residues_rows_kernel<T><<<grid, 256, 0, st>>>(nvec, K, kp, X, ldx, ex, conj ? 1 : 0, mod0, nmod,
+                                                  (__nv_bfloat16*)planes);
+  } else {
+    CHASE_REQUIRE(nvec <= 65535, 1, "residues: too many vectors");
+    const dim3 grid(ceil_div(K, 512), (unsigned)nvec);
+    residues_cols_kernel<T><<<grid, 128, 0, st>>>(K, kp, nvec, X, ldx, ex, conj ? 1 : 0, mod0, nmod,
+                                                  (__nv_bfloat16*)planes);
+  }
+  CHASE_CHECK_LAUNCH();
+}
+
+template <int G> static void launch(cudaStream_t st, const Product* ops, int nops, bool cplx, int mod0, int nmod, int* err) {
+  static thread_local Params<G> gp;  // large for G > 1: built in thread-local host memory
+  const int np = planes(cplx);
+  int64_t units = 0;
+  for (int p = 0; p < nops; ++p) {
+    const Product& o = ops[p];
+    const int64_t kp = kpad(o.K);
+    const int nblk = (int)ceil_div(o.N, 32), nt = (int)ceil_div(nblk, TN / 32);
+    const int box = 16 * (int)ceil_div(nblk, nt);
+    gp.tmA[p] = make_tmap_bf16(o.lpl, o.K, kp, o.M, nmod * np, TK, 128, 1, CU_TENSOR_MAP_SWIZZLE_128B);
+    gp.tmB[p] = make_tmap_bf16(o.rpl, o.K, kp, o.N, NMOD * np, TK, box, 1, CU_TENSOR_MAP_SWIZZLE_128B);
+    gp.R[p] = (int16_t*)o.res;
+    gp.M[p] = (int)o.M;
+    gp.N[p] = (int)o.N;
+    gp.nkb[p] = (int)ceil_div(o.K, TK);
+    gp.mt[p] = (int)ceil_div(o.M, TM);
+    gp.nt[p] = nt;
+    gp.nblk[p] = nblk;
+    gp.box_b[p] = box;
+    gp.ldr[p] = (int)rpad(o.M);
+    gp.unit_begin[p] = (int)units;
+    units += (int64_t)gp.mt[p] * nt * np * nmod;
+    CHASE_REQUIRE(units <= 0x7fffffff, 1, "residue product: too many tiles");
+  }
+  gp.unit_begin[nops] = (int)units;
+  gp.nprob = nops;
+  gp.mod0 = mod0;
+  gp.np = np;
+  static std::once_flag once;
+  static cudaError_t attr_err = cudaSuccess;
+  static int max_clusters = 0;
+  std::call_once(once, []() {
+    attr_err = cudaFuncSetAttribute(crt_gemm_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+    if (attr_err != cudaSuccess) return;
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = 2;
+    at.val.clusterDim.y = 1;
+    at.val.clusterDim.z = 1;
+    cfg.gridDim = dim3(2, 1, 1);
+    cfg.blockDim = dim3(NTHREADS, 1, 1);
+    cfg.dynamicSmemBytes = SMEM_BYTES;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    attr_err = cudaOccupancyMaxActiveClusters(&max_clusters, crt_gemm_kernel<G>, &cfg);
+  });
+  CHASE_CUDA(attr_err);
+  const int clusters = (int)std::min<int64_t>(units, std::max(1, max_clusters));
+  crt_gemm_kernel<G><<<2 * clusters, NTHREADS, SMEM_BYTES, st>>>(gp, err);
+  CHASE_CHECK_LAUNCH();
+}
+
+template <bool CPLX>
+void multiply(cudaStream_t st, const Product* ops, int nops, int mod0, int nmod, int* err) {
+  for (int q0 = 0; q0 < nops; q0 += MAXG) {
+    const int cnt = std::min(MAXG, nops - q0);
+    if (cnt == 1)
+      launch<1>(st, ops + q0, 1, CPLX, mod0, nmod, err);
+    else
+      launch<MAXG>(st, ops + q0, cnt, CPLX, mod0, nmod, err);
+  }
+}
+
+template <bool CPLX> void combine(cudaStream_t st, const Product& op) {
+  CHASE_REQUIRE(op.N <= 65535, 1, "residue product: too many columns");
+  const dim3 grid(ceil_div(op.M, 256), (unsigned)op.N);
+  combine_kernel<CPLX><<<grid, 128, 0, st>>>((int)op.M, (int)op.N, (int)rpad(op.M), (const int16_t*)op.res, op.lex,
+                                             op.rex, op.e);
+  CHASE_CHECK_LAUNCH();
+}
+
+#define INST(T)                                                                                                  \
+  template void scales<T>(cudaStream_t, bool, int64_t, int64_t, const T*, int64_t, int*);                         \
+  template void residues<T>(cudaStream_t, bool, bool, int64_t, int64_t, const T*, int64_t, const int*, int, int, void*);
+INST(double)
+INST(double2)
+#undef INST
+template void multiply<false>(cudaStream_t, const Product*, int, int, int, int*);
+template void multiply<true>(cudaStream_t, const Product*, int, int, int, int*);
+template void combine<false>(cudaStream_t, const Product&);
+template void combine<true>(cudaStream_t, const Product&);
+
+}  // namespace crt
+}  // namespace chase

@@ -1,5 +1,5 @@
-// Split-BF16 tensor-core products (tcgen05) with FP64-accurate or mixed
-// precision accumulation: the production path of the large HEMM/GEMM products.
+// Split tensor-core products (tcgen05) of the eigensolver: FP64-class products through residues (crt.cu) and the
+// mixed-precision filter products through digit planes (oz_kernel.cuh), with their workspace.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -7,15 +7,16 @@
 #include <map>
 #include <vector>
 
+#include "crt.h"
 #include "kernels.h"
 
 namespace chase {
 namespace oz {
 
-// Launch configuration of the split-product kernel chosen by measurement (see tune_pick in oz_gemm.cu):
-// the tile width NT of the mixed modes (128 or 256 columns) and the tile-order group size.
+// Launch configuration of the mixed-precision product kernel chosen by measurement (see tune_pick in oz_gemm.cu):
+// the tile width NT (128 or 256 columns) and the tile-order group size.
 struct LaunchCfg {
-  int nt = 0;       // 0: the mode's fixed width
+  int nt = 128;
   int group_m = 8;
 };
 
@@ -27,35 +28,47 @@ struct TuneEntry {
   std::vector<cudaEvent_t> ev;  // start/stop pair per candidate
 };
 
+constexpr int MIXED_SLICES = 3;  // digit slices of A held for the mixed modes (BF16x3 uses the first two)
+
 struct Workspace {
   bool ready = false;
   bool complex_ = true;
-  int slices = 6;
   int64_t n_max = 0;
   int ne_max = 0;
-  void* a_planes = nullptr;   // bf16 digit planes of A
-  void* b_planes = nullptr;   // bf16 digit planes of the right operand
-  void* l_planes = nullptr;   // bf16 digit planes of a general left operand
+  // FP64-class products
+  void* a_res = nullptr;      // residue planes of A: a_mods moduli at a time
+  int a_mods = 0;             // crt::NMOD: all of them stay resident; fewer: converted per product in passes
+  void* l_res = nullptr;      // residue planes of a general left operand
+  void* residue = nullptr;    // residues of a product (residue_bytes)
+  int64_t residue_bytes = 0;
+  int* a_ex = nullptr;        // per-row exponents of A
+  int* l_ex = nullptr;        // of the general left operand
+  int* b_ex = nullptr;        // per-column exponents of the right operand
+  // mixed modes
+  void* a_planes = nullptr;   // bf16 digit planes of A (MIXED_SLICES slices)
   double* a_scale = nullptr;  // per-row power-of-two scale of A
-  double* l_scale = nullptr;  // per-row scale of the general left operand
   double* b_scale = nullptr;  // per-column scale of the right operand
-  int* flags = nullptr;       // device error flags of the bounded waits
   double* partial = nullptr;  // FP64 partial sums of products split along K
   int64_t partial_elems = 0;
-  int group_m = 8;            // row blocks per tile group of the split-product launch order (untuned launches)
+  void* b_planes = nullptr;   // planes of the right operand (residues or digits, b_bytes)
+  int64_t b_bytes = 0;
+  int* flags = nullptr;       // device error flags of the bounded waits
+  int group_m = 8;            // row blocks per tile group of the mixed launch order (untuned launches)
   bool autotune = true;       // choose LaunchCfg per size class by timing the candidates
   std::map<uint64_t, TuneEntry> tune;  // size class -> measurements and choice
   // optional CUDA-event timing of the product kernels (filter roofline)
   bool timing = false;
   std::vector<cudaEvent_t> ev;
   int ev_used = 0;
-  const void* a_src = nullptr;  // A whose planes are cached
-  int a_mode = -1;
+  // A whose exponents and residues (a_src) or digit planes (d_src) are held
+  const void* a_src = nullptr;
   int64_t a_n = 0;
+  const void* d_src = nullptr;
+  int64_t d_n = 0;
 };
 
-// One product C = L R of a grouped launch: digit planes and scales of both operands, sizes, epilogue and
-// the tile-order group size.
+// One product C = L R of a grouped mixed-precision launch: digit planes and scales of both operands, sizes,
+// epilogue and the tile-order group size.
 struct ProductOp {
   const void* lpl;
   const double* lsc;
@@ -71,8 +84,11 @@ struct ProductOp {
 };
 
 bool available();
-int64_t workspace_bytes(int64_t n_max, int ne_max, bool complex_, int slices);
-void create(Workspace& w, int64_t n_max, int ne_max, bool complex_, int slices);
+// Bytes of a workspace that holds the residue planes of A for a_mods moduli (0: the fewest it works with).
+int64_t workspace_bytes(int64_t n_max, int ne_max, bool complex_, int a_mods);
+// Moduli of A that `budget` bytes hold, between the fewest and all.
+int a_mods_within(int64_t n_max, bool complex_, int64_t budget);
+void create(Workspace& w, int64_t n_max, int ne_max, bool complex_, int a_mods);
 void destroy(Workspace& w);
 // the tuner's choices so far: (size-class key, candidate index) pairs, for reports
 std::vector<std::pair<uint64_t, int>> tuned(const Workspace& w);
@@ -81,22 +97,29 @@ void invalidate(Workspace& w);
 void timing_begin(Workspace& w);
 double timing_collect(Workspace& w, int* launches);
 int read_flags(cudaStream_t st, Workspace& w);
-// digit planes of the right operand B (n x k, ld ldb) into w's right-operand buffer, for the given mode
-template <typename T>
-void split_right(cudaStream_t st, Workspace& w, int mode, const T* B, int64_t ldb, int k, int64_t n);
-// one launch (per 64 products) over the tiles of all the products; w supplies the error flags and timing.
-// Every op's planes must have been split with the mode's slice count (left: at least that many slices).
-template <bool CPLX> void launch_group(cudaStream_t st, Workspace& w, int mode, const ProductOp* ops, int nops);
+// planes of A for the given mode (cached until invalidate)
 template <typename T>
 void prepare_A(cudaStream_t st, Workspace& w, const T* A, int64_t n, int64_t lda, int mode);
+// C = A B with epilogue (prepare_A first)
 template <typename T>
 void hemm(cudaStream_t st, Workspace& w, const T* A, int64_t n, int64_t lda, const T* B, int64_t ldb, int k,
           const Epi& e, int mode);
-// C = op(A) op(B) (M x N, inner K) through split products; op(A) = A (M x K) or A^H (A: K x M),
-// op(B) = B (K x N) or B^H (B: N x K).
+// C = op(A) op(B) (M x N, inner K), FP64 class; op(A) = A (M x K) or A^H (A: K x M), op(B) = B (K x N) or B^H
+// (B: N x K).  C may be A's storage.
 template <typename T>
 void gemm(cudaStream_t st, Workspace& w, Op opA, const T* A, int64_t lda, Op opB, const T* B, int64_t ldb, int64_t M,
-          int64_t N, int64_t K, const Epi& e, int mode);
+          int64_t N, int64_t K, const Epi& e);
+
+// Grouped launches over several problems' workspaces.  Mixed modes: digit planes of the right operand B
+// (n x k, ld ldb) into w's right-operand buffer, then one launch (per 64 products) over the tiles of all products.
+template <typename T>
+void split_right(cudaStream_t st, Workspace& w, int mode, const T* B, int64_t ldb, int k, int64_t n);
+template <bool CPLX> void launch_group(cudaStream_t st, Workspace& w, int mode, const ProductOp* ops, int nops);
+// FP64: whether w's next product C = A B of k columns can join a group; its operands; and the group's launches.
+bool groupable(const Workspace& w, int64_t n, int k);
+template <typename T>
+crt::Product group_product(cudaStream_t st, Workspace& w, const T* B, int64_t ldb, int k, int64_t n, const Epi& e);
+template <bool CPLX> void multiply_group(cudaStream_t st, Workspace& w, const crt::Product* ops, int nops);
 
 }  // namespace oz
 }  // namespace chase

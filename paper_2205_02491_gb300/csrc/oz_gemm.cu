@@ -1,14 +1,13 @@
-// Split-BF16 products, host side and digit planes: the per-row / per-column power-of-two scales and the
-// digit-plane split kernels of the operands, the workspace, the launch-configuration tuner, the K-split
-// planning and the dispatch of products (single, grouped) to the tcgen05 kernel of oz_kernel.cuh, whose
-// instantiations live in the oz_inst_*.cu units.  The digit arithmetic, the exact-level accumulation and
-// the kernel's roles are described in oz_kernel.cuh.
+// Split tensor-core products, host side: the workspace, the FP64-class products (residue planes, crt.cu) in passes
+// over A's moduli and panels of columns, and the mixed modes' digit planes, launch-configuration tuner, K-split
+// planning and dispatch to the tcgen05 kernel of oz_kernel.cuh, whose instantiations live in the oz_inst_*.cu units.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
 #include <mutex>
 
 #include "common.cuh"
+#include "crt.h"
 #include "oz.h"
 #include "oz_kernel.cuh"
 
@@ -84,66 +83,8 @@ __global__ void split_cols_kernel(int64_t K, int64_t Kpad, int ncols, const T* _
   }
 }
 
-// Per-row power-of-two scale of a column-major X (vector i = row i, K along columns).
-template <typename T>
-__global__ void row_scale_kernel(int64_t nvec, int64_t K, const T* __restrict__ X, int64_t ldx, double* scale) {
-  int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nvec) return;
-  double m = 0.0;
-  for (int64_t kk = 0; kk < K; ++kk) {
-    T v = X[i + kk * ldx];
-    m = fmax(m, fmax(fabs(S<T>::re(v)), fabs(S<T>::im(v))));
-  }
-  int e = 0;
-  if (m > 0.0 && isfinite(m)) frexp(m, &e);
-  scale[i] = m > 0.0 ? ldexp(1.0, e) : 1.0;
-}
-
-// Planes of the vectors i = rows of X (K along columns), via a 32x32 shared-memory transpose.
-template <typename T, int NS, int KIND>
-__global__ void split_rows_kernel(int64_t nvec, int64_t K, int64_t Kpad, const T* __restrict__ X, int64_t ldx,
-                                  const double* __restrict__ scale, int conj, __nv_bfloat16* planes) {
-  constexpr bool CPLX = S<T>::cplx;
-  __shared__ T tile[32][33];
-  const int64_t i0 = (int64_t)blockIdx.y * 32, k0 = (int64_t)blockIdx.x * 32;
-  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-    int64_t kk = k0 + r, i = i0 + threadIdx.x;
-    tile[r][threadIdx.x] = (kk < K && i < nvec) ? X[i + kk * ldx] : S<T>::zero();
-  }
-  __syncthreads();
-  for (int r = threadIdx.y; r < 32; r += blockDim.y) {
-    int64_t i = i0 + r, kk = k0 + threadIdx.x;
-    if (i >= nvec || kk >= K) continue;
-    T v = tile[threadIdx.x][r];
-    const double inv = 1.0 / scale[i];
-    double re = S<T>::re(v) * inv;
-    double im = (conj ? -S<T>::im(v) : S<T>::im(v)) * inv;
-    __nv_bfloat16 dr[NS], di[NS];
-    digits<NS>(re, dr);
-    if (CPLX) digits<NS>(im, di);
-#pragma unroll
-    for (int t = 0; t < NS; ++t) {
-      if (!CPLX) {
-        planes[((int64_t)t * nvec + i) * Kpad + kk] = dr[t];
-      } else if (KIND == 0) {
-        planes[((int64_t)(t * 2 + 0) * nvec + i) * Kpad + kk] = dr[t];
-        planes[((int64_t)(t * 2 + 1) * nvec + i) * Kpad + kk] = di[t];
-      } else {
-        planes[((int64_t)(t * 3 + 0) * nvec + i) * Kpad + kk] = __hneg(di[t]);
-        planes[((int64_t)(t * 3 + 1) * nvec + i) * Kpad + kk] = dr[t];
-        planes[((int64_t)(t * 3 + 2) * nvec + i) * Kpad + kk] = di[t];
-      }
-    }
-  }
-}
-
 // ---------------------------------------------------------------- host side
-static int slices_for(int mode, int fp64_slices) {
-  if (mode == 2) return 2;   // BF16x3
-  if (mode == 3) return 3;   // BF16x6
-  return fp64_slices;        // FP64
-}
-
+static int slices_for(int mode) { return mode == 2 ? 2 : MIXED_SLICES; }  // BF16x3, BF16x6
 
 bool available() {
   // thread-safe one-time probe (batched solves call this from several host threads)
@@ -157,43 +98,79 @@ bool available() {
   return ok;
 }
 
-static int64_t left_elems(int64_t n_max, int ne_max) {
-  return std::max<int64_t>(n_max * kpad(ne_max), (int64_t)ne_max * kpad(n_max));
+// ---------------------------------------------------------------- workspace
+// Residues of a product are kept for panels of its columns: at most this many bytes, but at least 256 columns.
+// 6 GB hold the n = 30000, 1600-column block (4 GB) whole.
+constexpr int64_t RESIDUE_PANEL_BYTES = 6ll << 30;
+
+// The fewest moduli of A's residue planes a workspace holds at a time: with the mixed modes' three digit slices
+// their memory is 24 bytes per complex element of A (16 for real); all 14 moduli take 84 more than those digits
+// (28 for real).
+static int fewest_mods(bool complex_) { return complex_ ? 2 : 4; }
+
+static int panel_cols(int64_t n_max, int ne_max, bool complex_) {
+  const int64_t per = crt::residue_bytes(n_max, 1, complex_);
+  const int64_t fit = RESIDUE_PANEL_BYTES / per / 256 * 256;
+  return (int)std::min<int64_t>(ne_max, std::max<int64_t>(256, fit));
 }
 
-int64_t workspace_bytes(int64_t n_max, int ne_max, bool complex_, int slices) {
-  int ap = complex_ ? 2 : 1, bp = complex_ ? 3 : 1;
-  int64_t kp = kpad(n_max);
-  int64_t a = (int64_t)slices * ap * n_max * kp * 2;
-  int64_t l = (int64_t)slices * ap * left_elems(n_max, ne_max) * 2;
-  int64_t b = (int64_t)slices * bp * ne_max * kp * 2;
-  return a + l + b + (2 * n_max + 2 * ne_max) * 8 + 64 + (8ll << 20) * 8;
+static int64_t left_bytes(int64_t n_max, int ne_max, bool complex_) {
+  return std::max(crt::plane_bytes(n_max, ne_max, complex_, crt::NMOD), crt::plane_bytes(ne_max, n_max, complex_, crt::NMOD));
 }
 
-void create(Workspace& w, int64_t n_max, int ne_max, bool complex_, int slices) {
+static int64_t right_bytes(int64_t n_max, int ne_max, bool complex_) {
+  const int64_t digits = (int64_t)MIXED_SLICES * (complex_ ? 3 : 1) * ne_max * kpad(n_max) * 2;
+  return std::max(digits, crt::plane_bytes(panel_cols(n_max, ne_max, complex_), n_max, complex_, crt::NMOD));
+}
+
+static int64_t digit_bytes(int64_t n_max, bool complex_) {
+  return (int64_t)MIXED_SLICES * (complex_ ? 2 : 1) * n_max * kpad(n_max) * 2;
+}
+
+// partial sums of K-split mixed products: up to about 4 waves of 128 x 64 complex tiles
+constexpr int64_t PARTIAL_ELEMS = 8ll << 20;
+
+int a_mods_within(int64_t n_max, bool complex_, int64_t budget) {
+  const int64_t fit = budget / crt::plane_bytes(n_max, n_max, complex_, 1);
+  return (int)std::max<int64_t>(fewest_mods(complex_), std::min<int64_t>(fit, crt::NMOD));
+}
+
+int64_t workspace_bytes(int64_t n_max, int ne_max, bool complex_, int a_mods) {
+  if (a_mods == 0) a_mods = fewest_mods(complex_);
+  return crt::plane_bytes(n_max, n_max, complex_, a_mods) + left_bytes(n_max, ne_max, complex_) +
+         right_bytes(n_max, ne_max, complex_) +
+         crt::residue_bytes(n_max, panel_cols(n_max, ne_max, complex_), complex_) + digit_bytes(n_max, complex_) +
+         (2 * n_max + 2 * (int64_t)ne_max) * 8 + 64 + PARTIAL_ELEMS * 8;
+}
+
+void create(Workspace& w, int64_t n_max, int ne_max, bool complex_, int a_mods) {
   w.n_max = n_max;
   w.ne_max = ne_max;
   w.complex_ = complex_;
-  w.slices = slices;
   if (!available()) return;
-  int ap = complex_ ? 2 : 1, bp = complex_ ? 3 : 1;
-  int64_t kp = kpad(n_max);
-  CHASE_CUDA(cudaMalloc(&w.a_planes, (size_t)slices * ap * n_max * kp * 2));
-  CHASE_CUDA(cudaMalloc(&w.l_planes, (size_t)slices * ap * left_elems(n_max, ne_max) * 2));
-  CHASE_CUDA(cudaMalloc(&w.b_planes, (size_t)slices * bp * ne_max * kp * 2));
+  w.a_mods = a_mods;
+  w.b_bytes = right_bytes(n_max, ne_max, complex_);
+  w.residue_bytes = crt::residue_bytes(n_max, panel_cols(n_max, ne_max, complex_), complex_);
+  CHASE_CUDA(cudaMalloc(&w.a_res, crt::plane_bytes(n_max, n_max, complex_, a_mods)));
+  CHASE_CUDA(cudaMalloc(&w.l_res, left_bytes(n_max, ne_max, complex_)));
+  CHASE_CUDA(cudaMalloc(&w.b_planes, w.b_bytes));
+  CHASE_CUDA(cudaMalloc(&w.residue, w.residue_bytes));
+  CHASE_CUDA(cudaMalloc(&w.a_planes, digit_bytes(n_max, complex_)));
+  CHASE_CUDA(cudaMalloc(&w.a_ex, n_max * sizeof(int)));
+  CHASE_CUDA(cudaMalloc(&w.l_ex, std::max<int64_t>(n_max, ne_max) * sizeof(int)));
+  CHASE_CUDA(cudaMalloc(&w.b_ex, std::max<int64_t>(n_max, ne_max) * sizeof(int)));
   CHASE_CUDA(cudaMalloc(&w.a_scale, n_max * sizeof(double)));
-  CHASE_CUDA(cudaMalloc(&w.l_scale, std::max<int64_t>(n_max, ne_max) * sizeof(double)));
   CHASE_CUDA(cudaMalloc(&w.b_scale, ne_max * sizeof(double)));
   CHASE_CUDA(cudaMalloc(&w.flags, 16 * sizeof(int)));
   CHASE_CUDA(cudaMemset(w.flags, 0, 16 * sizeof(int)));
-  // partial sums of K-split products: up to about 4 waves of 128 x 40 complex tiles
-  w.partial_elems = 8ll << 20;
+  w.partial_elems = PARTIAL_ELEMS;
   CHASE_CUDA(cudaMalloc(&w.partial, (size_t)w.partial_elems * sizeof(double)));
   w.ready = true;
 }
 
 void destroy(Workspace& w) {
-  void* ps[] = {w.a_planes, w.l_planes, w.b_planes, w.a_scale, w.l_scale, w.b_scale, w.flags, w.partial};
+  void* ps[] = {w.a_res,   w.l_res,   w.b_planes, w.residue, w.a_planes, w.a_ex,
+                w.l_ex,    w.b_ex,    w.a_scale,  w.b_scale, w.flags,    w.partial};
   for (void* p : ps)
     if (p) cudaFree(p);
   for (auto& e : w.ev) cudaEventDestroy(e);
@@ -203,59 +180,41 @@ void destroy(Workspace& w) {
   w = Workspace{};
 }
 
-// Split nvec vectors of length K taken from a column-major X: by columns (vector = column,
-// optionally conjugated) or by rows (vector = row).  kind 0: left-operand planes (re, im);
-// kind 1: right-operand planes (-im, re, im).
+// Digit planes of nvec columns of length K of a column-major X (optionally conjugated).
+// kind 0: left-operand planes (re, im); kind 1: right-operand planes (-im, re, im).
 template <typename T>
-static void split(cudaStream_t st, int S_, int kind, bool by_rows, bool conj, const T* X, int64_t ld, int64_t nvec,
-                  int64_t K, void* planes, double* scale) {
+static void split(cudaStream_t st, int S_, int kind, bool conj, const T* X, int64_t ld, int64_t nvec, int64_t K,
+                  void* planes, double* scale) {
   const int64_t kp = kpad(K);
-  if (!by_rows) {
-    col_scale_kernel<T><<<(unsigned)nvec, 256, 0, st>>>(K, X, ld, scale);
-    CHASE_CHECK_LAUNCH();
-    dim3 grid(std::min<unsigned>(ceil_div(K, 256), 32), (unsigned)nvec);
+  col_scale_kernel<T><<<(unsigned)nvec, 256, 0, st>>>(K, X, ld, scale);
+  CHASE_CHECK_LAUNCH();
+  dim3 grid(std::min<unsigned>(ceil_div(K, 256), 32), (unsigned)nvec);
 #define SC(SS, KD) split_cols_kernel<T, SS, KD><<<grid, 256, 0, st>>>(K, kp, (int)nvec, X, ld, scale, conj ? 1 : 0, (__nv_bfloat16*)planes)
-#define SWK(SS) if (kind == 0) SC(SS, 0); else SC(SS, 1);
-    switch (S_) {
-      case 2: SWK(2); break;
-      case 3: SWK(3); break;
-      case 6: SWK(6); break;
-      case 7: SWK(7); break;
-      default: CHASE_REQUIRE(false, 1, "unsupported slice count");
-    }
-#undef SWK
+  if (S_ == 2 && kind == 1) SC(2, 1);
+  else if (S_ == 3 && kind == 1) SC(3, 1);
+  else if (S_ == 3 && kind == 0) SC(3, 0);
+  else CHASE_REQUIRE(false, 1, "unsupported slice count");
 #undef SC
-  } else {
-    row_scale_kernel<T><<<ceil_div(nvec, 128), 128, 0, st>>>(nvec, K, X, ld, scale);
-    CHASE_CHECK_LAUNCH();
-    dim3 grid(ceil_div(K, 32), ceil_div(nvec, 32));
-    CHASE_REQUIRE(grid.y <= 65535, 1, "split: too many vectors");
-#define SR(SS, KD) split_rows_kernel<T, SS, KD><<<grid, dim3(32, 8), 0, st>>>(nvec, K, kp, X, ld, scale, conj ? 1 : 0, (__nv_bfloat16*)planes)
-#define SWK(SS) if (kind == 0) SR(SS, 0); else SR(SS, 1);
-    switch (S_) {
-      case 2: SWK(2); break;
-      case 3: SWK(3); break;
-      case 6: SWK(6); break;
-      case 7: SWK(7); break;
-      default: CHASE_REQUIRE(false, 1, "unsupported slice count");
-    }
-#undef SWK
-#undef SR
-  }
   CHASE_CHECK_LAUNCH();
 }
 
 template <typename T>
 void prepare_A(cudaStream_t st, Workspace& w, const T* A, int64_t n, int64_t lda, int mode) {
   CHASE_REQUIRE(w.ready, 9, "split products not initialised");
-  // planes of all slices are nested: the S-slice split's first slices are the 2- and 3-slice splits
-  if (w.a_src == (const void*)A && w.a_n == n && w.a_mode == w.slices) return;
-  (void)mode;
   // A Hermitian: K-major row i of A = conjugate of column i of its column-major storage
-  split<T>(st, w.slices, 0, false, true, A, lda, n, n, w.a_planes, w.a_scale);
+  if (mode == 2 || mode == 3) {
+    // the three-slice split's first slices are the two-slice split
+    if (w.d_src == (const void*)A && w.d_n == n) return;
+    split<T>(st, MIXED_SLICES, 0, true, A, lda, n, n, w.a_planes, w.a_scale);
+    w.d_src = A;
+    w.d_n = n;
+    return;
+  }
+  if (w.a_src == (const void*)A && w.a_n == n) return;
+  crt::scales<T>(st, false, n, n, A, lda, w.a_ex);
+  if (w.a_mods == crt::NMOD) crt::residues<T>(st, false, true, n, n, A, lda, w.a_ex, 0, crt::NMOD, w.a_res);
   w.a_src = A;
   w.a_n = n;
-  w.a_mode = w.slices;
 }
 
 void timing_begin(Workspace& w) {
@@ -282,20 +241,71 @@ double timing_collect(Workspace& w, int* launches) {
 }
 
 void invalidate(Workspace& w) {
-  w.a_src = nullptr;
-  w.a_n = 0;
-  w.a_mode = -1;
+  w.a_src = w.d_src = nullptr;
+  w.a_n = w.d_n = 0;
   if (w.flags) CHASE_CUDA(cudaMemset(w.flags, 0, 16 * sizeof(int)));  // a new call starts clean
 }
 
-// C(M x N) = L(M x K) R(K x N) from digit planes (left: rows = M vectors of length K, right:
-// rows = N vectors of length K), split with l_slices_total / S slices respectively.
+// ---------------------------------------------------------------- FP64-class products
+// event pair around one product's kernels (filter roofline)
+struct ProductTimer {
+  cudaStream_t st;
+  Workspace& w;
+  bool on;
+  ProductTimer(cudaStream_t s, Workspace& ws) : st(s), w(ws), on(ws.timing && ws.ev_used + 2 <= (int)ws.ev.size()) {
+    if (on) CHASE_CUDA(cudaEventRecord(w.ev[w.ev_used], st));
+  }
+  void stop() {
+    if (!on) return;
+    CHASE_CUDA(cudaEventRecord(w.ev[w.ev_used + 1], st));
+    w.ev_used += 2;
+  }
+};
+
+// columns of a product (M rows, inner length K) whose right planes and residues fit the workspace
+static int64_t panel_fit(const Workspace& w, int64_t M, int64_t K) {
+  const int64_t by_res = w.residue_bytes / crt::residue_bytes(M, 1, w.complex_);
+  const int64_t by_rhs = w.b_bytes / crt::plane_bytes(1, K, w.complex_, crt::NMOD);
+  return std::min(by_res, by_rhs);
+}
+
+static Epi at_column(const Epi& e, int64_t j, size_t esz) {
+  Epi o = e;
+  o.C = (char*)e.C + (size_t)(j * e.ldc) * esz;
+  if (e.Y) o.Y = (const char*)e.Y + (size_t)(j * e.ldy) * esz;
+  if (e.Z) o.Z = (const char*)e.Z + (size_t)(j * e.ldz) * esz;
+  if (e.ycol) o.ycol = e.ycol + j;
+  return o;
+}
+
+// C = L R by panels of columns.  lconv(mod0, nmod): makes the left planes of those moduli current (called for passes
+// of `mods` moduli); the right operand's columns (rows when by_rows) are converted per panel.
+template <typename T, typename LeftConv>
+static void product(cudaStream_t st, Workspace& w, const void* lpl, const int* lex, int mods, LeftConv lconv, bool by_rows,
+                    const T* B, int64_t ldb, int64_t M, int64_t N, int64_t K, const Epi& e) {
+  const int64_t fit = panel_fit(w, M, K);
+  CHASE_REQUIRE(fit >= 1, 1, "split product exceeds the workspace");
+  for (int64_t j = 0; j < N; j += fit) {
+    const int64_t nc = std::min(fit, N - j);
+    const T* Bj = by_rows ? B + j : B + j * ldb;
+    crt::scales<T>(st, by_rows, nc, K, Bj, ldb, w.b_ex);
+    crt::residues<T>(st, by_rows, by_rows, nc, K, Bj, ldb, w.b_ex, 0, crt::NMOD, w.b_planes);
+    const crt::Product op{lpl, lex, w.b_planes, w.b_ex, w.residue, M, nc, K, at_column(e, j, sizeof(T))};
+    ProductTimer t(st, w);
+    for (int m0 = 0; m0 < crt::NMOD; m0 += mods) {
+      const int nm = std::min(mods, crt::NMOD - m0);
+      lconv(m0, nm);
+      crt::multiply<S<T>::cplx>(st, &op, 1, m0, nm, w.flags);
+    }
+    crt::combine<S<T>::cplx>(st, op);
+    t.stop();
+  }
+}
+
 // ---------------------------------------------------------------- launch-configuration tuner
-// Candidates per arithmetic: the FP64 kernels (NT fixed at 80 by TMEM) try the tile-order group sizes;
-// the mixed kernels (one accumulator) also try the 256-column tile, which halves the instructions per
-// unit of tensor work.
-static const LaunchCfg kCandFP64[] = {{0, 2}, {0, 4}, {0, 8}, {0, 16}, {0, 32}};
-static const LaunchCfg kCandMixed[] = {{128, 4}, {128, 16}, {256, 4}, {256, 16}};
+// Candidates of the mixed kernels: the tile-order group size and the tile width (256 columns halve the instructions
+// per unit of tensor work).
+static const LaunchCfg kCand[] = {{128, 4}, {128, 16}, {256, 4}, {256, 16}};
 
 static int log2_bucket(int64_t x) {
   int b = 0;
@@ -315,15 +325,11 @@ static uint64_t tune_key(int S_, bool cplx, bool grouped, int64_t M, int64_t N, 
 // The configuration for the next launch of a size class.  Until every candidate has been timed, each
 // launch takes the next candidate and gets an event pair (*ev_out); the first launch after that reads
 // the times (one event synchronisation per size class and context) and keeps the fastest.
-static LaunchCfg tune_pick(Workspace& w, uint64_t key, bool mixed, cudaEvent_t** ev_out) {
-  const LaunchCfg* cand = mixed ? kCandMixed : kCandFP64;
-  const int nc = mixed ? (int)(sizeof(kCandMixed) / sizeof(kCandMixed[0]))
-                       : (int)(sizeof(kCandFP64) / sizeof(kCandFP64[0]));
+static LaunchCfg tune_pick(Workspace& w, uint64_t key, cudaEvent_t** ev_out) {
+  const LaunchCfg* cand = kCand;
+  const int nc = (int)(sizeof(kCand) / sizeof(kCand[0]));
   *ev_out = nullptr;
-  if (!w.autotune) {
-    LaunchCfg d = mixed ? LaunchCfg{128, w.group_m} : LaunchCfg{0, w.group_m};
-    return d;
-  }
+  if (!w.autotune) return LaunchCfg{128, w.group_m};
   TuneEntry& t = w.tune[key];
   if (t.best >= 0) return cand[t.best];
   if (t.ev.empty()) {
@@ -386,100 +392,102 @@ static void plan_ksplit(Workspace& w, ProductOp& op, int ncols_tile, bool cplx) 
   }
 }
 
-template <int S, int NEX, bool CPLX, int NTT>
-static void launch(cudaStream_t st, Workspace& w, const void* lpl, const double* lsc, int l_slices_total,
-                   const void* rpl, const double* rsc, int64_t M, int64_t N, int64_t K, const Epi& e,
-                   int group_m, cudaEvent_t* tune_ev) {
-  ProductOp op{lpl, lsc, l_slices_total, rpl, rsc, M, N, K, e, group_m};
-  plan_ksplit(w, op, Cfg<S, NEX, CPLX, NTT>::NCOLS, CPLX);
-  launch_ops<S, NEX, CPLX, NTT, 1>(st, w, &op, 1, tune_ev);
-}
-
-template <bool CPLX>
-static void dispatch(cudaStream_t st, Workspace& w, int S_, const void* lpl, const double* lsc, int l_slices_total,
-                     int64_t M, int64_t N, int64_t K, const Epi& e) {
-  CHASE_REQUIRE(K <= 65472, 1, "split products support K <= 65472 (int64 exact-level sums)");
-  // a narrow right operand (up to 8 complex or 16 real columns: the Lanczos block) takes the N = 16 tile, so
-  // the launch streams the left planes once without computing unused accumulator columns
-  const bool narrow = N <= (CPLX ? 8 : 16);
-  const void* rp = w.b_planes;
-  const double* rs = w.b_scale;
-  if (narrow && S_ >= 6) {
-    // one column tile: the tile order is irrelevant
-    if (S_ == 7) launch<7, 5, CPLX, 16>(st, w, lpl, lsc, l_slices_total, rp, rs, M, N, K, e, 1, nullptr);
-    else launch<6, 5, CPLX, 16>(st, w, lpl, lsc, l_slices_total, rp, rs, M, N, K, e, 1, nullptr);
-    return;
-  }
-  cudaEvent_t* ev = nullptr;
-  const LaunchCfg cfg = tune_pick(w, tune_key(S_, CPLX, false, M, N, K), S_ <= 3, &ev);
-  if (S_ == 7) launch<7, 5, CPLX, 80>(st, w, lpl, lsc, l_slices_total, rp, rs, M, N, K, e, cfg.group_m, ev);
-  else if (S_ == 6) launch<6, 5, CPLX, 80>(st, w, lpl, lsc, l_slices_total, rp, rs, M, N, K, e, cfg.group_m, ev);
-  else if (S_ == 3 && cfg.nt == 256) launch<3, 0, CPLX, 256>(st, w, lpl, lsc, l_slices_total, rp, rs, M, N, K, e, cfg.group_m, ev);
-  else if (S_ == 3) launch<3, 0, CPLX, 128>(st, w, lpl, lsc, l_slices_total, rp, rs, M, N, K, e, cfg.group_m, ev);
-  else if (cfg.nt == 256) launch<2, 0, CPLX, 256>(st, w, lpl, lsc, l_slices_total, rp, rs, M, N, K, e, cfg.group_m, ev);
-  else launch<2, 0, CPLX, 128>(st, w, lpl, lsc, l_slices_total, rp, rs, M, N, K, e, cfg.group_m, ev);
+template <int S, bool CPLX, int NTT>
+static void launch(cudaStream_t st, Workspace& w, int64_t M, int64_t N, int64_t K, const Epi& e, int group_m,
+                   cudaEvent_t* tune_ev) {
+  ProductOp op{w.a_planes, w.a_scale, MIXED_SLICES, w.b_planes, w.b_scale, M, N, K, e, group_m};
+  plan_ksplit(w, op, Cfg<S, CPLX, NTT>::NCOLS, CPLX);
+  launch_ops<S, CPLX, NTT, 1>(st, w, &op, 1, tune_ev);
 }
 
 template <typename T>
 void split_right(cudaStream_t st, Workspace& w, int mode, const T* B, int64_t ldb, int k, int64_t n) {
   CHASE_REQUIRE(w.ready, 9, "split products not initialised");
   CHASE_REQUIRE(k <= w.ne_max && n <= w.n_max, 1, "split_right: size exceeds the workspace");
-  split<T>(st, slices_for(mode, w.slices), 1, false, false, B, ldb, k, n, w.b_planes, w.b_scale);
+  split<T>(st, slices_for(mode), 1, false, B, ldb, k, n, w.b_planes, w.b_scale);
 }
 
 template <bool CPLX>
 void launch_group(cudaStream_t st, Workspace& w, int mode, const ProductOp* ops, int nops) {
   constexpr int G = 64;
-  const int S_ = slices_for(mode, w.slices);
+  const int S_ = slices_for(mode);
   std::vector<ProductOp> chunk;
   for (int q0 = 0; q0 < nops; q0 += G) {
     const int cnt = std::min(G, nops - q0);
     // size class of a grouped launch: its total work in row blocks x columns x K
     int64_t rows = 0, cols = 0, kk = 0;
     for (int q = q0; q < q0 + cnt; ++q) {
-      CHASE_REQUIRE(ops[q].K <= 65472, 1, "split products support K <= 65472 (int64 exact-level sums)");
       rows += ops[q].M;
       cols = std::max(cols, ops[q].N);
       kk = std::max(kk, ops[q].K);
     }
     cudaEvent_t* ev = nullptr;
-    const LaunchCfg cfg = tune_pick(w, tune_key(S_, CPLX, true, rows, cols, kk), S_ <= 3, &ev);
+    const LaunchCfg cfg = tune_pick(w, tune_key(S_, CPLX, true, rows, cols, kk), &ev);
     chunk.assign(ops + q0, ops + q0 + cnt);
     for (auto& o : chunk) o.group_m = cfg.group_m;
     const ProductOp* cp = chunk.data();
-    if (S_ == 7) launch_ops<7, 5, CPLX, 80, G>(st, w, cp, cnt, ev);
-    else if (S_ == 6) launch_ops<6, 5, CPLX, 80, G>(st, w, cp, cnt, ev);
-    else if (S_ == 3 && cfg.nt == 256) launch_ops<3, 0, CPLX, 256, G>(st, w, cp, cnt, ev);
-    else if (S_ == 3) launch_ops<3, 0, CPLX, 128, G>(st, w, cp, cnt, ev);
-    else if (cfg.nt == 256) launch_ops<2, 0, CPLX, 256, G>(st, w, cp, cnt, ev);
-    else launch_ops<2, 0, CPLX, 128, G>(st, w, cp, cnt, ev);
+    if (S_ == 3 && cfg.nt == 256) launch_ops<3, CPLX, 256, G>(st, w, cp, cnt, ev);
+    else if (S_ == 3) launch_ops<3, CPLX, 128, G>(st, w, cp, cnt, ev);
+    else if (cfg.nt == 256) launch_ops<2, CPLX, 256, G>(st, w, cp, cnt, ev);
+    else launch_ops<2, CPLX, 128, G>(st, w, cp, cnt, ev);
   }
+}
+
+bool groupable(const Workspace& w, int64_t n, int k) { return w.a_mods == crt::NMOD && k <= panel_fit(w, n, n); }
+
+template <typename T>
+crt::Product group_product(cudaStream_t st, Workspace& w, const T* B, int64_t ldb, int k, int64_t n, const Epi& e) {
+  CHASE_REQUIRE(w.ready, 9, "split products not initialised");
+  crt::scales<T>(st, false, k, n, B, ldb, w.b_ex);
+  crt::residues<T>(st, false, false, k, n, B, ldb, w.b_ex, 0, crt::NMOD, w.b_planes);
+  return crt::Product{w.a_res, w.a_ex, w.b_planes, w.b_ex, w.residue, n, k, n, e};
+}
+
+template <bool CPLX> void multiply_group(cudaStream_t st, Workspace& w, const crt::Product* ops, int nops) {
+  crt::multiply<CPLX>(st, ops, nops, 0, crt::NMOD, w.flags);
+  for (int q = 0; q < nops; ++q) crt::combine<CPLX>(st, ops[q]);
 }
 
 template <typename T>
 void hemm(cudaStream_t st, Workspace& w, const T* A, int64_t n, int64_t lda, const T* B, int64_t ldb, int k,
           const Epi& e, int mode) {
+  constexpr bool CPLX = S<T>::cplx;
   CHASE_REQUIRE(w.ready, 9, "split products not initialised");
-  CHASE_REQUIRE(w.a_src == (const void*)A && w.a_n == n, 7, "prepare_A must precede hemm");
   CHASE_REQUIRE(k <= w.ne_max && n <= w.n_max, 1, "hemm size exceeds the workspace");
-  const int S_ = slices_for(mode, w.slices);
-  split<T>(st, S_, 1, false, false, B, ldb, k, n, w.b_planes, w.b_scale);
-  dispatch<S<T>::cplx>(st, w, S_, w.a_planes, w.a_scale, w.slices, n, k, n, e);
+  CHASE_REQUIRE(n <= 65472, 1, "split products support K <= 65472");
+  if (mode != 2 && mode != 3) {
+    CHASE_REQUIRE(w.a_src == (const void*)A && w.a_n == n, 7, "prepare_A must precede hemm");
+    auto conv = [&](int m0, int nm) {
+      if (w.a_mods < crt::NMOD) crt::residues<T>(st, false, true, n, n, A, lda, w.a_ex, m0, nm, w.a_res);
+    };
+    product<T>(st, w, w.a_res, w.a_ex, w.a_mods, conv, false, B, ldb, n, k, n, e);
+    return;
+  }
+  CHASE_REQUIRE(w.d_src == (const void*)A && w.d_n == n, 7, "prepare_A must precede hemm");
+  const int S_ = slices_for(mode);
+  split<T>(st, S_, 1, false, B, ldb, k, n, w.b_planes, w.b_scale);
+  cudaEvent_t* ev = nullptr;
+  const LaunchCfg cfg = tune_pick(w, tune_key(S_, CPLX, false, n, k, n), &ev);
+  if (S_ == 3 && cfg.nt == 256) launch<3, CPLX, 256>(st, w, n, k, n, e, cfg.group_m, ev);
+  else if (S_ == 3) launch<3, CPLX, 128>(st, w, n, k, n, e, cfg.group_m, ev);
+  else if (cfg.nt == 256) launch<2, CPLX, 256>(st, w, n, k, n, e, cfg.group_m, ev);
+  else launch<2, CPLX, 128>(st, w, n, k, n, e, cfg.group_m, ev);
 }
 
 template <typename T>
 void gemm(cudaStream_t st, Workspace& w, Op opA, const T* A, int64_t lda, Op opB, const T* B, int64_t ldb, int64_t M,
-          int64_t N, int64_t K, const Epi& e, int mode) {
+          int64_t N, int64_t K, const Epi& e) {
+  constexpr bool CPLX = S<T>::cplx;
   CHASE_REQUIRE(w.ready, 9, "split products not initialised");
   if (M <= 0 || N <= 0) return;
-  CHASE_REQUIRE(N <= w.ne_max && M * kpad(K) <= left_elems(w.n_max, w.ne_max) && N * kpad(K) <= (int64_t)w.ne_max * kpad(w.n_max),
+  CHASE_REQUIRE(N <= w.ne_max && M <= std::max<int64_t>(w.n_max, w.ne_max) &&
+                    crt::plane_bytes(M, K, CPLX, crt::NMOD) <= left_bytes(w.n_max, w.ne_max, CPLX),
                 1, "split product exceeds the workspace");
-  const int S_ = slices_for(mode, w.slices);
-  // left operand: OP_N rows of A (M x K), OP_C conjugated columns of A (K x M)
-  split<T>(st, S_, 0, opA == OP_N, opA == OP_C, A, lda, M, K, w.l_planes, w.l_scale);
-  // right operand: OP_N columns of B (K x N), OP_C conjugated rows of B (N x K)
-  split<T>(st, S_, 1, opB == OP_C, opB == OP_C, B, ldb, N, K, w.b_planes, w.b_scale);
-  dispatch<S<T>::cplx>(st, w, S_, w.l_planes, w.l_scale, S_, M, N, K, e);
+  // left operand: OP_N rows of A (M x K), OP_C conjugated columns of A (K x M); right operand: OP_N columns of B
+  // (K x N), OP_C conjugated rows of B (N x K).  The left planes of all moduli are made first, so C may overwrite A.
+  crt::scales<T>(st, opA == OP_N, M, K, A, lda, w.l_ex);
+  crt::residues<T>(st, opA == OP_N, opA == OP_C, M, K, A, lda, w.l_ex, 0, crt::NMOD, w.l_res);
+  product<T>(st, w, w.l_res, w.l_ex, crt::NMOD, [](int, int) {}, opB == OP_C, B, ldb, M, N, K, e);
 }
 
 int read_flags(cudaStream_t st, Workspace& w) {
@@ -495,9 +503,13 @@ template void prepare_A<double2>(cudaStream_t, Workspace&, const double2*, int64
 template void hemm<double>(cudaStream_t, Workspace&, const double*, int64_t, int64_t, const double*, int64_t, int,
                            const Epi&, int);
 template void gemm<double>(cudaStream_t, Workspace&, Op, const double*, int64_t, Op, const double*, int64_t, int64_t,
-                           int64_t, int64_t, const Epi&, int);
+                           int64_t, int64_t, const Epi&);
 template void gemm<double2>(cudaStream_t, Workspace&, Op, const double2*, int64_t, Op, const double2*, int64_t, int64_t,
-                            int64_t, int64_t, const Epi&, int);
+                            int64_t, int64_t, const Epi&);
+template crt::Product group_product<double>(cudaStream_t, Workspace&, const double*, int64_t, int, int64_t, const Epi&);
+template crt::Product group_product<double2>(cudaStream_t, Workspace&, const double2*, int64_t, int, int64_t, const Epi&);
+template void multiply_group<false>(cudaStream_t, Workspace&, const crt::Product*, int);
+template void multiply_group<true>(cudaStream_t, Workspace&, const crt::Product*, int);
 template void hemm<double2>(cudaStream_t, Workspace&, const double2*, int64_t, int64_t, const double2*, int64_t, int,
                             const Epi&, int);
 template void split_right<double>(cudaStream_t, Workspace&, int, const double*, int64_t, int, int64_t);

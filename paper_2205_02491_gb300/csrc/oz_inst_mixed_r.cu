@@ -5,14 +5,14 @@
 namespace chase {
 namespace oz {
 
-template void launch_ops<3, 0, false, 256, 1>(cudaStream_t, Workspace&, const ProductOp*, int, cudaEvent_t*);
-template void launch_ops<3, 0, false, 128, 1>(cudaStream_t, Workspace&, const ProductOp*, int, cudaEvent_t*);
-template void launch_ops<3, 0, false, 256, 64>(cudaStream_t, Workspace&, const ProductOp*, int, cudaEvent_t*);
-template void launch_ops<3, 0, false, 128, 64>(cudaStream_t, Workspace&, const ProductOp*, int, cudaEvent_t*);
-template void launch_ops<2, 0, false, 256, 1>(cudaStream_t, Workspace&, const ProductOp*, int, cudaEvent_t*);
-template void launch_ops<2, 0, false, 128, 1>(cudaStream_t, Workspace&, const ProductOp*, int, cudaEvent_t*);
-template void launch_ops<2, 0, false, 256, 64>(cudaStream_t, Workspace&, const ProductOp*, int, cudaEvent_t*);
-template void launch_ops<2, 0, false, 128, 64>(cudaStream_t, Workspace&, const ProductOp*, int, cudaEvent_t*);
+template void launch_ops<3, false, 256, 1>(cudaStream_t, Workspace&, const ProductOp*, int, cudaEvent_t*);
+template void launch_ops<3, false, 128, 1>(cudaStream_t, Workspace&, const ProductOp*, int, cudaEvent_t*);
+template void launch_ops<3, false, 256, 64>(cudaStream_t, Workspace&, const ProductOp*, int, cudaEvent_t*);
+template void launch_ops<3, false, 128, 64>(cudaStream_t, Workspace&, const ProductOp*, int, cudaEvent_t*);
+template void launch_ops<2, false, 256, 1>(cudaStream_t, Workspace&, const ProductOp*, int, cudaEvent_t*);
+template void launch_ops<2, false, 128, 1>(cudaStream_t, Workspace&, const ProductOp*, int, cudaEvent_t*);
+template void launch_ops<2, false, 256, 64>(cudaStream_t, Workspace&, const ProductOp*, int, cudaEvent_t*);
+template void launch_ops<2, false, 128, 64>(cudaStream_t, Workspace&, const ProductOp*, int, cudaEvent_t*);
 
 }  // namespace oz
 }  // namespace chase
