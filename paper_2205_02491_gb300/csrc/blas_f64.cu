@@ -6,6 +6,8 @@
 // reference path of the Chebyshev filter product.  On GB300 FP64 runs on the
 // CUDA cores only (about 1.2 TFLOP/s), so the large products of the
 // production path go through the split-BF16 tensor-core kernels instead.
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.h"
 

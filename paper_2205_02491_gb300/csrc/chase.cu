@@ -863,18 +863,7 @@ template <typename T> struct Solver {
     // Lanczos (line 2)
     {
       Timer t(c, 1, &S.ms_lanczos);
-      // large problems: the Lanczos matvecs use the FP64-class split tensor-core product (the digit
-      // planes of A are then reused by the filter); small ones and the native mode use DFMA
-      MatvecFn<T> mv = [&](const T* X, int64_t ldx, T* Wout) {
-        Epi e;
-        e.C = Wout;
-        e.ldc = n;
-        hemm(A, n, lda, X, ldx, runs, e, CHASE_FP64);
-      };
-      const bool lz_split = runs <= c->ne_max && use_split(mode == CHASE_FP64_NATIVE ? CHASE_FP64_NATIVE : CHASE_FP64,
-                                                           n, runs, n);
-      lanczos<T>(st(), A, n, lda, ne, L0, runs, steps, c->dwork, W(), c->work_elems, c->dwork + 8,
-                 lz_split ? &mv : nullptr);
+      lanczos<T>(st(), A, n, lda, ne, L0, runs, steps, c->dwork, W(), c->work_elems, c->dwork + 8);
       init_bounds_kernel<<<1, 1, 0, st()>>>(c->dwork, c->bounds);
       CHASE_CHECK_LAUNCH();
       t.stop();
@@ -1135,16 +1124,12 @@ void chase_default_opts(chase_opts* o) {
   o->batch_grouped = 1;
 }
 
-static int64_t lanczos_elems(int64_t n, int runs, int steps) {
-  int64_t nchunk = (n + 255) / 256;
-  int64_t part = std::max<int64_t>(nchunk * runs * n, (int64_t)runs * 64 * 64);
-  return (int64_t)runs * steps * n + runs * n + part + 2 * runs * 64;
-}
-
-static int64_t work_elems_for(int64_t n, int ne, const chase_opts& o) {
+static int64_t work_elems_for(int64_t n, int ne, bool cplx, const chase_opts& o) {
   // FP64 Jacobi: ne^2 + 3 ne + 8 scalars; FP32 first pass: 3 ne^2 + 3 ne + 8 half-size scalars
   int64_t jac = 2 * (int64_t)ne * ne + 3 * (int64_t)ne + 16;
-  int64_t lz = lanczos_elems(n, o.lanczos_runs, std::min<int>(o.lanczos_steps, (int)n));
+  // the context's own Lanczos settings, and any settings chase_lanczos takes for small n
+  int64_t lz = std::max(lanczos_work_elems(n, o.lanczos_runs, std::min<int>(o.lanczos_steps, (int)n), cplx),
+                        lanczos_work_elems(std::min<int64_t>(n, 4096), 8, 64, cplx));
   int64_t split = 2 * 1024 * 1024;
   return std::max(std::max(jac, lz), split);
 }
@@ -1154,7 +1139,7 @@ int64_t chase_workspace_bytes(int64_t n_max, int ne_max, chase_dtype dtype, cons
   chase_default_opts(&o);
   if (opts) o = *opts;
   int64_t esz = dtype == CHASE_C128 ? 16 : 8;
-  int64_t b = 3 * n_max * ne_max * esz + 2 * (int64_t)ne_max * ne_max * esz + work_elems_for(n_max, ne_max, o) * esz;
+  int64_t b = 3 * n_max * ne_max * esz + 3 * (int64_t)ne_max * ne_max * esz + work_elems_for(n_max, ne_max, dtype == CHASE_C128, o) * esz;
   b += (3 * 32 * (int64_t)ne_max + ne_max + 1024) * esz;  // Householder QR scratch
   b += oz::workspace_bytes(n_max, ne_max, dtype == CHASE_C128, 0);
   return b;
@@ -1203,9 +1188,9 @@ static chase_status create_ctx(chase_ctx** out, int64_t n_max, int ne_max, chase
     CHASE_CUDA(cudaMalloc(&c->V, blk));
     CHASE_CUDA(cudaMalloc(&c->T1, blk));
     CHASE_CUDA(cudaMalloc(&c->T2, blk));
-    CHASE_CUDA(cudaMalloc(&c->G, (size_t)ne_max * ne_max * c->esz));
+    CHASE_CUDA(cudaMalloc(&c->G, 2 * (size_t)ne_max * ne_max * c->esz));  // [G; I] of the Cholesky factorisations
     CHASE_CUDA(cudaMalloc(&c->Z, (size_t)ne_max * ne_max * c->esz));
-    c->work_elems = work_elems_for(n_max, ne_max, c->opts);
+    c->work_elems = work_elems_for(n_max, ne_max, dtype == CHASE_C128, c->opts);
     CHASE_CUDA(cudaMalloc(&c->work, (size_t)c->work_elems * c->esz));
     c->dwork_elems = 8 + 5 * 8 * 64 + 4 * (int64_t)ne_max + 16;
     CHASE_CUDA(cudaMalloc(&c->dwork, c->dwork_elems * sizeof(double)));

@@ -158,6 +158,19 @@ inline unsigned long long grid_wait_limit_ns() {
   return v ? v : 2000000000ull;
 }
 
+// 1 / sqrt(q), q > 0, from the FP32 estimate by two Newton steps: six dependent FP64 operations (each about 100 cycles
+// on GB300) instead of the twenty or so of a square root and a division
+__device__ __forceinline__ double fast_rsqrt(double q) {
+  if (!(q > 1e-30 && q < 1e30)) return rsqrt(q);
+  double y = (double)rsqrtf((float)q);
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const double r = fma(-q * y, y, 1.0);
+    y = fma(0.5 * y, r, y);
+  }
+  return y;
+}
+
 // warp-level FP64 sum
 __device__ inline double warp_sum(double v) {
 #pragma unroll

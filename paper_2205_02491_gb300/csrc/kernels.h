@@ -1,6 +1,5 @@
 // Internal launch interface of the FP64 kernels (host side).  Not part of the C ABI.
 #pragma once
-#include <functional>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -89,12 +88,11 @@ template <typename T>
 void sort_pairs(cudaStream_t st, int k, double* w, T* Z, int64_t ldz, T* tmp, double* wtmp, int* perm);
 
 // Lanczos bounds (Algorithm 1, line 2).  out4 (device) = {b_sup, mu_1, mu_ne, theta_max}.
-// matvec (nullable): W (n x runs, ld n) = A X (X: n x runs, ld ldx) on stream st, replacing the
-// DFMA multi-vector HEMV (used with the FP64-class split tensor-core products).
-template <typename T> using MatvecFn = std::function<void(const T* X, int64_t ldx, T* W)>;
+// work: at least lanczos_work_elems scalars (monotone in n).
+int64_t lanczos_work_elems(int64_t n, int runs, int steps, bool cplx);
 template <typename T>
 void lanczos(cudaStream_t st, const T* A, int64_t n, int64_t lda, int ne, const T* L0, int runs, int steps,
-             double* out4, T* work, int64_t work_elems, double* dwork, const MatvecFn<T>* matvec = nullptr);
+             double* out4, T* work, int64_t work_elems, double* dwork);
 
 // Input generator from compact-WY factors.
 template <typename T>

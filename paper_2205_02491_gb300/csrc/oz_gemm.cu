@@ -6,6 +6,8 @@
 
 #include <mutex>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "crt.h"
 #include "oz.h"
