@@ -14,7 +14,11 @@
 namespace chase {
 
 // ============================================================== GEMM
-constexpr int GB_M = 64, GB_N = 64;
+// GB300's FP64 units run 2 multiply-adds per SM and clock: any tile keeps them busy, and what a product costs is the
+// share of the SMs its blocks cover and the padding of its tiles.  16 x 16 tiles (2 x 2 per thread) and K chunks down
+// to two stages spread even small products: the 64 x 64 tiles they replace took 211 us for a 24 x 24 x 512 Gram
+// matrix, on 8 SMs and with 86 % of the arithmetic on padding.
+constexpr int GB = 16;
 
 template <typename T> struct GK { static constexpr int BK = 8; };
 template <> struct GK<double> { static constexpr int BK = 16; };
@@ -32,39 +36,38 @@ __device__ inline void epi_store(const Epi& e, int64_t i, int64_t j, T acc) {
 }
 
 template <typename T, int OPA, int OPB>
-__global__ void __launch_bounds__(256) gemm_f64_kernel(int64_t M, int64_t N, int64_t K, const T* __restrict__ A,
-                                                       int64_t lda, const T* __restrict__ B, int64_t ldb, Epi epi,
-                                                       T* __restrict__ work, int64_t kchunk) {
+__global__ void __launch_bounds__(64) gemm_f64_kernel(int64_t M, int64_t N, int64_t K, const T* __restrict__ A,
+                                                      int64_t lda, const T* __restrict__ B, int64_t ldb, Epi epi,
+                                                      T* __restrict__ work, int64_t kchunk) {
   using s = S<T>;
   constexpr int BK = GK<T>::BK;
-  __shared__ T As[BK][GB_M + 1];
-  __shared__ T Bs[BK][GB_N + 1];
+  __shared__ T As[BK][GB + 1];
+  __shared__ T Bs[BK][GB + 1];
   const int tid = threadIdx.x;
-  const int tx = tid % 16, ty = tid / 16;
-  const int64_t m0 = (int64_t)blockIdx.x * GB_M, n0 = (int64_t)blockIdx.y * GB_N;
+  const int tx = tid % 8, ty = tid / 8;
+  const int64_t m0 = (int64_t)blockIdx.x * GB, n0 = (int64_t)blockIdx.y * GB;
   const int64_t kb = (int64_t)blockIdx.z * kchunk;
   const int64_t ke = min(K, kb + kchunk);
-  T acc[4][4];
+  T acc[2][2];
 #pragma unroll
-  for (int r = 0; r < 4; ++r)
+  for (int r = 0; r < 2; ++r)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) acc[r][c] = s::zero();
+    for (int c = 0; c < 2; ++c) acc[r][c] = s::zero();
 
   for (int64_t k0 = kb; k0 < ke; k0 += BK) {
-    // A tile: BM x BK
 #pragma unroll
-    for (int t = tid; t < GB_M * BK; t += 256) {
+    for (int t = tid; t < GB * BK; t += 64) {
       int i, kk;
-      if (OPA == OP_N) { i = t % GB_M; kk = t / GB_M; } else { kk = t % BK; i = t / BK; }
+      if (OPA == OP_N) { i = t % GB; kk = t / GB; } else { kk = t % BK; i = t / BK; }
       int64_t gi = m0 + i, gk = k0 + kk;
       T v = s::zero();
       if (gi < M && gk < ke) v = (OPA == OP_N) ? A[gi + gk * lda] : s::conj(A[gk + gi * lda]);
       As[kk][i] = v;
     }
 #pragma unroll
-    for (int t = tid; t < GB_N * BK; t += 256) {
+    for (int t = tid; t < GB * BK; t += 64) {
       int j, kk;
-      if (OPB == OP_N) { kk = t % BK; j = t / BK; } else { j = t % GB_N; kk = t / GB_N; }
+      if (OPB == OP_N) { kk = t % BK; j = t / BK; } else { j = t % GB; kk = t / GB; }
       int64_t gj = n0 + j, gk = k0 + kk;
       T v = s::zero();
       if (gj < N && gk < ke) v = (OPB == OP_N) ? B[gk + gj * ldb] : s::conj(B[gj + gk * ldb]);
@@ -73,23 +76,23 @@ __global__ void __launch_bounds__(256) gemm_f64_kernel(int64_t M, int64_t N, int
     __syncthreads();
 #pragma unroll
     for (int kk = 0; kk < BK; ++kk) {
-      T a[4], b[4];
+      T a[2], b[2];
 #pragma unroll
-      for (int r = 0; r < 4; ++r) a[r] = As[kk][ty + 16 * r];
+      for (int r = 0; r < 2; ++r) a[r] = As[kk][ty + 8 * r];
 #pragma unroll
-      for (int c = 0; c < 4; ++c) b[c] = Bs[kk][tx + 16 * c];
+      for (int c = 0; c < 2; ++c) b[c] = Bs[kk][tx + 8 * c];
 #pragma unroll
-      for (int r = 0; r < 4; ++r)
+      for (int r = 0; r < 2; ++r)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) acc[r][c] = s::fma(a[r], b[c], acc[r][c]);
+        for (int c = 0; c < 2; ++c) acc[r][c] = s::fma(a[r], b[c], acc[r][c]);
     }
     __syncthreads();
   }
 #pragma unroll
-  for (int r = 0; r < 4; ++r)
+  for (int r = 0; r < 2; ++r)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      int64_t i = m0 + ty + 16 * r, j = n0 + tx + 16 * c;
+    for (int c = 0; c < 2; ++c) {
+      int64_t i = m0 + ty + 8 * r, j = n0 + tx + 8 * c;
       if (i < M && j < N) {
         if (work)
           work[(int64_t)blockIdx.z * M * N + i + j * M] = acc[r][c];
@@ -114,11 +117,11 @@ void gemm_f64(cudaStream_t st, Op opA, Op opB, int64_t M, int64_t N, int64_t K, 
               int64_t ldb, const Epi& epi, T* work, int64_t work_elems) {
   if (M <= 0 || N <= 0) return;
   constexpr int BK = GK<T>::BK;
-  int64_t tiles = (int64_t)ceil_div(M, GB_M) * ceil_div(N, GB_N);
+  int64_t tiles = (int64_t)ceil_div(M, GB) * ceil_div(N, GB);
   int nsplit = 1;
   if (K > 0) {
-    int64_t want = (2 * 152 + tiles - 1) / tiles;  // aim for >= 2 waves of blocks
-    int64_t maxsplit = K / (8 * BK);
+    int64_t want = (4 * 152 + tiles - 1) / tiles;  // four blocks per SM
+    int64_t maxsplit = K / (2 * BK);
     nsplit = (int)std::max<int64_t>(1, std::min<int64_t>(want, std::min<int64_t>(maxsplit, 64)));
     if (work == nullptr || work_elems < nsplit * M * N) nsplit = 1;
   }
@@ -127,9 +130,10 @@ void gemm_f64(cudaStream_t st, Op opA, Op opB, int64_t M, int64_t N, int64_t K, 
     // C = epilogue with acc = 0
     nsplit = 1;
   }
-  dim3 grid(ceil_div(M, GB_M), ceil_div(N, GB_N), nsplit);
+  CHASE_REQUIRE(ceil_div(N, GB) <= 65535, 1, "gemm_f64: too many columns");
+  dim3 grid(ceil_div(M, GB), ceil_div(N, GB), nsplit);
   T* w = nsplit > 1 ? work : nullptr;
-#define LAUNCH(OA, OB) gemm_f64_kernel<T, OA, OB><<<grid, 256, 0, st>>>(M, N, std::max<int64_t>(K, 0), A, lda, B, ldb, epi, w, kchunk)
+#define LAUNCH(OA, OB) gemm_f64_kernel<T, OA, OB><<<grid, 64, 0, st>>>(M, N, std::max<int64_t>(K, 0), A, lda, B, ldb, epi, w, kchunk)
   if (opA == OP_N && opB == OP_N) LAUNCH(OP_N, OP_N);
   else if (opA == OP_C && opB == OP_N) LAUNCH(OP_C, OP_N);
   else if (opA == OP_N && opB == OP_C) LAUNCH(OP_N, OP_C);

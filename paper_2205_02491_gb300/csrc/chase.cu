@@ -816,7 +816,7 @@ template <typename T> struct Solver {
     Epi ga;
     ga.C = gA;
     ga.ldc = ldga;
-    gemm_f64<T>(st(), OP_N, OP_C, n, n, nev, Tb, n, Vs, n, ga, W(), c->work_elems);
+    gemm(OP_N, Tb, n, OP_C, Vs, n, n, n, nev, ga, CHASE_FP64);
     hermitianize<T>(st(), (int)n, gA, ldga);
     CHASE_CUDA(cudaStreamSynchronize(st()));
     CHASE_REQUIRE(oz::read_flags(st(), c->ozw) == 0, CHASE_ERR_TIMEOUT, "a tensor-core product hit its wait limit");

@@ -482,7 +482,7 @@ void gemm(cudaStream_t st, Workspace& w, Op opA, const T* A, int64_t lda, Op opB
   constexpr bool CPLX = S<T>::cplx;
   CHASE_REQUIRE(w.ready, 9, "split products not initialised");
   if (M <= 0 || N <= 0) return;
-  CHASE_REQUIRE(N <= w.ne_max && M <= std::max<int64_t>(w.n_max, w.ne_max) &&
+  CHASE_REQUIRE(N <= w.n_max && M <= w.n_max &&
                     crt::plane_bytes(M, K, CPLX, crt::NMOD) <= left_bytes(w.n_max, w.ne_max, CPLX),
                 1, "split product exceeds the workspace");
   // left operand: OP_N rows of A (M x K), OP_C conjugated columns of A (K x M); right operand: OP_N columns of B
