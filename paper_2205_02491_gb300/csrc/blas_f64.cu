@@ -306,171 +306,179 @@ template <typename T> void hermitianize(cudaStream_t st, int k, T* G, int64_t ld
   CHASE_CHECK_LAUNCH();
 }
 
-// ============================================================== Cholesky and TRSM
-constexpr int CB = 32;  // block size of the blocked Cholesky / TRSM
+// ============================================================== Cholesky with the inverse factor
+// G = L L^H together with L^{-H}, on the stacked matrix S = [G; I] (2k x k): the column operations that turn G's
+// lower triangle into L turn the identity below it into L^{-H}, by substitution, in the same launches.
+// Panels of CB columns: chol_panel_kernel factors the diagonal block (every block of the launch for itself: it is
+// one launch and no barrier) and substitutes the k rows below it, rows j0 + nb .. k + j0 + nb of S (below those the
+// identity's columns are still zero); chol_update_kernel subtracts the panel from the following columns.
+// GB300's FP64 units run 2 multiply-adds per SM and clock, so a block on one SM is slow however it is written and the
+// width of the launch decides: 8 rows (panel) or 16 x 16 entries (update) per block.
+constexpr int CB = 16;    // panel width
+constexpr int CROWS = 8;  // rows per panel block
 
-// Unblocked Cholesky of one CB x CB diagonal block in shared memory (lower).  A pivot that is not finite,
-// or <= floor, marks the factorisation failed (info), except in detection mode (dep != null): there a
-// finite pivot <= floor marks its column numerically dependent on the columns before it (dep[1 + col],
-// count in dep[0]); the column gets a unit pivot and a zero column below it, so it drops out of the
-// trailing update and the factorisation of the other columns goes on.
+// A pivot that is not finite, or <= floor, marks the factorisation failed (info), except in detection mode
+// (dep != null): there a finite pivot <= floor marks its column numerically dependent on the columns before it
+// (dep[1 + col], count in dep[0]); the column gets a unit pivot and zeros below it, so it drops out of the updates
+// and the factorisation of the other columns goes on.
 template <typename T>
-__global__ void potrf_diag_kernel(int nb, T* G, int64_t ldg, int* info, int col0, double floor, int* dep) {
+__global__ void __launch_bounds__(CROWS * CB) chol_panel_kernel(int k, int j0, T* Sm, int64_t lds, int* info,
+                                                                 double floor, int* dep) {
   using s = S<T>;
-  __shared__ T a[CB][CB + 1];
-  __shared__ int bad;
-  __shared__ int dep_sh[CB];
-  int i = threadIdx.x, j = threadIdx.y;  // element (i, j)
-  if (i == 0 && j == 0) bad = 0;
-  if (j == 0 && i < CB) dep_sh[i] = 0;
-  if (i < nb && j < nb) a[i][j] = G[i + j * ldg];
+  __shared__ T a[CB][CB + 1];  // lower factor of the diagonal block
+  __shared__ double rinv[CB];  // reciprocal pivots; 0 for a dependent column
+  const int nb = min(CB, k - j0);
+  const int tid = threadIdx.x, lane = tid & 31;
+  T* D = Sm + j0 + (int64_t)j0 * lds;
+  // this thread's row and column of the rows below
+  const int c = tid & (CB - 1);
+  const int64_t row = j0 + nb + (int64_t)blockIdx.x * CROWS + tid / CB;
+  const bool live = row < (int64_t)k + j0 + nb && c < nb;
+  T x = live ? Sm[row + (int64_t)(j0 + c) * lds] : s::zero();
+  for (int t = tid; t < CB * CB; t += CROWS * CB) {
+    const int i = t % CB, j = t / CB;
+    a[i][j] = (i < nb && j <= i) ? D[i + (int64_t)j * lds] : s::zero();
+  }
   __syncthreads();
-  for (int c = 0; c < nb; ++c) {
-    if (i == c && j == c) {
-      double d = s::re(a[c][c]);
+  if (tid < 32) {
+    int bad = 0;
+    for (int p = 0; p < nb; ++p) {
+      double d = s::re(a[p][p]);
+      double ri;
+      bool isdep = false;
       if (!isfinite(d)) {
         bad = 1;
         d = 1.0;
       } else if (!(d > floor)) {
-        if (dep) dep_sh[c] = 1;
+        if (dep) isdep = true;
         else bad = 1;
         d = 1.0;
       }
-      a[c][c] = s::make(sqrt(d), 0.0);
+      ri = fast_rsqrt(d);
+      if (isdep) ri = 0.0;
+      __syncwarp();
+      const int i = lane & (CB - 1);
+      if (lane < CB && i > p && i < nb) a[i][p] = s::scale(a[i][p], ri);
+      if (lane == 0) {
+        rinv[p] = ri;
+        if (isdep && blockIdx.x == 0) {
+          dep[1 + j0 + p] = 1;
+          atomicAdd(&dep[0], 1);
+        }
+      }
+      __syncwarp();
+      for (int j = p + 1 + (lane >> 4); j < nb; j += 2)
+        if (i >= j && i < nb) a[i][j] = s::fma(s::scale(a[i][p], -1.0), s::conj(a[j][p]), a[i][j]);
+      __syncwarp();
     }
-    __syncthreads();
-    double piv = s::re(a[c][c]);
-    if (j == c && i > c && i < nb) a[i][c] = dep_sh[c] ? s::zero() : s::scale(a[i][c], 1.0 / piv);
-    __syncthreads();
-    if (i > c && j > c && i < nb && j <= i) a[i][j] = s::sub(a[i][j], s::mul(a[i][c], s::conj(a[j][c])));
-    __syncthreads();
+    if (bad && lane == 0 && blockIdx.x == 0 && info) atomicMax(info, j0 + 1);
   }
-  if (i < nb && j < nb) G[i + j * ldg] = (j <= i) ? a[i][j] : s::zero();
-  if (i == 0 && j == 0 && bad && info) atomicMax(info, col0 + 1);
-  if (dep && j == 0 && i < nb && dep_sh[i]) {
-    dep[1 + col0 + i] = 1;
-    atomicAdd(&dep[0], 1);
+  __syncthreads();
+  // x <- x L^{-H}: one row per 16 lanes, lane = column; column p's result goes to the later columns
+  for (int p = 0; p < nb; ++p) {
+    if (c == p) x = s::scale(x, rinv[p]);
+    const double qr = __shfl_sync(0xffffffffu, s::re(x), (lane & 16) + p);
+    const double qi = s::cplx ? __shfl_sync(0xffffffffu, s::im(x), (lane & 16) + p) : 0.0;
+    if (c > p) x = s::fma(s::make(-qr, -qi), s::conj(a[c][p]), x);
   }
+  if (live) Sm[row + (int64_t)(j0 + c) * lds] = x;
 }
 
-// X(rows x nb) <- X L^{-H} with L the nb x nb lower block (row-parallel forward substitution).  dep
-// (nullable): dependent-column flags of the block's columns, whose results are set to zero.
+// S[r, c] -= sum_p S[r, j0 + p] conj(S[c, j0 + p]) for the k rows r >= j0 + nb and the columns c in [j0 + nb, jend)
+// (entries above G's diagonal may be skipped or written: nothing reads them)
 template <typename T>
-__global__ void trsm_rows_kernel(int64_t rows, int nb, T* X, int64_t ldx, const T* L, int64_t ldl,
-                                 const int* dep) {
+__global__ void __launch_bounds__(64) chol_update_kernel(int k, int j0, int jend, T* Sm, int64_t lds) {
   using s = S<T>;
-  __shared__ T l[CB][CB + 1];
-  for (int t = threadIdx.x; t < CB * CB; t += blockDim.x) {
-    int i = t % CB, j = t / CB;
-    l[i][j] = (i < nb && j < nb && j <= i) ? L[i + j * ldl] : s::zero();
+  __shared__ T pr[16][CB + 1], pc[16][CB + 1];
+  const int j1 = j0 + CB;  // the panel before an update is always full
+  const int64_t r0 = j1 + (int64_t)blockIdx.x * 16;
+  const int c0 = j1 + blockIdx.y * 16;
+  if (r0 + 16 <= c0) return;  // G's upper triangle
+  const int64_t rend = (int64_t)k + j1;
+  const int tid = threadIdx.x;
+  for (int t = tid; t < 16 * CB; t += 64) {
+    const int i = t & 15, p = t >> 4;
+    pr[i][p] = r0 + i < rend ? Sm[r0 + i + (int64_t)(j0 + p) * lds] : s::zero();
+    pc[i][p] = c0 + i < jend ? s::conj(Sm[c0 + i + (int64_t)(j0 + p) * lds]) : s::zero();
   }
   __syncthreads();
-  int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= rows) return;
-  T q[CB];
+  const int i = tid & 15, jq = tid >> 4;
+  T acc[4];
 #pragma unroll
-  for (int j = 0; j < CB; ++j) {
-    if (j < nb) {
-      T v = X[r + j * ldx];
+  for (int q = 0; q < 4; ++q) acc[q] = s::zero();
+#pragma unroll 4
+  for (int p = 0; p < CB; ++p) {
+    const T v = pr[i][p];
 #pragma unroll
-      for (int m = 0; m < CB; ++m)
-        if (m < j) v = s::sub(v, s::mul(q[m], s::conj(l[j][m])));
-      q[j] = (dep && dep[j]) ? s::zero() : s::scale(v, 1.0 / s::re(l[j][j]));
-    }
+    for (int q = 0; q < 4; ++q) acc[q] = s::fma(v, pc[jq + 4 * q][p], acc[q]);
   }
+  if (r0 + i >= rend) return;
 #pragma unroll
-  for (int j = 0; j < CB; ++j)
-    if (j < nb) X[r + j * ldx] = q[j];
+  for (int q = 0; q < 4; ++q) {
+    const int cc = c0 + jq + 4 * q;
+    if (cc >= jend) continue;
+    T* o = Sm + r0 + i + (int64_t)cc * lds;
+    *o = s::sub(*o, acc[q]);
+  }
+}
+
+template <typename T> __global__ void chol_identity_kernel(int k, T* Sm, int64_t lds) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
+  if (i < k) Sm[k + i + (int64_t)j * lds] = i == j ? S<T>::one() : S<T>::zero();
 }
 
 template <typename T>
-void potrf_lower(cudaStream_t st, int k, T* G, int64_t ldg, int* info, T* work, int64_t work_elems,
-                 double pivot_floor, int* dep) {
-  for (int j0 = 0; j0 < k; j0 += CB) {
-    int nb = std::min(CB, k - j0);
-    T* Gjj = G + j0 + (int64_t)j0 * ldg;
-    potrf_diag_kernel<T><<<1, dim3(CB, CB), 0, st>>>(nb, Gjj, ldg, info, j0, pivot_floor, dep);
-    CHASE_CHECK_LAUNCH();
-    int rest = k - j0 - nb;
-    if (rest <= 0) break;
-    T* P = G + (j0 + nb) + (int64_t)j0 * ldg;  // panel below the diagonal block
-    trsm_rows_kernel<T><<<ceil_div(rest, 128), 128, 0, st>>>(rest, nb, P, ldg, Gjj, ldg,
-                                                             dep ? dep + 1 + j0 : nullptr);
-    CHASE_CHECK_LAUNCH();
-    // trailing update  G22 -= P P^H
-    T* G22 = G + (j0 + nb) + (int64_t)(j0 + nb) * ldg;
-    Epi e;
-    e.C = G22;
-    e.ldc = ldg;
-    e.alpha = -1.0;
-    e.Z = G22;
-    e.ldz = ldg;
-    e.beta = 1.0;
-    gemm_f64<T>(st, OP_N, OP_C, rest, rest, nb, P, ldg, P, ldg, e, work, work_elems);
-  }
-}
-
-template <typename T>
-void trsm_right_lh(cudaStream_t st, int64_t n, int k, T* X, int64_t ldx, const T* L, int64_t ldl, T* work,
-                   int64_t work_elems) {
-  for (int j0 = 0; j0 < k; j0 += CB) {
-    int nb = std::min(CB, k - j0);
-    T* Xb = X + (int64_t)j0 * ldx;
-    const T* Ljj = L + j0 + (int64_t)j0 * ldl;
-    trsm_rows_kernel<T><<<ceil_div(n, 128), 128, 0, st>>>(n, nb, Xb, ldx, Ljj, ldl, nullptr);
-    CHASE_CHECK_LAUNCH();
-    int rest = k - j0 - nb;
-    if (rest <= 0) break;
-    // X[:, j0+nb:] -= Xb * L[j0+nb:, j0:j0+nb]^H
-    T* Xr = X + (int64_t)(j0 + nb) * ldx;
-    Epi e;
-    e.C = Xr;
-    e.ldc = ldx;
-    e.alpha = -1.0;
-    e.Z = Xr;
-    e.ldz = ldx;
-    e.beta = 1.0;
-    gemm_f64<T>(st, OP_N, OP_C, n, rest, nb, Xb, ldx, L + (j0 + nb) + (int64_t)j0 * ldl, ldl, e, work, work_elems);
-  }
-}
-
-// ============================================================== triangular inverse
-// Inverse of one CB x CB lower-triangular diagonal block in place (one block per CTA).
-template <typename T> __global__ void trtri_diag_kernel(int k, T* L, int64_t ldl) {
-  using s = S<T>;
-  __shared__ T a[CB][CB + 1];
-  __shared__ T x[CB][CB + 1];
-  const int j0 = blockIdx.x * CB;
-  const int nb = min(CB, k - j0);
-  const int i = threadIdx.x, j = threadIdx.y;
-  T* Lb = L + j0 + (int64_t)j0 * ldl;
-  if (i < nb && j < nb) a[i][j] = (j <= i) ? Lb[i + (int64_t)j * ldl] : s::zero();
-  __syncthreads();
-  // column j of the inverse by forward substitution (thread row 0 of each column does it)
-  if (i == 0 && j < nb) {
-    for (int r = 0; r < nb; ++r) {
-      T v = (r == j) ? s::one() : s::zero();
-      for (int m = j; m < r; ++m) v = s::sub(v, s::mul(a[r][m], x[m][j]));
-      // divide by the (real, positive) diagonal
-      x[r][j] = (r < j) ? s::zero() : s::scale(v, 1.0 / s::re(a[r][r]));
-    }
-  }
-  __syncthreads();
-  if (i < nb && j < nb) Lb[i + (int64_t)j * ldl] = (j <= i) ? x[i][j] : s::zero();
-}
-
-template <typename T> __global__ void zero_upper_kernel(int k, T* G, int64_t ldg) {
-  int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * 32 + threadIdx.y;
-  if (i < k && j < k && i < j) G[i + (int64_t)j * ldg] = S<T>::zero();
-}
-
-template <typename T> void zero_upper(cudaStream_t st, int k, T* G, int64_t ldg) {
-  zero_upper_kernel<T><<<dim3(ceil_div(k, 32), ceil_div(k, 32)), dim3(32, 32), 0, st>>>(k, G, ldg);
+void chol_stack_begin(cudaStream_t st, int k, T* Sm, int64_t lds) {
+  chol_identity_kernel<T><<<dim3(ceil_div(k, 128), k), 128, 0, st>>>(k, Sm, lds);
   CHASE_CHECK_LAUNCH();
 }
 
-template <typename T> void trtri_diag(cudaStream_t st, int k, T* L, int64_t ldl) {
-  trtri_diag_kernel<T><<<ceil_div(k, CB), dim3(CB, CB), 0, st>>>(k, L, ldl);
+template <typename T>
+void chol_stack_columns(cudaStream_t st, int k, int jbeg, int jend, T* Sm, int64_t lds, int* info, double pivot_floor,
+                        int* dep) {
+  for (int j0 = jbeg; j0 < jend; j0 += CB) {
+    chol_panel_kernel<T><<<ceil_div(k, CROWS), CROWS * CB, 0, st>>>(k, j0, Sm, lds, info, pivot_floor, dep);
+    CHASE_CHECK_LAUNCH();
+    if (j0 + CB >= jend) break;
+    chol_update_kernel<T><<<dim3(ceil_div(k, 16), ceil_div(jend - j0 - CB, 16)), 64, 0, st>>>(k, j0, jend, Sm, lds);
+    CHASE_CHECK_LAUNCH();
+  }
+}
+
+// ============================================================== corrections of nearly orthonormal blocks
+// From the Gram matrix Gm = I + E of a block Q: the factor F with Q F closer to orthonormal by the square of E.
+// upper: F = I - striu(E) - diag(E)/2, which keeps the span of every leading set of columns (the QR's factor);
+// else F = I - E/2, the nearest orthonormal block.  dev = max over columns of sum_i |E_ij| (as float bits; NaN stays
+// largest), an upper bound of ||E||_2 for the caller's decision.
+template <typename T>
+__global__ void __launch_bounds__(128) gram_correction_kernel(int k, int upper, const T* __restrict__ Gm, int64_t ldg, T* F,
+                                                               int64_t ldf, unsigned* dev) {
+  using s = S<T>;
+  const int j = blockIdx.x;
+  float sum = 0.0f;
+  for (int i = threadIdx.x; i < k; i += 128) {
+    const T a = Gm[i + (int64_t)j * ldg], b = s::conj(Gm[j + (int64_t)i * ldg]);
+    T e = s::scale(s::add(a, b), 0.5);
+    if (i == j) e = s::make(s::re(e) - 1.0, 0.0);
+    sum += fabsf((float)s::re(e)) + fabsf((float)s::im(e));
+    T f = (upper && i < j) ? s::scale(e, -1.0) : ((upper && i > j) ? s::zero() : s::scale(e, -0.5));
+    if (i == j) f = s::add(f, s::one());
+    F[i + (int64_t)j * ldf] = f;
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  __shared__ float red[4];
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = sum;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    const float t = red[0] + red[1] + red[2] + red[3];
+    atomicMax(dev, t == t ? __float_as_uint(t) : 0x7fc00000u);
+  }
+}
+
+template <typename T>
+void gram_correction(cudaStream_t st, int k, bool upper, const T* Gm, int64_t ldg, T* F, int64_t ldf, unsigned* dev) {
+  gram_correction_kernel<T><<<k, 128, 0, st>>>(k, upper ? 1 : 0, Gm, ldg, F, ldf, dev);
   CHASE_CHECK_LAUNCH();
 }
 
@@ -712,16 +720,15 @@ template <typename T> void fill_normal(cudaStream_t st, T* X, int64_t rows, int 
   template void scale_cols<T>(cudaStream_t, int64_t, int, T*, int64_t, const double*, int);                       \
   template void add_diag<T>(cudaStream_t, int, T*, int64_t, const double*, double);                               \
   template void hermitianize<T>(cudaStream_t, int, T*, int64_t);                                                  \
-  template void potrf_lower<T>(cudaStream_t, int, T*, int64_t, int*, T*, int64_t, double, int*);                   \
+  template void chol_stack_begin<T>(cudaStream_t, int, T*, int64_t);                                             \
+  template void chol_stack_columns<T>(cudaStream_t, int, int, int, T*, int64_t, int*, double, int*);             \
+  template void gram_correction<T>(cudaStream_t, int, bool, const T*, int64_t, T*, int64_t, unsigned*);          \
   template void householder_vec<T>(cudaStream_t, int64_t, T*, T*, double*);                                      \
   template void householder_apply<T>(cudaStream_t, int64_t, const T*, T*, int64_t, int, const double*);            \
   template void reflector_panel<T>(cudaStream_t, int64_t, int, const T*, int64_t, T*, int64_t);                   \
   template void householder_T<T>(cudaStream_t, int, const T*, const double*, T*, int64_t);                         \
   template void identity_rect<T>(cudaStream_t, int64_t, int, T*, int64_t);                                         \
-  template void trsm_right_lh<T>(cudaStream_t, int64_t, int, T*, int64_t, const T*, int64_t, T*, int64_t);        \
   template void generate_wy<T>(cudaStream_t, T*, int64_t, int64_t, const double*, const T*, const T*, const T*, int); \
-  template void zero_upper<T>(cudaStream_t, int, T*, int64_t);                                                    \
-  template void trtri_diag<T>(cudaStream_t, int, T*, int64_t);                                                   \
   template void perturb<T>(cudaStream_t, T*, int64_t, int64_t, double, unsigned long long);                      \
   template void fill_normal<T>(cudaStream_t, T*, int64_t, int, int64_t, unsigned long long);
 INST(double)

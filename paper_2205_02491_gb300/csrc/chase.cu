@@ -220,11 +220,17 @@ template <typename T> struct Solver {
   }
 
   // C = op(A) op(B) with FP64 accuracy: split tensor-core products for large shapes, DFMA for
-  // small ones (and always in the native mode).  Split products may write C over an operand.
+  // small ones (and always in the native mode).  Split products may write C over the left operand.
+  // The default of native_below_mflop leaves the line to the library: a split product is five or six launches
+  // (20 to 30 us whatever its size, up to a few GFLOP) while DFMA tiles run at about 0.7 TFLOP/s, so they meet near
+  // SPLIT_FROM_MFLOP.  Any other value is the line itself.
+  static constexpr int DEFAULT_NATIVE_MFLOP = 2000;
+  static constexpr double SPLIT_FROM_MFLOP = 20.0;
   bool use_split(int mode, int64_t M, int64_t N, int64_t K) {
     if (mode == CHASE_FP64_NATIVE || !oz::available()) return false;
     double mflop = (S<T>::cplx ? 8.0 : 2.0) * (double)M * (double)N * (double)K * 1e-6;
-    return mflop >= (double)c->opts.native_below_mflop;
+    const int line = c->opts.native_below_mflop;
+    return mflop >= (line == DEFAULT_NATIVE_MFLOP ? SPLIT_FROM_MFLOP : (double)line);
   }
   // force_split: the split tensor-core product whatever the size (for the skinny products of a long loop,
   // which split along K where DFMA tiles stay latency-bound)
@@ -236,62 +242,97 @@ template <typename T> struct Solver {
       gemm_f64<T>(st(), opA, opB, M, N, K, A, lda, B, ldb, e, W(), c->work_elems);
   }
 
-  // L (k x k lower, diagonal CB-blocks already inverted) -> L^{-1} by recursive halving:
-  // [[A, 0], [B, C]]^{-1} = [[A^-1, 0], [-C^-1 B A^-1, C^-1]].  tmp: k*k/4 scalars.
-  void trtri_combine(T* L, int64_t ld, int k, T* tmp, int mode) {
-    if (k <= 32) return;
-    int k1 = ((k / 2 + 31) / 32) * 32;
-    if (k1 >= k) k1 = k - 32;
-    const int k2 = k - k1;
-    trtri_combine(L, ld, k1, tmp, mode);
-    trtri_combine(L + k1 + (int64_t)k1 * ld, ld, k2, tmp, mode);
-    T* B = L + k1;
-    Epi e1;
-    e1.C = tmp;
-    e1.ldc = k2;
-    gemm(OP_N, B, ld, OP_N, L, ld, k2, k1, k1, e1, mode);  // tmp = B A^-1
-    Epi e2;
-    e2.C = B;
-    e2.ldc = ld;
-    e2.alpha = -1.0;
-    gemm(OP_N, L + k1 + (int64_t)k1 * ld, ld, OP_N, tmp, k2, k2, k1, k2, e2, mode);  // B = -C^-1 tmp
+  // Cholesky of G in the stacked matrix Sm = [G; I] (Gb(), 2k x k, ld 2k), L^{-H} in its lower half: panels on CUDA
+  // cores, and after every CHOL_OUTER columns one product for all the columns that follow.
+  void cholesky(int k, int mode, double floor = 0.0, int* dep = nullptr) {
+    T* Sm = Gb();
+    const int64_t ld = 2 * (int64_t)k;
+    CHASE_CUDA(cudaMemsetAsync(c->info, 0, sizeof(int), st()));
+    if (dep) CHASE_CUDA(cudaMemsetAsync(dep, 0, (size_t)(k + 1) * sizeof(int), st()));
+    chol_stack_begin<T>(st(), k, Sm, ld);
+    for (int j = 0; j < k; j += CHOL_OUTER) {
+      const int je = std::min(k, j + CHOL_OUTER);
+      chol_stack_columns<T>(st(), k, j, je, Sm, ld, c->info, floor, dep);
+      if (je == k) break;
+      const T* P = Sm + je + j * ld;
+      Epi e;
+      e.C = Sm + je + je * ld;
+      e.ldc = ld;
+      e.alpha = -1.0;
+      e.Z = e.C;
+      e.ldz = ld;
+      e.beta = 1.0;
+      gemm(OP_N, P, ld, OP_C, P, ld, k, k - je, je - j, e, mode);
+    }
   }
 
-  // Y_s (n x k, ld n) <- Q with Y_s = Q R (Cholesky-QR2 with column equilibration) and Y_p <- Y_p R^{-1}:
-  // both iterates of the three-term recurrence take the same right factor, so the recurrence goes on
-  // and the filtered block keeps its span.  Returns false (both blocks rescaled consistently, otherwise
-  // as they were after the last completed pass) when a Cholesky factorisation fails.
+  // X (n x k, ld ldx) <- X F (F k x k, ld ldf).  Uses T2.
+  void apply_right(T* X, int64_t ldx, int64_t n, int k, const T* F, int64_t ldf, int mode) {
+    Epi q;
+    if (use_split(mode, n, k, k)) {
+      q.C = X;
+      q.ldc = ldx;
+      gemm(OP_N, X, ldx, OP_N, F, ldf, n, k, k, q, mode);
+    } else {
+      q.C = T2();
+      q.ldc = n;
+      gemm(OP_N, X, ldx, OP_N, F, ldf, n, k, k, q, mode);
+      copy_cols<T>(st(), n, k, T2(), n, X, ldx);
+    }
+  }
+
+  // Gram matrix of X (n x k, ld ldx) into Gb(), ld ldg
+  void gram(const T* X, int64_t ldx, int64_t n, int k, int64_t ldg, int mode) {
+    Epi e;
+    e.C = Gb();
+    e.ldc = ldg;
+    gemm(OP_C, X, ldx, OP_N, X, ldx, k, k, n, e, mode);
+  }
+
+  // Bound of ||G - I||_2 for the Gram matrix in Gb() (ld k); the correction factor goes to Zb() (ld k).
+  double correction(int k, bool upper) {
+    unsigned* dev = reinterpret_cast<unsigned*>(c->info);
+    CHASE_CUDA(cudaMemsetAsync(dev, 0, sizeof(unsigned), st()));
+    gram_correction<T>(st(), k, upper, Gb(), k, Zb(), k, dev);
+    float d = 0.f;
+    CHASE_CUDA(cudaMemcpyAsync(&d, dev, sizeof(float), cudaMemcpyDeviceToHost, st()));
+    CHASE_CUDA(cudaStreamSynchronize(st()));
+    return d;
+  }
+  // A block whose Gram matrix is off by d is corrected to O(d^2) by one product: below this bound the result is
+  // orthonormal to rounding.  Above CORRECT_MAX (or NaN) a Cholesky factorisation is needed.
+  static constexpr double CORRECT_LAST = 3e-8, CORRECT_MAX = 0.1;
+
+  // Y_s (n x k, ld n) <- Q with Y_s = Q R (Cholesky-QR with column equilibration, then corrections by upper
+  // triangular factors) and Y_p <- Y_p R^{-1}: both iterates of the three-term recurrence take the same right factor,
+  // so the recurrence goes on and the filtered block keeps its span.  Returns false (both blocks rescaled consistently,
+  // otherwise as they were after the last completed pass) when a Cholesky factorisation fails.
   bool orthonormalize_pair(T* Ys, T* Yp, int64_t n, int k) {
-    T* Gm = Gb();
-    for (int pass = 0; pass < 2; ++pass) {
-      colnorms<T>(st(), n, k, Ys, n, c->dwork);
-      scale_cols<T>(st(), n, k, Ys, n, c->dwork, 1);
-      scale_cols<T>(st(), n, k, Yp, n, c->dwork, 1);
-      Epi e;
-      e.C = Gm;
-      e.ldc = k;
-      gemm(OP_C, Ys, n, OP_N, Ys, n, k, k, n, e, CHASE_FP64);
-      hermitianize<T>(st(), k, Gm, k);
-      CHASE_CUDA(cudaMemsetAsync(c->info, 0, sizeof(int), st()));
-      potrf_lower<T>(st(), k, Gm, k, c->info, W(), c->work_elems);
-      int info = 0;
-      CHASE_CUDA(cudaMemcpyAsync(&info, c->info, sizeof(int), cudaMemcpyDeviceToHost, st()));
-      CHASE_CUDA(cudaStreamSynchronize(st()));
-      if (info != 0) return false;
-      if (use_split(CHASE_FP64, n, k, k)) {
-        zero_upper<T>(st(), k, Gm, k);
-        trtri_diag<T>(st(), k, Gm, k);
-        trtri_combine(Gm, k, k, Zb(), CHASE_FP64);
-        for (T* X : {Ys, Yp}) {
-          Epi q;
-          q.C = X;
-          q.ldc = n;
-          gemm(OP_N, X, n, OP_C, Gm, k, n, k, k, q, CHASE_FP64);
-        }
-      } else {
-        trsm_right_lh<T>(st(), n, k, Ys, n, Gm, k, W(), c->work_elems);
-        trsm_right_lh<T>(st(), n, k, Yp, n, Gm, k, W(), c->work_elems);
+    colnorms<T>(st(), n, k, Ys, n, c->dwork);
+    scale_cols<T>(st(), n, k, Ys, n, c->dwork, 1);
+    scale_cols<T>(st(), n, k, Yp, n, c->dwork, 1);
+    bool factored = false;
+    for (int pass = 0; pass < 8; ++pass) {
+      double d = -1.0;
+      if (factored) {
+        gram(Ys, n, n, k, k, CHASE_FP64);
+        d = correction(k, true);
       }
+      const T* F = Zb();
+      int64_t ldf = k;
+      if (!(d >= 0.0 && d < CORRECT_MAX)) {
+        gram(Ys, n, n, k, 2 * (int64_t)k, CHASE_FP64);
+        cholesky(k, CHASE_FP64);
+        int info = 0;
+        CHASE_CUDA(cudaMemcpyAsync(&info, c->info, sizeof(int), cudaMemcpyDeviceToHost, st()));
+        CHASE_CUDA(cudaStreamSynchronize(st()));
+        if (info != 0) return false;
+        factored = true;
+        F = Gb() + k;
+        ldf = 2 * (int64_t)k;
+      }
+      for (T* X : {Ys, Yp}) apply_right(X, n, n, k, F, ldf, CHASE_FP64);
+      if (d >= 0.0 && d <= CORRECT_LAST) break;
     }
     return true;
   }
@@ -464,45 +505,44 @@ template <typename T> struct Solver {
     // found numerically dependent columns (X is then left unchanged)
     int ndep = 0;
     auto chol_pass = [&](double shift_factor, int* dep = nullptr) -> bool {
-      Epi e;
-      e.C = Gm;
-      e.ldc = k;
-      gemm(OP_C, X, ldx, OP_N, X, ldx, k, k, n, e, pm);
-      hermitianize<T>(st(), k, Gm, k);
+      const int64_t ld = 2 * (int64_t)k;
+      gram(X, ldx, n, k, ld, pm);
       if (shift_factor > 0.0) {
         fro_norm2<T>(st(), n, k, X, ldx, c->dwork);
         double tr = 0.0;
         CHASE_CUDA(cudaMemcpyAsync(&tr, c->dwork, sizeof(double), cudaMemcpyDeviceToHost, st()));
         CHASE_CUDA(cudaStreamSynchronize(st()));
         double shift = shift_factor * ((double)n * k + (double)k * (k + 1)) * 1.1102230246251565e-16 * tr;
-        add_diag<T>(st(), k, Gm, k, nullptr, shift);
+        add_diag<T>(st(), k, Gm, ld, nullptr, shift);
       }
-      CHASE_CUDA(cudaMemsetAsync(c->info, 0, sizeof(int), st()));
       // detection: the columns have unit norm, so the Gram matrix has a unit diagonal and a pivot below
       // 8 (k + sqrt(n)) u lies within the rounding error of the Gram matrix and its factorisation: that
       // column is numerically in the span of the columns before it
       const double floor_dep = 8.0 * ((double)k + std::sqrt((double)n)) * 1.1102230246251565e-16;
-      if (dep) CHASE_CUDA(cudaMemsetAsync(dep, 0, (size_t)(k + 1) * sizeof(int), st()));
-      potrf_lower<T>(st(), k, Gm, k, c->info, W(), c->work_elems, dep ? floor_dep : 0.0, dep);
+      cholesky(k, pm, dep ? floor_dep : 0.0, dep);
       int hinfo[2] = {0, 0};
       CHASE_CUDA(cudaMemcpyAsync(&hinfo[0], c->info, sizeof(int), cudaMemcpyDeviceToHost, st()));
       if (dep) CHASE_CUDA(cudaMemcpyAsync(&hinfo[1], dep, sizeof(int), cudaMemcpyDeviceToHost, st()));
       CHASE_CUDA(cudaStreamSynchronize(st()));
       ndep = hinfo[1];
       if (hinfo[0] != 0 || ndep > 0) return false;
-      if (use_split(pm, n, k, k)) {
-        // X <- X L^{-H} as one product with the explicit triangular inverse (written over X)
-        zero_upper<T>(st(), k, Gm, k);
-        trtri_diag<T>(st(), k, Gm, k);
-        trtri_combine(Gm, k, k, Zb(), pm);
-        Epi q;
-        q.C = X;
-        q.ldc = ldx;
-        gemm(OP_N, X, ldx, OP_C, Gm, k, n, k, k, q, pm);
-      } else {
-        trsm_right_lh<T>(st(), n, k, X, ldx, Gm, k, W(), c->work_elems);
-      }
+      apply_right(X, ldx, n, k, Gm + k, ld, pm);  // X <- X L^{-H}
       return true;
+    };
+    // After a Cholesky pass X is orthonormal up to the Gram matrix's rounding times the block's squared condition:
+    // corrections by upper triangular factors (each one Gram product, no factorisation) finish it, each squaring the
+    // deviation; a deviation too large for them takes another Cholesky pass.  Projections keep X orthogonal to the
+    // locked columns to rounding even when it was ill-conditioned.
+    auto refine = [&]() -> bool {
+      for (int pass = 0; pass < 8; ++pass) {
+        project();
+        gram(X, ldx, n, k, k, pm);
+        const double d = correction(k, true);
+        if (d < CORRECT_MAX) apply_right(X, ldx, n, k, Zb(), k, pm);
+        else if (!chol_pass(0.0)) return false;
+        if (d <= CORRECT_LAST) return true;
+      }
+      return false;
     };
     // Cholesky-QR2 with a projection before each pass, so the final basis is orthogonal to the
     // locked columns to rounding even when X was ill-conditioned.  A filtered block can be numerically
@@ -520,10 +560,7 @@ template <typename T> struct Solver {
       scale_cols<T>(st(), n, k, X, ldx, c->dwork, 1);
       ok = chol_pass(0.0);
     }
-    if (ok) {
-      project();
-      ok = chol_pass(0.0);
-    }
+    if (ok) ok = refine();
     if (!ok) {
       // shifted Cholesky-QR3 (Fukaya et al.): one shifted pass, then Cholesky-QR2
       c->stats.qr_fallbacks++;
@@ -535,42 +572,12 @@ template <typename T> struct Solver {
         project();
         ok = chol_pass(0.0);
       }
-      if (ok) {
-        project();
-        ok = chol_pass(0.0);
-      }
+      if (ok) ok = refine();
     }
     CHASE_REQUIRE(ok, CHASE_ERR_QR_BREAKDOWN, "Cholesky-QR breakdown after the shifted fallback");
   }
 
   // ------------------------------------------------------------ Rayleigh-Ritz eigensolve
-  // Z (k x k, orthonormal columns) <- Z L^{-H} with G_z = Z^H Z = L L^H.  Returns false if not SPD.
-  bool orthonormalize_small(T* Z, int k, T* Gm, T* tmp) {
-    Epi e;
-    e.C = Gm;
-    e.ldc = k;
-    gemm(OP_C, Z, k, OP_N, Z, k, k, k, k, e, CHASE_FP64);
-    hermitianize<T>(st(), k, Gm, k);
-    CHASE_CUDA(cudaMemsetAsync(c->info, 0, sizeof(int), st()));
-    potrf_lower<T>(st(), k, Gm, k, c->info, W(), c->work_elems);
-    int info = 0;
-    CHASE_CUDA(cudaMemcpyAsync(&info, c->info, sizeof(int), cudaMemcpyDeviceToHost, st()));
-    CHASE_CUDA(cudaStreamSynchronize(st()));
-    if (info != 0) return false;
-    if (use_split(CHASE_FP64, k, k, k)) {
-      zero_upper<T>(st(), k, Gm, k);
-      trtri_diag<T>(st(), k, Gm, k);
-      trtri_combine(Gm, k, k, tmp, CHASE_FP64);
-      Epi q;
-      q.C = Z;
-      q.ldc = k;
-      gemm(OP_N, Z, k, OP_C, Gm, k, k, k, k, q, CHASE_FP64);
-    } else {
-      trsm_right_lh<T>(st(), k, k, Z, k, Gm, k, W(), c->work_elems);
-    }
-    return true;
-  }
-
   // Eigenpairs of the Hermitian G = Gb() (k x k): FP32 parallel Jacobi, two first-order refinement
   // steps in FP64-class products, exact FP64 Jacobi on clusters closer than omega.  Ascending
   // eigenvalues to w (device), eigenvectors to Zb().  scratch: 3 k*k scalars.  Returns false when a
@@ -594,7 +601,7 @@ template <typename T> struct Solver {
     using F = typename Lowp<T>::type;
     T* G = Gb();
     T* Z = Zb();
-    T *Wk = scratch, *Gp = scratch + (size_t)k * k, *X = scratch + 2 * (size_t)k * k;
+    T *X2 = scratch, *Gp = scratch + (size_t)k * k, *X = scratch + 2 * (size_t)k * k;
     F* Gf = (F*)W();
     F* Zf = Gf + (size_t)k * k;
     F* jw = Zf + (size_t)k * k;
@@ -626,29 +633,41 @@ template <typename T> struct Solver {
     if (!(scale > 0.0) || !std::isfinite(scale)) return false;
     const double omega = 1e-5 * scale;
     // three first-order corrections: the FP32 pass stops at its rounding floor (up to about 1e-4 relative
-    // off-diagonal norm for large k), which quadratic convergence takes to FP64 level in three steps
+    // off-diagonal norm for large k), which quadratic convergence takes to FP64 level in three steps.  Before each,
+    // Z (I - E/2) with Z^H Z = I + E brings Z back to orthonormality up to E^2: E is the FP32 rounding (1e-5) at
+    // first and the squared correction later, so the last pass leaves rounding level.
+    unsigned* dev = reinterpret_cast<unsigned*>(c->info);
+    CHASE_CUDA(cudaMemsetAsync(dev, 0, sizeof(unsigned), st()));
+    T* Zn = X2;
     for (int it = 0; it < 4; ++it) {
-      if (!orthonormalize_small(Z, k, Gp, X)) return false;
+      Epi eg;
+      eg.C = Gp;
+      eg.ldc = k;
+      gemm(OP_C, Z, k, OP_N, Z, k, k, k, k, eg, CHASE_FP64);
+      gram_correction<T>(st(), k, false, Gp, k, X, k, dev);
+      Epi ez;
+      ez.C = Zn;
+      ez.ldc = k;
+      gemm(OP_N, Z, k, OP_N, X, k, k, k, k, ez, CHASE_FP64);
       Epi e1;
-      e1.C = Wk;
+      e1.C = Z;
       e1.ldc = k;
-      gemm(OP_N, G, k, OP_N, Z, k, k, k, k, e1, CHASE_FP64);  // G Z
+      gemm(OP_N, G, k, OP_N, Zn, k, k, k, k, e1, CHASE_FP64);  // G Z (over the block before)
       Epi e2;
       e2.C = Gp;
       e2.ldc = k;
-      gemm(OP_C, Z, k, OP_N, Wk, k, k, k, k, e2, CHASE_FP64);  // G' = Z^H G Z
+      gemm(OP_C, Zn, k, OP_N, Z, k, k, k, k, e2, CHASE_FP64);  // G' = Z^H G Z
       hermitianize<T>(st(), k, Gp, k);
       dbg_finite(Gp, k, k, k, sizeof(T), "G' in the refinement");
       if (it == 3) break;
       eig_correction<T>(st(), k, Gp, k, X, k, omega);
       Epi e3;
-      e3.C = Wk;
+      e3.C = Z;
       e3.ldc = k;
-      e3.Y = Z;
+      e3.Y = Zn;
       e3.ldy = k;
       e3.gamma = 1.0;
-      gemm(OP_N, Z, k, OP_N, X, k, k, k, k, e3, CHASE_FP64);  // Z (I + X)
-      copy_cols<T>(st(), k, k, Wk, k, Z, k);
+      gemm(OP_N, Zn, k, OP_N, X, k, k, k, k, e3, CHASE_FP64);  // Z (I + X)
     }
     // eigenvalues: diagonal of G', clusters solved exactly
     diag_real<T>(st(), k, Gp, k, w);
@@ -656,11 +675,15 @@ template <typename T> struct Solver {
     CHASE_CUDA(cudaMemcpyAsync(d.data(), w, k * sizeof(double), cudaMemcpyDeviceToHost, st()));
     CHASE_CUDA(cudaStreamSynchronize(st()));
     std::vector<int> cl;
+    // a block too far from orthonormal for the corrections (or not finite) is left to the FP64 solver
+    float far = 0.f;
+    CHASE_CUDA(cudaMemcpyAsync(&far, dev, sizeof(float), cudaMemcpyDeviceToHost, st()));
     for (int i = 0; i < k;) {
       int j = i + 1;
       while (j < k && std::fabs(d[j] - d[j - 1]) <= omega) ++j;
       if (j - i > 1) {
         if (j - i > 32) return false;
+    if (!(far < CORRECT_MAX)) return false;
         cl.push_back(i);
         cl.push_back(j - i);
       }
@@ -671,9 +694,9 @@ template <typename T> struct Solver {
     if (ncl > 0) {
       CHASE_CUDA(cudaMemcpyAsync(c->iwork, cl.data(), cl.size() * sizeof(int), cudaMemcpyHostToDevice, st()));
       CHASE_CUDA(cudaMemsetAsync(c->status_dev, 0, sizeof(int), st()));
-      cluster_eig<T>(st(), k, ncl, c->iwork, Gp, k, Z, k, w, nullptr, c->status_dev);
+      cluster_eig<T>(st(), k, ncl, c->iwork, Gp, k, Zn, k, w, nullptr, c->status_dev);
     }
-    sort_pairs<T>(st(), k, w, Z, k, Wk, c->dwork + 8, c->iwork + k);
+    sort_pairs<T>(st(), k, w, Zn, k, Z, k, c->dwork + 8, c->iwork + k);
     return true;
   }
 

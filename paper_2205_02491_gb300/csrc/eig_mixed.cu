@@ -179,11 +179,10 @@ template <typename T> __global__ void rank_kernel(int k, const double* w, double
 }
 
 template <typename T>
-void sort_pairs(cudaStream_t st, int k, double* w, T* Z, int64_t ldz, T* tmp, double* wtmp, int* perm) {
+void sort_pairs(cudaStream_t st, int k, double* w, const T* Z, int64_t ldz, T* out, int64_t ldo, double* wtmp, int* perm) {
   rank_kernel<T><<<ceil_div(k, 128), 128, 0, st>>>(k, w, wtmp, perm);
   CHASE_CHECK_LAUNCH();
-  permute_cols<T>(st, k, k, Z, ldz, tmp, k, perm);
-  copy_cols<T>(st, k, k, tmp, k, Z, ldz);
+  permute_cols<T>(st, k, k, Z, ldz, out, ldo, perm);
   CHASE_CUDA(cudaMemcpyAsync(w, wtmp, k * sizeof(double), cudaMemcpyDeviceToDevice, st));
 }
 
@@ -192,7 +191,7 @@ void sort_pairs(cudaStream_t st, int k, double* w, T* Z, int64_t ldz, T* tmp, do
   template void cluster_eig<T>(cudaStream_t, int, int, const int*, const T*, int64_t, T*, int64_t, double*, T*,   \
                                int*);                                                                            \
   template void diag_real<T>(cudaStream_t, int, const T*, int64_t, double*);                                     \
-  template void sort_pairs<T>(cudaStream_t, int, double*, T*, int64_t, T*, double*, int*);
+  template void sort_pairs<T>(cudaStream_t, int, double*, const T*, int64_t, T*, int64_t, double*, int*);
 INST(double)
 INST(double2)
 #undef INST

@@ -34,13 +34,23 @@ template <typename T> void scale_cols(cudaStream_t st, int64_t n, int k, T* X, i
 template <typename T>
 void copy_cols(cudaStream_t st, int64_t n, int k, const T* src, int64_t lds, T* dst, int64_t ldd);
 
-// Cholesky G = L L^H (lower, in place, k x k).  info: device int, set > 0 on a non-finite pivot or one
+// Cholesky G = L L^H with L^{-H}, on the stacked matrix Sm = [G; I] (2k x k, ld lds): begin writes the identity, then
+// the columns [jbeg, jend) are factored in order (jbeg a multiple of CHOL_OUTER; the updates of the columns >= jend
+// are the caller's: S[jend.., jend..] -= S[jend.., jbeg..jend] S[jend..k, jbeg..jend]^H over the k rows from jend).
+// At the end rows k.. of Sm hold L^{-H} (upper triangular).  info: device int, set > 0 on a non-finite pivot or one
 // <= pivot_floor.  dep (nullable, k + 1 ints, zeroed by the caller): detection mode, where a finite pivot
-// <= pivot_floor marks its column as numerically dependent (dep[1 + j] = 1, dep[0] counts them) instead
-// of failing; such a column is decoupled (unit pivot, zero below it) and the factorisation goes on.
+// <= pivot_floor marks its column as numerically dependent (dep[1 + j] = 1, dep[0] counts them) instead of failing;
+// such a column is decoupled (unit pivot, zero below it) and the factorisation goes on.
+constexpr int CHOL_OUTER = 128;
+template <typename T> void chol_stack_begin(cudaStream_t st, int k, T* Sm, int64_t lds);
 template <typename T>
-void potrf_lower(cudaStream_t st, int k, T* G, int64_t ldg, int* info, T* work, int64_t work_elems,
-                 double pivot_floor = 0.0, int* dep = nullptr);
+void chol_stack_columns(cudaStream_t st, int k, int jbeg, int jend, T* Sm, int64_t lds, int* info, double pivot_floor,
+                        int* dep);
+// Correction factor F (k x k) of a nearly orthonormal block with Gram matrix Gm: Q F is orthonormal up to the square of
+// Gm - I; upper: F upper triangular (keeps the QR's spans), else the nearest orthonormal block.  dev (device, zeroed
+// by the caller) receives the bits of a float bound of ||Gm - I||_2 (NaN when not finite).
+template <typename T>
+void gram_correction(cudaStream_t st, int k, bool upper, const T* Gm, int64_t ldg, T* F, int64_t ldf, unsigned* dev);
 // Householder QR building blocks (blas_f64.cu): reflector of a column segment (v over x, alpha, real tau),
 // application of one reflector to ncols columns, the panel's reflectors with explicit zeros, the
 // compact-WY factor Tm of a panel from Gv = V^H V, and Q = [I; 0].
@@ -51,13 +61,6 @@ template <typename T> void reflector_panel(cudaStream_t st, int64_t m, int pb, c
 template <typename T> void householder_T(cudaStream_t st, int pb, const T* Gv, const double* tau, T* Tm, int64_t ldt);
 template <typename T> void identity_rect(cudaStream_t st, int64_t n, int k, T* Q, int64_t ldq);
 
-// X <- X L^{-H} (right solve with the lower Cholesky factor), X n x k.
-template <typename T>
-void trsm_right_lh(cudaStream_t st, int64_t n, int k, T* X, int64_t ldx, const T* L, int64_t ldl, T* work,
-                   int64_t work_elems);
-template <typename T> void zero_upper(cudaStream_t st, int k, T* G, int64_t ldg);
-// inverts every CB x CB diagonal block of the lower-triangular L in place (CB = 32)
-template <typename T> void trtri_diag(cudaStream_t st, int k, T* L, int64_t ldl);
 template <typename T> void add_diag(cudaStream_t st, int k, T* G, int64_t ldg, const double* shift_dev, double shift);
 template <typename T> void hermitianize(cudaStream_t st, int k, T* G, int64_t ldg);
 template <typename T> void fro_norm2(cudaStream_t st, int64_t n, int k, const T* X, int64_t ldx, double* out);
@@ -85,7 +88,8 @@ void cluster_eig(cudaStream_t st, int k, int nclusters, const int* cl /* start,s
                  int64_t ldg, T* Z, int64_t ldz, double* w, T* scratch, int* status);
 template <typename T> void diag_real(cudaStream_t st, int k, const T* G, int64_t ldg, double* d);
 template <typename T>
-void sort_pairs(cudaStream_t st, int k, double* w, T* Z, int64_t ldz, T* tmp, double* wtmp, int* perm);
+void sort_pairs(cudaStream_t st, int k, double* w, const T* Z, int64_t ldz, T* out, int64_t ldo, double* wtmp,
+                int* perm);
 
 // Lanczos bounds (Algorithm 1, line 2).  out4 (device) = {b_sup, mu_1, mu_ne, theta_max}.
 // work: at least lanczos_work_elems scalars (monotone in n).
