@@ -606,17 +606,21 @@ template <typename T> struct Solver {
     F* Zf = Gf + (size_t)k * k;
     F* jw = Zf + (size_t)k * k;
     const int64_t jw_elems = (c->work_elems * (int64_t)sizeof(T)) / (int64_t)sizeof(F) - 2 * (int64_t)k * k;
-    if (jw_elems < (int64_t)k * k + 3 * (int64_t)k + 8) return false;
+    if (jw_elems < 2 * (int64_t)k * k) return false;
     dbg_finite(G, k, k, k, sizeof(T), "G before the FP32 pass");
     convert_mat<T, F>(st(), k, G, k, Gf, k);
+    int block_sweeps = 0;
     try {
-      // block Jacobi for quotients of a few blocks and more (its rounds scale with k / 32, not k); the scalar
-      // cooperative sweep below that
-      if (k >= 128 && jw_elems >= (int64_t)k * k + heev_block_workspace(k))
+      // up to 64 columns in one block; a cooperative launch per sweep of scalar rotations up to 127; block Jacobi
+      // beyond (its rounds scale with k / 32, not k)
+      if (k <= 64) {
+        heev_block<F>(st(), k, Gf, k, w, Zf, k, c->status_dev + 1, 3e-6f, 40);
+        CHASE_CUDA(cudaMemcpyAsync(&block_sweeps, c->status_dev + 1, sizeof(int), cudaMemcpyDeviceToHost, st()));
+      } else if (k >= 128 && jw_elems >= (int64_t)k * k + heev_block_workspace(k)) {
         c->stats.rr_sweeps += heev_block_jacobi<F>(st(), k, Gf, k, w, Zf, k, jw, jw_elems, c->dwork, c->iwork, 3e-6, 40);
-      else
-        c->stats.rr_sweeps += heev_jacobi<F>(st(), k, Gf, k, w, Zf, k, jw, jw_elems, c->dwork, c->iwork, 3e-6, 40,
-                                             false, true);
+      } else {
+        c->stats.rr_sweeps += heev_sweep<F>(st(), k, Gf, w, Zf, k, jw, jw_elems, c->dwork, c->iwork, 3e-6, 40);
+      }
     } catch (const Error& e) {
       // non-finite FP32 values: G itself is untouched and the FP64 solver takes over; a grid barrier
       // that hit its wait limit is reported as CHASE_ERR_TIMEOUT
@@ -629,6 +633,8 @@ template <typename T> struct Solver {
     CHASE_CUDA(cudaMemcpyAsync(&ends[0], w, sizeof(double), cudaMemcpyDeviceToHost, st()));
     CHASE_CUDA(cudaMemcpyAsync(&ends[1], w + (k - 1), sizeof(double), cudaMemcpyDeviceToHost, st()));
     CHASE_CUDA(cudaStreamSynchronize(st()));
+    if (block_sweeps < 0) return false;  // non-finite FP32 values
+    c->stats.rr_sweeps += block_sweeps;
     const double scale = std::max(std::fabs(ends[0]), std::fabs(ends[1]));
     if (!(scale > 0.0) || !std::isfinite(scale)) return false;
     const double omega = 1e-5 * scale;
@@ -669,21 +675,21 @@ template <typename T> struct Solver {
       e3.gamma = 1.0;
       gemm(OP_N, Zn, k, OP_N, X, k, k, k, k, e3, CHASE_FP64);  // Z (I + X)
     }
+    // a block too far from orthonormal for the corrections (or not finite) is left to the FP64 solver
+    float far = 0.f;
+    CHASE_CUDA(cudaMemcpyAsync(&far, dev, sizeof(float), cudaMemcpyDeviceToHost, st()));
     // eigenvalues: diagonal of G', clusters solved exactly
     diag_real<T>(st(), k, Gp, k, w);
     std::vector<double> d(k);
     CHASE_CUDA(cudaMemcpyAsync(d.data(), w, k * sizeof(double), cudaMemcpyDeviceToHost, st()));
     CHASE_CUDA(cudaStreamSynchronize(st()));
+    if (!(far < CORRECT_MAX)) return false;
     std::vector<int> cl;
-    // a block too far from orthonormal for the corrections (or not finite) is left to the FP64 solver
-    float far = 0.f;
-    CHASE_CUDA(cudaMemcpyAsync(&far, dev, sizeof(float), cudaMemcpyDeviceToHost, st()));
     for (int i = 0; i < k;) {
       int j = i + 1;
       while (j < k && std::fabs(d[j] - d[j - 1]) <= omega) ++j;
       if (j - i > 1) {
         if (j - i > 32) return false;
-    if (!(far < CORRECT_MAX)) return false;
         cl.push_back(i);
         cl.push_back(j - i);
       }
@@ -717,10 +723,10 @@ template <typename T> struct Solver {
     hermitianize<T>(st(), k, Gb(), k);
     dbg_finite(Gb(), k, k, k, sizeof(T), "the Rayleigh quotient");
     dbg_finite(Wb, n, k, n, sizeof(T), "A Q");
-    // FP32 Jacobi + FP64-class refinement for large quotients (scratch: the Ritz-vector buffer, unused
+    // FP32 Jacobi + FP64-class refinement from 8 columns on (scratch: the Ritz-vector buffer, unused
     // until the back-transform); the FP64 Jacobi otherwise and as the fallback
     bool done = false;
-    if (rmode != CHASE_FP64_NATIVE && k >= 64 && n >= 3 * (int64_t)k) {
+    if (rmode != CHASE_FP64_NATIVE && k >= 8 && n >= 3 * (int64_t)k) {
       done = eigh_mixed(k, ritz, Tv);  // leaves G intact, so the fallback below can still use it
       if (!done) {
         c->stats.rr_fallbacks++;

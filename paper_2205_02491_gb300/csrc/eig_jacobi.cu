@@ -194,91 +194,6 @@ __global__ void jacobi_apply_z_kernel(int k, int kp, int r, T* Z, int64_t ldz, c
   jacobi_apply_z<T>(k, kp, r, i, pi, Z, ldz, rot);
 }
 
-// ---------------------------------------------------------------- persistent sweep
-// One cooperative launch runs all kp-1 rounds of a sweep: rotation parameters, then the G and Z
-// updates, separated by grid-wide barriers (all blocks are co-resident under a cooperative
-// launch).  Every barrier wait is bounded by a wall-clock limit; on expiry, or when another block
-// has flagged an error, the block sets/keeps the error flag and returns.
-constexpr int SWEEP_THREADS = 256;  // up to four blocks per SM (measured faster than one 1024-thread block)
-// barrier words, each in its own 32-byte sector so that the pollers of the generation word do not
-// contend with the arrival atomics
-constexpr int BAR_COUNT = 0, BAR_GEN = 8, BAR_ERR = 16, BAR_WORDS = 17;
-
-__device__ __forceinline__ unsigned long long gtimer() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-// bar[BAR_COUNT]: arrivals, bar[BAR_GEN]: generation, bar[BAR_ERR]: error flag (all zero at launch);
-// wait_ns: wall-clock limit of one wait
-__device__ bool grid_barrier(unsigned* bar, unsigned nblocks, unsigned long long wait_ns) {
-  __shared__ int ok_sh;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    volatile unsigned* vb = bar;
-    int ok = vb[BAR_ERR] == 0u;
-    if (ok) {
-      const unsigned gen = vb[BAR_GEN];
-      __threadfence();
-      if (atomicAdd(&bar[BAR_COUNT], 1u) == nblocks - 1) {
-        atomicExch(&bar[BAR_COUNT], 0u);
-        __threadfence();
-        atomicAdd(&bar[BAR_GEN], 1u);
-      } else {
-        const unsigned long long t0 = gtimer();
-        while (vb[BAR_GEN] == gen) {
-          if (vb[BAR_ERR] != 0u) {
-            ok = 0;
-            break;
-          }
-          if (gtimer() - t0 > wait_ns) {
-            atomicOr(&bar[BAR_ERR], 1u);
-            ok = 0;
-            break;
-          }
-          __nanosleep(100);
-        }
-      }
-      __threadfence();
-    }
-    ok_sh = ok;
-  }
-  __syncthreads();
-  return ok_sh != 0;
-}
-
-template <typename T>
-__global__ void __launch_bounds__(SWEEP_THREADS, 4) jacobi_sweep_kernel(int k, int kp, T* G, int64_t ldg, T* Z,
-                                                                        int64_t ldz, Rot<T>* rot, unsigned* bar,
-                                                                        unsigned long long wait_ns) {
-  const int half = kp / 2;
-  const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t nthr = (int64_t)gridDim.x * blockDim.x;
-  const int64_t ng = (int64_t)half * half, nz = (int64_t)k * half;
-  for (int r = 0; r < kp - 1; ++r) {
-    for (int64_t idx = tid; idx < half; idx += nthr) jacobi_params<T>(k, kp, r, (int)idx, G, ldg, rot);
-    if (!grid_barrier(bar, gridDim.x, wait_ns)) return;
-    for (int64_t x = tid; x < ng; x += nthr) jacobi_apply_g<T>(k, kp, r, (int)(x % half), (int)(x / half), G, ldg, rot);
-    for (int64_t x = tid; x < nz; x += nthr) jacobi_apply_z<T>(k, kp, r, (int)(x % k), (int)(x / k), Z, ldz, rot);
-    if (!grid_barrier(bar, gridDim.x, wait_ns)) return;
-  }
-}
-
-// co-resident blocks of SWEEP_THREADS threads for the sweep kernel (0: no cooperative launch)
-template <typename T> static int sweep_grid() {
-  static const int nb = []() {
-    int dev = 0, sms = 0, per = 0, coop = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-    if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop) return 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, jacobi_sweep_kernel<T>, SWEEP_THREADS, 0) != cudaSuccess)
-      return 0;
-    return sms * std::min(per, 4);
-  }();
-  return nb;
-}
-
 template <typename T> __global__ void set_identity_kernel(int k, T* Z, int64_t ldz) {
   int i = blockIdx.x * blockDim.x + threadIdx.x, j = blockIdx.y;
   if (i < k) Z[i + (int64_t)j * ldz] = (i == j) ? S<T>::one() : S<T>::zero();
@@ -345,7 +260,7 @@ __global__ void diag_rank_kernel(int k, const T* __restrict__ G, int64_t ldg, do
 
 template <typename T>
 int heev_jacobi(cudaStream_t st, int k, T* G, int64_t ldg, double* w, T* Z, int64_t ldz, T* work, int64_t work_elems,
-                double* dwork, int* iwork, double tol, int max_sweeps, bool require_convergence, bool persistent) {
+                double* dwork, int* iwork, double tol, int max_sweeps) {
   // work: k*k scalars for the unsorted Z plus Rot array; dwork: 2k+2 doubles; iwork: k ints
   CHASE_REQUIRE(work_elems >= (int64_t)k * k + 3 * (int64_t)k + 8, 2, "heev_jacobi: workspace too small");
   if (k <= 0) return 0;
@@ -358,27 +273,13 @@ int heev_jacobi(cudaStream_t st, int k, T* G, int64_t ldg, double* w, T* Z, int6
   double hstat[2];
   int sweeps = 0;
   bool done = false;
-  // one cooperative launch per sweep; the barrier words live in iwork[0, BAR_WORDS) (k >= 64 ints;
-  // overwritten by the final ranking only after the sweeps)
-  // grid sized by the work of a round (about 4 rotation updates per thread), at most the co-resident
-  // maximum: small quotients take few SMs, which leaves room for other streams' kernels
-  int coop_grid = (persistent && k >= 64) ? sweep_grid<T>() : 0;
-  if (coop_grid > 0) {
-    const int64_t items = (int64_t)(kp / 2) * (kp / 2) + (int64_t)k * (kp / 2);
-    coop_grid = (int)std::max<int64_t>(1, std::min<int64_t>(coop_grid, ceil_div(items, 4 * SWEEP_THREADS)));
-  }
-  unsigned* bar = reinterpret_cast<unsigned*>(iwork);
-  unsigned bar_err = 0;
   for (; sweeps <= max_sweeps; ++sweeps) {
     offdiag_partial_kernel<T><<<k, 128, 0, st>>>(k, G, ldg, part);
     CHASE_CHECK_LAUNCH();
     offdiag_sum_kernel<<<1, 32, 0, st>>>(k, part, dwork);
     CHASE_CHECK_LAUNCH();
     CHASE_CUDA(cudaMemcpyAsync(hstat, dwork, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
-    if (coop_grid > 0 && sweeps > 0)
-      CHASE_CUDA(cudaMemcpyAsync(&bar_err, bar + BAR_ERR, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
     CHASE_CUDA(cudaStreamSynchronize(st));
-    CHASE_REQUIRE(bar_err == 0, 8, "heev_jacobi: a grid barrier of the sweep kernel hit its wait limit");
     CHASE_REQUIRE(isfinite(hstat[0]) && isfinite(hstat[1]), 5, "heev_jacobi: non-finite matrix");
     if (sqrt(hstat[0]) <= tol * sqrt(hstat[1]) || k == 1) {
       done = true;
@@ -388,34 +289,386 @@ int heev_jacobi(cudaStream_t st, int k, T* G, int64_t ldg, double* w, T* Z, int6
     int half = kp / 2;
     dim3 gblk(16, 16), ggrid(ceil_div(half, 16), ceil_div(half, 16));
     dim3 zgrid(ceil_div(k, 128), half);
-    if (coop_grid > 0) {
-      CHASE_CUDA(cudaMemsetAsync(bar, 0, BAR_WORDS * sizeof(unsigned), st));
-      int kk = k, kpp = kp;
-      int64_t ldgg = ldg, ldzz = k;
-      T* Gp = G;
-      T* Zp = Zu;
-      Rot<T>* rp = rot;
-      unsigned long long wait_ns = grid_wait_limit_ns();
-      void* args[] = {&kk, &kpp, &Gp, &ldgg, &Zp, &ldzz, &rp, &bar, &wait_ns};
-      CHASE_CUDA(cudaLaunchCooperativeKernel((const void*)jacobi_sweep_kernel<T>, dim3(coop_grid), dim3(SWEEP_THREADS),
-                                             args, 0, st));
+    for (int r = 0; r < kp - 1; ++r) {
+      jacobi_params_kernel<T><<<ceil_div(half, 128), 128, 0, st>>>(k, kp, r, G, ldg, rot);
       CHASE_CHECK_LAUNCH();
-    } else {
-      for (int r = 0; r < kp - 1; ++r) {
-        jacobi_params_kernel<T><<<ceil_div(half, 128), 128, 0, st>>>(k, kp, r, G, ldg, rot);
-        CHASE_CHECK_LAUNCH();
-        jacobi_apply_g_kernel<T><<<ggrid, gblk, 0, st>>>(k, kp, r, G, ldg, rot);
-        CHASE_CHECK_LAUNCH();
-        jacobi_apply_z_kernel<T><<<zgrid, 128, 0, st>>>(k, kp, r, Zu, k, rot);
-        CHASE_CHECK_LAUNCH();
-      }
+      jacobi_apply_g_kernel<T><<<ggrid, gblk, 0, st>>>(k, kp, r, G, ldg, rot);
+      CHASE_CHECK_LAUNCH();
+      jacobi_apply_z_kernel<T><<<zgrid, 128, 0, st>>>(k, kp, r, Zu, k, rot);
+      CHASE_CHECK_LAUNCH();
     }
   }
-  CHASE_REQUIRE(done || !require_convergence, 8, "heev_jacobi: sweep cap reached without convergence");
+  CHASE_REQUIRE(done, 8, "heev_jacobi: sweep cap reached without convergence");
   diag_rank_kernel<T><<<ceil_div(k, 128), 128, 0, st>>>(k, G, ldg, w, iwork);
   CHASE_CHECK_LAUNCH();
   permute_cols<T>(st, k, k, Zu, k, Z, ldz, iwork);
   return sweeps;
+}
+
+// ---------------------------------------------------------------- FP32 rotations
+// realness of a diagonal entry without a round trip through double
+__device__ __forceinline__ void bj_real(float& a) {}
+__device__ __forceinline__ void bj_real(float2& a) { a.y = 0.0f; }
+
+// Rotation that zeroes g in [[a, g], [conj g, b]]: phase ph = conj(g)/|g|, then c, sn.  All in FP32 (GB300's FP64 runs
+// at 1/64 of it, and this is the serial part of a round), but each pair is brought back to unit length by one Newton
+// step on a residual computed without cancellation, so c^2 + sn^2 and |ph| are off by their own rounding only, as if
+// rounded from FP64 (plain FP32 parameters raise the pass's rounding floor above what the FP64 corrections that follow
+// can absorb for close eigenvalues).
+template <typename F> struct Givens {
+  float c, sn;
+  F ph;
+};
+__device__ __forceinline__ float phase_of(float g, float& ag) {
+  ag = fabsf(g);
+  return g < 0.0f ? -1.0f : 1.0f;
+}
+__device__ __forceinline__ float2 phase_of(float2 g, float& ag) {
+  const float x = fabsf(g.x), y = fabsf(g.y), m = fmaxf(x, y), r = __fdividef(fminf(x, y), m);
+  ag = m * sqrtf(fmaf(r, r, 1.0f));
+  const float inv = 1.0f / ag;
+  float2 ph = make_float2(g.x * inv, -g.y * inv);
+  const float d = 0.5f * fmaf(-ph.y, ph.y, fmaf(-ph.x, ph.x, 1.0f));
+  return make_float2(fmaf(ph.x, d, ph.x), fmaf(ph.y, d, ph.y));
+}
+__device__ __forceinline__ float largest(float g) { return fabsf(g); }
+__device__ __forceinline__ float largest(float2 g) { return fmaxf(fabsf(g.x), fabsf(g.y)); }
+__device__ __forceinline__ float real_of(float g) { return g; }
+__device__ __forceinline__ float real_of(float2 g) { return g.x; }
+
+template <typename F> __device__ __forceinline__ Givens<F> givens(F a, F b, F g) {
+  Givens<F> o;
+  o.c = 1.0f;
+  o.sn = 0.0f;
+  o.ph = S<F>::one();
+  if (!(largest(g) > 1e-30f)) return o;
+  float ag;
+  o.ph = phase_of(g, ag);
+  const float z = (real_of(b) - real_of(a)) / (2.0f * ag);
+  const float az = fabsf(z);
+  // t = sign(z) / (|z| + sqrt(1 + z^2)); from |z| = 1e4 on the square root is |z| to FP32
+  const float t = copysignf(1.0f / (az + (az < 1e4f ? sqrtf(fmaf(z, z, 1.0f)) : az)), z);
+  const float c = rsqrtf(fmaf(t, t, 1.0f)), sn = t * c;
+  const float d = 0.5f * fmaf(-sn, sn, fmaf(-c, c, 1.0f));
+  o.c = fmaf(c, d, c);
+  o.sn = fmaf(sn, d, sn);
+  return o;
+}
+
+// (p, q) <- (c p - sn ph q, sn p + c ph q): columns p, q of a row times J = [[c, sn], [-sn ph, c ph]]; rows take conj(ph)
+__device__ __forceinline__ void rotate(float& p, float& q, float c, float sn, float ph) {
+  const float y = q * ph, x = p;
+  p = fmaf(c, x, -sn * y);
+  q = fmaf(sn, x, c * y);
+}
+__device__ __forceinline__ void rotate(float2& p, float2& q, float c, float sn, float2 ph) {
+  const float2 y = make_float2(fmaf(q.x, ph.x, -q.y * ph.y), fmaf(q.x, ph.y, q.y * ph.x)), x = p;
+  p = make_float2(fmaf(c, x.x, -sn * y.x), fmaf(c, x.y, -sn * y.y));
+  q = make_float2(fmaf(sn, x.x, c * y.x), fmaf(sn, x.y, c * y.y));
+}
+
+// ---------------------------------------------------------------- persistent sweep
+// FP32 first pass of quotients of 65 to 127 columns: one cooperative launch runs all kp-1 rounds of a sweep.  A round is
+// one phase and one grid-wide barrier (all blocks are co-resident under a cooperative launch): every item works
+// out the rotations it needs from the old G (FP32, a few tens of instructions) and writes the other of two copies, so
+// nothing waits for a parameter pass; Z items own their entries.  With a parameter phase in FP64 and two barriers a
+// round took 10 us.  Every barrier wait is bounded by a wall-clock limit; on expiry, or when another block has flagged an
+// error, the block sets/keeps the error flag and returns.
+constexpr int SWEEP_THREADS = 256;  // up to four blocks per SM (measured faster than one 1024-thread block)
+// barrier words, each in its own 32-byte sector so that the pollers of the generation word do not
+// contend with the arrival atomics
+constexpr int BAR_COUNT = 0, BAR_GEN = 8, BAR_ERR = 16, BAR_WORDS = 17;
+
+__device__ __forceinline__ unsigned long long gtimer() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
+// bar[BAR_COUNT]: arrivals, bar[BAR_GEN]: generation, bar[BAR_ERR]: error flag (all zero at launch);
+// wait_ns: wall-clock limit of one wait
+__device__ bool grid_barrier(unsigned* bar, unsigned nblocks, unsigned long long wait_ns) {
+  __shared__ int ok_sh;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    volatile unsigned* vb = bar;
+    int ok = vb[BAR_ERR] == 0u;
+    if (ok) {
+      const unsigned gen = vb[BAR_GEN];
+      __threadfence();
+      if (atomicAdd(&bar[BAR_COUNT], 1u) == nblocks - 1) {
+        atomicExch(&bar[BAR_COUNT], 0u);
+        __threadfence();
+        atomicAdd(&bar[BAR_GEN], 1u);
+      } else {
+        const unsigned long long t0 = gtimer();
+        while (vb[BAR_GEN] == gen) {
+          if (vb[BAR_ERR] != 0u) {
+            ok = 0;
+            break;
+          }
+          if (gtimer() - t0 > wait_ns) {
+            atomicOr(&bar[BAR_ERR], 1u);
+            ok = 0;
+            break;
+          }
+          __nanosleep(100);
+        }
+      }
+      __threadfence();
+    }
+    ok_sh = ok;
+  }
+  __syncthreads();
+  return ok_sh != 0;
+}
+
+template <typename F>
+__device__ __forceinline__ Givens<F> pair_rotation(int k, int p, int q, const F* G, int64_t ldg) {
+  // the dummy index of an odd k rotates nothing
+  if (p >= k || q >= k) return givens<F>(S<F>::zero(), S<F>::zero(), S<F>::zero());
+  return givens<F>(G[p + (int64_t)p * ldg], G[q + (int64_t)q * ldg], G[p + (int64_t)q * ldg]);
+}
+
+// Starts from Ga; the result of the kp - 1 (odd) rounds is in Gb.  Plain loads: other blocks write between barriers.
+template <typename F>
+__global__ void __launch_bounds__(SWEEP_THREADS, 4) jacobi_sweep_kernel(int k, int kp, F* Ga, F* Gb, F* Z, unsigned* bar,
+                                                                        unsigned long long wait_ns) {
+  using s = S<F>;
+  const int half = kp / 2;
+  const int tid = blockIdx.x * blockDim.x + threadIdx.x, nthr = gridDim.x * blockDim.x;
+  const int ng = half * half, nz = k * half;
+  const int64_t ld = k;
+  for (int r = 0; r < kp - 1; ++r) {
+    const F* Go = (r & 1) ? Gb : Ga;
+    F* Gn = (r & 1) ? Ga : Gb;
+    for (int x = tid; x < ng; x += nthr) {
+      const int i1 = x % half, i2 = x / half;
+      int p1, q1, p2, q2;
+      round_pair(r, i1, kp, p1, q1);
+      round_pair(r, i2, kp, p2, q2);
+      const Givens<F> jr = pair_rotation<F>(k, p1, q1, Go, ld), jc = pair_rotation<F>(k, p2, q2, Go, ld);
+      const bool a = p1 < k, b = q1 < k, c = p2 < k, d = q2 < k;
+      F tt = a && c ? Go[p1 + p2 * ld] : s::zero(), tb = a && d ? Go[p1 + q2 * ld] : s::zero();
+      F bt = b && c ? Go[q1 + p2 * ld] : s::zero(), bb = b && d ? Go[q1 + q2 * ld] : s::zero();
+      rotate(tt, tb, jc.c, jc.sn, jc.ph);
+      rotate(bt, bb, jc.c, jc.sn, jc.ph);
+      rotate(tt, bt, jr.c, jr.sn, s::conj(jr.ph));
+      rotate(tb, bb, jr.c, jr.sn, s::conj(jr.ph));
+      if (i1 == i2) {
+        bj_real(tt);
+        bj_real(bb);
+        tb = bt = s::zero();
+      }
+      if (a && c) Gn[p1 + p2 * ld] = tt;
+      if (a && d) Gn[p1 + q2 * ld] = tb;
+      if (b && c) Gn[q1 + p2 * ld] = bt;
+      if (b && d) Gn[q1 + q2 * ld] = bb;
+    }
+    for (int x = tid; x < nz; x += nthr) {
+      const int i = x % k;
+      int p, q;
+      round_pair(r, x / k, kp, p, q);
+      if (p >= k || q >= k) continue;
+      const Givens<F> j = pair_rotation<F>(k, p, q, Go, ld);
+      F zp = Z[i + p * ld], zq = Z[i + q * ld];
+      rotate(zp, zq, j.c, j.sn, j.ph);
+      Z[i + p * ld] = zp;
+      Z[i + q * ld] = zq;
+    }
+    if (!grid_barrier(bar, gridDim.x, wait_ns)) return;
+  }
+}
+
+// co-resident blocks of SWEEP_THREADS threads for the sweep kernel (0: no cooperative launch)
+template <typename F> static int sweep_grid() {
+  static const int nb = []() {
+    int dev = 0, sms = 0, per = 0, coop = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+    if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) != cudaSuccess || !coop) return 0;
+    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, jacobi_sweep_kernel<F>, SWEEP_THREADS, 0) != cudaSuccess)
+      return 0;
+    return sms * std::min(per, 4);
+  }();
+  return nb;
+}
+
+template <typename F>
+int heev_sweep(cudaStream_t st, int k, F* G, double* w, F* Z, int64_t ldz, F* work, int64_t work_elems, double* dwork,
+               int* iwork, double tol, int max_sweeps) {
+  CHASE_REQUIRE(k >= BAR_WORDS && work_elems >= 2 * (int64_t)k * k, 2, "heev_sweep: workspace too small");
+  F* Zu = work;
+  F* buf[2] = {G, work + (int64_t)k * k};
+  const int kp = k + (k & 1);
+  set_identity_kernel<F><<<dim3(ceil_div(k, 256), k), 256, 0, st>>>(k, Zu, k);
+  CHASE_CHECK_LAUNCH();
+  double* part = dwork + 2;
+  double hstat[2];
+  // grid sized by the work of a round (one item per thread), at most the co-resident maximum: small quotients take
+  // few SMs, which leaves room for other streams' kernels.  The barrier words live in iwork (k ints; overwritten by
+  // the final ranking only after the sweeps).
+  const int items = (kp / 2) * (kp / 2) + k * (kp / 2);
+  const int grid = std::min<int>(sweep_grid<F>(), (int)ceil_div(items, SWEEP_THREADS));
+  CHASE_REQUIRE(grid > 0, 9, "heev_sweep: no cooperative launch on this device");
+  unsigned* bar = reinterpret_cast<unsigned*>(iwork);
+  unsigned bar_err = 0;
+  int sweeps = 0;
+  for (; sweeps <= max_sweeps; ++sweeps) {
+    offdiag_partial_kernel<F><<<k, 128, 0, st>>>(k, buf[0], k, part);
+    CHASE_CHECK_LAUNCH();
+    offdiag_sum_kernel<<<1, 32, 0, st>>>(k, part, dwork);
+    CHASE_CHECK_LAUNCH();
+    CHASE_CUDA(cudaMemcpyAsync(hstat, dwork, 2 * sizeof(double), cudaMemcpyDeviceToHost, st));
+    if (sweeps > 0)
+      CHASE_CUDA(cudaMemcpyAsync(&bar_err, bar + BAR_ERR, sizeof(unsigned), cudaMemcpyDeviceToHost, st));
+    CHASE_CUDA(cudaStreamSynchronize(st));
+    CHASE_REQUIRE(bar_err == 0, 8, "heev_sweep: a grid barrier of the sweep kernel hit its wait limit");
+    CHASE_REQUIRE(isfinite(hstat[0]) && isfinite(hstat[1]), 5, "heev_sweep: non-finite matrix");
+    // the cap is not an error: the FP64 refinement follows
+    if (sqrt(hstat[0]) <= tol * sqrt(hstat[1]) || sweeps == max_sweeps) break;
+    CHASE_CUDA(cudaMemsetAsync(bar, 0, BAR_WORDS * sizeof(unsigned), st));
+    int kk = k, kpp = kp;
+    unsigned long long wait_ns = grid_wait_limit_ns();
+    void* args[] = {&kk, &kpp, &buf[0], &buf[1], &Zu, &bar, &wait_ns};
+    CHASE_CUDA(cudaLaunchCooperativeKernel((const void*)jacobi_sweep_kernel<F>, dim3(grid), dim3(SWEEP_THREADS), args, 0,
+                                           st));
+    CHASE_CHECK_LAUNCH();
+    std::swap(buf[0], buf[1]);
+  }
+  diag_rank_kernel<F><<<ceil_div(k, 128), 128, 0, st>>>(k, buf[0], k, w, iwork);
+  CHASE_CHECK_LAUNCH();
+  permute_cols<F>(st, k, k, Zu, k, Z, ldz, iwork);
+  return sweeps;
+}
+
+// ---------------------------------------------------------------- one-block Jacobi (FP32 first pass, k <= 64)
+// The whole solve in one launch of one CTA: G and Z in shared memory by position (the tournament of bj_solve_kernel
+// below, M = 32 or 64 indices, zero rows and columns past k), sweeps until the off-diagonal norm is below tol or stops
+// falling at FP32's floor.  A launch per round phase and a host check per sweep took about 2 ms for 24 columns.
+// out: sweeps used, or -1 for a non-finite matrix.
+template <typename F, int M>
+__global__ void __launch_bounds__(M * M / 4) jacobi_block_kernel(int k, const F* __restrict__ G, int64_t ldg, float tol,
+                                                                  int max_sweeps, double* w, F* Z, int64_t ldz, int* out) {
+  using s = S<F>;
+  constexpr int H = M / 2, NT = M * M / 4;
+  extern __shared__ __align__(16) unsigned char bj_smem[];
+  F* Sm = reinterpret_cast<F*>(bj_smem);  // [2][M][M]
+  F* Um = Sm + 2 * M * M;                 // [2][M][M]
+  __shared__ Givens<F> prm[2][H];
+  __shared__ double red_off[NT / 32], red_tot[NT / 32];
+  __shared__ float dg[M];
+  const int tid = threadIdx.x, i1 = tid / H, i2 = tid % H;
+  for (int e = tid; e < M * M; e += NT) {
+    const int l = e % M, m = e / M;
+    Sm[m * M + l] = (l < k && m < k) ? s::conj(G[l + (int64_t)m * ldg]) : s::zero();
+    Um[m * M + l] = (l == m) ? s::one() : s::zero();
+  }
+  auto next_top = [](int i) { return i == 0 ? 0 : (i == H - 1 ? M - 1 : i + 1); };
+  auto next_bot = [](int i) { return i == 0 ? 1 : H + i - 1; };
+  const int rt = next_top(i1) * M, rb = next_bot(i1) * M, ct = next_top(i2), cb = next_bot(i2);
+  int cur = 0, sweeps = 0;
+  double prev = 0.0;
+  __syncthreads();
+  for (;; ++sweeps) {
+    const F* Sc = Sm + cur * M * M;
+    double off = 0.0, tot = 0.0;
+    for (int e = tid; e < M * M; e += NT) {
+      const double v = s::abs2(Sc[e]);
+      tot += v;
+      if (e % M != e / M) off += v;
+    }
+    off = warp_sum(off);
+    tot = warp_sum(tot);
+    if ((tid & 31) == 0) {
+      red_off[tid >> 5] = off;
+      red_tot[tid >> 5] = tot;
+    }
+    __syncthreads();
+    off = tot = 0.0;
+    for (int i = 0; i < NT / 32; ++i) {
+      off += red_off[i];
+      tot += red_tot[i];
+    }
+    if (!isfinite(tot)) {
+      if (tid == 0) out[0] = -1;
+      return;
+    }
+    // FP32 floor as in heev_block_jacobi
+    if (off <= (double)tol * tol * tot || sweeps == max_sweeps || (sweeps >= 2 && off > 0.0625 * prev && off <= 1e-10 * tot))
+      break;
+    prev = off;
+    if (tid < H) prm[0][tid] = givens<F>(Sc[tid * (M + 1)], Sc[(H + tid) * (M + 1)], Sc[tid * M + H + tid]);
+    __syncthreads();
+    for (int rr = 0; rr < M - 1; ++rr, cur ^= 1) {
+      const int pb = rr & 1;
+      const F* S0 = Sm + cur * M * M;
+      F* S1 = Sm + (cur ^ 1) * M * M;
+      const F* U0 = Um + cur * M * M;
+      F* U1 = Um + (cur ^ 1) * M * M;
+      const Givens<F> pc = prm[pb][i2], pr = prm[pb][i1];
+      {
+        F tt = S0[i1 * M + i2], tb = S0[i1 * M + H + i2], bt = S0[(H + i1) * M + i2], bb = S0[(H + i1) * M + H + i2];
+        rotate(tt, tb, pc.c, pc.sn, pc.ph);
+        rotate(bt, bb, pc.c, pc.sn, pc.ph);
+        rotate(tt, bt, pr.c, pr.sn, s::conj(pr.ph));
+        rotate(tb, bb, pr.c, pr.sn, s::conj(pr.ph));
+        if (i1 == i2) {
+          bj_real(tt);
+          bj_real(bb);
+          tb = bt = s::zero();
+        }
+        S1[rt + ct] = tt;
+        S1[rt + cb] = tb;
+        S1[rb + ct] = bt;
+        S1[rb + cb] = bb;
+      }
+      __syncthreads();
+      if (tid < H && rr + 1 < M - 1)
+        prm[pb ^ 1][tid] = givens<F>(S1[tid * (M + 1)], S1[(H + tid) * (M + 1)], S1[tid * M + H + tid]);
+      if (tid >= 32) {
+        for (int x = tid - 32; x < M * H; x += NT - 32) {
+          const int l = x / H, c = x % H;
+          const Givens<F> pz = prm[pb][c];
+          F ut = U0[l * M + c], ub = U0[l * M + H + c];
+          rotate(ut, ub, pz.c, pz.sn, pz.ph);
+          U1[l * M + next_top(c)] = ut;
+          U1[l * M + next_bot(c)] = ub;
+        }
+      }
+      __syncthreads();
+    }
+  }
+  // ascending (stable) order of the first k diagonal entries
+  const F* Sf = Sm + cur * M * M;
+  const F* Uf = Um + cur * M * M;
+  if (tid < M) dg[tid] = real_of(Sf[tid * (M + 1)]);
+  __syncthreads();
+  for (int c = tid >> 5; c < k; c += NT / 32) {
+    int rank = 0;
+    for (int j = 0; j < k; ++j) rank += (dg[j] < dg[c]) || (dg[j] == dg[c] && j < c);
+    if ((tid & 31) == 0) w[rank] = dg[c];
+    for (int l = tid & 31; l < k; l += 32) Z[l + (int64_t)rank * ldz] = Uf[l * M + c];
+  }
+  if (tid == 0) out[0] = sweeps;
+}
+
+template <typename F>
+void heev_block(cudaStream_t st, int k, const F* G, int64_t ldg, double* w, F* Z, int64_t ldz, int* out, float tol,
+                int max_sweeps) {
+  CHASE_REQUIRE(k >= 1 && k <= 64, 1, "heev_block: 1 <= k <= 64");
+  static std::once_flag once;
+  static cudaError_t attr = cudaSuccess;
+  std::call_once(once, []() {
+    attr = cudaFuncSetAttribute(jacobi_block_kernel<F, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)(4 * 64 * 64 * sizeof(F)));
+  });
+  CHASE_CUDA(attr);
+  if (k <= 32)
+    jacobi_block_kernel<F, 32><<<1, 256, 4 * 32 * 32 * sizeof(F), st>>>(k, G, ldg, tol, max_sweeps, w, Z, ldz, out);
+  else
+    jacobi_block_kernel<F, 64><<<1, 1024, 4 * 64 * 64 * sizeof(F), st>>>(k, G, ldg, tol, max_sweeps, w, Z, ldz, out);
+  CHASE_CHECK_LAUNCH();
 }
 
 // ---------------------------------------------------------------- block Jacobi (FP32 first pass)
@@ -429,7 +682,6 @@ int heev_jacobi(cudaStream_t st, int k, T* G, int64_t ldg, double* w, T* Z, int6
 // the block width while the arithmetic per sweep stays 4 k^3 multiply-adds.
 constexpr int BJ_B = 32;          // block width
 constexpr int BJ_M = 2 * BJ_B;    // subproblem order
-constexpr int BJ_LD = BJ_M + 1;   // padded shared-memory row length
 constexpr int BJ_SOLVE_THREADS = 1024;
 constexpr int BJ_UPD_THREADS = 256;
 constexpr int BJ_TILE = 64;       // rows (columns) of G or Z per update CTA
@@ -439,146 +691,212 @@ __device__ __forceinline__ int bj_global(int I, int J, int l) {
   return l < BJ_B ? I * BJ_B + l : J * BJ_B + (l - BJ_B);
 }
 
-// realness of a diagonal entry without a round trip through double
-__device__ __forceinline__ void bj_real(float& a) {}
-__device__ __forceinline__ void bj_real(float2& a) { a.y = 0.0f; }
+// A block paired with the padding block has nothing to do, except in a sweep's first round, which annihilates the
+// entries inside the blocks too (the padding's rows and columns read as zero).
+__device__ __forceinline__ bool bj_idle(int I, int J, int nb, int r) {
+  return (I >= nb && J >= nb) || (r != 0 && (I >= nb || J >= nb));
+}
 
+// One block pair's subproblem.  Pair i of a round is (top i, bottom i): rows and columns of S, and columns of U, are
+// stored by position, top i at i and bottom i at 32 + i, and every round writes them to the positions of the next one
+// (two buffers), so that addresses are the same in all rounds, lanes touch consecutive words, and a thread's 2 x 2
+// block of S is its row pair (warp) by its column pair (lane).
+// full: all 63 rounds of the 64 indices' tournament (top 0 fixed, the others move one position around the circle top
+// 1 .. 31, bottom 31 .. 0).  Else only the 32 rounds that pair a top with a bottom index (bottoms move by one): within
+// the two blocks the entries were annihilated in the sweep's first round, and each cross pair is rotated once a sweep.
+// While one warp works out the next round's rotations from the new S, the others apply the current ones to U: a round
+// is bound by its shared-memory traffic (S and U read and written once), about 1250 cycles.
 template <typename F>
 __global__ void __launch_bounds__(BJ_SOLVE_THREADS) bj_solve_kernel(int k, int nbp, int r, const F* G, int64_t ldg,
-                                                                     F* Ubuf, int inner_sweeps) {
+                                                                     F* Ubuf, int full) {
   using s = S<F>;
   extern __shared__ __align__(16) unsigned char bj_smem[];
-  F* Sm = reinterpret_cast<F*>(bj_smem);  // S[l][m] at Sm[l * BJ_LD + m]
-  F* Um = Sm + BJ_M * BJ_LD;              // U[l][m] at Um[l * BJ_LD + m]
-  __shared__ F rself[BJ_M], rother[BJ_M];
+  F* Sm = reinterpret_cast<F*>(bj_smem);    // [2][64][64], row-major by position
+  F* Um = Sm + 2 * BJ_M * BJ_M;             // [2][64][64]: row l, column by position
+  __shared__ Givens<F> prm[2][BJ_B];
   const int nb = (k + BJ_B - 1) / BJ_B;
   int I, J;
   round_pair(r, blockIdx.x, nbp, I, J);
-  if (I >= nb || J >= nb) return;  // paired with the padding block: nothing to do this round
-  const int tid = threadIdx.x;
-  for (int e = tid; e < BJ_M * BJ_M; e += blockDim.x) {
+  if (bj_idle(I, J, nb, r)) return;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  for (int e = tid; e < BJ_M * BJ_M; e += BJ_SOLVE_THREADS) {
     const int l = e % BJ_M, m = e / BJ_M;
     const int gl = bj_global(I, J, l), gm = bj_global(I, J, m);
-    Sm[l * BJ_LD + m] = (gl < k && gm < k) ? G[gl + (int64_t)gm * ldg] : s::zero();
-    Um[l * BJ_LD + m] = (l == m) ? s::one() : s::zero();
+    // row m, column l: the conjugate of the Hermitian matrix's entry (l, m), so that lanes store consecutive words
+    Sm[m * BJ_M + l] = (gl < k && gm < k) ? s::conj(G[gl + (int64_t)gm * ldg]) : s::zero();
+    Um[m * BJ_M + l] = (l == m) ? s::one() : s::zero();
   }
+  // next position of (top | bottom) index i
+  auto next_top = [&](int i) { return !full || i == 0 ? i : (i == BJ_B - 1 ? BJ_M - 1 : i + 1); };
+  auto next_bot = [&](int i) { return full ? (i == 0 ? 1 : BJ_B + i - 1) : BJ_B + ((i + BJ_B - 1) & (BJ_B - 1)); };
+  const int rt = next_top(warp) * BJ_M, rb = next_bot(warp) * BJ_M, ct = next_top(lane), cb = next_bot(lane);
+  const int rounds = full ? BJ_M - 1 : BJ_B;
   __syncthreads();
-  for (int sw = 0; sw < inner_sweeps; ++sw) {
-    for (int rr = 0; rr < BJ_M - 1; ++rr) {
-      if (tid < BJ_M / 2) {
-        int a, b;
-        round_pair(rr, tid, BJ_M, a, b);
-        const int p = min(a, b), q = max(a, b);
-        const bool valid = bj_global(I, J, q) < k && bj_global(I, J, p) < k;
-        const F g = Sm[p * BJ_LD + q];
-        // parameters in FP64 (32 threads, a few operations per round): FP32 parameters raise the pass's
-        // rounding floor above what the FP64 corrections that follow can absorb for close eigenvalues
-        const double ag = sqrt(s::abs2(g));
-        const double app = s::re(Sm[p * BJ_LD + p]), aqq = s::re(Sm[q * BJ_LD + q]);
-        if (!valid || !(ag > 1e-30)) {
-          rself[p] = s::one();
-          rother[p] = s::zero();
-          rself[q] = s::one();
-          rother[q] = s::zero();
-        } else {
-          const double z = (aqq - app) / (2.0 * ag);
-          const double t = (z >= 0.0 ? 1.0 : -1.0) / (fabs(z) + sqrt(1.0 + z * z));
-          const double c = 1.0 / sqrt(1.0 + t * t), sn = t * c;
-          const F ph = s::scale(s::conj(g), 1.0 / ag);  // conj(g)/|g|
-          // J = [[c, sn], [-sn ph, c ph]] on (p, q): J[p][p], J[q][p] for p; J[q][q], J[p][q] for q
-          rself[p] = s::make(c, 0.0);
-          rother[p] = s::scale(ph, -sn);
-          rself[q] = s::scale(ph, c);
-          rother[q] = s::make(sn, 0.0);
-        }
+  if (warp == 0) prm[0][lane] = givens<F>(Sm[lane * BJ_M + lane], Sm[(BJ_B + lane) * (BJ_M + 1)], Sm[lane * BJ_M + BJ_B + lane]);
+  __syncthreads();
+  for (int rr = 0; rr < rounds; ++rr) {
+    const int cur = rr & 1;
+    const F* S0 = Sm + cur * BJ_M * BJ_M;
+    F* S1 = Sm + (cur ^ 1) * BJ_M * BJ_M;
+    const F* U0 = Um + cur * BJ_M * BJ_M;
+    F* U1 = Um + (cur ^ 1) * BJ_M * BJ_M;
+    const Givens<F> pc = prm[cur][lane], pr = prm[cur][warp];
+    {
+      F tt = S0[warp * BJ_M + lane], tb = S0[warp * BJ_M + BJ_B + lane];
+      F bt = S0[(BJ_B + warp) * BJ_M + lane], bb = S0[(BJ_B + warp) * BJ_M + BJ_B + lane];
+      rotate(tt, tb, pc.c, pc.sn, pc.ph);
+      rotate(bt, bb, pc.c, pc.sn, pc.ph);
+      rotate(tt, bt, pr.c, pr.sn, s::conj(pr.ph));
+      rotate(tb, bb, pr.c, pr.sn, s::conj(pr.ph));
+      if (warp == lane) {
+        bj_real(tt);
+        bj_real(bb);
+        tb = bt = s::zero();
       }
-      __syncthreads();
-      // S <- J^H S J on every (row pair, column pair) 2x2 block, U <- U J; each item owns its entries
-      for (int it = tid; it < (BJ_M / 2) * (BJ_M / 2); it += blockDim.x) {
-        const int i1 = it % (BJ_M / 2), i2 = it / (BJ_M / 2);
-        int rows[2], cols[2];
-        round_pair(rr, i1, BJ_M, rows[0], rows[1]);
-        round_pair(rr, i2, BJ_M, cols[0], cols[1]);
-        F in[2][2], cu[2][2];
-#pragma unroll
-        for (int u = 0; u < 2; ++u)
-#pragma unroll
-          for (int v = 0; v < 2; ++v) in[u][v] = Sm[rows[u] * BJ_LD + cols[v]];
-#pragma unroll
-        for (int u = 0; u < 2; ++u)
-#pragma unroll
-          for (int v = 0; v < 2; ++v)
-            cu[u][v] = s::add(s::mul(in[u][v], rself[cols[v]]), s::mul(in[u][1 - v], rother[cols[v]]));
-#pragma unroll
-        for (int u = 0; u < 2; ++u)
-#pragma unroll
-          for (int v = 0; v < 2; ++v) {
-            F o = s::add(s::mul(s::conj(rself[rows[u]]), cu[u][v]), s::mul(s::conj(rother[rows[u]]), cu[1 - u][v]));
-            if (rows[u] == cols[v]) bj_real(o);
-            if (i1 == i2 && u != v) o = s::zero();
-            Sm[rows[u] * BJ_LD + cols[v]] = o;
-          }
+      S1[rt + ct] = tt;
+      S1[rt + cb] = tb;
+      S1[rb + ct] = bt;
+      S1[rb + cb] = bb;
+    }
+    __syncthreads();
+    if (warp == 0) {
+      if (rr + 1 < rounds)
+        prm[cur ^ 1][lane] =
+            givens<F>(S1[lane * BJ_M + lane], S1[(BJ_B + lane) * (BJ_M + 1)], S1[lane * BJ_M + BJ_B + lane]);
+    } else {
+      for (int l = warp - 1; l < BJ_M; l += BJ_SOLVE_THREADS / 32 - 1) {
+        F ut = U0[l * BJ_M + lane], ub = U0[l * BJ_M + BJ_B + lane];
+        rotate(ut, ub, pc.c, pc.sn, pc.ph);
+        U1[l * BJ_M + ct] = ut;
+        U1[l * BJ_M + cb] = ub;
       }
-      for (int it = tid; it < BJ_M * (BJ_M / 2); it += blockDim.x) {
-        const int i = it % BJ_M, pi = it / BJ_M;
-        int a, b;
-        round_pair(rr, pi, BJ_M, a, b);
-        const F ua = Um[i * BJ_LD + a], ub = Um[i * BJ_LD + b];
-        Um[i * BJ_LD + a] = s::add(s::mul(ua, rself[a]), s::mul(ub, rother[a]));
-        Um[i * BJ_LD + b] = s::add(s::mul(ub, rself[b]), s::mul(ua, rother[b]));
+    }
+    __syncthreads();
+  }
+  // after all rounds every index is back at its position
+  const F* Uf = Um + (rounds & 1) * BJ_M * BJ_M;
+  F* U = Ubuf + (int64_t)blockIdx.x * BJ_M * BJ_M;  // row-major
+  for (int e = tid; e < BJ_M * BJ_M; e += BJ_SOLVE_THREADS) U[e] = Uf[e];
+}
+
+// The updates' 64 x 64 x 64 products: out = sum_m v[m][4 consecutive] * w[m][4], per thread 4 x 4 outputs, on packed
+// FP32 pairs (two multiply-adds per instruction).  v is read as it is (re, im pairs, or two reals); w is held twice
+// ({re, re}, {im, im} or {x, x}) so that it multiplies both halves.  Complex outputs are kept as
+// A = sum re(w) v and B = sum im(w) v until the end.
+__device__ __forceinline__ uint64_t pair2(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void unpair2(uint64_t v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t ffma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+template <typename F> struct Tile;
+template <> struct Tile<float2> {
+  static constexpr int DUP = 2;  // 64-bit words per doubled entry
+  uint64_t A[4][4], B[4][4];     // [w index][v index]
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+      for (int j = 0; j < 4; ++j) A[i][j] = B[i][j] = 0ull;
+  }
+  static __device__ __forceinline__ void dup(uint64_t* o, float2 x) {
+    o[0] = pair2(x.x, x.x);
+    o[1] = pair2(x.y, x.y);
+  }
+  // v: 4 consecutive entries; w[i]: doubled entries
+  __device__ __forceinline__ void add(const float2* v, const uint64_t* const (&w)[4]) {
+    const ulonglong2 v01 = *reinterpret_cast<const ulonglong2*>(v), v23 = *reinterpret_cast<const ulonglong2*>(v + 2);
+    const uint64_t vv[4] = {v01.x, v01.y, v23.x, v23.y};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const ulonglong2 d = *reinterpret_cast<const ulonglong2*>(w[i]);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        A[i][j] = ffma2(d.x, vv[j], A[i][j]);
+        B[i][j] = ffma2(d.y, vv[j], B[i][j]);
       }
-      __syncthreads();
     }
   }
-  F* U = Ubuf + (int64_t)blockIdx.x * BJ_M * BJ_M;
-  for (int e = tid; e < BJ_M * BJ_M; e += blockDim.x) {
-    const int l = e % BJ_M, m = e / BJ_M;
-    U[l + m * BJ_M] = Um[l * BJ_LD + m];
+  // conj_v: the product was to take conj(v)
+  __device__ __forceinline__ float2 get(int i, int j, bool conj_v) const {
+    float ar, ai, br, bi;
+    unpair2(A[i][j], ar, ai);
+    unpair2(B[i][j], br, bi);
+    return conj_v ? make_float2(ar + bi, br - ai) : make_float2(ar - bi, ai + br);
   }
-}
+};
+template <> struct Tile<float> {
+  static constexpr int DUP = 1;
+  uint64_t A[4][2];
+  __device__ __forceinline__ void clear() {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) A[i][0] = A[i][1] = 0ull;
+  }
+  static __device__ __forceinline__ void dup(uint64_t* o, float x) { o[0] = pair2(x, x); }
+  __device__ __forceinline__ void add(const float* v, const uint64_t* const (&w)[4]) {
+    const ulonglong2 vv = *reinterpret_cast<const ulonglong2*>(v);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const uint64_t d = *w[i];
+      A[i][0] = ffma2(d, vv.x, A[i][0]);
+      A[i][1] = ffma2(d, vv.y, A[i][1]);
+    }
+  }
+  __device__ __forceinline__ float get(int i, int j, bool) const {
+    float a, b;
+    unpair2(A[i][j >> 1], a, b);
+    return (j & 1) ? b : a;
+  }
+};
 
 // X[:, IJ] <- X[:, IJ] U for a tile of BJ_TILE rows (X = G for blockIdx.z == 0, Z for 1)
 template <typename F>
 __global__ void __launch_bounds__(BJ_UPD_THREADS) bj_cols_kernel(int k, int nbp, int r, F* G, int64_t ldg, F* Z,
                                                                   int64_t ldz, const F* __restrict__ Ubuf) {
   using s = S<F>;
+  using T = Tile<F>;
   extern __shared__ __align__(16) unsigned char bj_smem[];
-  F* Us = reinterpret_cast<F*>(bj_smem);   // BJ_M x BJ_LD
-  F* Xs = Us + BJ_M * BJ_LD;               // BJ_TILE x BJ_LD
+  uint64_t* Us = reinterpret_cast<uint64_t*>(bj_smem);             // [m][c] doubled
+  F* Xs = reinterpret_cast<F*>(Us + BJ_M * BJ_M * T::DUP);         // [m][row]
   const int nb = (k + BJ_B - 1) / BJ_B;
   int I, J;
   round_pair(r, blockIdx.y, nbp, I, J);
-  if (I >= nb || J >= nb) return;
+  if (bj_idle(I, J, nb, r)) return;
   F* X = blockIdx.z == 0 ? G : Z;
   const int64_t ldx = blockIdx.z == 0 ? ldg : ldz;
   const int r0 = blockIdx.x * BJ_TILE;
   const F* U = Ubuf + (int64_t)blockIdx.y * BJ_M * BJ_M;
   const int tid = threadIdx.x;
-  for (int e = tid; e < BJ_M * BJ_M; e += blockDim.x) Us[(e % BJ_M) * BJ_LD + e / BJ_M] = U[e];
-  for (int e = tid; e < BJ_TILE * BJ_M; e += blockDim.x) {
+  for (int e = tid; e < BJ_M * BJ_M; e += BJ_UPD_THREADS) T::dup(Us + e * T::DUP, U[e]);
+  for (int e = tid; e < BJ_TILE * BJ_M; e += BJ_UPD_THREADS) {
     const int i = e % BJ_TILE, l = e / BJ_TILE;
     const int gi = r0 + i, gl = bj_global(I, J, l);
-    Xs[i * BJ_LD + l] = (gi < k && gl < k) ? X[gi + (int64_t)gl * ldx] : s::zero();
+    Xs[l * BJ_TILE + i] = (gi < k && gl < k) ? X[gi + (int64_t)gl * ldx] : s::zero();
   }
   __syncthreads();
-  // thread: one row, BJ_M / 4 columns (c = cq + 4 j)
-  const int i = tid % BJ_TILE, cq = tid / BJ_TILE;
-  F acc[BJ_M / 4];
-#pragma unroll
-  for (int j = 0; j < BJ_M / 4; ++j) acc[j] = s::zero();
+  const int i4 = (tid % 16) * 4, c4 = (tid / 16) * 4;
+  T acc;
+  acc.clear();
+#pragma unroll 4
   for (int m = 0; m < BJ_M; ++m) {
-    const F xv = Xs[i * BJ_LD + m];
-#pragma unroll
-    for (int j = 0; j < BJ_M / 4; ++j) acc[j] = s::fma(xv, Us[m * BJ_LD + cq + 4 * j], acc[j]);
+    const uint64_t* u = Us + (m * BJ_M + c4) * T::DUP;
+    const uint64_t* const w[4] = {u, u + T::DUP, u + 2 * T::DUP, u + 3 * T::DUP};
+    acc.add(Xs + m * BJ_TILE + i4, w);
   }
-  __syncthreads();
 #pragma unroll
-  for (int j = 0; j < BJ_M / 4; ++j) Xs[i * BJ_LD + cq + 4 * j] = acc[j];
-  __syncthreads();
-  for (int e = tid; e < BJ_TILE * BJ_M; e += blockDim.x) {
-    const int ii = e % BJ_TILE, l = e / BJ_TILE;
-    const int gi = r0 + ii, gl = bj_global(I, J, l);
-    if (gi < k && gl < k) X[gi + (int64_t)gl * ldx] = Xs[ii * BJ_LD + l];
+  for (int c = 0; c < 4; ++c) {
+    const int gl = bj_global(I, J, c4 + c);
+    if (gl >= k) continue;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (r0 + i4 + i < k) X[r0 + i4 + i + (int64_t)gl * ldx] = acc.get(c, i, false);
   }
 }
 
@@ -587,45 +905,48 @@ template <typename F>
 __global__ void __launch_bounds__(BJ_UPD_THREADS) bj_rows_kernel(int k, int nbp, int r, F* G, int64_t ldg,
                                                                   const F* __restrict__ Ubuf) {
   using s = S<F>;
+  using T = Tile<F>;
   extern __shared__ __align__(16) unsigned char bj_smem[];
-  F* Us = reinterpret_cast<F*>(bj_smem);   // BJ_M x BJ_LD
-  F* Xs = Us + BJ_M * BJ_LD;               // Xs[l][j]: row l of the pair, column c0 + j (BJ_M x BJ_LD)
+  uint64_t* Xs = reinterpret_cast<uint64_t*>(bj_smem);             // [column j][m] doubled
+  F* Us = reinterpret_cast<F*>(Xs + BJ_M * BJ_TILE * T::DUP);      // [m][l]
   const int nb = (k + BJ_B - 1) / BJ_B;
   int I, J;
   round_pair(r, blockIdx.y, nbp, I, J);
-  if (I >= nb || J >= nb) return;
+  if (bj_idle(I, J, nb, r)) return;
   const int c0 = blockIdx.x * BJ_TILE;
   const F* U = Ubuf + (int64_t)blockIdx.y * BJ_M * BJ_M;
   const int tid = threadIdx.x;
-  for (int e = tid; e < BJ_M * BJ_M; e += blockDim.x) Us[(e % BJ_M) * BJ_LD + e / BJ_M] = U[e];
-  for (int e = tid; e < BJ_M * BJ_TILE; e += blockDim.x) {
+  for (int e = tid; e < BJ_M * BJ_M; e += BJ_UPD_THREADS) Us[e] = U[e];
+  for (int e = tid; e < BJ_M * BJ_TILE; e += BJ_UPD_THREADS) {
     const int l = e % BJ_M, j = e / BJ_M;
     const int gl = bj_global(I, J, l), gj = c0 + j;
-    Xs[l * BJ_LD + j] = (gl < k && gj < k) ? G[gl + (int64_t)gj * ldg] : s::zero();
+    T::dup(Xs + e * T::DUP, (gl < k && gj < k) ? G[gl + (int64_t)gj * ldg] : s::zero());
   }
   __syncthreads();
-  // thread: one column j, BJ_M / 4 rows (l = lq + 4 q); out[l][j] = sum_m conj(U[m][l]) X[m][j]
-  const int j = tid % BJ_TILE, lq = tid / BJ_TILE;
-  F acc[BJ_M / 4];
-#pragma unroll
-  for (int q = 0; q < BJ_M / 4; ++q) acc[q] = s::zero();
+  // out[l][j] = sum_m conj(U[m][l]) X[m][j]
+  const int l4 = (tid % 16) * 4, j4 = (tid / 16) * 4;
+  T acc;
+  acc.clear();
+#pragma unroll 4
   for (int m = 0; m < BJ_M; ++m) {
-    const F xv = Xs[m * BJ_LD + j];
-#pragma unroll
-    for (int q = 0; q < BJ_M / 4; ++q) acc[q] = s::fma(s::conj(Us[m * BJ_LD + lq + 4 * q]), xv, acc[q]);
+    const uint64_t* x = Xs + (j4 * BJ_M + m) * T::DUP;
+    const uint64_t* const w[4] = {x, x + BJ_M * T::DUP, x + 2 * BJ_M * T::DUP, x + 3 * BJ_M * T::DUP};
+    acc.add(Us + m * BJ_M + l4, w);
   }
-  __syncthreads();
 #pragma unroll
-  for (int q = 0; q < BJ_M / 4; ++q) Xs[(lq + 4 * q) * BJ_LD + j] = acc[q];
-  __syncthreads();
-  for (int e = tid; e < BJ_M * BJ_TILE; e += blockDim.x) {
-    const int l = e % BJ_M, jj = e / BJ_M;
-    const int gl = bj_global(I, J, l), gj = c0 + jj;
-    if (gl < k && gj < k) G[gl + (int64_t)gj * ldg] = Xs[l * BJ_LD + jj];
+  for (int j = 0; j < 4; ++j) {
+    const int gj = c0 + j4 + j;
+    if (gj >= k) continue;
+#pragma unroll
+    for (int l = 0; l < 4; ++l) {
+      const int gl = bj_global(I, J, l4 + l);
+      if (gl < k) G[gl + (int64_t)gj * ldg] = acc.get(j, l, true);
+    }
   }
 }
 
-template <typename F> static size_t bj_smem_bytes() { return (size_t)2 * BJ_M * BJ_LD * sizeof(F); }
+template <typename F> static size_t bj_smem_bytes() { return (size_t)BJ_M * BJ_M * (sizeof(F) + 8 * Tile<F>::DUP); }
+template <typename F> static size_t bj_solve_smem_bytes() { return (size_t)4 * BJ_M * BJ_M * sizeof(F); }
 
 int heev_block_workspace(int k) {
   const int nb = (k + BJ_B - 1) / BJ_B;
@@ -647,7 +968,8 @@ int heev_block_jacobi(cudaStream_t st, int k, F* G, int64_t ldg, double* w, F* Z
   static cudaError_t attr = cudaSuccess;
   std::call_once(once, []() {
     const int b = (int)bj_smem_bytes<F>();
-    attr = cudaFuncSetAttribute(bj_solve_kernel<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
+    attr = cudaFuncSetAttribute(bj_solve_kernel<F>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)bj_solve_smem_bytes<F>());
     if (attr == cudaSuccess) attr = cudaFuncSetAttribute(bj_cols_kernel<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
     if (attr == cudaSuccess) attr = cudaFuncSetAttribute(bj_rows_kernel<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
   });
@@ -675,7 +997,7 @@ int heev_block_jacobi(cudaStream_t st, int k, F* G, int64_t ldg, double* w, F* Z
     if (sweeps >= 2 && hstat[0] > 0.0625 * prev_off && sqrt(hstat[0]) <= 1e-5 * sqrt(hstat[1])) break;
     prev_off = hstat[0];
     for (int r = 0; r < nbp - 1; ++r) {
-      bj_solve_kernel<F><<<npairs, BJ_SOLVE_THREADS, bj_smem_bytes<F>(), st>>>(k, nbp, r, G, ldg, Ubuf, 1);
+      bj_solve_kernel<F><<<npairs, BJ_SOLVE_THREADS, bj_solve_smem_bytes<F>(), st>>>(k, nbp, r, G, ldg, Ubuf, r == 0);
       CHASE_CHECK_LAUNCH();
       bj_cols_kernel<F><<<dim3(tiles, npairs, 2), BJ_UPD_THREADS, bj_smem_bytes<F>(), st>>>(k, nbp, r, G, ldg, Zu, k,
                                                                                           Ubuf);
@@ -696,12 +1018,14 @@ template int heev_block_jacobi<float2>(cudaStream_t, int, float2*, int64_t, doub
                                        int64_t, double*, int*, double, int);
 
 template int heev_jacobi<double>(cudaStream_t, int, double*, int64_t, double*, double*, int64_t, double*, int64_t,
-                                 double*, int*, double, int, bool, bool);
+                                 double*, int*, double, int);
 template int heev_jacobi<double2>(cudaStream_t, int, double2*, int64_t, double*, double2*, int64_t, double2*, int64_t,
-                                  double*, int*, double, int, bool, bool);
-template int heev_jacobi<float>(cudaStream_t, int, float*, int64_t, double*, float*, int64_t, float*, int64_t, double*,
-                                int*, double, int, bool, bool);
-template int heev_jacobi<float2>(cudaStream_t, int, float2*, int64_t, double*, float2*, int64_t, float2*, int64_t,
-                                 double*, int*, double, int, bool, bool);
+                                  double*, int*, double, int);
+template int heev_sweep<float>(cudaStream_t, int, float*, double*, float*, int64_t, float*, int64_t, double*, int*, double,
+                               int);
+template int heev_sweep<float2>(cudaStream_t, int, float2*, double*, float2*, int64_t, float2*, int64_t, double*, int*,
+                                double, int);
+template void heev_block<float>(cudaStream_t, int, const float*, int64_t, double*, float*, int64_t, int*, float, int);
+template void heev_block<float2>(cudaStream_t, int, const float2*, int64_t, double*, float2*, int64_t, int*, float, int);
 
 }  // namespace chase

@@ -65,11 +65,20 @@ template <typename T> void add_diag(cudaStream_t st, int k, T* G, int64_t ldg, c
 template <typename T> void hermitianize(cudaStream_t st, int k, T* G, int64_t ldg);
 template <typename T> void fro_norm2(cudaStream_t st, int64_t n, int k, const T* X, int64_t ldx, double* out);
 
-// Parallel cyclic Jacobi: G (k x k, destroyed) -> w ascending, Z.  Returns sweeps used; throws on cap.
+// Parallel cyclic Jacobi (FP64): G (k x k, destroyed) -> w ascending, Z.  Returns sweeps used; throws on cap.
 template <typename T>
 int heev_jacobi(cudaStream_t st, int k, T* G, int64_t ldg, double* w, T* Z, int64_t ldz, T* work,
-                int64_t work_elems, double* dwork, int* iwork, double tol, int max_sweeps,
-                bool require_convergence = true, bool persistent = false);
+                int64_t work_elems, double* dwork, int* iwork, double tol, int max_sweeps);
+
+// FP32 first passes of the mixed eigensolve (the cap on sweeps is not an error: the FP64 refinement follows).
+// heev_block: k <= 64, one launch, nothing waits; out (device int) receives the sweeps, -1 for a non-finite matrix.
+// heev_sweep: one cooperative launch per sweep; G (ld k) destroyed; work: 2 k*k scalars.
+template <typename F>
+void heev_block(cudaStream_t st, int k, const F* G, int64_t ldg, double* w, F* Z, int64_t ldz, int* out, float tol,
+                int max_sweeps);
+template <typename F>
+int heev_sweep(cudaStream_t st, int k, F* G, double* w, F* Z, int64_t ldz, F* work, int64_t work_elems, double* dwork,
+               int* iwork, double tol, int max_sweeps);
 
 // Two-sided block Jacobi (blocks of 32, one CTA per block pair per round) for the FP32 first pass of the
 // mixed eigensolve: G (k x k, destroyed) -> w ascending, Z.  work: k*k + heev_block_workspace(k) scalars.
