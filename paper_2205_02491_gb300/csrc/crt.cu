@@ -2,18 +2,21 @@
 //
 // Every left row / right column x is scaled by a power of two so that its 2-norm is below 2^62 and rounded to
 // integers X (at most half a unit each).  The integer product then satisfies |C_ij| <= ||X_i|| ||Y_j|| < 2^124
-// (Cauchy-Schwarz), and it is determined by its residues modulo NMOD = 14 pairwise coprime moduli m_i <= 512 whose
-// product is M = 2^125.25 (Chinese remainder theorem): 2^124 = 0.42 M < M / 2.  Each residue of X lies in
-// [-256, 256] and is exact in bf16, a product of two residues is at most 2^16, and 256 of them sum to at most 2^24,
-// so FP32 accumulators are exact over chunks of 256 along K.  Complex operands take three real products per modulus
+// (Cauchy-Schwarz), and it is determined by its residues modulo NMOD = 16 pairwise coprime moduli m_i <= 256 whose
+// product is M = 2^125.6 (Chinese remainder theorem): 2^124 = 0.33 M < M / 2.  Each residue of X lies in
+// [-128, 128] and is exact in bf16, a product of two residues is at most 2^14, and 1024 of them sum to at most 2^24,
+// so FP32 accumulators are exact over chunks of 1024 along K.  Complex operands take three real products per modulus
 // instead of four, P1 = Xr Yr, P2 = Xi Yi, P3 = (Xr + Xi)(Yr + Yi): modulo m_i nothing is lost to the sums or to
 // Re = P1 - P2, Im = P3 - P1 - P2.
 //
 // Why residues and not digits: splitting FP64 operands into seven 8-bit digits takes 28 digit-pair products (112 for
 // complex operands) and one accumulator per digit level, which caps the MMA width at 80 columns (44 cycles per MMA,
-// the instruction's floor, for 40 cycles of math).  Residues take 14 (42 complex) products, each a plain bf16 GEMM
+// the instruction's floor, for 40 cycles of math).  Residues take 16 (48 complex) products, each a plain bf16 GEMM
 // with the widest MMA (256 x 256 x 16 on a CTA pair), and round the operands no more coarsely: an entry keeps
 // 62 - log2(norm / |entry|) bits.
+// Why moduli up to 256 and not 512 (residues up to 256 are exact in bf16 too, and 14 moduli suffice): chunks would
+// hold 256 along K, and reading TMEM four times as often stalls the MMAs (n = 8192, 512 columns, 14 real planes:
+// 863 us, against 588 us with a read per 1024), which outweighs the two planes saved.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -39,19 +42,19 @@ using oz::smem_u32;
 // ---------------------------------------------------------------- moduli and reconstruction constants
 typedef unsigned __int128 u128;
 
-// The 14 pairwise coprime integers <= 512 with the largest product (exhaustive search from the top).
-#define CRT_MODULI {512, 511, 509, 505, 503, 501, 499, 493, 491, 487, 481, 479, 473, 467}
+// The 16 pairwise coprime integers <= 256 with the largest product (exhaustive search from the top).
+#define CRT_MODULI {256, 253, 251, 249, 247, 241, 239, 235, 233, 229, 227, 223, 217, 211, 199, 197}
 
 struct Tables {
   int m[NMOD];           // moduli
-  int inv[NMOD];         // round(2^39 / m): nearest-integer quotients of |t| < 2^31 by a multiply and a shift
-  int c1[NMOD], c2[NMOD];  // 2^21 and 2^42 modulo m, in [-256, 256]
+  int inv[NMOD];         // round(2^38 / m): nearest-integer quotients of |t| < 2^30 by a multiply and a shift
+  int c1[NMOD], c2[NMOD];  // 2^21 and 2^42 modulo m, in [-128, 128]
   uint32_t w[NMOD][4];   // (M / m_i) ((M / m_i)^-1 mod m_i): the CRT weights, 32-bit limbs
   uint32_t off[4];       // -BIAS sum_i w_i mod M
   uint64_t Mlo, Mhi;
   float q;               // 2^112 / M
 };
-constexpr int BIAS = 1024;  // added to every residue (at most 3 * 256 + 2 in size) so that the limb products are unsigned
+constexpr int BIAS = 512;  // added to every residue (at most 3 * 128 in size) so that the limb products are unsigned
 
 constexpr int sym_mod(u128 x, int m) {
   int r = (int)(x % (u128)m);
@@ -67,7 +70,7 @@ constexpr Tables make_tables() {
   for (int i = 0; i < NMOD; ++i) {
     const int m = ms[i];
     t.m[i] = m;
-    t.inv[i] = (int)((((uint64_t)1 << 39) + (uint64_t)m / 2) / (uint64_t)m);
+    t.inv[i] = (int)((((uint64_t)1 << 38) + (uint64_t)m / 2) / (uint64_t)m);
     t.c1[i] = sym_mod((u128)1 << 21, m);
     t.c2[i] = sym_mod((u128)1 << 42, m);
     const u128 Mi = M / (u128)m;
@@ -247,21 +250,21 @@ __device__ __forceinline__ Limbs limbs(long long x) {
   return Limbs{(int)(x & 0x1fffff), (int)((x >> 21) & 0x1fffff), (int)(x >> 42)};
 }
 
-// x mod m_i in [-256, 256]: the limbs' residue sum t (|t| < 2^31), then t - m round(t / m).  The quotient's error is
-// below 2^-9 / 2, so |r| <= m / 2 + 1 / 2, which is 256 at most for odd m <= 511 and for m = 512.
+// x mod m_i in [-128, 128]: the limbs' residue sum t (|t| < 2^30), then t - m round(t / m).  The quotient's error is
+// below 2^-9 / 2, so |r| < m / 2 + 1 / 2: at most (m - 1) / 2 for odd m, at most 128 for m = 256.
 __device__ __forceinline__ int residue(const Limbs& x, int i) {
   const int t = x.x0 + x.x1 * cT.c1[i] + x.x2 * cT.c2[i];
-  const int q = (int)(((long long)t * cT.inv[i] + (1ll << 38)) >> 39);
+  const int q = (int)(((long long)t * cT.inv[i] + (1ll << 37)) >> 38);
   return t - q * cT.m[i];
 }
-// sum of two residues brought back to [-256, 256]
+// sum of two residues brought back to [-128, 128]
 __device__ __forceinline__ int residue_sum(int a, int b, int i) {
   int r = a + b;
-  if (r > 256) r -= cT.m[i];
-  if (r < -256) r += cT.m[i];
+  if (r > 128) r -= cT.m[i];
+  if (r < -128) r += cT.m[i];
   return r;
 }
-// two integers |r| <= 256 as packed bf16 (exact: the upper halves of their FP32 images)
+// two integers |r| <= 128 as packed bf16 (exact: the upper halves of their FP32 images)
 __device__ __forceinline__ uint32_t pack_bf16(int a, int b) {
   const float fa = __int_as_float(0x4b400000 + a) - 12582912.0f;
   const float fb = __int_as_float(0x4b400000 + b) - 12582912.0f;
@@ -345,7 +348,7 @@ __global__ void __launch_bounds__(256) residues_rows_kernel(int64_t nvec, int64_
 constexpr int TM = 256;           // rows of a tile: 128 per CTA of the pair
 constexpr int TN = 256;           // columns of a tile at most
 constexpr int TK = 64;            // K per stage: 128 bytes of bf16 (the 128-byte swizzle atom)
-constexpr int CHUNK = 4;          // stages per exact FP32 accumulation (256 along K)
+constexpr int CHUNK = 16;         // stages per exact FP32 accumulation (1024 along K)
 constexpr int STAGES = 6;
 constexpr int STAGE_BYTES = (128 + 128) * TK * 2;  // this CTA's 128 left rows and up to 128 right rows
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
@@ -357,7 +360,7 @@ constexpr unsigned long long TIMEOUT_NS = 2000000000ull;
 template <int G> struct Params {
   CUtensorMap tmA[G];
   CUtensorMap tmB[G];
-  int16_t* R[G];
+  int8_t* R[G];
   int M[G], N[G], nkb[G], mt[G], nt[G], ldr[G];
   int nblk[G];                   // 32-column blocks of the product's columns
   int box_b[G];                  // right rows per copy
@@ -444,7 +447,17 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r) {
         "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
       : "r"(taddr));
 }
-__device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+// waits for this thread's loads; r: the registers read next (in and out, so that no use moves before the wait)
+__device__ __forceinline__ void tmem_wait_ld(uint32_t* r) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]),
+                 "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]),
+                 "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]),
+                 "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
+               :
+               : "memory");
+}
 
 // two FP32 lanes per instruction
 __device__ __forceinline__ uint64_t pack2(uint32_t a, uint32_t b) {
@@ -479,7 +492,7 @@ struct Mod2 {
 // its 128 left rows and half of the right rows of a stage; the leader issues the pair's MMAs into one of two
 // accumulator sets (2 x 256 TMEM columns) and the eight reduction warps of each CTA take a finished chunk modulo m
 // into FP32 registers while the next chunk accumulates in the other set.  At a unit's end they write residues
-// (16-bit); the copies and MMAs of the next unit run meanwhile.
+// (8-bit); the copies and MMAs of the next unit run meanwhile.
 // Register split: 384 threads at 168 (64512 at launch); warps 0-3 give down to 40, warps 4-11 take 232.
 template <int G>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
@@ -644,20 +657,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
         if (!ok) break;
         fence_after();
         const uint32_t src = lane_addr + (uint32_t)(b * 256 + half * hc);
+        // the next 32 columns load while these are reduced (a load's wait covers every load issued before it)
+        uint32_t r[2][32];
+        tmem_ld32(src, r[0]);
 #pragma unroll
         for (int g = 0; g < 4; ++g) {
           if (g * 32 >= hc) continue;
-          uint32_t r[32];
-          tmem_ld32(src + (uint32_t)(g * 32), r);
-          tmem_wait_ld();
-          if (g * 32 + 32 >= hc) {  // the last read of this set: release it before the arithmetic
+          tmem_wait_ld(r[g & 1]);
+          if (g * 32 + 32 < hc) {
+            tmem_ld32(src + (uint32_t)(g * 32 + 32), r[(g + 1) & 1]);
+          } else {  // every read of this set is done: release it before the arithmetic
             fence_before();
             __syncwarp();
             if (lane == 0) arrive_cluster(b ? rel1 : rel0);
           }
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
-            const uint64_t v = pack2(r[2 * j], r[2 * j + 1]);
+            const uint64_t v = pack2(r[g & 1][2 * j], r[g & 1][2 * j + 1]);
             acc[g * 16 + j] = add2(acc[g * 16 + j], mod(v));
           }
         }
@@ -667,14 +683,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
       if (row < gp.M[prob]) {
         const int N = gp.N[prob], ldr = gp.ldr[prob];
         const int c0 = n0 + half * hc;
-        int16_t* out = gp.R[prob] + ((int64_t)(gp.mod0 * gp.np + plane) * N + c0) * ldr + row;
+        int8_t* out = gp.R[prob] + ((int64_t)(gp.mod0 * gp.np + plane) * N + c0) * ldr + row;
 #pragma unroll
         for (int j = 0; j < 64; ++j) {
-          // integers of at most 2^24 / 257 chunks of 257: exact in FP32; residue at most 257 in size
+          // sums of at most 128 per chunk: exact in FP32; residues at most 128 in size, +128 (modulo 256 only) wraps
           const uint64_t v = mod(acc[j]);
           const float lo = __uint_as_float((uint32_t)v), hi = __uint_as_float((uint32_t)(v >> 32));
-          if (2 * j < hc && c0 + 2 * j < N) out[(int64_t)(2 * j) * ldr] = (int16_t)(int)lo;
-          if (2 * j + 1 < hc && c0 + 2 * j + 1 < N) out[(int64_t)(2 * j + 1) * ldr] = (int16_t)(int)hi;
+          if (2 * j < hc && c0 + 2 * j < N) out[(int64_t)(2 * j) * ldr] = (int8_t)(int)lo;
+          if (2 * j + 1 < hc && c0 + 2 * j + 1 < N) out[(int64_t)(2 * j + 1) * ldr] = (int8_t)(int)hi;
         }
       }
     }
@@ -728,7 +744,7 @@ __device__ __forceinline__ double reconstruct(const uint64_t (&a)[4], int e) {
   const uint64_t s1 = a[1] + cT.off[1] + (s0 >> 32);
   const uint64_t s2 = a[2] + cT.off[2] + (s1 >> 32);
   const uint64_t s3 = a[3] + cT.off[3] + (s2 >> 32);
-  // T = s3 2^96 + ...; T / M < 2^15 lies within 0.42 of an integer; FP32 of its top 31 bits is off by 2^-9 at most
+  // T = s3 2^96 + ...; T / M < 2^14 lies within 0.33 of an integer; FP32 of its top 28 bits is off by 2^-9 at most
   const uint32_t q = (uint32_t)__float2int_rn((float)(uint32_t)(s3 >> 16) * cT.q);
   u128 t = ((u128)((s3 << 32) | (uint32_t)s2) << 64) | (u128)((s1 << 32) | (uint32_t)s0);
   const u128 M = ((u128)cT.Mhi << 64) | cT.Mlo;
@@ -736,34 +752,35 @@ __device__ __forceinline__ double reconstruct(const uint64_t (&a)[4], int e) {
   return to_double((__int128)t, e);
 }
 
-// Two rows per thread (one 4-byte load per plane).  HBM-bound on the residues (2 bytes per plane and entry); the
+// Four rows per thread (one 4-byte load per plane).  HBM-bound on the residues (1 byte per plane and entry); the
 // weights' limb products run on the integer pipe.
 template <bool CPLX>
-__global__ void __launch_bounds__(128) combine_kernel(int M, int N, int ldr, const int16_t* __restrict__ R,
-                                                       const int* __restrict__ lex, const int* __restrict__ rex, Epi ep) {
+__global__ void __launch_bounds__(64) combine_kernel(int M, int N, int ldr, const int8_t* __restrict__ R,
+                                                      const int* __restrict__ lex, const int* __restrict__ rex, Epi ep) {
   constexpr int NP = CPLX ? 3 : 1, NC = CPLX ? 2 : 1;
-  const int i0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x), j = blockIdx.y;
+  const int i0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x), j = blockIdx.y;
   if (i0 >= M) return;
-  const int16_t* src = R + (int64_t)j * ldr + i0;
+  const int8_t* src = R + (int64_t)j * ldr + i0;
   const int64_t plane = (int64_t)N * ldr;
-  uint64_t acc[2][NC][4];
+  uint64_t acc[4][NC][4];
 #pragma unroll
-  for (int r = 0; r < 2; ++r)
+  for (int r = 0; r < 4; ++r)
 #pragma unroll
     for (int c = 0; c < NC; ++c)
 #pragma unroll
       for (int l = 0; l < 4; ++l) acc[r][c][l] = 0ull;
-#pragma unroll
+#pragma unroll 4
   for (int i = 0; i < NMOD; ++i) {
-    short2 p[NP];
+    char4 p[NP];
 #pragma unroll
-    for (int k = 0; k < NP; ++k) p[k] = *reinterpret_cast<const short2*>(src + (int64_t)(i * NP + k) * plane);
+    for (int k = 0; k < NP; ++k) p[k] = *reinterpret_cast<const char4*>(src + (int64_t)(i * NP + k) * plane);
 #pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      const int p0 = r ? p[0].y : p[0].x;
+    for (int r = 0; r < 4; ++r) {
+      auto byte = [&](const char4& v) -> int { return r == 0 ? v.x : r == 1 ? v.y : r == 2 ? v.z : v.w; };
+      const int p0 = byte(p[0]);
       uint32_t v[NC];
       if (CPLX) {
-        const int p1 = r ? p[NP - 2].y : p[NP - 2].x, p2 = r ? p[NP - 1].y : p[NP - 1].x;
+        const int p1 = byte(p[NP - 2]), p2 = byte(p[NP - 1]);
         v[0] = (uint32_t)(p0 - p1 + BIAS);
         v[NC - 1] = (uint32_t)(p2 - p0 - p1 + BIAS);
       } else {
@@ -777,7 +794,7 @@ __global__ void __launch_bounds__(128) combine_kernel(int M, int N, int ldr, con
   }
   const int ej = rex[j];
 #pragma unroll
-  for (int r = 0; r < 2; ++r) {
+  for (int r = 0; r < 4; ++r) {
     const int i = i0 + r;
     if (i >= M) return;
     const int ei = lex[i];
@@ -834,7 +851,7 @@ template <int G> static void launch(cudaStream_t st, const Product* ops, int nop
     const int box = 16 * (int)ceil_div(nblk, nt);
     gp.tmA[p] = make_tmap_bf16(o.lpl, o.K, kp, o.M, nmod * np, TK, 128, 1, CU_TENSOR_MAP_SWIZZLE_128B);
     gp.tmB[p] = make_tmap_bf16(o.rpl, o.K, kp, o.N, NMOD * np, TK, box, 1, CU_TENSOR_MAP_SWIZZLE_128B);
-    gp.R[p] = (int16_t*)o.res;
+    gp.R[p] = (int8_t*)o.res;
     gp.M[p] = (int)o.M;
     gp.N[p] = (int)o.N;
     gp.nkb[p] = (int)ceil_div(o.K, TK);
@@ -890,7 +907,7 @@ void multiply(cudaStream_t st, const Product* ops, int nops, int mod0, int nmod,
 template <bool CPLX> void combine(cudaStream_t st, const Product& op) {
   CHASE_REQUIRE(op.N <= 65535, 1, "residue product: too many columns");
   const dim3 grid(ceil_div(op.M, 256), (unsigned)op.N);
-  combine_kernel<CPLX><<<grid, 128, 0, st>>>((int)op.M, (int)op.N, (int)rpad(op.M), (const int16_t*)op.res, op.lex,
+  combine_kernel<CPLX><<<grid, 64, 0, st>>>((int)op.M, (int)op.N, (int)rpad(op.M), (const int8_t*)op.res, op.lex,
                                              op.rex, op.e);
   CHASE_CHECK_LAUNCH();
 }

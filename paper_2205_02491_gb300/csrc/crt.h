@@ -8,18 +8,18 @@
 namespace chase {
 namespace crt {
 
-constexpr int NMOD = 14;  // moduli
+constexpr int NMOD = 16;  // moduli
 // residue planes per modulus: real operands one; complex ones re, im and re + im
 constexpr int planes(bool cplx) { return cplx ? 3 : 1; }
 inline int64_t kpad(int64_t K) { return (K + 7) / 8 * 8; }   // plane row pitch (16-byte rows for TMA)
-inline int64_t rpad(int64_t M) { return (M + 7) / 8 * 8; }   // pitch of the product's residue columns
+inline int64_t rpad(int64_t M) { return (M + 15) / 16 * 16; }   // pitch of the product's residue columns
 
 // Bytes of the residue planes of nvec vectors of length K for nmod moduli
 inline int64_t plane_bytes(int64_t nvec, int64_t K, bool cplx, int nmod) {
   return (int64_t)nmod * planes(cplx) * nvec * kpad(K) * 2;
 }
 // Bytes of the residues of an M x N product (all moduli)
-inline int64_t residue_bytes(int64_t M, int64_t N, bool cplx) { return (int64_t)NMOD * planes(cplx) * N * rpad(M) * 2; }
+inline int64_t residue_bytes(int64_t M, int64_t N, bool cplx) { return (int64_t)NMOD * planes(cplx) * N * rpad(M); }
 
 // Exponents ex[v] with the 2-norm of vector v below 2^ex[v] (NONFINITE when the vector holds a NaN or an
 // infinity): vector = column of the column-major X (K rows), or row when by_rows.

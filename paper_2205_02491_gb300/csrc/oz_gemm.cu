@@ -102,12 +102,12 @@ bool available() {
 
 // ---------------------------------------------------------------- workspace
 // Residues of a product are kept for panels of its columns: at most this many bytes, but at least 256 columns.
-// 6 GB hold the n = 30000, 1600-column block (4 GB) whole.
+// 6 GB hold the n = 30000, 1600-column block (2.3 GB) whole.
 constexpr int64_t RESIDUE_PANEL_BYTES = 6ll << 30;
 
 // The fewest moduli of A's residue planes a workspace holds at a time: with the mixed modes' three digit slices
-// their memory is 24 bytes per complex element of A (16 for real); all 14 moduli take 84 more than those digits
-// (28 for real).
+// their memory is 24 bytes per complex element of A (14 for real); all 16 moduli take 96 bytes beside those digits
+// (32 for real).
 static int fewest_mods(bool complex_) { return complex_ ? 2 : 4; }
 
 static int panel_cols(int64_t n_max, int ne_max, bool complex_) {

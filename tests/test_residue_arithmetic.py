@@ -14,14 +14,14 @@ M = math.prod(MODULI)
 
 
 def test_moduli_are_coprime_and_wide_enough():
-    assert len(MODULI) == 14 and max(MODULI) <= 512
+    assert len(MODULI) == 16 and max(MODULI) <= 256
     for i, a in enumerate(MODULI):
         for b in MODULI[i + 1:]:
             assert math.gcd(a, b) == 1
-    # |C| <= 2^62 2^62 lies inside (-M/2, M/2), 0.08 M away from its ends (the FP32 quotient's slack)
-    assert 2 ** 124 < 0.42 * M and 2 ** 125 <= M < 2 ** 126
-    # 256 products of residues are an exact FP32 sum
-    assert 256 * 256 * 256 <= 2 ** 24
+    # |C| <= 2^62 2^62 lies inside (-M/2, M/2), well away from its ends (the FP32 quotient's slack)
+    assert 2 ** 124 < 0.33 * M and 2 ** 125 <= M < 2 ** 126
+    # 1024 products of residues are an exact FP32 sum
+    assert 1024 * 128 * 128 <= 2 ** 24
 
 
 def sym(x, m):
@@ -33,10 +33,10 @@ def residue(x, m):
     """The kernel's residue of a 63-bit integer: 21-bit limbs, 32-bit sums, quotient by multiply and shift."""
     x0, x1, x2 = x & 0x1fffff, (x >> 21) & 0x1fffff, x >> 42
     t = x0 + x1 * sym(2 ** 21, m) + x2 * sym(2 ** 42, m)
-    assert -2 ** 31 <= t < 2 ** 31
-    inv = (2 ** 39 + m // 2) // m
+    assert -2 ** 30 < t < 2 ** 30
+    inv = (2 ** 38 + m // 2) // m
     assert inv < 2 ** 31
-    q = (t * inv + 2 ** 38) >> 39
+    q = (t * inv + 2 ** 37) >> 38
     return t - q * m
 
 
@@ -48,7 +48,7 @@ def test_residues_stay_in_bf16_range(m):
     xs += [int(v) * m + m // 2 for v in g.integers(-2 ** 52, 2 ** 52, size=1000)]
     for x in xs:
         r = residue(x, m)
-        assert abs(r) <= 256 and (r - x) % m == 0
+        assert abs(r) <= 128 and (r - x) % m == 0
 
 
 def test_products_come_back_exactly():
@@ -70,10 +70,10 @@ def test_products_come_back_exactly():
             p2 = sum(residue(b, m) * residue(d, m) for b, d in zip(xi, yi))
             p3 = sum(residue(a + b, m) * residue(c + d, m) for a, b, c, d in zip(xr, xi, yr, yi))
             p1, p2, p3 = (sym(p, m) for p in (p1, p2, p3))
-            sr += (p1 - p2 + 1024) * wi
-            si += (p3 - p1 - p2 + 1024) * wi
-            assert p1 - p2 + 1024 > 0 and p3 - p1 - p2 + 1024 > 0
-        off = (-1024 * sum(w)) % M
+            sr += (p1 - p2 + 512) * wi
+            si += (p3 - p1 - p2 + 512) * wi
+            assert p1 - p2 + 512 > 0 and p3 - p1 - p2 + 512 > 0
+        off = (-512 * sum(w)) % M
         for s, c in ((sr, cr), (si, ci)):
             t = s + off
             q = int(np.rint(np.float32((t >> 112) & 0xffffffff) * np.float32(2.0 ** 48 / float(M >> 64))))
