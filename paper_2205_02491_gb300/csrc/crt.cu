@@ -347,11 +347,13 @@ __global__ void __launch_bounds__(256) residues_rows_kernel(int64_t nvec, int64_
 // ---------------------------------------------------------------- product kernel
 constexpr int TM = 256;           // rows of a tile: 128 per CTA of the pair
 constexpr int TN = 256;           // columns of a tile at most
-constexpr int TK = 64;            // K per stage: 128 bytes of bf16 (the 128-byte swizzle atom)
-constexpr int CHUNK = 16;         // stages per exact FP32 accumulation (1024 along K)
-constexpr int STAGES = 6;
-constexpr int STAGE_BYTES = (128 + 128) * TK * 2;  // this CTA's 128 left rows and up to 128 right rows
-constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024 + 256;
+constexpr int TK = 64;            // K per copy: 128 bytes of bf16 (the 128-byte swizzle atom)
+constexpr int SK = 2 * TK;        // K per stage
+constexpr int CHUNK = 8;          // stages per exact FP32 accumulation (1024 along K)
+constexpr int A_HALF = 128 * TK * 2;  // this CTA's left rows of a stage, half of its K
+constexpr int MAX_STAGES = 6;
+constexpr int SMEM_RING = 216 * 1024;
+constexpr int SMEM_BYTES = SMEM_RING + 1024 + 256;
 constexpr int NTHREADS = 384;     // warps 0-3: copies, MMA issue, TMEM; warps 4-11: accumulator reduction
 constexpr int EPI_WARPS = 8;
 constexpr int MAXG = 64;          // products per launch
@@ -361,11 +363,13 @@ template <int G> struct Params {
   CUtensorMap tmA[G];
   CUtensorMap tmB[G];
   int8_t* R[G];
-  int M[G], N[G], nkb[G], mt[G], nt[G], ldr[G];
+  int M[G], N[G], K[G], mt[G], nt[G], ldr[G];  // mt: row tiles, in units of `pairs`
   int nblk[G];                   // 32-column blocks of the product's columns
   int box_b[G];                  // right rows per copy
   int unit_begin[G + 1];
   int nprob, mod0, np;           // np: planes per modulus
+  int pairs;                     // CTA pairs per cluster (1 or 2)
+  int stages, stage_bytes;       // ring of the launch (as many stages as its widest right copy leaves room for)
 };
 
 // column blocks of tile n: the nblk 32-column blocks spread evenly over nt tiles
@@ -380,10 +384,10 @@ __device__ __forceinline__ uint32_t cluster_rank() {
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
 }
-// shared::cluster address of this CTA-local address in CTA 0 (the leader) of the pair
-__device__ __forceinline__ uint32_t leader_addr(uint32_t a) {
+// shared::cluster address of this CTA-local address in the given CTA of the cluster
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t a, uint32_t cta) {
   uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(r) : "r"(a));
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(cta));
   return r;
 }
 __device__ __forceinline__ void cluster_sync() {
@@ -391,6 +395,16 @@ __device__ __forceinline__ void cluster_sync() {
 }
 __device__ __forceinline__ void arrive_cluster(uint32_t bar) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+// whether the phase is complete, without waiting
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+  uint32_t done;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(done)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return done != 0;
 }
 // bounded wait: false on expiry (which sets the launch's error flag) or when another role set it
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int* err) {
@@ -415,16 +429,25 @@ __device__ __forceinline__ void tma_load_pair(uint32_t dst, const CUtensorMap* m
       "l"((unsigned long long)map), "r"(bar), "r"(x), "r"(y), "r"(z)
       : "memory");
 }
+// the same into every CTA of the mask, each of which signals its own pair's leader (bar lies in an even CTA)
+__device__ __forceinline__ void tma_load_multicast(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y, int z,
+                                                   uint32_t mask) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes.multicast::cluster "
+      "[%0], [%1, {%3, %4, %5}], [%2], %6;" ::"r"(dst),
+      "l"((unsigned long long)map), "r"(bar), "r"(x), "r"(y), "r"(z), "h"((uint16_t)mask)
+      : "memory");
+}
 __device__ __forceinline__ void mma_pair(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
   asm volatile(
       "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
       "l"(a), "l"(b), "r"(idesc), "r"(acc));
 }
-// arrives on the barrier at this offset in both CTAs when every MMA issued so far has completed
-__device__ __forceinline__ void commit_pair(uint32_t bar) {
+// arrives on the barrier at this offset in the mask's CTAs when every MMA issued so far has completed
+__device__ __forceinline__ void commit_to(uint32_t bar, uint32_t mask) {
   asm volatile(
       "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
-      "h"((uint16_t)3)
+      "h"((uint16_t)mask)
       : "memory");
 }
 // K-major operand tile, 128-byte swizzle: 8-row groups 1024 bytes apart
@@ -493,27 +516,37 @@ struct Mod2 {
 // accumulator sets (2 x 256 TMEM columns) and the eight reduction warps of each CTA take a finished chunk modulo m
 // into FP32 registers while the next chunk accumulates in the other set.  At a unit's end they write residues
 // (8-bit); the copies and MMAs of the next unit run meanwhile.
+// Two pairs may form a cluster: they take neighbouring row tiles of the same columns, and each CTA copies one half (along
+// K) of its right rows for both (multicast), which takes a quarter off the copies' L2 traffic.  A slot is then free
+// when both pairs' MMAs on it are done.
+// What bounds it: the issuing thread, and L2 traffic.  Without any copy, a stage of four MMAs took 720 cycles at any width up to 256
+// columns (512 cycles of math): a barrier check costs it about 200 cycles and the MMA queue is only a few instructions
+// deep.  So a stage holds 128 along K (eight MMAs), and the next stage's barrier is looked at between its halves,
+// while four MMAs are queued.
 // Register split: 384 threads at 168 (64512 at launch); warps 0-3 give down to 40, warps 4-11 take 232.
 template <int G>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
+__global__ void __launch_bounds__(NTHREADS, 1)
     crt_gemm_kernel(const __grid_constant__ Params<G> gp, int* err) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  uint64_t* full = (uint64_t*)(smem + STAGES * STAGE_BYTES);  // leader's: both CTAs' copies of a stage have landed
-  uint64_t* empty = full + STAGES;                            // each CTA's: the stage's MMAs are done
-  uint64_t* acc_full = empty + STAGES;                        // each CTA's: a chunk is complete in set b
+  uint64_t* full = (uint64_t*)(smem + SMEM_RING);             // leader's: both CTAs' copies of a stage have landed
+  uint64_t* empty = full + MAX_STAGES;                        // each CTA's: the stage's MMAs are done
+  uint64_t* acc_full = empty + MAX_STAGES;                    // each CTA's: a chunk is complete in set b
   uint64_t* acc_empty = acc_full + 2;                         // leader's: both CTAs have read set b
   uint64_t* drain = acc_empty + 2;
   uint32_t* tmem_slot = (uint32_t*)(drain + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t rank = cluster_rank();
-  const int cluster = blockIdx.x >> 1, nclusters = gridDim.x >> 1;
+  const uint32_t cta = cluster_rank(), rank = cta & 1, pair = cta >> 1, leader = cta & ~1u;
+  const int pairs = gp.pairs;
+  const int cluster = blockIdx.x / (2 * pairs), nclusters = gridDim.x / (2 * pairs);
+  const uint32_t pair_mask = 3u << (2 * pair), all_mask = (1u << (2 * pairs)) - 1;
   const int total = gp.unit_begin[gp.nprob];
+  const int stages = gp.stages, stage_bytes = gp.stage_bytes;
 
   if (threadIdx.x == 0) {
-    for (int i = 0; i < STAGES; ++i) {
+    for (int i = 0; i < MAX_STAGES; ++i) {
       mbar_init(smem_u32(&full[i]), 1);
-      mbar_init(smem_u32(&empty[i]), 1);
+      mbar_init(smem_u32(&empty[i]), pairs);
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(smem_u32(&acc_full[i]), 1);
@@ -537,9 +570,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
     asm volatile("setmaxnreg.dec.sync.aligned.u32 40;");
     if (warp == 0 && lane == 0) {
       // ---------------------------------------------------------- copies
-      int it = 0;
+      int it = 0, sl = 0;  // stages so far, slot
+      uint32_t ph = 0;     // parity of the slot's round
       bool ok = true;
       int prob = 0;
+      auto advance = [&]() {
+        ++it;
+        if (++sl == stages) {
+          sl = 0;
+          ph ^= 1;
+        }
+      };
       for (int unit = cluster; unit < total && ok; unit += nclusters) {
         while (G > 1 && unit >= gp.unit_begin[prob + 1]) ++prob;
         const int tiles = gp.mt[prob] * gp.nt[prob];
@@ -548,38 +589,49 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
         const int m = t / gp.nt[prob], n = t - m * gp.nt[prob];
         int n0, width;
         tile_cols(gp.nblk[prob], gp.nt[prob], n, n0, width);
-        const int box = gp.box_b[prob];
-        const int y_a = m * TM + (int)rank * 128, y_b = n0 + (int)rank * (width >> 1);
+        const int box = gp.box_b[prob], K = gp.K[prob];
+        const int y_a = (m * pairs + (int)pair) * TM + (int)rank * 128, y_b = n0 + (int)rank * (width >> 1);
         const int z_b = gp.mod0 * gp.np + plane;
-        const uint32_t bytes = 2u * (uint32_t)(128 + box) * TK * 2;
-        const int nkb = gp.nkb[prob];
-        for (int kb = 0; kb < nkb; ++kb, ++it) {
-          const int s = it % STAGES;
-          if (!mbar_wait(smem_u32(&empty[s]), ((it / STAGES) & 1) ^ 1, err)) {
+        const uint32_t half_bytes = (uint32_t)(A_HALF + box * TK * 2);
+        for (int k0 = 0; k0 < K; k0 += SK) {
+          if (!mbar_wait(smem_u32(&empty[sl]), ph ^ 1, err)) {
             ok = false;
             break;
           }
-          if (rank == 0) mbar_expect_tx(smem_u32(&full[s]), bytes);
-          const uint32_t dst = smem_u32(smem + s * STAGE_BYTES), bar = leader_addr(smem_u32(&full[s]));
-          tma_load_pair(dst, &gp.tmA[prob], bar, kb * TK, y_a, plane);
-          tma_load_pair(dst + 128 * TK * 2, &gp.tmB[prob], bar, kb * TK, y_b, z_b);
+          const bool two = k0 + TK < K;  // a second half within K
+          if (rank == 0) mbar_expect_tx(smem_u32(&full[sl]), 2 * (two ? 2 * half_bytes : half_bytes));
+          const uint32_t dst = smem_u32(smem + sl * stage_bytes), bar = cluster_addr(smem_u32(&full[sl]), leader);
+          const uint32_t dst_b = dst + 2 * A_HALF, b_half = (uint32_t)(box * TK * 2);
+          tma_load_pair(dst, &gp.tmA[prob], bar, k0, y_a, plane);
+          if (pairs == 1) {
+            tma_load_pair(dst_b, &gp.tmB[prob], bar, k0, y_b, z_b);
+            if (two) tma_load_pair(dst_b + b_half, &gp.tmB[prob], bar, k0 + TK, y_b, z_b);
+          } else if (pair == 0 || two) {
+            tma_load_multicast(dst_b + pair * b_half, &gp.tmB[prob], bar, k0 + (int)pair * TK, y_b, z_b, 5u << rank);
+          }
+          if (two) tma_load_pair(dst + A_HALF, &gp.tmA[prob], bar, k0 + TK, y_a, plane);
+          advance();
         }
       }
       if (ok) {
         // every stage's release has arrived in this CTA before it may exit
-        for (int i = 0; i < STAGES && ok; ++i, ++it)
-          ok = mbar_wait(smem_u32(&empty[it % STAGES]), ((it / STAGES) & 1) ^ 1, err);
+        for (int i = 0; i < stages && ok; ++i) {
+          ok = mbar_wait(smem_u32(&empty[sl]), ph ^ 1, err);
+          advance();
+        }
       } else if (rank == 0) {
         // aborted: the copies in flight (this CTA's and its peer's) land before the pair exits
-        for (int j = it > STAGES ? it - STAGES : 0; j < it; ++j) {
+        for (int j = it > stages ? it - stages : 0; j < it; ++j) {
           const unsigned long long t0 = globaltimer();
-          while (!mbar_try(smem_u32(&full[j % STAGES]), (j / STAGES) & 1) && globaltimer() - t0 < TIMEOUT_NS) {
+          while (!mbar_try(smem_u32(&full[j % stages]), (j / stages) & 1) && globaltimer() - t0 < TIMEOUT_NS) {
           }
         }
       }
     } else if (warp == 1 && lane == 0 && rank == 0) {
       // ---------------------------------------------------------- MMA issue
-      int it = 0, chunk = 0;
+      int chunk = 0, sl = 0;
+      uint32_t ph = 0;
+      bool ready = false;  // the slot's copies are known to have landed
       bool ok = true;
       int prob = 0;
       for (int unit = cluster; unit < total && ok; unit += nclusters) {
@@ -590,37 +642,51 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
         int n0, width;
         tile_cols(gp.nblk[prob], gp.nt[prob], n, n0, width);
         const uint32_t idesc = oz::idesc_bf16(TM, width);
-        const int nkb = gp.nkb[prob];
-        for (int kb = 0; kb < nkb; ++kb, ++it) {
+        const int K = gp.K[prob];
+        const uint32_t b_half = (uint32_t)(gp.box_b[prob] * TK * 2);
+        int in_chunk = 0;
+        for (int k0 = 0; k0 < K; k0 += SK) {
           const int b = chunk & 1;
-          if (kb % CHUNK == 0) {
+          if (in_chunk == 0) {
             if (!mbar_wait(smem_u32(&acc_empty[b]), ((chunk >> 1) & 1) ^ 1, err)) {
               ok = false;
               break;
             }
             fence_after();
           }
-          const int s = it % STAGES;
-          if (!mbar_wait(smem_u32(&full[s]), (it / STAGES) & 1, err)) {
+          if (!ready && !mbar_wait(smem_u32(&full[sl]), ph, err)) {
             ok = false;
             break;
           }
           fence_after();
-          const uint32_t base = smem_u32(smem + s * STAGE_BYTES);
-          const uint64_t ad = sw128_desc(base), bd = sw128_desc(base + 128 * TK * 2);
+          const uint32_t base = smem_u32(smem + sl * stage_bytes);
+          const uint64_t ad = sw128_desc(base), bd = sw128_desc(base + 2 * A_HALF);
           const uint32_t d = tmem + (uint32_t)(b * 256);
 #pragma unroll
           for (int ks = 0; ks < TK / 16; ++ks)
-            mma_pair(d, ad + (uint64_t)(ks * 2), bd + (uint64_t)(ks * 2), idesc, (kb % CHUNK != 0 || ks != 0) ? 1u : 0u);
-          commit_pair(smem_u32(&empty[s]));
-          if (kb % CHUNK == CHUNK - 1 || kb == nkb - 1) {
-            commit_pair(smem_u32(&acc_full[b]));
+            mma_pair(d, ad + (uint64_t)(ks * 2), bd + (uint64_t)(ks * 2), idesc, (in_chunk != 0 || ks != 0) ? 1u : 0u);
+          // the next stage's barrier, while these run
+          const uint32_t slot = smem_u32(&empty[sl]);
+          if (++sl == stages) {
+            sl = 0;
+            ph ^= 1;
+          }
+          ready = mbar_test(smem_u32(&full[sl]), ph);
+          if (k0 + TK < K) {
+            const uint64_t ad2 = ad + (uint64_t)(A_HALF >> 4), bd2 = bd + (uint64_t)(b_half >> 4);
+#pragma unroll
+            for (int ks = 0; ks < TK / 16; ++ks) mma_pair(d, ad2 + (uint64_t)(ks * 2), bd2 + (uint64_t)(ks * 2), idesc, 1u);
+          }
+          commit_to(slot, all_mask);
+          if (++in_chunk == CHUNK || k0 + SK >= K) {
+            commit_to(smem_u32(&acc_full[b]), pair_mask);
             ++chunk;
+            in_chunk = 0;
           }
         }
       }
       // every MMA is done before TMEM is freed
-      commit_pair(smem_u32(drain));
+      commit_to(smem_u32(drain), pair_mask);
       const unsigned long long t0 = globaltimer();
       while (!mbar_try(smem_u32(drain), 0) && globaltimer() - t0 < TIMEOUT_NS) {
       }
@@ -631,7 +697,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
     // ------------------------------------------------------------ chunk reduction
     const int ew = warp - 4, q = ew & 3, half = ew >> 2;  // TMEM lane quadrant, column half
     const uint32_t lane_addr = tmem + ((uint32_t)(q * 32) << 16);
-    const uint32_t rel0 = leader_addr(smem_u32(&acc_empty[0])), rel1 = leader_addr(smem_u32(&acc_empty[1]));
+    const uint32_t rel0 = cluster_addr(smem_u32(&acc_empty[0]), leader), rel1 = cluster_addr(smem_u32(&acc_empty[1]), leader);
     int chunk = 0;
     bool ok = true;
     int prob = 0;
@@ -646,7 +712,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
       tile_cols(gp.nblk[prob], nt, n, n0, width);
       const int hc = width >> 1;  // this warp's columns: [half hc, half hc + hc)
       const Mod2 mod(cT.m[gp.mod0 + plane / gp.np]);
-      const int nchunk = (gp.nkb[prob] + CHUNK - 1) / CHUNK;
+      const int nchunk = (gp.K[prob] + CHUNK * SK - 1) / (CHUNK * SK);
       uint64_t acc[64];
 #pragma unroll
       for (int j = 0; j < 64; ++j) acc[j] = 0ull;
@@ -679,7 +745,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
         }
       }
       if (!ok) break;
-      const int row = m * TM + (int)rank * 128 + q * 32 + lane;
+      const int row = (m * pairs + (int)pair) * TM + (int)rank * 128 + q * 32 + lane;
       if (row < gp.M[prob]) {
         const int N = gp.N[prob], ldr = gp.ldr[prob];
         const int c0 = n0 + half * hc;
@@ -840,10 +906,50 @@ void residues(cudaStream_t st, bool by_rows, bool conj, int64_t nvec, int64_t K,
   CHASE_CHECK_LAUNCH();
 }
 
+// clusters of one or two CTA pairs the device keeps resident (0: none)
+template <int G> static int max_clusters(int pairs) {
+  static std::once_flag once;
+  static cudaError_t err = cudaSuccess;
+  static int got[2] = {0, 0};
+  std::call_once(once, []() {
+    err = cudaFuncSetAttribute(crt_gemm_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+    for (int p = 1; p <= 2 && err == cudaSuccess; ++p) {
+      cudaLaunchConfig_t cfg{};
+      cudaLaunchAttribute at{};
+      at.id = cudaLaunchAttributeClusterDimension;
+      at.val.clusterDim.x = 2 * p;
+      at.val.clusterDim.y = at.val.clusterDim.z = 1;
+      cfg.gridDim = dim3(2 * p, 1, 1);
+      cfg.blockDim = dim3(NTHREADS, 1, 1);
+      cfg.dynamicSmemBytes = SMEM_BYTES;
+      cfg.attrs = &at;
+      cfg.numAttrs = 1;
+      err = cudaOccupancyMaxActiveClusters(&got[p - 1], crt_gemm_kernel<G>, &cfg);
+    }
+  });
+  CHASE_CUDA(err);
+  return got[pairs - 1];
+}
+
 template <int G> static void launch(cudaStream_t st, const Product* ops, int nops, bool cplx, int mod0, int nmod, int* err) {
   static thread_local Params<G> gp;  // large for G > 1: built in thread-local host memory
   const int np = planes(cplx);
+  // units and rounds over the resident clusters, with one and with two pairs per cluster
+  int64_t u[2] = {0, 0};
+  int64_t cols = 0;
+  for (int p = 0; p < nops; ++p) {
+    const int64_t nt = ceil_div(ceil_div(ops[p].N, 32), TN / 32), mt = ceil_div(ops[p].M, TM);
+    u[0] += mt * nt * np * nmod;
+    u[1] += (mt + 1) / 2 * nt * np * nmod;
+    cols = std::max(cols, std::min<int64_t>(TN, ops[p].N / nt));
+  }
+  const int c1 = std::max(1, max_clusters<G>(1)), c2 = max_clusters<G>(2);
+  // Narrow tiles are bound by the left planes' HBM traffic, which sharing does not lower; else two pairs unless their
+  // last round is emptier by more than the tenth that sharing gains
+  const double r1 = (double)ceil_div(u[0], c1), r2 = c2 > 0 ? (double)ceil_div(u[1], c2) : 1e30;
+  const int pairs = cols >= 128 && r2 <= 1.1 * r1 ? 2 : 1;
   int64_t units = 0;
+  int box_max = 0;
   for (int p = 0; p < nops; ++p) {
     const Product& o = ops[p];
     const int64_t kp = kpad(o.K);
@@ -854,8 +960,9 @@ template <int G> static void launch(cudaStream_t st, const Product* ops, int nop
     gp.R[p] = (int8_t*)o.res;
     gp.M[p] = (int)o.M;
     gp.N[p] = (int)o.N;
-    gp.nkb[p] = (int)ceil_div(o.K, TK);
-    gp.mt[p] = (int)ceil_div(o.M, TM);
+    gp.K[p] = (int)o.K;
+    box_max = std::max(box_max, box);
+    gp.mt[p] = (int)ceil_div(ceil_div(o.M, TM), pairs);
     gp.nt[p] = nt;
     gp.nblk[p] = nblk;
     gp.box_b[p] = box;
@@ -868,28 +975,21 @@ template <int G> static void launch(cudaStream_t st, const Product* ops, int nop
   gp.nprob = nops;
   gp.mod0 = mod0;
   gp.np = np;
-  static std::once_flag once;
-  static cudaError_t attr_err = cudaSuccess;
-  static int max_clusters = 0;
-  std::call_once(once, []() {
-    attr_err = cudaFuncSetAttribute(crt_gemm_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-    if (attr_err != cudaSuccess) return;
-    cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = 2;
-    at.val.clusterDim.y = 1;
-    at.val.clusterDim.z = 1;
-    cfg.gridDim = dim3(2, 1, 1);
-    cfg.blockDim = dim3(NTHREADS, 1, 1);
-    cfg.dynamicSmemBytes = SMEM_BYTES;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    attr_err = cudaOccupancyMaxActiveClusters(&max_clusters, crt_gemm_kernel<G>, &cfg);
-  });
-  CHASE_CUDA(attr_err);
-  const int clusters = (int)std::min<int64_t>(units, std::max(1, max_clusters));
-  crt_gemm_kernel<G><<<2 * clusters, NTHREADS, SMEM_BYTES, st>>>(gp, err);
+  gp.pairs = pairs;
+  gp.stage_bytes = 2 * (A_HALF + box_max * TK * 2);
+  gp.stages = std::min(MAX_STAGES, SMEM_RING / gp.stage_bytes);
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = 2 * pairs;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.gridDim = dim3((unsigned)(2 * pairs * std::min<int64_t>(units, pairs == 2 ? c2 : c1)), 1, 1);
+  cfg.blockDim = dim3(NTHREADS, 1, 1);
+  cfg.dynamicSmemBytes = SMEM_BYTES;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  CHASE_CUDA(cudaLaunchKernelEx(&cfg, crt_gemm_kernel<G>, gp, err));
   CHASE_CHECK_LAUNCH();
 }
 

@@ -684,7 +684,7 @@ constexpr int BJ_B = 32;          // block width
 constexpr int BJ_M = 2 * BJ_B;    // subproblem order
 constexpr int BJ_SOLVE_THREADS = 1024;
 constexpr int BJ_UPD_THREADS = 256;
-constexpr int BJ_TILE = 64;       // rows (columns) of G or Z per update CTA
+constexpr int BJ_TILE = 16;       // rows (columns) of G or Z per update CTA
 
 // global index of local index l of block pair (I, J)
 __device__ __forceinline__ int bj_global(int I, int J, int l) {
@@ -779,124 +779,46 @@ __global__ void __launch_bounds__(BJ_SOLVE_THREADS) bj_solve_kernel(int k, int n
   for (int e = tid; e < BJ_M * BJ_M; e += BJ_SOLVE_THREADS) U[e] = Uf[e];
 }
 
-// The updates' 64 x 64 x 64 products: out = sum_m v[m][4 consecutive] * w[m][4], per thread 4 x 4 outputs, on packed
-// FP32 pairs (two multiply-adds per instruction).  v is read as it is (re, im pairs, or two reals); w is held twice
-// ({re, re}, {im, im} or {x, x}) so that it multiplies both halves.  Complex outputs are kept as
-// A = sum re(w) v and B = sum im(w) v until the end.
-__device__ __forceinline__ uint64_t pair2(float a, float b) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ void unpair2(uint64_t v, float& a, float& b) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-}
-__device__ __forceinline__ uint64_t ffma2(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-template <typename F> struct Tile;
-template <> struct Tile<float2> {
-  static constexpr int DUP = 2;  // 64-bit words per doubled entry
-  uint64_t A[4][4], B[4][4];     // [w index][v index]
-  __device__ __forceinline__ void clear() {
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) A[i][j] = B[i][j] = 0ull;
-  }
-  static __device__ __forceinline__ void dup(uint64_t* o, float2 x) {
-    o[0] = pair2(x.x, x.x);
-    o[1] = pair2(x.y, x.y);
-  }
-  // v: 4 consecutive entries; w[i]: doubled entries
-  __device__ __forceinline__ void add(const float2* v, const uint64_t* const (&w)[4]) {
-    const ulonglong2 v01 = *reinterpret_cast<const ulonglong2*>(v), v23 = *reinterpret_cast<const ulonglong2*>(v + 2);
-    const uint64_t vv[4] = {v01.x, v01.y, v23.x, v23.y};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const ulonglong2 d = *reinterpret_cast<const ulonglong2*>(w[i]);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        A[i][j] = ffma2(d.x, vv[j], A[i][j]);
-        B[i][j] = ffma2(d.y, vv[j], B[i][j]);
-      }
-    }
-  }
-  // conj_v: the product was to take conj(v)
-  __device__ __forceinline__ float2 get(int i, int j, bool conj_v) const {
-    float ar, ai, br, bi;
-    unpair2(A[i][j], ar, ai);
-    unpair2(B[i][j], br, bi);
-    return conj_v ? make_float2(ar + bi, br - ai) : make_float2(ar - bi, ai + br);
-  }
-};
-template <> struct Tile<float> {
-  static constexpr int DUP = 1;
-  uint64_t A[4][2];
-  __device__ __forceinline__ void clear() {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) A[i][0] = A[i][1] = 0ull;
-  }
-  static __device__ __forceinline__ void dup(uint64_t* o, float x) { o[0] = pair2(x, x); }
-  __device__ __forceinline__ void add(const float* v, const uint64_t* const (&w)[4]) {
-    const ulonglong2 vv = *reinterpret_cast<const ulonglong2*>(v);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const uint64_t d = *w[i];
-      A[i][0] = ffma2(d, vv.x, A[i][0]);
-      A[i][1] = ffma2(d, vv.y, A[i][1]);
-    }
-  }
-  __device__ __forceinline__ float get(int i, int j, bool) const {
-    float a, b;
-    unpair2(A[i][j >> 1], a, b);
-    return (j & 1) ? b : a;
-  }
-};
-
+// The updates: 64 x 64 times 64 x 16 products, 4 outputs per thread.  Their arithmetic is 2 to 3 us for 437 complex
+// columns; what they cost is latency, so tiles are small (several CTAs per SM).  Doubled operands for packed FP32
+// multiply-adds and 64 x 64 tiles with 4 x 4 outputs per thread took 20 us a launch, one CTA per SM.
 // X[:, IJ] <- X[:, IJ] U for a tile of BJ_TILE rows (X = G for blockIdx.z == 0, Z for 1)
 template <typename F>
 __global__ void __launch_bounds__(BJ_UPD_THREADS) bj_cols_kernel(int k, int nbp, int r, F* G, int64_t ldg, F* Z,
                                                                   int64_t ldz, const F* __restrict__ Ubuf) {
   using s = S<F>;
-  using T = Tile<F>;
-  extern __shared__ __align__(16) unsigned char bj_smem[];
-  uint64_t* Us = reinterpret_cast<uint64_t*>(bj_smem);             // [m][c] doubled
-  F* Xs = reinterpret_cast<F*>(Us + BJ_M * BJ_M * T::DUP);         // [m][row]
+  __shared__ __align__(16) F Us[BJ_M][BJ_M];    // U[m][c]
+  __shared__ F Xs[BJ_M][BJ_TILE];               // X[row][m] at Xs[m][row]
   const int nb = (k + BJ_B - 1) / BJ_B;
   int I, J;
   round_pair(r, blockIdx.y, nbp, I, J);
   if (bj_idle(I, J, nb, r)) return;
   F* X = blockIdx.z == 0 ? G : Z;
   const int64_t ldx = blockIdx.z == 0 ? ldg : ldz;
-  const int r0 = blockIdx.x * BJ_TILE;
+  const int tid = threadIdx.x, i = tid % BJ_TILE, q = tid / BJ_TILE;
+  const int gi = blockIdx.x * BJ_TILE + i;
   const F* U = Ubuf + (int64_t)blockIdx.y * BJ_M * BJ_M;
-  const int tid = threadIdx.x;
-  for (int e = tid; e < BJ_M * BJ_M; e += BJ_UPD_THREADS) T::dup(Us + e * T::DUP, U[e]);
-  for (int e = tid; e < BJ_TILE * BJ_M; e += BJ_UPD_THREADS) {
-    const int i = e % BJ_TILE, l = e / BJ_TILE;
-    const int gi = r0 + i, gl = bj_global(I, J, l);
-    Xs[l * BJ_TILE + i] = (gi < k && gl < k) ? X[gi + (int64_t)gl * ldx] : s::zero();
+#pragma unroll
+  for (int e = 0; e < BJ_M * BJ_M / BJ_UPD_THREADS; ++e) (&Us[0][0])[tid + e * BJ_UPD_THREADS] = U[tid + e * BJ_UPD_THREADS];
+#pragma unroll
+  for (int e = 0; e < BJ_M * BJ_TILE / BJ_UPD_THREADS; ++e) {
+    const int l = q + e * (BJ_UPD_THREADS / BJ_TILE), gl = bj_global(I, J, l);
+    Xs[l][i] = (gi < k && gl < k) ? X[gi + (int64_t)gl * ldx] : s::zero();
   }
   __syncthreads();
-  const int i4 = (tid % 16) * 4, c4 = (tid / 16) * 4;
-  T acc;
-  acc.clear();
-#pragma unroll 4
+  F acc[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) acc[c] = s::zero();
+#pragma unroll 8
   for (int m = 0; m < BJ_M; ++m) {
-    const uint64_t* u = Us + (m * BJ_M + c4) * T::DUP;
-    const uint64_t* const w[4] = {u, u + T::DUP, u + 2 * T::DUP, u + 3 * T::DUP};
-    acc.add(Xs + m * BJ_TILE + i4, w);
+    const F x = Xs[m][i];
+#pragma unroll
+    for (int c = 0; c < 4; ++c) acc[c] = s::fma(x, Us[m][4 * q + c], acc[c]);
   }
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
-    const int gl = bj_global(I, J, c4 + c);
-    if (gl >= k) continue;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-      if (r0 + i4 + i < k) X[r0 + i4 + i + (int64_t)gl * ldx] = acc.get(c, i, false);
+    const int gl = bj_global(I, J, 4 * q + c);
+    if (gi < k && gl < k) X[gi + (int64_t)gl * ldx] = acc[c];
   }
 }
 
@@ -905,47 +827,38 @@ template <typename F>
 __global__ void __launch_bounds__(BJ_UPD_THREADS) bj_rows_kernel(int k, int nbp, int r, F* G, int64_t ldg,
                                                                   const F* __restrict__ Ubuf) {
   using s = S<F>;
-  using T = Tile<F>;
-  extern __shared__ __align__(16) unsigned char bj_smem[];
-  uint64_t* Xs = reinterpret_cast<uint64_t*>(bj_smem);             // [column j][m] doubled
-  F* Us = reinterpret_cast<F*>(Xs + BJ_M * BJ_TILE * T::DUP);      // [m][l]
+  __shared__ F Us[BJ_M][BJ_M + 1];      // U[m][l]
+  __shared__ F Xs[BJ_TILE][BJ_M];       // X[m][column] at Xs[column][m]
   const int nb = (k + BJ_B - 1) / BJ_B;
   int I, J;
   round_pair(r, blockIdx.y, nbp, I, J);
   if (bj_idle(I, J, nb, r)) return;
-  const int c0 = blockIdx.x * BJ_TILE;
+  const int tid = threadIdx.x, l = tid % BJ_M, q = tid / BJ_M;
+  const int c0 = blockIdx.x * BJ_TILE, gl = bj_global(I, J, l);
   const F* U = Ubuf + (int64_t)blockIdx.y * BJ_M * BJ_M;
-  const int tid = threadIdx.x;
-  for (int e = tid; e < BJ_M * BJ_M; e += BJ_UPD_THREADS) Us[e] = U[e];
-  for (int e = tid; e < BJ_M * BJ_TILE; e += BJ_UPD_THREADS) {
-    const int l = e % BJ_M, j = e / BJ_M;
-    const int gl = bj_global(I, J, l), gj = c0 + j;
-    T::dup(Xs + e * T::DUP, (gl < k && gj < k) ? G[gl + (int64_t)gj * ldg] : s::zero());
+#pragma unroll
+  for (int e = 0; e < BJ_M * BJ_M / BJ_UPD_THREADS; ++e) Us[q + e * (BJ_UPD_THREADS / BJ_M)][l] = U[tid + e * BJ_UPD_THREADS];
+#pragma unroll
+  for (int e = 0; e < BJ_M * BJ_TILE / BJ_UPD_THREADS; ++e) {
+    const int j = q + e * (BJ_UPD_THREADS / BJ_M);
+    Xs[j][l] = (gl < k && c0 + j < k) ? G[gl + (int64_t)(c0 + j) * ldg] : s::zero();
   }
   __syncthreads();
-  // out[l][j] = sum_m conj(U[m][l]) X[m][j]
-  const int l4 = (tid % 16) * 4, j4 = (tid / 16) * 4;
-  T acc;
-  acc.clear();
-#pragma unroll 4
+  // thread: row l of the pair, columns 4 q .. 4 q + 3; out[l][j] = sum_m conj(U[m][l]) X[m][j]
+  F acc[4];
+#pragma unroll
+  for (int j = 0; j < 4; ++j) acc[j] = s::zero();
+#pragma unroll 8
   for (int m = 0; m < BJ_M; ++m) {
-    const uint64_t* x = Xs + (j4 * BJ_M + m) * T::DUP;
-    const uint64_t* const w[4] = {x, x + BJ_M * T::DUP, x + 2 * BJ_M * T::DUP, x + 3 * BJ_M * T::DUP};
-    acc.add(Us + m * BJ_M + l4, w);
+    const F u = s::conj(Us[m][l]);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[j] = s::fma(u, Xs[4 * q + j][m], acc[j]);
   }
 #pragma unroll
-  for (int j = 0; j < 4; ++j) {
-    const int gj = c0 + j4 + j;
-    if (gj >= k) continue;
-#pragma unroll
-    for (int l = 0; l < 4; ++l) {
-      const int gl = bj_global(I, J, l4 + l);
-      if (gl < k) G[gl + (int64_t)gj * ldg] = acc.get(j, l, true);
-    }
-  }
+  for (int j = 0; j < 4; ++j)
+    if (gl < k && c0 + 4 * q + j < k) G[gl + (int64_t)(c0 + 4 * q + j) * ldg] = acc[j];
 }
 
-template <typename F> static size_t bj_smem_bytes() { return (size_t)BJ_M * BJ_M * (sizeof(F) + 8 * Tile<F>::DUP); }
 template <typename F> static size_t bj_solve_smem_bytes() { return (size_t)4 * BJ_M * BJ_M * sizeof(F); }
 
 int heev_block_workspace(int k) {
@@ -967,11 +880,8 @@ int heev_block_jacobi(cudaStream_t st, int k, F* G, int64_t ldg, double* w, F* Z
   static std::once_flag once;
   static cudaError_t attr = cudaSuccess;
   std::call_once(once, []() {
-    const int b = (int)bj_smem_bytes<F>();
     attr = cudaFuncSetAttribute(bj_solve_kernel<F>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 (int)bj_solve_smem_bytes<F>());
-    if (attr == cudaSuccess) attr = cudaFuncSetAttribute(bj_cols_kernel<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
-    if (attr == cudaSuccess) attr = cudaFuncSetAttribute(bj_rows_kernel<F>, cudaFuncAttributeMaxDynamicSharedMemorySize, b);
   });
   CHASE_CUDA(attr);
   set_identity_kernel<F><<<dim3(ceil_div(k, 256), k), 256, 0, st>>>(k, Zu, k);
@@ -999,10 +909,10 @@ int heev_block_jacobi(cudaStream_t st, int k, F* G, int64_t ldg, double* w, F* Z
     for (int r = 0; r < nbp - 1; ++r) {
       bj_solve_kernel<F><<<npairs, BJ_SOLVE_THREADS, bj_solve_smem_bytes<F>(), st>>>(k, nbp, r, G, ldg, Ubuf, r == 0);
       CHASE_CHECK_LAUNCH();
-      bj_cols_kernel<F><<<dim3(tiles, npairs, 2), BJ_UPD_THREADS, bj_smem_bytes<F>(), st>>>(k, nbp, r, G, ldg, Zu, k,
+      bj_cols_kernel<F><<<dim3(tiles, npairs, 2), BJ_UPD_THREADS, 0, st>>>(k, nbp, r, G, ldg, Zu, k,
                                                                                           Ubuf);
       CHASE_CHECK_LAUNCH();
-      bj_rows_kernel<F><<<dim3(tiles, npairs), BJ_UPD_THREADS, bj_smem_bytes<F>(), st>>>(k, nbp, r, G, ldg, Ubuf);
+      bj_rows_kernel<F><<<dim3(tiles, npairs), BJ_UPD_THREADS, 0, st>>>(k, nbp, r, G, ldg, Ubuf);
       CHASE_CHECK_LAUNCH();
     }
   }

@@ -461,55 +461,61 @@ __global__ void __launch_bounds__(STEP_THREADS) lanczos_step_kernel(int64_t n, i
 }
 
 // ---------------------------------------------------------------- Ritz values
-// Implicit QL with Wilkinson shifts on the run's tridiagonal T (steps <= 64), one thread per run: eigenvalues, and the
+// Implicit QL with Wilkinson shifts on the run's tridiagonal T (steps <= 64), one warp per run: eigenvalues, and the
 // first row of the eigenvectors' matrix, which is all the density of states needs (Golub and Welsch 1969).  About
-// 1.7 QL sweeps per eigenvalue of at most `steps` rotations: a short serial chain (a two-sided Jacobi over the whole
-// block took 5.6 ms for 25 steps; this takes 0.1 to 0.2).  Output theta ascending and tau2 = squared first components.
+// 1.7 QL sweeps per eigenvalue of at most `steps` rotations, a serial chain in lane 0; the search for a negligible
+// off-diagonal before each sweep is one step of the whole warp.  Output theta ascending and tau2 = squared first
+// components.  (A two-sided Jacobi over the block took 5.6 ms for 25 steps.)
 __global__ void tridiag_ql_kernel(int steps, const double* alpha, const double* beta, double* theta, double* tau2,
                                   int* status) {
-  const int r = blockIdx.x, k = steps;
+  const int r = blockIdx.x, k = steps, lane = threadIdx.x;
   __shared__ double d[LZ_MAXS], e[LZ_MAXS], z[LZ_MAXS];
-  __shared__ int ex;
-  for (int i = threadIdx.x; i < k; i += blockDim.x) {
+  // scaled by a power of two to norm about 1, so that squares neither overflow nor vanish
+  double m = 0.0;
+  for (int i = lane; i < k; i += 32) {
     d[i] = alpha[r * LZ_MAXS + i];
     e[i] = i + 1 < k ? beta[r * LZ_MAXS + i] : 0.0;
     z[i] = i == 0 ? 1.0 : 0.0;
+    m = fmax(m, fmax(fabs(d[i]), fabs(e[i])));
   }
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    // scaled by a power of two to norm about 1, so that squares neither overflow nor vanish
-    double m = 0.0;
-    for (int i = 0; i < k; ++i) m = fmax(m, fmax(fabs(d[i]), fabs(e[i])));
-    int sc = 0;
-    if (m > 0.0 && isfinite(m)) frexp(m, &sc);
-    for (int i = 0; i < k; ++i) {
-      d[i] = ldexp(d[i], -sc);
-      e[i] = ldexp(e[i], -sc);
-    }
-    ex = sc;
-    const double eps = 1.1102230246251565e-16;
-    for (int l = 0; l < k; ++l) {
-      for (int iter = 0;; ++iter) {
-        int mm = l;
-        for (; mm < k - 1; ++mm)
-          if (fabs(e[mm]) <= eps * (fabs(d[mm]) + fabs(d[mm + 1])) || fabs(e[mm]) < 1e-150) break;
-        if (mm == l) break;
-        if (iter == 60) {
-          atomicMax(status, 1);
-          break;
-        }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+  int sc = 0;
+  if (m > 0.0 && isfinite(m)) frexp(m, &sc);
+  for (int i = lane; i < k; i += 32) {
+    d[i] = ldexp(d[i], -sc);
+    e[i] = ldexp(e[i], -sc);
+  }
+  __syncwarp();
+  const double eps = 1.1102230246251565e-16;
+  for (int l = 0; l < k; ++l) {
+    for (int iter = 0;; ++iter) {
+      // first mm >= l whose off-diagonal entry is negligible (k - 1 at the latest)
+      auto small = [&](int i) {
+        return i >= k - 1 || (i >= l && (fabs(e[i]) <= eps * (fabs(d[i]) + fabs(d[i + 1])) || fabs(e[i]) < 1e-150));
+      };
+      const unsigned lo = __ballot_sync(0xffffffffu, small(lane));
+      const unsigned hi = __ballot_sync(0xffffffffu, small(lane + 32));
+      const int mm = min(k - 1, lo ? __ffs((int)lo) - 1 : 31 + __ffs((int)hi));
+      if (mm == l) break;
+      if (iter == 60) {
+        if (lane == 0) atomicMax(status, 1);
+        break;
+      }
+      if (lane == 0) {
         double g = (d[l + 1] - d[l]) / (2.0 * e[l]);
-        double h = sqrt(g * g + 1.0);
+        const double h = sqrt(g * g + 1.0);
         g = d[mm] - d[l] + e[l] / (g + (g >= 0.0 ? h : -h));
         double sn = 1.0, cs = 1.0, p = 0.0;
+        double di1 = d[mm];
         int i = mm - 1;
         for (; i >= l; --i) {
-          double f = sn * e[i];
-          const double b = cs * e[i];
-          const double q = f * f + g * g;
+          const double ei = e[i], di = d[i], zi = z[i], zi1 = z[i + 1];
+          const double f = sn * ei, b = cs * ei;
+          const double q = fma(f, f, g * g);
           if (!(q > 1e-300)) {  // the rotation is undefined: the matrix splits here
             e[i + 1] = 0.0;
-            d[i + 1] -= p;
+            d[i + 1] = di1 - p;
             e[mm] = 0.0;
             break;
           }
@@ -517,29 +523,31 @@ __global__ void tridiag_ql_kernel(int steps, const double* alpha, const double* 
           e[i + 1] = q * ri;
           sn = f * ri;
           cs = g * ri;
-          g = d[i + 1] - p;
-          const double t = (d[i] - g) * sn + 2.0 * cs * b;
+          g = di1 - p;
+          const double t = fma(di - g, sn, 2.0 * cs * b);
           p = sn * t;
           d[i + 1] = g + p;
-          g = cs * t - b;
-          f = z[i + 1];
-          z[i + 1] = sn * z[i] + cs * f;
-          z[i] = cs * z[i] - sn * f;
+          g = fma(cs, t, -b);
+          z[i + 1] = fma(sn, zi, cs * zi1);
+          z[i] = fma(cs, zi, -sn * zi1);
+          di1 = di;
         }
-        if (i >= l) continue;
-        d[l] -= p;
-        e[l] = g;
-        e[mm] = 0.0;
+        if (i < l) {
+          d[l] -= p;
+          e[l] = g;
+          e[mm] = 0.0;
+        }
       }
+      __syncwarp();
     }
+    __syncwarp();
   }
-  __syncthreads();
   // ascending (stable) order
-  for (int i = threadIdx.x; i < k; i += blockDim.x) {
+  for (int i = lane; i < k; i += 32) {
     const double wi = d[i];
     int rank = 0;
     for (int q = 0; q < k; ++q) rank += (d[q] < wi) || (d[q] == wi && q < i);
-    theta[r * LZ_MAXS + rank] = ldexp(wi, ex);
+    theta[r * LZ_MAXS + rank] = ldexp(wi, sc);
     tau2[r * LZ_MAXS + rank] = z[i] * z[i];
   }
 }
