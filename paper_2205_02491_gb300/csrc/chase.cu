@@ -1766,13 +1766,13 @@ static void solve_batched_grouped(chase_ctx* c, int nprob, const void* const* A,
           ops_lo.push_back(oz::ProductOp{sc->ozw.a_planes, sc->ozw.a_scale, oz::MIXED_SLICES, sc->ozw.b_planes,
                                          sc->ozw.b_scale, r.n, cols, r.n, e, c->ozw.group_m});
         } else if (oz::groupable(sc->ozw, r.n, cols)) {
-          ops_hi.push_back(oz::group_product<T>(fs, sc->ozw, in, r.n, cols, r.n, e));
+          ops_hi.push_back(oz::group_product<T>(sc->ozw, in, r.n, cols, r.n, e));
         } else {
           oz::hemm<T>(fs, sc->ozw, r.A, r.n, r.lda, in, r.n, cols, e, CHASE_FP64);  // A's planes in passes
         }
         sc->stats.filter_launches++;
       }
-      if (!ops_hi.empty()) oz::multiply_group<CPLX>(fs, c->ozw, ops_hi.data(), (int)ops_hi.size());
+      if (!ops_hi.empty()) oz::multiply_group<T>(fs, c->ozw, ops_hi.data(), (int)ops_hi.size());
       // the low-precision problems of one batch share its mode
       if (!ops_lo.empty()) oz::launch_group<CPLX>(fs, c->ozw, mode, ops_lo.data(), (int)ops_lo.size());
     }

@@ -344,6 +344,112 @@ __global__ void __launch_bounds__(256) residues_rows_kernel(int64_t nvec, int64_
   write_residues<T>(v, e, conj != 0, mod0, nmod, nvec * Kp, planes + i * Kp + k0 + g);
 }
 
+// ---------------------------------------------------------------- right operands: norms and planes in one launch
+constexpr int MAXG = 64;  // products per launch
+// shared::cluster address of this CTA-local address in the given CTA of the cluster
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t a, uint32_t cta) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(cta));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
+template <int G> struct RightParams {
+  const void* X[G];
+  int64_t ldx[G];
+  int* ex[G];
+  void* planes[G];
+  int nvec[G], K[G];
+};
+
+// A right operand's columns, exponents and all residue planes; blockIdx.y runs over the products' columns.  A cluster
+// (1 to 8 CTAs, 512 elements each while K <= 4096) takes one column: the CTAs' partial sums of squares meet in
+// every CTA's shared memory, so that a short K needs one launch of a few microseconds and a few columns still spread
+// over the SMs.  What bounds it: latency and launch overhead at small sizes, instruction issue at large ones.
+// Complex, n = 512: 6.1 us where separate norm and plane launches took 8.0 and the gap between them; n = 8192 and 512
+// columns: 87 us instead of 130.
+template <typename T, int G>
+__global__ void __launch_bounds__(128) right_planes_kernel(const __grid_constant__ RightParams<G> rp) {
+  using s = S<T>;
+  const int q = G == 1 ? 0 : blockIdx.z;
+  const int col = blockIdx.y;
+  if (col >= rp.nvec[q]) return;  // the whole cluster
+  __shared__ double part[2][32];
+  __shared__ unsigned long long partm[32];
+  const int rank = (int)blockIdx.x, cs = (int)gridDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  const int64_t K = rp.K[q], kp = (K + 7) / 8 * 8;
+  const int64_t slice = ((K + cs - 1) / cs + 3) / 4 * 4;
+  const int64_t k0 = rank * slice, k1 = k0 + slice < K ? k0 + slice : K;
+  const T* x = (const T*)rp.X[q] + (int64_t)col * rp.ldx[q];
+  auto load4 = [&](T (&v)[4], int64_t i) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = i + j < k1 ? x[i + j] : s::zero();
+  };
+  // the sum (largest bit pattern) over the cluster of one value per warp
+  auto spread = [&](uint32_t slot, unsigned long long bits) {
+    if (lane < cs)
+      asm volatile("st.shared::cluster.b64 [%0], %1;" ::"r"(cluster_addr(slot + 8 * (4 * rank + warp), lane)), "l"(bits) : "memory");
+    cluster_sync();
+  };
+  auto cluster_sum = [&](double v, int set) {
+    v = warp_sum(v);
+    spread(smem_u32(part[set]), (unsigned long long)__double_as_longlong(v));
+    return warp_sum(lane < 4 * cs ? part[set][lane] : 0.0);
+  };
+  T v[4];
+  const int64_t i0 = k0 + 4 * tid;
+  load4(v, i0);  // stays in registers when the slice is 512 elements
+  double a = (s::abs2(v[0]) + s::abs2(v[1])) + (s::abs2(v[2]) + s::abs2(v[3]));
+  for (int64_t i = i0 + 512; i < k1; i += 512) {
+    T u[4];
+    load4(u, i);
+    a += (s::abs2(u[0]) + s::abs2(u[1])) + (s::abs2(u[2]) + s::abs2(u[3]));
+  }
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");  // every CTA of the cluster runs
+  const double ss = cluster_sum(a, 0);
+  int e;
+  if (ss > 1e-250 && ss < 1e250) {
+    e = norm_exponent(ss);
+  } else {
+    // largest magnitude (bit patterns, so that NaN and infinity compare largest), then scaled squares
+    unsigned long long m = 0ull;
+    for (int64_t i = k0 + tid; i < k1; i += 128) {
+      const unsigned long long br = (unsigned long long)__double_as_longlong(fabs(s::re(x[i])));
+      const unsigned long long bi = (unsigned long long)__double_as_longlong(fabs(s::im(x[i])));
+      m = m > br ? m : br;
+      m = m > bi ? m : bi;
+    }
+    for (int o = 16; o; o >>= 1) {
+      const unsigned long long t = __shfl_xor_sync(0xffffffffu, m, o);
+      m = m > t ? m : t;
+    }
+    spread(smem_u32(partm), m);
+    m = 0ull;
+    for (int w = 0; w < 4 * cs; ++w) m = m > partm[w] ? m : partm[w];
+    int em = 0;
+    if (m < 0x7ff0000000000000ull) frexp(__longlong_as_double((long long)m), &em);
+    double b = 0.0;
+    for (int64_t i = k0 + tid; i < k1; i += 128) {
+      const double r = ldexp(s::re(x[i]), -em), c = ldexp(s::im(x[i]), -em);
+      b += r * r + c * c;
+    }
+    b = cluster_sum(b, 1);
+    e = m >= 0x7ff0000000000000ull ? NONFINITE : m == 0ull ? 0 : em + norm_exponent(b);
+  }
+  if (rank == 0 && tid == 0) rp.ex[q][col] = e;
+  if (e == NONFINITE) e = 0;
+  const int64_t plane = (int64_t)rp.nvec[q] * kp;
+  __nv_bfloat16* out = (__nv_bfloat16*)rp.planes[q] + (int64_t)col * kp;
+  if (i0 < k1) write_residues<T>(v, e, false, 0, NMOD, plane, out + i0);
+  for (int64_t i = i0 + 512; i < k1; i += 512) {
+    load4(v, i);
+    write_residues<T>(v, e, false, 0, NMOD, plane, out + i);
+  }
+}
+
 // ---------------------------------------------------------------- product kernel
 constexpr int TM = 256;           // rows of a tile: 128 per CTA of the pair
 constexpr int TN = 256;           // columns of a tile at most
@@ -356,7 +462,6 @@ constexpr int SMEM_RING = 216 * 1024;
 constexpr int SMEM_BYTES = SMEM_RING + 1024 + 256;
 constexpr int NTHREADS = 384;     // warps 0-3: copies, MMA issue, TMEM; warps 4-11: accumulator reduction
 constexpr int EPI_WARPS = 8;
-constexpr int MAXG = 64;          // products per launch
 constexpr unsigned long long TIMEOUT_NS = 2000000000ull;
 
 template <int G> struct Params {
@@ -383,15 +488,6 @@ __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
   asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
   return r;
-}
-// shared::cluster address of this CTA-local address in the given CTA of the cluster
-__device__ __forceinline__ uint32_t cluster_addr(uint32_t a, uint32_t cta) {
-  uint32_t r;
-  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(cta));
-  return r;
-}
-__device__ __forceinline__ void cluster_sync() {
-  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 __device__ __forceinline__ void arrive_cluster(uint32_t bar) {
   asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
@@ -818,49 +914,75 @@ __device__ __forceinline__ double reconstruct(const uint64_t (&a)[4], int e) {
   return to_double((__int128)t, e);
 }
 
-// Four rows per thread (one 4-byte load per plane).  HBM-bound on the residues (1 byte per plane and entry); the
-// weights' limb products run on the integer pipe.
-template <bool CPLX>
-__global__ void __launch_bounds__(64) combine_kernel(int M, int N, int ldr, const int8_t* __restrict__ R,
-                                                      const int* __restrict__ lex, const int* __restrict__ rex, Epi ep) {
+// ROWS = 4: four rows per thread (one 4-byte load per plane); HBM-bound on the residues (1 byte per plane and entry), the
+// weights' limb products run on the integer pipe.  ROWS = 1: one row per thread, for products too small to fill the
+// SMs otherwise, with every plane's load in flight at once.
+template <int G> struct CombineParams {
+  const int8_t* R[G];
+  const int* lex[G];
+  const int* rex[G];
+  Epi e[G];
+  int M[G], N[G], ldr[G];
+};
+template <bool CPLX, int ROWS, int G>
+__global__ void __launch_bounds__(64) combine_kernel(const __grid_constant__ CombineParams<G> cp) {
   constexpr int NP = CPLX ? 3 : 1, NC = CPLX ? 2 : 1;
-  const int i0 = 4 * (blockIdx.x * blockDim.x + threadIdx.x), j = blockIdx.y;
-  if (i0 >= M) return;
-  const int8_t* src = R + (int64_t)j * ldr + i0;
+  const int prob = G == 1 ? 0 : blockIdx.z;
+  const int M = cp.M[prob], N = cp.N[prob], ldr = cp.ldr[prob];
+  const int i0 = ROWS * (blockIdx.x * blockDim.x + threadIdx.x), j = blockIdx.y;
+  if (i0 >= M || j >= N) return;
+  const int* __restrict__ lex = cp.lex[prob];
+  const Epi& ep = cp.e[prob];
+  const int8_t* __restrict__ src = cp.R[prob] + (int64_t)j * ldr + i0;
   const int64_t plane = (int64_t)N * ldr;
-  uint64_t acc[4][NC][4];
+  uint64_t acc[ROWS][NC][4];
 #pragma unroll
-  for (int r = 0; r < 4; ++r)
+  for (int r = 0; r < ROWS; ++r)
 #pragma unroll
     for (int c = 0; c < NC; ++c)
 #pragma unroll
       for (int l = 0; l < 4; ++l) acc[r][c][l] = 0ull;
-#pragma unroll 4
-  for (int i = 0; i < NMOD; ++i) {
-    char4 p[NP];
+  constexpr int BATCH = ROWS == 1 ? NMOD : 4;  // moduli whose loads are in flight together
 #pragma unroll
-    for (int k = 0; k < NP; ++k) p[k] = *reinterpret_cast<const char4*>(src + (int64_t)(i * NP + k) * plane);
+  for (int i0m = 0; i0m < NMOD; i0m += BATCH) {
+    int8_t p[BATCH][NP][ROWS];
 #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      auto byte = [&](const char4& v) -> int { return r == 0 ? v.x : r == 1 ? v.y : r == 2 ? v.z : v.w; };
-      const int p0 = byte(p[0]);
-      uint32_t v[NC];
-      if (CPLX) {
-        const int p1 = byte(p[NP - 2]), p2 = byte(p[NP - 1]);
-        v[0] = (uint32_t)(p0 - p1 + BIAS);
-        v[NC - 1] = (uint32_t)(p2 - p0 - p1 + BIAS);
-      } else {
-        v[0] = (uint32_t)(p0 + BIAS);
+    for (int b = 0; b < BATCH; ++b)
+#pragma unroll
+      for (int k = 0; k < NP; ++k) {
+        const int8_t* q = src + (int64_t)((i0m + b) * NP + k) * plane;
+        if (ROWS == 4) {
+          const char4 v = *reinterpret_cast<const char4*>(q);
+          p[b][k][0] = v.x;
+          p[b][k][ROWS > 1 ? 1 : 0] = v.y;
+          p[b][k][ROWS > 2 ? 2 : 0] = v.z;
+          p[b][k][ROWS > 3 ? 3 : 0] = v.w;
+        } else {
+          p[b][k][0] = *q;
+        }
       }
 #pragma unroll
-      for (int c = 0; c < NC; ++c)
+    for (int b = 0; b < BATCH; ++b)
 #pragma unroll
-        for (int l = 0; l < 4; ++l) acc[r][c][l] += (uint64_t)v[c] * cT.w[i][l];
-    }
+      for (int r = 0; r < ROWS; ++r) {
+        const int p0 = p[b][0][r];
+        uint32_t v[NC];
+        if (CPLX) {
+          const int p1 = p[b][NP - 2][r], p2 = p[b][NP - 1][r];
+          v[0] = (uint32_t)(p0 - p1 + BIAS);
+          v[NC - 1] = (uint32_t)(p2 - p0 - p1 + BIAS);
+        } else {
+          v[0] = (uint32_t)(p0 + BIAS);
+        }
+#pragma unroll
+        for (int c = 0; c < NC; ++c)
+#pragma unroll
+          for (int l = 0; l < 4; ++l) acc[r][c][l] += (uint64_t)v[c] * cT.w[i0m + b][l];
+      }
   }
-  const int ej = rex[j];
+  const int ej = cp.rex[prob][j];
 #pragma unroll
-  for (int r = 0; r < 4; ++r) {
+  for (int r = 0; r < ROWS; ++r) {
     const int i = i0 + r;
     if (i >= M) return;
     const int ei = lex[i];
@@ -1004,24 +1126,92 @@ void multiply(cudaStream_t st, const Product* ops, int nops, int mod0, int nmod,
   }
 }
 
-template <bool CPLX> void combine(cudaStream_t st, const Product& op) {
-  CHASE_REQUIRE(op.N <= 65535, 1, "residue product: too many columns");
-  const dim3 grid(ceil_div(op.M, 256), (unsigned)op.N);
-  combine_kernel<CPLX><<<grid, 64, 0, st>>>((int)op.M, (int)op.N, (int)rpad(op.M), (const int8_t*)op.res, op.lex,
-                                             op.rex, op.e);
+template <bool CPLX, int ROWS, int G> static void launch_combine(cudaStream_t st, const Product* ops, int nops) {
+  static thread_local CombineParams<G> cp;
+  int64_t M = 0, N = 0;
+  for (int p = 0; p < nops; ++p) {
+    const Product& o = ops[p];
+    CHASE_REQUIRE(o.N <= 65535, 1, "residue product: too many columns");
+    cp.R[p] = (const int8_t*)o.res;
+    cp.lex[p] = o.lex;
+    cp.rex[p] = o.rex;
+    cp.e[p] = o.e;
+    cp.M[p] = (int)o.M;
+    cp.N[p] = (int)o.N;
+    cp.ldr[p] = (int)rpad(o.M);
+    M = std::max(M, o.M);
+    N = std::max(N, o.N);
+  }
+  combine_kernel<CPLX, ROWS, G><<<dim3(ceil_div(M, 64 * ROWS), (unsigned)N, (unsigned)nops), 64, 0, st>>>(cp);
   CHASE_CHECK_LAUNCH();
+}
+
+template <bool CPLX> void combine(cudaStream_t st, const Product* ops, int nops) {
+  for (int q0 = 0; q0 < nops; q0 += MAXG) {
+    const int cnt = std::min(MAXG, nops - q0);
+    int64_t entries = 0;
+    for (int q = q0; q < q0 + cnt; ++q) entries += ops[q].M * ops[q].N;
+    // One row per thread up to 2^19 entries (four rows make about 8 two-warp blocks per SM there): complex,
+    // 512 x 40 entries 4.3 us instead of 12, 3001 x 100 7.5 instead of 14; four rows read the planes in wider loads
+    // and win above.
+    const bool small = entries <= (1 << 19);
+    if (cnt == 1 && small) launch_combine<CPLX, 1, 1>(st, ops + q0, 1);
+    else if (cnt == 1) launch_combine<CPLX, 4, 1>(st, ops + q0, 1);
+    else if (small) launch_combine<CPLX, 1, MAXG>(st, ops + q0, cnt);
+    else launch_combine<CPLX, 4, MAXG>(st, ops + q0, cnt);
+  }
+}
+
+template <typename T, int G> static void launch_right(cudaStream_t st, const Product* ops, int nops) {
+  static thread_local RightParams<G> rp;
+  int64_t K = 0, N = 0;
+  for (int p = 0; p < nops; ++p) {
+    const Product& o = ops[p];
+    CHASE_REQUIRE(o.N <= 65535, 1, "residues: too many vectors");
+    rp.X[p] = o.X;
+    rp.ldx[p] = o.ldx;
+    rp.ex[p] = o.rex;
+    rp.planes[p] = o.rpl;
+    rp.nvec[p] = (int)o.N;
+    rp.K[p] = (int)o.K;
+    K = std::max(K, o.K);
+    N = std::max(N, o.N);
+  }
+  int cs = 1;
+  while (cs < 8 && 512 * cs < K) cs *= 2;
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeClusterDimension;
+  at.val.clusterDim.x = cs;
+  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cfg.gridDim = dim3(cs, (unsigned)N, (unsigned)nops);
+  cfg.blockDim = dim3(128, 1, 1);
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  CHASE_CUDA(cudaLaunchKernelEx(&cfg, right_planes_kernel<T, G>, rp));
+  CHASE_CHECK_LAUNCH();
+}
+
+template <typename T> void right_planes(cudaStream_t st, const Product* ops, int nops) {
+  for (int q0 = 0; q0 < nops; q0 += MAXG) {
+    const int cnt = std::min(MAXG, nops - q0);
+    if (cnt == 1) launch_right<T, 1>(st, ops + q0, 1);
+    else launch_right<T, MAXG>(st, ops + q0, cnt);
+  }
 }
 
 #define INST(T)                                                                                                  \
   template void scales<T>(cudaStream_t, bool, int64_t, int64_t, const T*, int64_t, int*);                         \
-  template void residues<T>(cudaStream_t, bool, bool, int64_t, int64_t, const T*, int64_t, const int*, int, int, void*);
+  template void residues<T>(cudaStream_t, bool, bool, int64_t, int64_t, const T*, int64_t, const int*, int, int, void*); \
+  template void right_planes<T>(cudaStream_t, const Product*, int);
 INST(double)
 INST(double2)
 #undef INST
 template void multiply<false>(cudaStream_t, const Product*, int, int, int, int*);
 template void multiply<true>(cudaStream_t, const Product*, int, int, int, int*);
-template void combine<false>(cudaStream_t, const Product&);
-template void combine<true>(cudaStream_t, const Product&);
+template void combine<false>(cudaStream_t, const Product*, int);
+template void combine<true>(cudaStream_t, const Product*, int);
 
 }  // namespace crt
 }  // namespace chase

@@ -38,18 +38,23 @@ void residues(cudaStream_t st, bool by_rows, bool conj, int64_t nvec, int64_t K,
 struct Product {
   const void* lpl;
   const int* lex;
-  const void* rpl;
-  const int* rex;
+  void* rpl;
+  int* rex;
   void* res;
   int64_t M, N, K;
   Epi e;
+  const void* X;  // the right operand (K x N, column-major), for right_planes
+  int64_t ldx;
 };
+
+// exponents and planes (all moduli) of the products' right operands, one launch per 64 products
+template <typename T> void right_planes(cudaStream_t st, const Product* ops, int nops);
 
 // residues of the products for the moduli [mod0, mod0 + nmod), one launch per 64 products
 template <bool CPLX>
 void multiply(cudaStream_t st, const Product* ops, int nops, int mod0, int nmod, int* err);
-// C = alpha * product + gamma ycol Y + beta Z from the residues of all moduli
-template <bool CPLX> void combine(cudaStream_t st, const Product& op);
+// C = alpha * product + gamma ycol Y + beta Z from the residues of all moduli, one launch per 64 products
+template <bool CPLX> void combine(cudaStream_t st, const Product* ops, int nops);
 
 }  // namespace crt
 }  // namespace chase

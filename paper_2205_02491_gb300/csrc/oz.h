@@ -118,8 +118,8 @@ template <bool CPLX> void launch_group(cudaStream_t st, Workspace& w, int mode, 
 // FP64: whether w's next product C = A B of k columns can join a group; its operands; and the group's launches.
 bool groupable(const Workspace& w, int64_t n, int k);
 template <typename T>
-crt::Product group_product(cudaStream_t st, Workspace& w, const T* B, int64_t ldb, int k, int64_t n, const Epi& e);
-template <bool CPLX> void multiply_group(cudaStream_t st, Workspace& w, const crt::Product* ops, int nops);
+crt::Product group_product(Workspace& w, const T* B, int64_t ldb, int k, int64_t n, const Epi& e);
+template <typename T> void multiply_group(cudaStream_t st, Workspace& w, const crt::Product* ops, int nops);
 
 }  // namespace oz
 }  // namespace chase

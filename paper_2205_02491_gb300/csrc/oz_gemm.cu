@@ -290,16 +290,20 @@ static void product(cudaStream_t st, Workspace& w, const void* lpl, const int* l
   for (int64_t j = 0; j < N; j += fit) {
     const int64_t nc = std::min(fit, N - j);
     const T* Bj = by_rows ? B + j : B + j * ldb;
-    crt::scales<T>(st, by_rows, nc, K, Bj, ldb, w.b_ex);
-    crt::residues<T>(st, by_rows, by_rows, nc, K, Bj, ldb, w.b_ex, 0, crt::NMOD, w.b_planes);
-    const crt::Product op{lpl, lex, w.b_planes, w.b_ex, w.residue, M, nc, K, at_column(e, j, sizeof(T))};
+    const crt::Product op{lpl, lex, w.b_planes, w.b_ex, w.residue, M, nc, K, at_column(e, j, sizeof(T)), Bj, ldb};
+    if (by_rows) {
+      crt::scales<T>(st, true, nc, K, Bj, ldb, w.b_ex);
+      crt::residues<T>(st, true, true, nc, K, Bj, ldb, w.b_ex, 0, crt::NMOD, w.b_planes);
+    } else {
+      crt::right_planes<T>(st, &op, 1);
+    }
     ProductTimer t(st, w);
     for (int m0 = 0; m0 < crt::NMOD; m0 += mods) {
       const int nm = std::min(mods, crt::NMOD - m0);
       lconv(m0, nm);
       crt::multiply<S<T>::cplx>(st, &op, 1, m0, nm, w.flags);
     }
-    crt::combine<S<T>::cplx>(st, op);
+    crt::combine<S<T>::cplx>(st, &op, 1);
     t.stop();
   }
 }
@@ -438,16 +442,15 @@ void launch_group(cudaStream_t st, Workspace& w, int mode, const ProductOp* ops,
 bool groupable(const Workspace& w, int64_t n, int k) { return w.a_mods == crt::NMOD && k <= panel_fit(w, n, n); }
 
 template <typename T>
-crt::Product group_product(cudaStream_t st, Workspace& w, const T* B, int64_t ldb, int k, int64_t n, const Epi& e) {
+crt::Product group_product(Workspace& w, const T* B, int64_t ldb, int k, int64_t n, const Epi& e) {
   CHASE_REQUIRE(w.ready, 9, "split products not initialised");
-  crt::scales<T>(st, false, k, n, B, ldb, w.b_ex);
-  crt::residues<T>(st, false, false, k, n, B, ldb, w.b_ex, 0, crt::NMOD, w.b_planes);
-  return crt::Product{w.a_res, w.a_ex, w.b_planes, w.b_ex, w.residue, n, k, n, e};
+  return crt::Product{w.a_res, w.a_ex, w.b_planes, w.b_ex, w.residue, n, k, n, e, B, ldb};
 }
 
-template <bool CPLX> void multiply_group(cudaStream_t st, Workspace& w, const crt::Product* ops, int nops) {
-  crt::multiply<CPLX>(st, ops, nops, 0, crt::NMOD, w.flags);
-  for (int q = 0; q < nops; ++q) crt::combine<CPLX>(st, ops[q]);
+template <typename T> void multiply_group(cudaStream_t st, Workspace& w, const crt::Product* ops, int nops) {
+  crt::right_planes<T>(st, ops, nops);
+  crt::multiply<S<T>::cplx>(st, ops, nops, 0, crt::NMOD, w.flags);
+  crt::combine<S<T>::cplx>(st, ops, nops);
 }
 
 template <typename T>
@@ -508,10 +511,10 @@ template void gemm<double>(cudaStream_t, Workspace&, Op, const double*, int64_t,
                            int64_t, int64_t, const Epi&);
 template void gemm<double2>(cudaStream_t, Workspace&, Op, const double2*, int64_t, Op, const double2*, int64_t, int64_t,
                             int64_t, int64_t, const Epi&);
-template crt::Product group_product<double>(cudaStream_t, Workspace&, const double*, int64_t, int, int64_t, const Epi&);
-template crt::Product group_product<double2>(cudaStream_t, Workspace&, const double2*, int64_t, int, int64_t, const Epi&);
-template void multiply_group<false>(cudaStream_t, Workspace&, const crt::Product*, int);
-template void multiply_group<true>(cudaStream_t, Workspace&, const crt::Product*, int);
+template crt::Product group_product<double>(Workspace&, const double*, int64_t, int, int64_t, const Epi&);
+template crt::Product group_product<double2>(Workspace&, const double2*, int64_t, int, int64_t, const Epi&);
+template void multiply_group<double>(cudaStream_t, Workspace&, const crt::Product*, int);
+template void multiply_group<double2>(cudaStream_t, Workspace&, const crt::Product*, int);
 template void hemm<double2>(cudaStream_t, Workspace&, const double2*, int64_t, int64_t, const double2*, int64_t, int,
                             const Epi&, int);
 template void split_right<double>(cudaStream_t, Workspace&, int, const double*, int64_t, int, int64_t);
