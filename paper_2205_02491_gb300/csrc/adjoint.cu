@@ -91,6 +91,7 @@ __device__ inline double block_sum(double v, double* red) {
 __global__ void minres_update_kernel(int64_t n, const double* __restrict__ Y, double* R1, const double* R2,
                                      double* Vv, double* Wn /* in: w1, out: new w */, const double* Wc /* w */,
                                      double* X, MinresState* st, double tol) {
+  grid_dependency_wait();
   const int j = blockIdx.x;
   __shared__ double red[32];
   __shared__ double sh[8];
@@ -153,6 +154,7 @@ __global__ void minres_update_kernel(int64_t n, const double* __restrict__ Y, do
 }
 
 __global__ void count_done_kernel(int nev, const MinresState* st, int* out) {
+  grid_dependency_wait();
   int c = 0;
   for (int j = threadIdx.x; j < nev; j += 32) c += st[j].done;
   for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
@@ -178,12 +180,12 @@ void minres_init(cudaStream_t st, int64_t n, int nev, const double* B, int64_t l
 
 void minres_update(cudaStream_t st, int64_t n, int nev, const double* Y, double* R1, const double* R2, double* Vv,
                    double* Wn, const double* Wc, double* X, void* state, double tol) {
-  minres_update_kernel<<<nev, 1024, 0, st>>>(n, Y, R1, R2, Vv, Wn, Wc, X, (MinresState*)state, tol);
+  launch_pdl(minres_update_kernel, nev, 1024, 0, st, n, Y, R1, R2, Vv, Wn, Wc, X, (MinresState*)state, tol);
   CHASE_CHECK_LAUNCH();
 }
 
 void minres_count_done(cudaStream_t st, int nev, const void* state, int* out) {
-  count_done_kernel<<<1, 32, 0, st>>>(nev, (const MinresState*)state, out);
+  launch_pdl(count_done_kernel, 1, 32, 0, st, nev, (const MinresState*)state, out);
   CHASE_CHECK_LAUNCH();
 }
 

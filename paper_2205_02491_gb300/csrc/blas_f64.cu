@@ -39,6 +39,7 @@ template <typename T, int OPA, int OPB>
 __global__ void __launch_bounds__(64) gemm_f64_kernel(int64_t M, int64_t N, int64_t K, const T* __restrict__ A,
                                                       int64_t lda, const T* __restrict__ B, int64_t ldb, Epi epi,
                                                       T* __restrict__ work, int64_t kchunk) {
+  grid_dependency_wait();
   using s = S<T>;
   constexpr int BK = GK<T>::BK;
   __shared__ T As[BK][GB + 1];
@@ -104,6 +105,7 @@ __global__ void __launch_bounds__(64) gemm_f64_kernel(int64_t M, int64_t N, int6
 
 template <typename T>
 __global__ void splitk_reduce_kernel(int64_t M, int64_t N, int nsplit, const T* __restrict__ work, Epi epi) {
+  grid_dependency_wait();
   using s = S<T>;
   int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (idx >= M * N) return;
@@ -133,7 +135,7 @@ void gemm_f64(cudaStream_t st, Op opA, Op opB, int64_t M, int64_t N, int64_t K, 
   CHASE_REQUIRE(ceil_div(N, GB) <= 65535, 1, "gemm_f64: too many columns");
   dim3 grid(ceil_div(M, GB), ceil_div(N, GB), nsplit);
   T* w = nsplit > 1 ? work : nullptr;
-#define LAUNCH(OA, OB) gemm_f64_kernel<T, OA, OB><<<grid, 64, 0, st>>>(M, N, std::max<int64_t>(K, 0), A, lda, B, ldb, epi, w, kchunk)
+#define LAUNCH(OA, OB) launch_pdl(gemm_f64_kernel<T, OA, OB>, grid, 64, 0, st, M, N, std::max<int64_t>(K, 0), A, lda, B, ldb, epi, w, kchunk)
   if (opA == OP_N && opB == OP_N) LAUNCH(OP_N, OP_N);
   else if (opA == OP_C && opB == OP_N) LAUNCH(OP_C, OP_N);
   else if (opA == OP_N && opB == OP_C) LAUNCH(OP_N, OP_C);
@@ -141,7 +143,7 @@ void gemm_f64(cudaStream_t st, Op opA, Op opB, int64_t M, int64_t N, int64_t K, 
 #undef LAUNCH
   CHASE_CHECK_LAUNCH();
   if (nsplit > 1) {
-    splitk_reduce_kernel<T><<<ceil_div(M * N, 256), 256, 0, st>>>(M, N, nsplit, work, epi);
+    launch_pdl(splitk_reduce_kernel<T>, ceil_div(M * N, 256), 256, 0, st, M, N, nsplit, work, epi);
     CHASE_CHECK_LAUNCH();
   }
 }
@@ -149,6 +151,7 @@ void gemm_f64(cudaStream_t st, Op opA, Op opB, int64_t M, int64_t N, int64_t K, 
 // ============================================================== column reductions
 template <typename T>
 __global__ void colnorms_kernel(int64_t n, const T* __restrict__ X, int64_t ldx, double* out) {
+  grid_dependency_wait();
   using s = S<T>;
   const T* x = X + (int64_t)blockIdx.x * ldx;
   double acc = 0.0;
@@ -166,7 +169,7 @@ __global__ void colnorms_kernel(int64_t n, const T* __restrict__ X, int64_t ldx,
 
 template <typename T> void colnorms(cudaStream_t st, int64_t n, int k, const T* X, int64_t ldx, double* out) {
   if (k <= 0) return;
-  colnorms_kernel<T><<<k, 256, 0, st>>>(n, X, ldx, out);
+  launch_pdl(colnorms_kernel<T>, k, 256, 0, st, n, X, ldx, out);
   CHASE_CHECK_LAUNCH();
 }
 
@@ -235,6 +238,7 @@ template <typename T> void fro_norm2(cudaStream_t st, int64_t n, int k, const T*
 template <typename T>
 __global__ void permute_cols_kernel(int64_t n, const T* __restrict__ src, int64_t lds, T* __restrict__ dst,
                                     int64_t ldd, const int* __restrict__ perm) {
+  grid_dependency_wait();
   int a = blockIdx.y;
   int p = perm ? perm[a] : a;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
@@ -245,7 +249,7 @@ template <typename T>
 void permute_cols(cudaStream_t st, int64_t n, int k, const T* src, int64_t lds, T* dst, int64_t ldd, const int* perm) {
   if (k <= 0 || n <= 0) return;
   dim3 grid(std::min<unsigned>(ceil_div(n, 256), 64), k);
-  permute_cols_kernel<T><<<grid, 256, 0, st>>>(n, src, lds, dst, ldd, perm);
+  launch_pdl(permute_cols_kernel<T>, grid, 256, 0, st, n, src, lds, dst, ldd, perm);
   CHASE_CHECK_LAUNCH();
 }
 
@@ -258,6 +262,7 @@ void copy_cols(cudaStream_t st, int64_t n, int k, const T* src, int64_t lds, T* 
 
 template <typename T>
 __global__ void scale_cols_kernel(int64_t n, T* X, int64_t ldx, const double* s, int invert) {
+  grid_dependency_wait();
   int a = blockIdx.y;
   double f = s[a];
   if (invert) f = (f > 0.0) ? 1.0 / f : 0.0;
@@ -268,7 +273,7 @@ __global__ void scale_cols_kernel(int64_t n, T* X, int64_t ldx, const double* s,
 template <typename T> void scale_cols(cudaStream_t st, int64_t n, int k, T* X, int64_t ldx, const double* s, int invert) {
   if (k <= 0 || n <= 0) return;
   dim3 grid(std::min<unsigned>(ceil_div(n, 256), 64), k);
-  scale_cols_kernel<T><<<grid, 256, 0, st>>>(n, X, ldx, s, invert);
+  launch_pdl(scale_cols_kernel<T>, grid, 256, 0, st, n, X, ldx, s, invert);
   CHASE_CHECK_LAUNCH();
 }
 
@@ -287,6 +292,7 @@ template <typename T> void add_diag(cudaStream_t st, int k, T* G, int64_t ldg, c
 }
 
 template <typename T> __global__ void hermitianize_kernel(int k, T* G, int64_t ldg) {
+  grid_dependency_wait();
   int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y * 32 + threadIdx.y;
   if (i >= k || j >= k || i < j) return;
   using s = S<T>;
@@ -302,7 +308,7 @@ template <typename T> __global__ void hermitianize_kernel(int k, T* G, int64_t l
 
 template <typename T> void hermitianize(cudaStream_t st, int k, T* G, int64_t ldg) {
   dim3 grid(ceil_div(k, 32), ceil_div(k, 32));
-  hermitianize_kernel<T><<<grid, dim3(32, 32), 0, st>>>(k, G, ldg);
+  launch_pdl(hermitianize_kernel<T>, grid, dim3(32, 32), 0, st, k, G, ldg);
   CHASE_CHECK_LAUNCH();
 }
 
@@ -324,6 +330,7 @@ constexpr int CROWS = 8;  // rows per panel block
 template <typename T>
 __global__ void __launch_bounds__(CROWS * CB) chol_panel_kernel(int k, int j0, T* Sm, int64_t lds, int* info,
                                                                  double floor, int* dep) {
+  grid_dependency_wait();
   using s = S<T>;
   __shared__ T a[CB][CB + 1];  // lower factor of the diagonal block
   __shared__ double rinv[CB];  // reciprocal pivots; 0 for a dependent column
@@ -388,6 +395,7 @@ __global__ void __launch_bounds__(CROWS * CB) chol_panel_kernel(int k, int j0, T
 // (entries above G's diagonal may be skipped or written: nothing reads them)
 template <typename T>
 __global__ void __launch_bounds__(64) chol_update_kernel(int k, int j0, int jend, T* Sm, int64_t lds) {
+  grid_dependency_wait();
   using s = S<T>;
   __shared__ T pr[16][CB + 1], pc[16][CB + 1];
   const int j1 = j0 + CB;  // the panel before an update is always full
@@ -437,10 +445,10 @@ template <typename T>
 void chol_stack_columns(cudaStream_t st, int k, int jbeg, int jend, T* Sm, int64_t lds, int* info, double pivot_floor,
                         int* dep) {
   for (int j0 = jbeg; j0 < jend; j0 += CB) {
-    chol_panel_kernel<T><<<ceil_div(k, CROWS), CROWS * CB, 0, st>>>(k, j0, Sm, lds, info, pivot_floor, dep);
+    launch_pdl(chol_panel_kernel<T>, ceil_div(k, CROWS), CROWS * CB, 0, st, k, j0, Sm, lds, info, pivot_floor, dep);
     CHASE_CHECK_LAUNCH();
     if (j0 + CB >= jend) break;
-    chol_update_kernel<T><<<dim3(ceil_div(k, 16), ceil_div(jend - j0 - CB, 16)), 64, 0, st>>>(k, j0, jend, Sm, lds);
+    launch_pdl(chol_update_kernel<T>, dim3(ceil_div(k, 16), ceil_div(jend - j0 - CB, 16)), 64, 0, st, k, j0, jend, Sm, lds);
     CHASE_CHECK_LAUNCH();
   }
 }
@@ -453,6 +461,7 @@ void chol_stack_columns(cudaStream_t st, int k, int jbeg, int jend, T* Sm, int64
 template <typename T>
 __global__ void __launch_bounds__(128) gram_correction_kernel(int k, int upper, const T* __restrict__ Gm, int64_t ldg, T* F,
                                                                int64_t ldf, unsigned* dev) {
+  grid_dependency_wait();
   using s = S<T>;
   const int j = blockIdx.x;
   float sum = 0.0f;
@@ -478,7 +487,7 @@ __global__ void __launch_bounds__(128) gram_correction_kernel(int k, int upper, 
 
 template <typename T>
 void gram_correction(cudaStream_t st, int k, bool upper, const T* Gm, int64_t ldg, T* F, int64_t ldf, unsigned* dev) {
-  gram_correction_kernel<T><<<k, 128, 0, st>>>(k, upper ? 1 : 0, Gm, ldg, F, ldf, dev);
+  launch_pdl(gram_correction_kernel<T>, k, 128, 0, st, k, upper ? 1 : 0, Gm, ldg, F, ldf, dev);
   CHASE_CHECK_LAUNCH();
 }
 

@@ -108,6 +108,7 @@ __device__ __forceinline__ int norm_exponent(double ss) {
 template <typename T>
 __global__ void __launch_bounds__(256) col_exponent_kernel(int64_t K, const T* __restrict__ X, int64_t ldx, int* ex) {
   using s = S<T>;
+  grid_dependency_wait();
   const T* x = X + (int64_t)blockIdx.x * ldx;
   __shared__ double red[8];
   __shared__ double sum_sh;
@@ -178,6 +179,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) row_exponent_kernel(int64_t nvec, int64_t K, const T* __restrict__ X, int64_t ldx,
                                                             int* ex) {
   using s = S<T>;
+  grid_dependency_wait();
   const int r = threadIdx.x & 31, c = threadIdx.x >> 5;
   const int64_t i = (int64_t)blockIdx.x * 32 + r;
   __shared__ double red[8][33];
@@ -310,6 +312,7 @@ __global__ void __launch_bounds__(128) residues_cols_kernel(int64_t K, int64_t K
                                                              int64_t ldx, const int* __restrict__ ex, int conj, int mod0,
                                                              int nmod, __nv_bfloat16* planes) {
   const int64_t col = blockIdx.y;
+  grid_dependency_wait();
   const T* x = X + col * ldx;
   int e = ex[col];
   if (e == NONFINITE) e = 0;
@@ -327,6 +330,7 @@ __global__ void __launch_bounds__(256) residues_rows_kernel(int64_t nvec, int64_
                                                              int64_t ldx, const int* __restrict__ ex, int conj, int mod0,
                                                              int nmod, __nv_bfloat16* planes) {
   __shared__ T tile[32][33];
+  grid_dependency_wait();
   const int64_t i0 = (int64_t)blockIdx.x * 32, k0 = (int64_t)blockIdx.y * 32;
   for (int r = threadIdx.x >> 5; r < 32; r += 8) {
     const int64_t kk = k0 + r, i = i0 + (threadIdx.x & 31);
@@ -373,6 +377,7 @@ template <int G> struct RightParams {
 template <typename T, int G>
 __global__ void __launch_bounds__(128) right_planes_kernel(const __grid_constant__ RightParams<G> rp) {
   using s = S<T>;
+  grid_dependency_wait();
   const int q = G == 1 ? 0 : blockIdx.z;
   const int col = blockIdx.y;
   if (col >= rp.nvec[q]) return;  // the whole cluster
@@ -651,6 +656,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     mbar_init(smem_u32(drain), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  grid_dependency_wait();
   }
   if (warp == 2) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(tmem_slot)));
@@ -917,6 +923,7 @@ __device__ __forceinline__ double reconstruct(const uint64_t (&a)[4], int e) {
 // ROWS = 4: four rows per thread (one 4-byte load per plane); HBM-bound on the residues (1 byte per plane and entry), the
 // weights' limb products run on the integer pipe.  ROWS = 1: one row per thread, for products too small to fill the
 // SMs otherwise, with every plane's load in flight at once.
+  grid_dependency_wait();
 template <int G> struct CombineParams {
   const int8_t* R[G];
   const int* lex[G];
@@ -1004,9 +1011,9 @@ __global__ void __launch_bounds__(64) combine_kernel(const __grid_constant__ Com
 template <typename T>
 void scales(cudaStream_t st, bool by_rows, int64_t nvec, int64_t K, const T* X, int64_t ldx, int* ex) {
   if (by_rows)
-    row_exponent_kernel<T><<<ceil_div(nvec, 32), 256, 0, st>>>(nvec, K, X, ldx, ex);
+    launch_pdl(row_exponent_kernel<T>, ceil_div(nvec, 32), 256, 0, st, nvec, K, X, ldx, ex);
   else
-    col_exponent_kernel<T><<<(unsigned)nvec, 256, 0, st>>>(K, X, ldx, ex);
+    launch_pdl(col_exponent_kernel<T>, (unsigned)nvec, 256, 0, st, K, X, ldx, ex);
   CHASE_CHECK_LAUNCH();
 }
 
@@ -1017,12 +1024,12 @@ void residues(cudaStream_t st, bool by_rows, bool conj, int64_t nvec, int64_t K,
   if (by_rows) {
     const dim3 grid(ceil_div(nvec, 32), ceil_div(K, 32));
     CHASE_REQUIRE(grid.y <= 65535, 1, "residues: vectors too long");
-    residues_rows_kernel<T><<<grid, 256, 0, st>>>(nvec, K, kp, X, ldx, ex, conj ? 1 : 0, mod0, nmod,
+    launch_pdl(residues_rows_kernel<T>, grid, 256, 0, st, nvec, K, kp, X, ldx, ex, conj ? 1 : 0, mod0, nmod,
                                                   (__nv_bfloat16*)planes);
   } else {
     CHASE_REQUIRE(nvec <= 65535, 1, "residues: too many vectors");
     const dim3 grid(ceil_div(K, 512), (unsigned)nvec);
-    residues_cols_kernel<T><<<grid, 128, 0, st>>>(K, kp, nvec, X, ldx, ex, conj ? 1 : 0, mod0, nmod,
+    launch_pdl(residues_cols_kernel<T>, grid, 128, 0, st, K, kp, nvec, X, ldx, ex, conj ? 1 : 0, mod0, nmod,
                                                   (__nv_bfloat16*)planes);
   }
   CHASE_CHECK_LAUNCH();
@@ -1101,16 +1108,16 @@ template <int G> static void launch(cudaStream_t st, const Product* ops, int nop
   gp.stage_bytes = 2 * (A_HALF + box_max * TK * 2);
   gp.stages = std::min(MAX_STAGES, SMEM_RING / gp.stage_bytes);
   cudaLaunchConfig_t cfg{};
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = 2 * pairs;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cudaLaunchAttribute at[2] = {{}, pdl_attribute()};
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 2 * pairs;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
   cfg.gridDim = dim3((unsigned)(2 * pairs * std::min<int64_t>(units, pairs == 2 ? c2 : c1)), 1, 1);
   cfg.blockDim = dim3(NTHREADS, 1, 1);
   cfg.dynamicSmemBytes = SMEM_BYTES;
   cfg.stream = st;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
   CHASE_CUDA(cudaLaunchKernelEx(&cfg, crt_gemm_kernel<G>, gp, err));
   CHASE_CHECK_LAUNCH();
 }
@@ -1142,7 +1149,7 @@ template <bool CPLX, int ROWS, int G> static void launch_combine(cudaStream_t st
     M = std::max(M, o.M);
     N = std::max(N, o.N);
   }
-  combine_kernel<CPLX, ROWS, G><<<dim3(ceil_div(M, 64 * ROWS), (unsigned)N, (unsigned)nops), 64, 0, st>>>(cp);
+  launch_pdl(combine_kernel<CPLX, ROWS, G>, dim3(ceil_div(M, 64 * ROWS), (unsigned)N, (unsigned)nops), 64, 0, st, cp);
   CHASE_CHECK_LAUNCH();
 }
 
@@ -1180,15 +1187,15 @@ template <typename T, int G> static void launch_right(cudaStream_t st, const Pro
   int cs = 1;
   while (cs < 8 && 512 * cs < K) cs *= 2;
   cudaLaunchConfig_t cfg{};
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = cs;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  cudaLaunchAttribute at[2] = {{}, pdl_attribute()};
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cs;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
   cfg.gridDim = dim3(cs, (unsigned)N, (unsigned)nops);
   cfg.blockDim = dim3(128, 1, 1);
   cfg.stream = st;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
   CHASE_CUDA(cudaLaunchKernelEx(&cfg, right_planes_kernel<T, G>, rp));
   CHASE_CHECK_LAUNCH();
 }

@@ -709,6 +709,7 @@ __device__ __forceinline__ bool bj_idle(int I, int J, int nb, int r) {
 template <typename F>
 __global__ void __launch_bounds__(BJ_SOLVE_THREADS) bj_solve_kernel(int k, int nbp, int r, const F* G, int64_t ldg,
                                                                      F* Ubuf, int full) {
+  grid_dependency_wait();
   using s = S<F>;
   extern __shared__ __align__(16) unsigned char bj_smem[];
   F* Sm = reinterpret_cast<F*>(bj_smem);    // [2][64][64], row-major by position
@@ -786,6 +787,7 @@ __global__ void __launch_bounds__(BJ_SOLVE_THREADS) bj_solve_kernel(int k, int n
 template <typename F>
 __global__ void __launch_bounds__(BJ_UPD_THREADS) bj_cols_kernel(int k, int nbp, int r, F* G, int64_t ldg, F* Z,
                                                                   int64_t ldz, const F* __restrict__ Ubuf) {
+  grid_dependency_wait();
   using s = S<F>;
   __shared__ __align__(16) F Us[BJ_M][BJ_M];    // U[m][c]
   __shared__ F Xs[BJ_M][BJ_TILE];               // X[row][m] at Xs[m][row]
@@ -826,6 +828,7 @@ __global__ void __launch_bounds__(BJ_UPD_THREADS) bj_cols_kernel(int k, int nbp,
 template <typename F>
 __global__ void __launch_bounds__(BJ_UPD_THREADS) bj_rows_kernel(int k, int nbp, int r, F* G, int64_t ldg,
                                                                   const F* __restrict__ Ubuf) {
+  grid_dependency_wait();
   using s = S<F>;
   __shared__ F Us[BJ_M][BJ_M + 1];      // U[m][l]
   __shared__ F Xs[BJ_TILE][BJ_M];       // X[m][column] at Xs[column][m]
@@ -907,12 +910,12 @@ int heev_block_jacobi(cudaStream_t st, int k, F* G, int64_t ldg, double* w, F* Z
     if (sweeps >= 2 && hstat[0] > 0.0625 * prev_off && sqrt(hstat[0]) <= 1e-5 * sqrt(hstat[1])) break;
     prev_off = hstat[0];
     for (int r = 0; r < nbp - 1; ++r) {
-      bj_solve_kernel<F><<<npairs, BJ_SOLVE_THREADS, bj_solve_smem_bytes<F>(), st>>>(k, nbp, r, G, ldg, Ubuf, r == 0);
+      launch_pdl(bj_solve_kernel<F>, npairs, BJ_SOLVE_THREADS, bj_solve_smem_bytes<F>(), st, k, nbp, r, G, ldg, Ubuf, r == 0);
       CHASE_CHECK_LAUNCH();
-      bj_cols_kernel<F><<<dim3(tiles, npairs, 2), BJ_UPD_THREADS, 0, st>>>(k, nbp, r, G, ldg, Zu, k,
+      launch_pdl(bj_cols_kernel<F>, dim3(tiles, npairs, 2), BJ_UPD_THREADS, 0, st, k, nbp, r, G, ldg, Zu, k,
                                                                                           Ubuf);
       CHASE_CHECK_LAUNCH();
-      bj_rows_kernel<F><<<dim3(tiles, npairs), BJ_UPD_THREADS, 0, st>>>(k, nbp, r, G, ldg, Ubuf);
+      launch_pdl(bj_rows_kernel<F>, dim3(tiles, npairs), BJ_UPD_THREADS, 0, st, k, nbp, r, G, ldg, Ubuf);
       CHASE_CHECK_LAUNCH();
     }
   }

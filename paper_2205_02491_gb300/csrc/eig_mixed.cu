@@ -31,6 +31,7 @@ template <typename T, typename F> void convert_mat(cudaStream_t st, int k, const
 
 template <typename T>
 __global__ void correction_kernel(int k, const T* Gp, int64_t ldg, T* X, int64_t ldx, double omega) {
+  grid_dependency_wait();
   using s = S<T>;
   int p = blockIdx.x * blockDim.x + threadIdx.x, q = blockIdx.y;
   if (p >= k) return;
@@ -45,7 +46,7 @@ __global__ void correction_kernel(int k, const T* Gp, int64_t ldg, T* X, int64_t
 
 template <typename T>
 void eig_correction(cudaStream_t st, int k, const T* Gp, int64_t ldg, T* X, int64_t ldx, double omega) {
-  correction_kernel<T><<<dim3(ceil_div(k, 128), k), 128, 0, st>>>(k, Gp, ldg, X, ldx, omega);
+  launch_pdl(correction_kernel<T>, dim3(ceil_div(k, 128), k), 128, 0, st, k, Gp, ldg, X, ldx, omega);
   CHASE_CHECK_LAUNCH();
 }
 

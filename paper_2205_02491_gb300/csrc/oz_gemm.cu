@@ -19,6 +19,7 @@ namespace oz {
 // Per-column power-of-two scale s = 2^e with max|re|,|im| = f 2^e, f in [0.5, 1).
 template <typename T>
 __global__ void col_scale_kernel(int64_t K, const T* __restrict__ X, int64_t ldx, double* scale) {
+  grid_dependency_wait();
   const T* x = X + (int64_t)blockIdx.x * ldx;
   double m = 0.0;
   for (int64_t i = threadIdx.x; i < K; i += blockDim.x) {
@@ -58,6 +59,7 @@ template <int NS> __device__ __forceinline__ void digits(double xs, __nv_bfloat1
 template <typename T, int NS, int KIND>
 __global__ void split_cols_kernel(int64_t K, int64_t Kpad, int ncols, const T* __restrict__ X, int64_t ldx,
                                   const double* __restrict__ scale, int conj, __nv_bfloat16* planes) {
+  grid_dependency_wait();
   constexpr bool CPLX = S<T>::cplx;
   const int col = blockIdx.y;
   const T* x = X + (int64_t)col * ldx;
@@ -188,10 +190,10 @@ template <typename T>
 static void split(cudaStream_t st, int S_, int kind, bool conj, const T* X, int64_t ld, int64_t nvec, int64_t K,
                   void* planes, double* scale) {
   const int64_t kp = kpad(K);
-  col_scale_kernel<T><<<(unsigned)nvec, 256, 0, st>>>(K, X, ld, scale);
+  launch_pdl(col_scale_kernel<T>, (unsigned)nvec, 256, 0, st, K, X, ld, scale);
   CHASE_CHECK_LAUNCH();
   dim3 grid(std::min<unsigned>(ceil_div(K, 256), 32), (unsigned)nvec);
-#define SC(SS, KD) split_cols_kernel<T, SS, KD><<<grid, 256, 0, st>>>(K, kp, (int)nvec, X, ld, scale, conj ? 1 : 0, (__nv_bfloat16*)planes)
+#define SC(SS, KD) launch_pdl(split_cols_kernel<T, SS, KD>, grid, 256, 0, st, K, kp, (int)nvec, X, ld, scale, conj ? 1 : 0, (__nv_bfloat16*)planes)
   if (S_ == 2 && kind == 1) SC(2, 1);
   else if (S_ == 3 && kind == 1) SC(3, 1);
   else if (S_ == 3 && kind == 0) SC(3, 0);

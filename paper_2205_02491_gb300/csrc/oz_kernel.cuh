@@ -216,6 +216,7 @@ __global__ void __maxnreg__(168) oz_gemm_kernel(const __grid_constant__ GroupPar
   fence_before();
   __syncthreads();
   fence_after();
+  grid_dependency_wait();
   const uint32_t tmem = *tmem_slot;
 
   if (warp == 0 && lane == 0) {
@@ -392,6 +393,7 @@ __global__ void __maxnreg__(168) oz_gemm_kernel(const __grid_constant__ GroupPar
 // result does not depend on scheduling).
 template <bool CPLX>
 __global__ void split_reduce_kernel(int M, int N, int ksplit, const double* __restrict__ part, EpiArgs ep) {
+  grid_dependency_wait();
   constexpr int comp = CPLX ? 2 : 1;
   const int64_t total = (int64_t)M * N * comp;
   for (int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; idx < total; idx += (int64_t)gridDim.x * blockDim.x) {
@@ -458,12 +460,12 @@ void launch_ops(cudaStream_t st, Workspace& w, const ProductOp* ops, int nops, c
   const bool timed = w.timing && w.ev_used + 2 <= (int)w.ev.size();
   if (timed) CHASE_CUDA(cudaEventRecord(w.ev[w.ev_used], st));
   if (tune_ev) CHASE_CUDA(cudaEventRecord(tune_ev[0], st));
-  oz_gemm_kernel<S, CPLX, NTT, G><<<(unsigned)tiles, NTHREADS, Cf::SMEM_BYTES, st>>>(gp, w.flags);
+  launch_pdl(oz_gemm_kernel<S, CPLX, NTT, G>, (unsigned)tiles, NTHREADS, Cf::SMEM_BYTES, st, gp, w.flags);
   CHASE_CHECK_LAUNCH();
   for (int q = 0; q < nops; ++q) {
     if (gp.ksplit[q] <= 1) continue;
     const int64_t total = ops[q].M * ops[q].N * (CPLX ? 2 : 1);
-    split_reduce_kernel<CPLX><<<(unsigned)std::min<int64_t>(ceil_div(total, 256), 4096), 256, 0, st>>>(
+    launch_pdl(split_reduce_kernel<CPLX>, (unsigned)std::min<int64_t>(ceil_div(total, 256), 4096), 256, 0, st, 
         (int)ops[q].M, (int)ops[q].N, gp.ksplit[q], ops[q].part, gp.ep[q]);
     CHASE_CHECK_LAUNCH();
   }
