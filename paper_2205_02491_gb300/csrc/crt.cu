@@ -107,8 +107,8 @@ __device__ __forceinline__ int norm_exponent(double ss) {
 // bits to underflow (or a non-finite one) takes a second, scaled pass.  HBM/L2-bound, one block per column.
 template <typename T>
 __global__ void __launch_bounds__(256) col_exponent_kernel(int64_t K, const T* __restrict__ X, int64_t ldx, int* ex) {
-  using s = S<T>;
   grid_dependency_wait();
+  using s = S<T>;
   const T* x = X + (int64_t)blockIdx.x * ldx;
   __shared__ double red[8];
   __shared__ double sum_sh;
@@ -178,8 +178,8 @@ __global__ void __launch_bounds__(256) col_exponent_kernel(int64_t K, const T* _
 template <typename T>
 __global__ void __launch_bounds__(256) row_exponent_kernel(int64_t nvec, int64_t K, const T* __restrict__ X, int64_t ldx,
                                                             int* ex) {
-  using s = S<T>;
   grid_dependency_wait();
+  using s = S<T>;
   const int r = threadIdx.x & 31, c = threadIdx.x >> 5;
   const int64_t i = (int64_t)blockIdx.x * 32 + r;
   __shared__ double red[8][33];
@@ -311,8 +311,8 @@ template <typename T>
 __global__ void __launch_bounds__(128) residues_cols_kernel(int64_t K, int64_t Kp, int64_t nvec, const T* __restrict__ X,
                                                              int64_t ldx, const int* __restrict__ ex, int conj, int mod0,
                                                              int nmod, __nv_bfloat16* planes) {
-  const int64_t col = blockIdx.y;
   grid_dependency_wait();
+  const int64_t col = blockIdx.y;
   const T* x = X + col * ldx;
   int e = ex[col];
   if (e == NONFINITE) e = 0;
@@ -329,8 +329,8 @@ template <typename T>
 __global__ void __launch_bounds__(256) residues_rows_kernel(int64_t nvec, int64_t K, int64_t Kp, const T* __restrict__ X,
                                                              int64_t ldx, const int* __restrict__ ex, int conj, int mod0,
                                                              int nmod, __nv_bfloat16* planes) {
-  __shared__ T tile[32][33];
   grid_dependency_wait();
+  __shared__ T tile[32][33];
   const int64_t i0 = (int64_t)blockIdx.x * 32, k0 = (int64_t)blockIdx.y * 32;
   for (int r = threadIdx.x >> 5; r < 32; r += 8) {
     const int64_t kk = k0 + r, i = i0 + (threadIdx.x & 31);
@@ -376,8 +376,8 @@ template <int G> struct RightParams {
 // columns: 87 us instead of 130.
 template <typename T, int G>
 __global__ void __launch_bounds__(128) right_planes_kernel(const __grid_constant__ RightParams<G> rp) {
-  using s = S<T>;
   grid_dependency_wait();
+  using s = S<T>;
   const int q = G == 1 ? 0 : blockIdx.z;
   const int col = blockIdx.y;
   if (col >= rp.nvec[q]) return;  // the whole cluster
@@ -656,7 +656,6 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     mbar_init(smem_u32(drain), 1);
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-  grid_dependency_wait();
   }
   if (warp == 2) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(tmem_slot)));
@@ -666,6 +665,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   __syncthreads();
   cluster_sync();
   fence_after();
+  grid_dependency_wait();
   const uint32_t tmem = *tmem_slot;
 
   if (warp < 4) {
@@ -923,7 +923,6 @@ __device__ __forceinline__ double reconstruct(const uint64_t (&a)[4], int e) {
 // ROWS = 4: four rows per thread (one 4-byte load per plane); HBM-bound on the residues (1 byte per plane and entry), the
 // weights' limb products run on the integer pipe.  ROWS = 1: one row per thread, for products too small to fill the
 // SMs otherwise, with every plane's load in flight at once.
-  grid_dependency_wait();
 template <int G> struct CombineParams {
   const int8_t* R[G];
   const int* lex[G];
@@ -933,6 +932,7 @@ template <int G> struct CombineParams {
 };
 template <bool CPLX, int ROWS, int G>
 __global__ void __launch_bounds__(64) combine_kernel(const __grid_constant__ CombineParams<G> cp) {
+  grid_dependency_wait();
   constexpr int NP = CPLX ? 3 : 1, NC = CPLX ? 2 : 1;
   const int prob = G == 1 ? 0 : blockIdx.z;
   const int M = cp.M[prob], N = cp.N[prob], ldr = cp.ldr[prob];
