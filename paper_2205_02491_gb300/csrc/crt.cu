@@ -38,6 +38,7 @@ using oz::mbar_expect_tx;
 using oz::mbar_init;
 using oz::mbar_try;
 using oz::smem_u32;
+using oz::sw128_desc;
 
 // ---------------------------------------------------------------- moduli and reconstruction constants
 typedef unsigned __int128 u128;
@@ -550,16 +551,6 @@ __device__ __forceinline__ void commit_to(uint32_t bar, uint32_t mask) {
       "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar),
       "h"((uint16_t)mask)
       : "memory");
-}
-// K-major operand tile, 128-byte swizzle: 8-row groups 1024 bytes apart
-__device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr >> 4) & 0x3FFF);
-  d |= (uint64_t)1 << 16;
-  d |= (uint64_t)(1024 >> 4) << 32;
-  d |= (uint64_t)1 << 46;
-  d |= (uint64_t)2 << 61;
-  return d;
 }
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t* r) {
   asm volatile(

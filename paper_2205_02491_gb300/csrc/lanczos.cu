@@ -1,6 +1,6 @@
 // Lanczos spectral-bound estimation (Algorithm 1, line 2) on the device.
 //
-// All runs advance together, two launches per step: the product of A with one vector per run (hemv_mma_kernel, A
+// All runs advance together, two launches per step: the product of A with one vector per run (hemv_kernel, A
 // streamed once per step), and the rest of the step (lanczos_step_kernel, one cluster of CTAs per run): three-term
 // update, one classical Gram-Schmidt reorthogonalisation against the run's basis, normalisation.  The tridiagonal T
 // of each run is diagonalised by implicit QL, and one block computes b_sup = max(theta_max + |beta_last|),
@@ -13,6 +13,7 @@
 
 #include "common.cuh"
 #include "kernels.h"
+#include "tcgen05.cuh"
 
 namespace chase {
 
@@ -20,8 +21,9 @@ constexpr int LZ_MAXR = 8;      // runs
 constexpr int LZ_MAXS = 64;     // steps
 
 // ---------------------------------------------------------------- fixed-point operands
-// A value x with |x| < 2^e is held as r = round(x 2^(54 - e)), |r| <= 2^54, in balanced base-256 digits
-// r = sum_t d_t 256^t, t = 0..6, d_t in [-128, 127]: adding 128 to every digit makes them the bytes of an integer.
+// An entry x of a vector with |x| < 2^e is held as r = round(x 2^(54 - e)), |r| <= 2^54, in balanced base-256 digits
+// r = sum_t d_t 256^t, t = 0..6, d_t in [-128, 127]: adding 128 to every digit makes them the bytes of an integer.  An
+// entry of A is cut to 56 bits and a sign, seven plain base-256 digits: most of the work is cutting A, once per step.
 constexpr int LZ_NONFINITE = 0x7fffffff;
 constexpr int NDIG = 7;
 constexpr unsigned long long DIGIT_BIAS = 0x80808080808080ull;
@@ -68,216 +70,425 @@ __global__ void __launch_bounds__(128) row_max_kernel(int64_t n, const T* __rest
   atomicMax(&rmax[i], (unsigned)(m >> 32));
 }
 
-// part[c][r][i] = sum_{j in chunk c} A[i,j] X[j,r] for up to 8 real columns (4 complex runs, re and im interleaved).
-// FP64 multiply-adds bound a plain version (GB300: 2 per SM and clock; four complex vectors take 16 per element of A,
-// 1.78 ms at n = 8192 where reading A takes 0.16 ms), and 64-bit integer ones are only 8 times faster (1.03 ms).
-// Here A (per row) and X (per run) are 55-bit fixed-point numbers in seven 8-bit digits; the digits of A are made in
-// registers, straight into the fragments of mma.sync m16n8k16 (f16 digits, FP32 sums), whose 8 columns are the
-// vectors.  Digit pairs up to level 7 (34 of 49; the rest is below 2^-56 of the scales' product) go to one accumulator
-// per level, exact over 64 columns (at most 8 pairs x 2 planes x 64 products of 2^14 < 2^24), then to integers.
-constexpr int HEMV_ROWS = 64;    // 16 per warp
-constexpr int HEMV_FOLD = 4;     // 16-column steps between folds
-constexpr int NLEV = 8;
-
-__device__ __forceinline__ void mma_16816(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-               : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-               : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+// |x| 2^(56 - e) cut to an integer below 2^56 for |x| < 2^e, c = 1029 + e: the mantissa with its leading bit at 62, shifted
+// right by c minus the biased exponent.  Exact zero for x = 0; subnormal x only with e below -966, which the caller scales.
+__device__ __forceinline__ unsigned long long cut56(uint32_t lo, uint32_t hi, int c) {
+  const uint32_t mh = (__funnelshift_l(lo, hi, 10) & 0x3fffffffu) | 0x40000000u;
+  const uint32_t n = min((uint32_t)(c - (int)((hi >> 20) & 0x7ffu)), 63u);
+  return ((unsigned long long)mh << 32 | (lo << 10)) >> n;
 }
-
-// digits t = 0..6 of two fixed-point numbers as f16 pairs (exact: 1024 + byte - 1152)
-__device__ __forceinline__ void digit_pairs(long long r0, long long r1, uint32_t (&out)[NDIG]) {
-  const unsigned long long w0 = (unsigned long long)r0 + DIGIT_BIAS, w1 = (unsigned long long)r1 + DIGIT_BIAS;
-  const uint32_t l0 = (uint32_t)w0, l1 = (uint32_t)w1, h0 = (uint32_t)(w0 >> 32), h1 = (uint32_t)(w1 >> 32);
-  const uint32_t b[4] = {__byte_perm(l0, l1, 0x5140), __byte_perm(l0, l1, 0x7362), __byte_perm(h0, h1, 0x5140),
-                         __byte_perm(h0, h1, 0x7362)};
-  const __half2 off = __half2(__ushort_as_half(0x6480), __ushort_as_half(0x6480));  // 1152
+// base-256 digits t = 0..6 of two numbers as f16 pairs in units of 2^-24: a digit's byte with the number's sign bit is
+// that f16 subnormal, exactly, without a conversion
+__device__ __forceinline__ void digit_pairs(double x0, double x1, int c, uint32_t (&out)[NDIG]) {
+  const uint32_t h0 = (uint32_t)__double2hiint(x0), h1 = (uint32_t)__double2hiint(x1);
+  const unsigned long long r0 = cut56((uint32_t)__double2loint(x0), h0, c), r1 = cut56((uint32_t)__double2loint(x1), h1, c);
+  const uint32_t sgn = __byte_perm(h0, h1, 0x7632) & 0x80008000u;
+  const uint32_t l0 = (uint32_t)r0, l1 = (uint32_t)r1, u0 = (uint32_t)(r0 >> 32), u1 = (uint32_t)(r1 >> 32);
+  const uint32_t p[3] = {__byte_perm(l0, l1, 0x5410), __byte_perm(l0, l1, 0x7632), __byte_perm(u0, u1, 0x5410)};
 #pragma unroll
-  for (int t = 0; t < NDIG; ++t) {
-    const uint32_t v = __byte_perm(b[t >> 1], 0x64646464u, (t & 1) ? 0x4342 : 0x4140);
-    const __half2 h = __hsub2(*reinterpret_cast<const __half2*>(&v), off);
-    out[t] = *reinterpret_cast<const uint32_t*>(&h);
-  }
+  for (int t = 0; t < 6; ++t) out[t] = ((t & 1 ? p[t >> 1] >> 8 : p[t >> 1]) & 0x00ff00ffu) | sgn;
+  out[6] = __byte_perm(u0, u1, 0x7632) | sgn;
 }
 
-// Vectors as B fragments: for every 16 columns of A (rows of X), digit and lane the lane's registers
-// (k = 2t, 2t + 1 | 2t + 8, 2t + 9 of vector column g; lane = 4 g + t).  Complex: form 0 multiplies Re A
-// (columns re, im of each run), form 1 multiplies Im A (columns -im, re).
+// Vectors as the products' right operand: for every 64 columns of A (rows of X) and form, 64 rows of 64 f16 digits in
+// the 128-byte-swizzled K-major layout that the MMA reads, so that one bulk copy brings a block to shared memory.  Row
+// (6 - u) 8 + c is digit u of vector column c (8 real columns: up to 8 runs; complex: re and im of up to 4).  Complex:
+// form 0 multiplies Re A (columns re, im of each run), form 1 multiplies Im A (columns -im, re).
+constexpr int HK = 64;                    // columns of A per block
+constexpr int FORM_HALVES = 64 * HK;
 template <typename T> struct Frag {
   static constexpr int FORMS = S<T>::cplx ? 2 : 1;
   static constexpr int RUNS = S<T>::cplx ? 4 : 8;       // runs per group of 8 columns
-  static constexpr int LANE_HALVES = FORMS * 4;         // halves per lane and digit
-  static constexpr int STEP_HALVES = NDIG * 32 * LANE_HALVES;
+  static constexpr int BLOCK_HALVES = FORMS * FORM_HALVES;
 };
 inline int64_t frag_halves(int64_t n, bool cplx, int runs) {
   const int per = cplx ? 4 : 8;
-  return (n + 15) / 16 * ((runs + per - 1) / per) * (NDIG * 32 * (cplx ? 8 : 4));
+  return (n + HK - 1) / HK * ((runs + per - 1) / per) * ((cplx ? 2 : 1) * FORM_HALVES);
 }
 // writes digit t = 0..6 of entry j of a run's vector
 template <typename T>
-__device__ __forceinline__ void write_frag(__half* X, int64_t nk16, int64_t j, int run, long long re, long long im) {
+__device__ __forceinline__ void write_frag(__half* X, int64_t nkb, int64_t j, int run, long long re, long long im) {
   using F = Frag<T>;
-  const int grp = run / F::RUNS, r = run % F::RUNS, kk = (int)(j & 15);
-  __half* base = X + ((int64_t)grp * nk16 + (j >> 4)) * F::STEP_HALVES;
-  const int reg = kk >> 3, t4 = (kk & 7) >> 1, half = kk & 1;
+  const int grp = run / F::RUNS, r = run % F::RUNS, kk = (int)(j & (HK - 1));
+  __half* base = X + ((int64_t)grp * nkb + j / HK) * F::BLOCK_HALVES;
+  auto at = [&](int row) { return base + row * HK + (((kk >> 3) ^ (row & 7)) << 3) + (kk & 7); };
   unsigned long long wr = (unsigned long long)re + DIGIT_BIAS, wi = (unsigned long long)im + DIGIT_BIAS;
   for (int t = 0; t < NDIG; ++t, wr >>= 8, wi >>= 8) {
+    const int row = (NDIG - 1 - t) * 8;
     const __half dr = __int2half_rn((int)(wr & 0xff) - 128);
-    __half* o = base + (int64_t)t * 32 * F::LANE_HALVES;
     if (F::FORMS == 2) {
       const __half di = __int2half_rn((int)(wi & 0xff) - 128);
-      __half* c0 = o + ((2 * r) * 4 + t4) * F::LANE_HALVES + reg * 2 + half;
-      __half* c1 = o + ((2 * r + 1) * 4 + t4) * F::LANE_HALVES + reg * 2 + half;
+      __half* c0 = at(row + 2 * r);
+      __half* c1 = at(row + 2 * r + 1);
       c0[0] = dr;
       c1[0] = di;
-      c0[4] = __hneg(di);
-      c1[4] = dr;
+      c0[FORM_HALVES] = __hneg(di);
+      c1[FORM_HALVES] = dr;
     } else {
-      o[(r * 4 + t4) * F::LANE_HALVES + reg * 2 + half] = dr;
+      *at(row + r) = dr;
     }
   }
+}
+
+// part[c][r][i] = sum_{j in chunk c} A[i,j] X[j,r] for up to 8 real columns (4 complex runs, re and im interleaved).
+// FP64 multiply-adds bound a plain version (GB300: 2 per SM and clock; four complex vectors take 16 per element of A,
+// 1.78 ms at n = 8192 where reading A takes 0.16 ms).  Here both are fixed-point numbers in seven 8-bit digits,
+// multiplied on the tensor cores (f16 digits, FP32 sums).  With mma.sync the 34 digit pairs that count bound it (0.44
+// ms).  tcgen05 takes digit t of A (128 rows x 16 columns in TMEM) against all digits of X at once: X's digits are the
+// MMA's columns, and accumulator columns of one level t + u coincide when digit t's window starts 6 - t groups of 8
+// columns along, so seven MMAs per form do all pairs; levels past 7 (below 2^-56 of the scales' product) fall into
+// columns nobody reads.  Sums are exact over 32 columns (at most 7 pairs x 2 planes x 32 products of 255 x 128 < 2^24),
+// then go to integers (at most 128 of them).
+// Warps 0-3 add up the accumulators; warps 4-11 (two groups of 128 threads, one row per thread, alternating 16-column
+// steps) make digits in registers and store them to their group's TMEM operand; warp 12 issues MMAs, warp 13 copies X.
+// Each thread brings its own entries of A through shared memory with cp.async (64 KB in flight per SM), so no barrier
+// guards them.  Registers: 512 threads at 128; the sums take 160, the digits 136, the rest keep 80.
+// What bounds it: the integer instructions that cut A's entries into digits, next to the HBM time: complex, n = 8192,
+// 4 runs: 208 us a step (5.2 TB/s), 436 with mma.sync.
+constexpr int HEMV_ROWS = 128;
+constexpr int HEMV_THREADS = 512;        // warps 14, 15 idle: whole warpgroups
+constexpr int HSTEP = 16;                // columns per MMA step
+constexpr int H_XSTAGES = 4;
+constexpr int NLEV = 8;
+constexpr int H_ACC = 80;                // TMEM columns per accumulator: 72 written
+constexpr int H_A0 = 2 * H_ACC;          // then one operand per producer group
+constexpr int H_ASLOT = 2 * NDIG * 8;    // 14 digit planes of 8 columns
+constexpr unsigned long long H_TIMEOUT_NS = 2000000000ull;
+template <typename T> struct Hemv {
+  static constexpr int SLOTS = S<T>::cplx ? 2 : 4;                            // steps of A in flight per thread
+  static constexpr int A_BYTES = SLOTS * 2 * HSTEP * 128 * (int)sizeof(T);   // 128 KB
+  static constexpr int X_BYTES = Frag<T>::BLOCK_HALVES * 2;
+  static constexpr int SMEM = 1024 + H_XSTAGES * X_BYTES + A_BYTES + 256;
+};
+
+// bounded wait: false on timeout or when another role gave up
+__device__ __forceinline__ bool hemv_wait(uint32_t bar, uint32_t parity, volatile int* gave_up) {
+  unsigned long long t0 = 0;
+  for (uint32_t it = 0;; ++it) {
+    if (oz::mbar_try(bar, parity)) return true;
+    if ((it & 255) == 255) {
+      if (*gave_up) return false;
+      const unsigned long long t = oz::globaltimer();
+      if (t0 == 0) t0 = t;
+      else if (t - t0 > H_TIMEOUT_NS) {
+        *gave_up = 1;
+        return false;
+      }
+    }
+  }
+}
+// D (+)= A B, A (f16, 128 x 16) in TMEM
+__device__ __forceinline__ void mma_tmem_a(uint32_t d, uint32_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d),
+      "r"(a), "l"(b), "r"(idesc), "r"(acc));
+}
+__device__ __forceinline__ void tmem_st(uint32_t a, const uint32_t (&r)[4]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x4.b32 [%0], {%1,%2,%3,%4};" ::"r"(a), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3])
+               : "memory");
+}
+__device__ __forceinline__ void tmem_st(uint32_t a, const uint32_t (&r)[8]) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"r"(a), "r"(r[0]), "r"(r[1]),
+               "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+               : "memory");
+}
+// 16 accumulator columns; the wait takes the registers in and out, so that no use moves before it
+__device__ __forceinline__ void tmem_ld16(uint32_t a, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(a));
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]), "+r"(r[8]),
+                 "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+               :
+               : "memory");
 }
 
 template <typename T>
-__global__ void __launch_bounds__(2 * HEMV_ROWS) hemv_mma_kernel(int64_t n, const T* __restrict__ A, int64_t lda,
-                                                                  const unsigned* __restrict__ rmax,
-                                                                  const __half* __restrict__ X,
-                                                                  const int* __restrict__ xe, int cols, int runs,
-                                                                  T* part) {
+__global__ void __launch_bounds__(HEMV_THREADS, 1) hemv_kernel(int64_t n, const T* __restrict__ A, int64_t lda,
+                                                                const unsigned* __restrict__ rmax,
+                                                                const __half* __restrict__ X,
+                                                                const int* __restrict__ xe, int cols, int runs, T* part) {
   using s = S<T>;
   using F = Frag<T>;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t4 = lane & 3;
-  const int64_t row0 = (int64_t)blockIdx.x * HEMV_ROWS + warp * 16 + g, row1 = row0 + 8;
+  using H = Hemv<T>;
+  using oz::smem_u32;
+  extern __shared__ __align__(1024) unsigned char hemv_smem[];
+  unsigned char* smem = (unsigned char*)(((uintptr_t)hemv_smem + 1023) & ~(uintptr_t)1023);
+  unsigned char* abuf = smem + H_XSTAGES * H::X_BYTES;
+  uint64_t* xfull = (uint64_t*)(abuf + H::A_BYTES);  // a block of X has landed
+  uint64_t* xempty = xfull + H_XSTAGES;              // its MMAs are done
+  uint64_t* afull = xempty + H_XSTAGES;              // a group's digits are in TMEM
+  uint64_t* aempty = afull + 2;                      // their MMAs are done
+  uint64_t* dfull = aempty + 2;                      // an accumulator is complete
+  uint64_t* dempty = dfull + 2;                      // it has been read
+  uint64_t* drain = dempty + 2;
+  uint32_t* tmem_slot = (uint32_t*)(drain + 1);
+  volatile int* gave_up = (volatile int*)(tmem_slot + 1);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < H_XSTAGES; ++i) {
+      oz::mbar_init(smem_u32(&xfull[i]), 1);
+      oz::mbar_init(smem_u32(&xempty[i]), 1);
+    }
+    for (int i = 0; i < 2; ++i) {
+      oz::mbar_init(smem_u32(&afull[i]), 4);
+      oz::mbar_init(smem_u32(&aempty[i]), 1);
+      oz::mbar_init(smem_u32(&dfull[i]), 1);
+      oz::mbar_init(smem_u32(&dempty[i]), 4);
+    }
+    oz::mbar_init(smem_u32(drain), 1);
+    *gave_up = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(tmem_slot)));
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+  }
+  oz::fence_before();
+  __syncthreads();
+  oz::fence_after();
+  grid_dependency_wait();
+  const uint32_t tmem = *tmem_slot;
+
+  const int64_t row = (int64_t)blockIdx.x * HEMV_ROWS + (warp & 3) * 32 + lane;  // warps 0-11
   const int64_t jbeg = (int64_t)blockIdx.y * cols, jend = jbeg + cols < n ? jbeg + cols : n;
   const int grp = blockIdx.z;
-  const int64_t nk16 = (n + 15) / 16;
-  const bool l0 = row0 < n, l1 = row1 < n;
-  const int e0 = l0 ? exponent_of_bits((unsigned long long)rmax[row0] << 32 | 0xffffffffull) : 0;
-  const int e1 = l1 ? exponent_of_bits((unsigned long long)rmax[row1] << 32 | 0xffffffffull) : 0;
-  const int s0 = e0 == LZ_NONFINITE ? 0 : e0, s1 = e1 == LZ_NONFINITE ? 0 : e1;
-  float acc[NLEV][4];
-  int sum[NLEV][4];
+  const int nblk = (int)((jend - jbeg + HK - 1) / HK);  // blocks of 64 columns
+  const int ea = row < n && warp < 12 ? exponent_of_bits((unsigned long long)rmax[row] << 32 | 0xffffffffull) : 0;
+  const uint32_t lane_addr = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+
+  if (warp < 4) {
+    // ------------------------------------------------------------ sums of the accumulators
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 160;");
+    int sum[NLEV][8];
 #pragma unroll
-  for (int l = 0; l < NLEV; ++l)
+    for (int l = 0; l < NLEV; ++l)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      acc[l][q] = 0.0f;
-      sum[l][q] = 0;
+      for (int q = 0; q < 8; ++q) sum[l][q] = 0;
+    bool ok = true;
+    for (int k = 0; k < 2 * nblk; ++k) {
+      const int b = k & 1;
+      ok = __all_sync(0xffffffffu, hemv_wait(smem_u32(&dfull[b]), (k >> 1) & 1, gave_up));
+      if (!ok) break;
+      oz::fence_after();
+#pragma unroll
+      for (int h = 0; h < 4; ++h) {
+        uint32_t r[16];
+        tmem_ld16(lane_addr + (uint32_t)(b * H_ACC + h * 16), r);
+#pragma unroll
+        for (int q = 0; q < 16; ++q) sum[2 * h + (q >> 3)][q & 7] += __float2int_rn(__uint_as_float(r[q]) * 16777216.0f);
+      }
+      oz::fence_before();
+      __syncwarp();
+      if (lane == 0) oz::mbar_arrive(smem_u32(&dempty[b]));
     }
-  const __half* xb = X + ((int64_t)grp * nk16 + jbeg / 16) * F::STEP_HALVES + lane * F::LANE_HALVES;
-  const T* a0 = A + row0 + (jbeg + 2 * t4) * lda;
-  int fold = 0;
-  // this lane's 2 x 4 entries of the step: rows row0, row1; columns 2t, 2t + 1, 2t + 8, 2t + 9
-  T v[2][4], w[2][4];
-  auto load = [&](int64_t j, const T* a, T (&o)[2][4]) {
+    // levels 0-3 and 4-7 as two integers; value = (hi 2^32 + lo) 2^40, in units of 2^(ea + ex - 110)
+    if (row < n) {
+      double o[8];
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int dj = (q & 1) + 8 * (q >> 1);
-      const bool in = j + 2 * t4 + dj < jend;
-      o[0][q] = in && l0 ? a[dj * lda] : s::zero();
-      o[1][q] = in && l1 ? a[dj * lda + 8] : s::zero();
-    }
-  };
-  load(jbeg, a0, v);
-  for (int64_t j = jbeg; j < jend; j += 16) {
-    a0 += 16 * lda;
-    load(j + 16, a0, w);  // past the end: zeros, no access
-    uint32_t bf[NDIG][F::FORMS][2];
+      for (int q = 0; q < 8; ++q) {
+        const long long hi = ((long long)sum[0][q] << 24) + ((long long)sum[1][q] << 16) + ((long long)sum[2][q] << 8) + sum[3][q];
+        const long long lo = ((long long)sum[4][q] << 24) + ((long long)sum[5][q] << 16) + ((long long)sum[6][q] << 8) + sum[7][q];
+        o[q] = (double)hi * 4294967296.0 + (double)lo;
+      }
+      T* out = part + (int64_t)blockIdx.y * runs * n + row;
 #pragma unroll
-    for (int u = 0; u < NDIG; ++u) {
-      const __half* p = xb + u * 32 * F::LANE_HALVES;
-      if (F::FORMS == 2) {
-        const uint4 q = *reinterpret_cast<const uint4*>(p);
-        bf[u][0][0] = q.x;
-        bf[u][0][1] = q.y;
-        bf[u][F::FORMS - 1][0] = q.z;
-        bf[u][F::FORMS - 1][1] = q.w;
-      } else {
-        const uint2 q = *reinterpret_cast<const uint2*>(p);
-        bf[u][0][0] = q.x;
-        bf[u][0][1] = q.y;
+      for (int q = 0; q < F::RUNS; ++q) {
+        const int run = grp * F::RUNS + q;
+        if (run >= runs) break;
+        const int ex = xe[run];
+        const bool bad = !ok || ea == LZ_NONFINITE || ex == LZ_NONFINITE;  // also a wait that ran out
+        const double nan = __longlong_as_double(0x7ff8000000000000ll);
+        const int c = F::FORMS * q;
+        const double re = bad ? nan : ldexp(o[c], ea + ex - 70);
+        const double im = F::FORMS == 1 ? 0.0 : bad ? nan : ldexp(o[c + F::FORMS - 1], ea + ex - 70);
+        out[(int64_t)run * n] = s::make(re, im);
       }
     }
-    xb += F::STEP_HALVES;
+  } else if (warp < 12) {
+    // ------------------------------------------------------------ digits of A
+    asm volatile("setmaxnreg.inc.sync.aligned.u32 136;");
+    const int g = (warp >> 2) - 1;
+    const uint32_t dst = lane_addr + (uint32_t)(H_A0 + g * H_ASLOT);
+    constexpr int ESZ = (int)sizeof(T), UNIT = 16 / F::FORMS;  // columns per pass (56 registers of digits)
+    const uint32_t buf = smem_u32(abuf) + (uint32_t)((g * HSTEP * 128 + (warp & 3) * 32 + lane) * ESZ);
+    const int count = 2 * nblk;  // this group's steps: columns jbeg + 16 (2 it + g) ...
+    // rows of tiny entries (subnormal ones cannot be cut) are scaled by 2^600 first
+    const bool tiny = ea < -900, any_tiny = __any_sync(0xffffffffu, tiny);
+    const double up = tiny ? 4.149515568880993e180 : 1.0;
+    const int c0 = 1029 + (ea == LZ_NONFINITE ? 0 : tiny ? ea + 600 : ea);
+    const T* src = A + (row < n ? row : 0) + (jbeg + HSTEP * g) * lda;
+    auto copy = [&](uint32_t to, const T* p, int bytes) {
+      if (ESZ == 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(to), "l"(p), "r"(bytes) : "memory");
+      else
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(to), "l"(p), "r"(bytes) : "memory");
+    };
+    auto issue = [&](int it) {
+      const int64_t j = jbeg + (int64_t)HSTEP * (2 * it + g);
+      const uint32_t to = buf + (uint32_t)(it % H::SLOTS * (2 * HSTEP * 128 * ESZ));
+      if (j + HSTEP <= jend && row < n) {
+        const T* p = src;
 #pragma unroll
-    for (int f = 0; f < F::FORMS; ++f) {
-      uint32_t ad[4][NDIG];  // A registers 0..3 (row0 | row1, then columns + 8) by digit
-#pragma unroll
-      for (int r = 0; r < 4; ++r) {
-        const int rr = r & 1, c = (r >> 1) * 2, sc = rr ? s1 : s0;
-        const double x0 = f ? s::im(v[rr][c]) : s::re(v[rr][c]), x1 = f ? s::im(v[rr][c + 1]) : s::re(v[rr][c + 1]);
-        digit_pairs(to_fixed(x0, sc), to_fixed(x1, sc), ad[r]);
-      }
-#pragma unroll
-      for (int t = NDIG - 1; t >= 0; --t) {
-        const uint32_t a[4] = {ad[0][t], ad[1][t], ad[2][t], ad[3][t]};
-#pragma unroll
-        for (int u = NDIG - 1; u >= 0; --u) {
-          const int lev = 2 * (NDIG - 1) - t - u;
-          if (lev < NLEV) mma_16816(acc[lev], a, bf[u][f][0], bf[u][f][1]);
+        for (int q = 0; q < HSTEP; ++q, p += lda) copy(to + (uint32_t)(q * 128 * ESZ), p, ESZ);
+      } else if (it < count) {  // zeros outside the matrix
+#pragma unroll 1
+        for (int q = 0; q < HSTEP; ++q) {
+          const bool in = row < n && j + q < jend;
+          copy(to + (uint32_t)(q * 128 * ESZ), in ? src + q * lda : A, in ? ESZ : 0);
         }
       }
-    }
-    if (++fold == HEMV_FOLD || j + 16 >= jend) {
-      fold = 0;
+      src += 2 * HSTEP * lda;
+      asm volatile("cp.async.commit_group;" ::: "memory");
+    };
 #pragma unroll
-      for (int l = 0; l < NLEV; ++l)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          sum[l][q] += __float2int_rn(acc[l][q]);
-          acc[l][q] = 0.0f;
+    for (int it = 0; it < H::SLOTS - 1; ++it) issue(it);
+    for (int it = 0; it < count; ++it) {
+      issue(it + H::SLOTS - 1);
+      asm volatile("cp.async.wait_group %0;" ::"n"(H::SLOTS - 1) : "memory");
+      const uint32_t from = buf + (uint32_t)(it % H::SLOTS * (2 * HSTEP * 128 * ESZ));
+      if (any_tiny) {  // a loop of its own: inline, its FP64 multiplications are issued for every entry and bound the kernel
+#pragma unroll 1
+        for (int q = 0; q < HSTEP * F::FORMS; ++q) {
+          const uint32_t at = from + (uint32_t)((q / F::FORMS) * 128 * ESZ + (q % F::FORMS) * 8);
+          double v;
+          asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(at) : "memory");
+          asm volatile("st.shared.f64 [%0], %1;" ::"r"(at), "d"(v * up) : "memory");
         }
+      }
+      bool ok = true;
+#pragma unroll
+      for (int h = 0; h < F::FORMS; ++h) {
+        uint32_t dig[F::FORMS][NDIG][UNIT / 2];
+#pragma unroll
+        for (int c = 0; c < UNIT; c += 2) {
+          double x[2][2];
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            const uint32_t at = from + (uint32_t)((h * UNIT + c + k) * 128 * ESZ);
+            if (F::FORMS == 2)
+              asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(x[k][0]), "=d"(x[k][1]) : "r"(at) : "memory");
+            else
+              asm volatile("ld.shared.f64 %0, [%1];" : "=d"(x[k][0]) : "r"(at) : "memory");
+          }
+#pragma unroll
+          for (int f = 0; f < F::FORMS; ++f) {
+            uint32_t d[NDIG];
+            digit_pairs(x[0][f], x[1][f], c0, d);
+#pragma unroll
+            for (int t = 0; t < NDIG; ++t) dig[f][t][c / 2] = d[t];
+          }
+        }
+        if (h == 0) {
+          ok = __all_sync(0xffffffffu, hemv_wait(smem_u32(&aempty[g]), (it & 1) ^ 1, gave_up));
+          if (!ok) break;
+          oz::fence_after();
+        }
+#pragma unroll
+        for (int f = 0; f < F::FORMS; ++f)
+#pragma unroll
+          for (int t = 0; t < NDIG; ++t) tmem_st(dst + (uint32_t)((f * NDIG + t) * 8 + h * (UNIT / 2)), dig[f][t]);
+      }
+      if (!ok) break;
+      asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+      oz::fence_before();
+      __syncwarp();
+      if (lane == 0) oz::mbar_arrive(smem_u32(&afull[g]));
     }
-#pragma unroll
-    for (int r = 0; r < 2; ++r)
-#pragma unroll
-      for (int q = 0; q < 4; ++q) v[r][q] = w[r][q];
-  }
-  // levels 0-3 and 4-7 as two integers; value = (hi 2^32 + lo) 2^40, in units of 2^(ea + ex - 108)
-  double o[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const long long hi = ((long long)sum[0][q] << 24) + ((long long)sum[1][q] << 16) + ((long long)sum[2][q] << 8) + sum[3][q];
-    const long long lo = ((long long)sum[4][q] << 24) + ((long long)sum[5][q] << 16) + ((long long)sum[6][q] << 8) + sum[7][q];
-    o[q] = (double)hi * 4294967296.0 + (double)lo;
-  }
-#pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    // accumulator columns 2t, 2t + 1: complex, one run's re and im; real, two runs
-    const int run = F::FORMS == 2 ? grp * F::RUNS + t4 : grp * F::RUNS + 2 * t4 + (q & 1);
-    const int ea = q < 2 ? e0 : e1;
-    if (run >= runs) continue;
-    const int ex = xe[run];
-    o[q] = ea == LZ_NONFINITE || ex == LZ_NONFINITE ? __longlong_as_double(0x7ff8000000000000ll) : ldexp(o[q], ea + ex - 68);
-  }
-  T* out = part + (int64_t)blockIdx.y * runs * n;
-  if (F::FORMS == 2) {
-    const int run = grp * F::RUNS + t4;
-    if (run < runs) {
-      if (l0) out[(int64_t)run * n + row0] = s::make(o[0], o[1]);
-      if (l1) out[(int64_t)run * n + row1] = s::make(o[2], o[3]);
-    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
   } else {
+    asm volatile("setmaxnreg.dec.sync.aligned.u32 80;");
+    if (warp == 12 && lane == 0) {
+      // ------------------------------------------------------------ MMA issue
+      bool ok = true;
+      for (int kb = 0; kb < nblk && ok; ++kb) {
+        const int st = kb % H_XSTAGES;
+        ok = hemv_wait(smem_u32(&xfull[st]), (kb / H_XSTAGES) & 1, gave_up);
+        if (!ok) break;
+        const uint64_t xd = oz::sw128_desc(smem_u32(smem + st * H::X_BYTES));
+#pragma unroll 1
+        for (int k = 0; k < HK / HSTEP; ++k) {
+          // accumulator: two steps each
+          const int g = k & 1, b = k >> 1, it = 2 * kb + (k >> 1);
+          ok = (g != 0 || hemv_wait(smem_u32(&dempty[b]), (kb & 1) ^ 1, gave_up)) &&
+               hemv_wait(smem_u32(&afull[g]), it & 1, gave_up);
+          if (!ok) break;
+          oz::fence_after();
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int run = grp * F::RUNS + 2 * t4 + (q & 1);
-      const bool in = q < 2 ? l0 : l1;
-      if (run < runs && in) out[(int64_t)run * n + (q < 2 ? row0 : row1)] = s::make(o[q], 0.0);
+          for (int f = 0; f < F::FORMS; ++f)
+#pragma unroll
+            for (int t = NDIG - 1; t >= 0; --t) {
+              // digit t's window: levels 6 - t .. 7, in MMAs of a multiple of 16 columns
+              const int first = NDIG - 1 - t, groups = NLEV - first;
+              const int N = (groups * 8 + 15) / 16 * 16;
+              const uint32_t idesc = (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(HEMV_ROWS >> 4) << 24);
+              mma_tmem_a(tmem + (uint32_t)(b * H_ACC + first * 8), tmem + (uint32_t)(H_A0 + g * H_ASLOT + (f * NDIG + t) * 8),
+                         xd + (uint64_t)(f * (FORM_HALVES * 2 >> 4) + k * (HSTEP * 2 >> 4)), idesc,
+                         g == 0 && f == 0 && t == NDIG - 1 ? 0u : 1u);
+            }
+          oz::mma_commit(smem_u32(&aempty[g]));
+          if (g == 1) oz::mma_commit(smem_u32(&dfull[b]));
+        }
+        if (ok) oz::mma_commit(smem_u32(&xempty[st]));
+      }
+      // every MMA is done before TMEM is freed
+      oz::mma_commit(smem_u32(drain));
+      const unsigned long long t0 = oz::globaltimer();
+      while (!oz::mbar_try(smem_u32(drain), 0) && oz::globaltimer() - t0 < H_TIMEOUT_NS) {
+      }
+    } else if (warp == 13 && lane == 0) {
+      // ------------------------------------------------------------ copies of X
+      const int64_t nkb = (n + HK - 1) / HK;
+      const __half* src = X + ((int64_t)grp * nkb + jbeg / HK) * F::BLOCK_HALVES;
+      int issued = 0;
+      for (; issued < nblk; ++issued) {
+        const int st = issued % H_XSTAGES;
+        if (!hemv_wait(smem_u32(&xempty[st]), ((issued / H_XSTAGES) & 1) ^ 1, gave_up)) break;
+        oz::mbar_expect_tx(smem_u32(&xfull[st]), H::X_BYTES);
+        asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                         smem_u32(smem + st * H::X_BYTES)),
+                     "l"(src + (int64_t)issued * F::BLOCK_HALVES), "r"(H::X_BYTES), "r"(smem_u32(&xfull[st]))
+                     : "memory");
+      }
+      // the copies in flight land before the CTA exits
+      for (int i = issued > H_XSTAGES ? issued - H_XSTAGES : 0; i < issued; ++i) {
+        const unsigned long long t0 = oz::globaltimer();
+        while (!oz::mbar_try(smem_u32(&xfull[i % H_XSTAGES]), (i / H_XSTAGES) & 1) && oz::globaltimer() - t0 < H_TIMEOUT_NS) {
+        }
+      }
     }
   }
+  __syncwarp();
+  oz::fence_before();
+  __syncthreads();
+  oz::fence_after();
+  if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
 }
 
-// Columns per hemv block (a multiple of 64): enough blocks for a few waves on small problems, at most 512 columns
+// Columns per hemv block (a multiple of 64): row blocks times column chunks in full waves of one block per SM, a block
+// costing about two column blocks more than its columns (set-up, pipeline fill).  At most 64 column blocks (the
+// integer sums) and, unless those need more, at most 608 blocks in all (the partial sums' space).
 static int hemv_cols(int64_t n) {
-  const int64_t row_blocks = (n + HEMV_ROWS - 1) / HEMV_ROWS;
-  const int64_t want = std::max<int64_t>(1, 152 * 8 / row_blocks);
-  const int64_t c = ((n + want - 1) / want + 63) / 64 * 64;
-  return (int)std::min<int64_t>(512, std::max<int64_t>(64, c));
+  const int64_t rb = (n + HEMV_ROWS - 1) / HEMV_ROWS, kb = (n + HK - 1) / HK;
+  const int64_t least = (kb + 63) / 64, most = std::max(least, std::min(kb, 608 / rb));
+  int64_t best = least, cost = INT64_MAX;
+  for (int64_t nc = least; nc <= most; ++nc) {
+    const int64_t c = (rb * nc + 151) / 152 * ((kb + nc - 1) / nc + 2);
+    if (c < cost) {
+      cost = c;
+      best = nc;
+    }
+  }
+  return (int)((kb + best - 1) / best * HK);
 }
 
-// Bound of nchunk * n over all sizes up to n (the hemv partial sums of one run): the wanted blocks' rows, or n rows
-// per 512 columns.
-static int64_t hemv_part_rows(int64_t n) { return std::max<int64_t>(152 * 8 * HEMV_ROWS, n * (n / 512 + 1)); }
+// Bound of nchunk * n over all sizes up to n (the hemv partial sums of one run): 608 blocks' rows, or n rows per 4096
+// columns.
+static int64_t hemv_part_rows(int64_t n) { return std::max<int64_t>(608 * HEMV_ROWS, n * (n / 4096 + 1)); }
 
 int64_t lanczos_work_elems(int64_t n, int runs, int steps, bool cplx) {
   // basis | W | hemv partial sums | vector fragments | row maxima | exponents
@@ -323,6 +534,7 @@ __global__ void __launch_bounds__(STEP_THREADS) lanczos_step_kernel(int64_t n, i
                                                                      const T* __restrict__ part,
                                                                      const T* __restrict__ L0, T* Vb, T* Wb,
                                                                      double* alpha, double* beta, __half* X, int* xe) {
+  grid_dependency_wait();
   using s = S<T>;
   constexpr int NC = s::cplx ? 2 : 1;
   constexpr int NW = STEP_THREADS / 32;
@@ -456,7 +668,7 @@ __global__ void __launch_bounds__(STEP_THREADS) lanczos_step_kernel(int64_t n, i
   for (int64_t i = i0 + tid; i < i1; i += STEP_THREADS) {
     const T v = s::scale(w[i], inv);
     vn[i] = v;
-    write_frag<T>(X, (n + 15) / 16, i, run, to_fixed(s::re(v), es), NC == 2 ? to_fixed(s::im(v), es) : 0ll);
+    write_frag<T>(X, (n + HK - 1) / HK, i, run, to_fixed(s::re(v), es), NC == 2 ? to_fixed(s::im(v), es) : 0ll);
   }
 }
 
@@ -619,6 +831,15 @@ template <typename T> static int step_ctas(int64_t n) {
   return n >= 2048 && big ? STEP_MAXC : 8;
 }
 
+template <typename T> static void hemv_attributes() {
+  static std::once_flag once;
+  static cudaError_t err = cudaSuccess;
+  std::call_once(once, []() {
+    err = cudaFuncSetAttribute(hemv_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, Hemv<T>::SMEM);
+  });
+  CHASE_CUDA(err);
+}
+
 template <typename T>
 void lanczos(cudaStream_t st, const T* A, int64_t n, int64_t lda, int ne, const T* L0, int runs, int steps,
              double* out4, T* work, int64_t work_elems, double* dwork) {
@@ -649,25 +870,26 @@ void lanczos(cudaStream_t st, const T* A, int64_t n, int64_t lda, int ne, const 
   CHASE_CHECK_LAUNCH();
 
   cudaLaunchConfig_t cfg{};
-  cudaLaunchAttribute at{};
+  cudaLaunchAttribute at[2] = {{}, pdl_attribute()};
   const int ctas = step_ctas<T>(n);
-  at.id = cudaLaunchAttributeClusterDimension;
-  at.val.clusterDim.x = ctas;
-  at.val.clusterDim.y = at.val.clusterDim.z = 1;
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = ctas;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
   cfg.gridDim = dim3(ctas, runs, 1);
   cfg.blockDim = dim3(STEP_THREADS, 1, 1);
   cfg.stream = st;
-  cfg.attrs = &at;
-  cfg.numAttrs = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
   auto step = [&](int j) {
     CHASE_CUDA(cudaLaunchKernelEx(&cfg, lanczos_step_kernel<T>, n, runs, steps, j, nchunk, (const T*)part, L0, Vb, W,
                                   alpha, beta, X, xe));
     CHASE_CHECK_LAUNCH();
   };
+  hemv_attributes<T>();
   step(-1);
   const dim3 g1(ceil_div(n, HEMV_ROWS), nchunk, ceil_div(runs, Frag<T>::RUNS));
   for (int j = 0; j < steps; ++j) {
-    hemv_mma_kernel<T><<<g1, 2 * HEMV_ROWS, 0, st>>>(n, A, lda, rmax, X, xe, cols, runs, part);
+    launch_pdl(hemv_kernel<T>, g1, HEMV_THREADS, Hemv<T>::SMEM, st, n, A, lda, rmax, X, xe, cols, runs, part);
     CHASE_CHECK_LAUNCH();
     step(j);
   }

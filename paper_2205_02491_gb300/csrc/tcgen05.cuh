@@ -1,6 +1,6 @@
 // Inline-PTX wrappers for sm_103a: shared-memory addresses, mbarriers, tcgen05.mma (kind::f16, bf16
-// operands, FP32 accumulators in TMEM), commits and the thread-sync fences.  Shared by the split-product
-// kernel and the issue-rate probe.
+// operands, FP32 accumulators in TMEM), commits and the thread-sync fences.  Shared by the product kernels and the
+// issue-rate probe.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -46,6 +46,17 @@ __device__ __forceinline__ uint64_t sw64_desc(uint32_t saddr) {
   d |= (uint64_t)(512 >> 4) << 32;    // stride byte offset
   d |= (uint64_t)1 << 46;             // descriptor version
   d |= (uint64_t)4 << 61;             // 64-byte swizzle
+  return d;
+}
+
+// K-major operand tile, 128-byte swizzle: 8-row groups 1024 bytes apart
+__device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr >> 4) & 0x3FFF);
+  d |= (uint64_t)1 << 16;
+  d |= (uint64_t)(1024 >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)2 << 61;
   return d;
 }
 
