@@ -763,13 +763,27 @@ template <typename T> struct Solver {
     CHASE_REQUIRE(gA && ldga >= n && lda >= n && (gV == nullptr || ldg >= n), CHASE_ERR_ARG, "bad backward arguments");
     CHASE_REQUIRE(tol > 0.0 && maxit >= 1, CHASE_ERR_ARG, "bad MINRES tolerance or iteration cap");
     const size_t need = 9 * (size_t)n * nev * sizeof(T) + minres_state_bytes(nev) + 256;
-    if (c->bwd_bytes < need) {
+    // V_S as the left operand of MINRES's projections, V_S^T (l x n) and V_S (n x l), converted once: with the rest
+    // where memory allows (n = 4096, l = 68: 36 MB), else per product
+    const size_t lp = crt::plane_bytes(l, n, S<T>::cplx, crt::NMOD), rp = crt::plane_bytes(n, l, S<T>::cplx, crt::NMOD);
+    const size_t planes_at = (need + 255) / 256 * 256, with_planes = planes_at + lp + rp + (size_t)(l + n) * sizeof(int);
+    if (c->bwd_bytes < with_planes) {
       if (c->bwd) CHASE_CUDA(cudaFree(c->bwd));
       c->bwd = nullptr;
       c->bwd_bytes = 0;
-      CHASE_CUDA(cudaMalloc(&c->bwd, need));
-      c->bwd_bytes = need;
+      size_t got = with_planes;
+      if (cudaMalloc(&c->bwd, got) != cudaSuccess) {
+        cudaGetLastError();
+        c->bwd = nullptr;
+        got = need;
+        CHASE_CUDA(cudaMalloc(&c->bwd, got));
+      }
+      c->bwd_bytes = got;
     }
+    const bool held = oz::available() && c->bwd_bytes >= with_planes;
+    char* vs_cols = (char*)c->bwd + planes_at;
+    char* vs_rows = vs_cols + lp;
+    int* vs_ex = (int*)(vs_rows + rp);  // l exponents of V_S^T's rows, then n of V_S's
     T* base = (T*)c->bwd;
     const int64_t blk = n * nev;
     T *Tb = base, *Bb = base + blk, *Vv = base + 2 * blk, *Yb = base + 3 * blk, *R1 = base + 4 * blk,
@@ -803,6 +817,10 @@ template <typename T> struct Solver {
       minres_init(st(), n, nev, (const double*)Bb, n, (double*)R1, (double*)R2, (double*)Vv, (double*)X,
                   (double*)Wa, (double*)Wb, state, tol);
       T* Mp = Gb();
+      if (held) {
+        oz::left_planes<T>(st(), OP_C, Vs, n, l, n, vs_cols, vs_ex);
+        oz::left_planes<T>(st(), OP_N, Vs, n, n, l, vs_rows, vs_ex + l);
+      }
       T *r1 = R1, *r2 = R2, *wc = Wa, *wn = Wb;  // wc: w_{t-1}, wn: w_{t-2}
       int it = 0;
       for (; it < maxit; ++it) {
@@ -817,7 +835,8 @@ template <typename T> struct Solver {
         Epi ep;
         ep.C = Mp;
         ep.ldc = l;
-        gemm(OP_C, Vs, n, OP_N, Yb, n, l, nev, n, ep, CHASE_FP64, true);
+        if (held) oz::gemm_planes<T>(st(), c->ozw, vs_cols, vs_ex, Yb, n, l, nev, n, ep);
+        else gemm(OP_C, Vs, n, OP_N, Yb, n, l, nev, n, ep, CHASE_FP64, true);
         Epi eu;
         eu.C = Yb;
         eu.ldc = n;
@@ -825,7 +844,9 @@ template <typename T> struct Solver {
         eu.Z = Yb;
         eu.ldz = n;
         eu.beta = 1.0;
-        gemm(OP_N, Vs, n, OP_N, Mp, l, n, nev, l, eu, CHASE_FP64, true);  // Y -= V_S (V_S^T Y)
+        // Y -= V_S (V_S^T Y)
+        if (held) oz::gemm_planes<T>(st(), c->ozw, vs_rows, vs_ex + l, Mp, l, n, nev, l, eu);
+        else gemm(OP_N, Vs, n, OP_N, Mp, l, n, nev, l, eu, CHASE_FP64, true);
         minres_update(st(), n, nev, (const double*)Yb, (double*)r1, (const double*)r2, (double*)Vv, (double*)wn,
                       (const double*)wc, (double*)X, state, tol);
         std::swap(r1, r2);

@@ -110,6 +110,14 @@ template <typename T>
 void gemm(cudaStream_t st, Workspace& w, Op opA, const T* A, int64_t lda, Op opB, const T* B, int64_t ldb, int64_t M,
           int64_t N, int64_t K, const Epi& e);
 
+// The same with a left operand that is converted once for several products: its planes (crt::plane_bytes(M, K, ...)
+// bytes, 16-byte aligned) and M exponents.
+template <typename T>
+void left_planes(cudaStream_t st, Op opA, const T* A, int64_t lda, int64_t M, int64_t K, void* planes, int* ex);
+template <typename T>
+void gemm_planes(cudaStream_t st, Workspace& w, const void* planes, const int* ex, const T* B, int64_t ldb, int64_t M,
+                 int64_t N, int64_t K, const Epi& e);
+
 // Grouped launches over several problems' workspaces.  Mixed modes: digit planes of the right operand B
 // (n x k, ld ldb) into w's right-operand buffer, then one launch (per 64 products) over the tiles of all products.
 template <typename T>

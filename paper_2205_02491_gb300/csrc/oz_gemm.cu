@@ -481,6 +481,21 @@ void hemm(cudaStream_t st, Workspace& w, const T* A, int64_t n, int64_t lda, con
   else launch<2, CPLX, 128>(st, w, n, k, n, e, cfg.group_m, ev);
 }
 
+// left operand: OP_N rows of A (M x K), OP_C conjugated columns of A (K x M)
+template <typename T>
+void left_planes(cudaStream_t st, Op opA, const T* A, int64_t lda, int64_t M, int64_t K, void* planes, int* ex) {
+  crt::scales<T>(st, opA == OP_N, M, K, A, lda, ex);
+  crt::residues<T>(st, opA == OP_N, opA == OP_C, M, K, A, lda, ex, 0, crt::NMOD, planes);
+}
+
+template <typename T>
+void gemm_planes(cudaStream_t st, Workspace& w, const void* planes, const int* ex, const T* B, int64_t ldb, int64_t M,
+                 int64_t N, int64_t K, const Epi& e) {
+  CHASE_REQUIRE(w.ready, 9, "split products not initialised");
+  if (M <= 0 || N <= 0) return;
+  product<T>(st, w, planes, ex, crt::NMOD, [](int, int) {}, false, B, ldb, M, N, K, e);
+}
+
 template <typename T>
 void gemm(cudaStream_t st, Workspace& w, Op opA, const T* A, int64_t lda, Op opB, const T* B, int64_t ldb, int64_t M,
           int64_t N, int64_t K, const Epi& e) {
@@ -490,10 +505,9 @@ void gemm(cudaStream_t st, Workspace& w, Op opA, const T* A, int64_t lda, Op opB
   CHASE_REQUIRE(N <= w.n_max && M <= w.n_max &&
                     crt::plane_bytes(M, K, CPLX, crt::NMOD) <= left_bytes(w.n_max, w.ne_max, CPLX),
                 1, "split product exceeds the workspace");
-  // left operand: OP_N rows of A (M x K), OP_C conjugated columns of A (K x M); right operand: OP_N columns of B
-  // (K x N), OP_C conjugated rows of B (N x K).  The left planes of all moduli are made first, so C may overwrite A.
-  crt::scales<T>(st, opA == OP_N, M, K, A, lda, w.l_ex);
-  crt::residues<T>(st, opA == OP_N, opA == OP_C, M, K, A, lda, w.l_ex, 0, crt::NMOD, w.l_res);
+  // right operand: OP_N columns of B (K x N), OP_C conjugated rows of B (N x K).  The left planes of all moduli are
+  // made first, so C may overwrite A.
+  left_planes<T>(st, opA, A, lda, M, K, w.l_res, w.l_ex);
   product<T>(st, w, w.l_res, w.l_ex, crt::NMOD, [](int, int) {}, opB == OP_C, B, ldb, M, N, K, e);
 }
 
@@ -513,6 +527,12 @@ template void gemm<double>(cudaStream_t, Workspace&, Op, const double*, int64_t,
                            int64_t, int64_t, const Epi&);
 template void gemm<double2>(cudaStream_t, Workspace&, Op, const double2*, int64_t, Op, const double2*, int64_t, int64_t,
                             int64_t, int64_t, const Epi&);
+template void left_planes<double>(cudaStream_t, Op, const double*, int64_t, int64_t, int64_t, void*, int*);
+template void left_planes<double2>(cudaStream_t, Op, const double2*, int64_t, int64_t, int64_t, void*, int*);
+template void gemm_planes<double>(cudaStream_t, Workspace&, const void*, const int*, const double*, int64_t, int64_t,
+                                  int64_t, int64_t, const Epi&);
+template void gemm_planes<double2>(cudaStream_t, Workspace&, const void*, const int*, const double2*, int64_t, int64_t,
+                                   int64_t, int64_t, const Epi&);
 template crt::Product group_product<double>(Workspace&, const double*, int64_t, int, int64_t, const Epi&);
 template crt::Product group_product<double2>(Workspace&, const double2*, int64_t, int, int64_t, const Epi&);
 template void multiply_group<double>(cudaStream_t, Workspace&, const crt::Product*, int);
