@@ -16,74 +16,134 @@
 namespace chase {
 namespace oz {
 // ---------------------------------------------------------------- split kernels
-// Per-column power-of-two scale s = 2^e with max|re|,|im| = f 2^e, f in [0.5, 1).
-template <typename T>
-__global__ void col_scale_kernel(int64_t K, const T* __restrict__ X, int64_t ldx, double* scale) {
-  grid_dependency_wait();
-  const T* x = X + (int64_t)blockIdx.x * ldx;
-  double m = 0.0;
-  for (int64_t i = threadIdx.x; i < K; i += blockDim.x) {
-    T v = x[i];
-    m = fmax(m, fmax(fabs(S<T>::re(v)), fabs(S<T>::im(v))));
-  }
-  __shared__ double red[32];
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double v = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) v = fmax(v, red[w]);
-    int e = 0;
-    if (v > 0.0 && isfinite(v)) frexp(v, &e);
-    scale[blockIdx.x] = v > 0.0 ? ldexp(1.0, e) : 1.0;
-  }
-}
-
-// Digits of one value: d_t = rint(r_t), r_0 = x/s * 2^7, r_{t+1} = (r_t - d_t) 2^8; plane stores d_t 2^-8t.
-template <int NS> __device__ __forceinline__ void digits(double xs, __nv_bfloat16 (&out)[NS]) {
-  double r = xs * 128.0;
-  float sc = 1.0f;
-#pragma unroll
-  for (int t = 0; t < NS; ++t) {
-    double d = rint(r);
-    out[t] = __float2bfloat16_rn((float)d * sc);
-    r = (r - d) * 256.0;
-    sc *= 0.00390625f;
-  }
-}
-
-// Left-operand planes (K-major rows = conjugated columns of X when conj, else columns):
-// plane (t, p), p in {re, im}.  Right-operand planes: p in {-im, re, im}.
-// Real: one plane per slice.  Layout planes[(t*P + p) * ncols + col][Kpad].
-template <typename T, int NS, int KIND>
-__global__ void split_cols_kernel(int64_t K, int64_t Kpad, int ncols, const T* __restrict__ X, int64_t ldx,
-                                  const double* __restrict__ scale, int conj, __nv_bfloat16* planes) {
-  grid_dependency_wait();
-  constexpr bool CPLX = S<T>::cplx;
-  const int col = blockIdx.y;
-  const T* x = X + (int64_t)col * ldx;
-  const double inv = 1.0 / scale[col];
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < K; i += (int64_t)gridDim.x * blockDim.x) {
-    T v = x[i];
-    double re = S<T>::re(v) * inv;
-    double im = (conj ? -S<T>::im(v) : S<T>::im(v)) * inv;
-    __nv_bfloat16 dr[NS], di[NS];
-    digits<NS>(re, dr);
-    if (CPLX) digits<NS>(im, di);
+// Digits of one value x with |x| < s = 2^e: d_t = rint(r_t), r_0 = x/s * 2^7, r_{t+1} = (r_t - d_t) 2^8; a plane stores
+// d_t 2^-8t.  Rounding to nearest even is symmetric and looks no further than 2^-16 of r_0, so the digits come exactly
+// from |r_0| in 32-bit fixed point (23 fraction bits, the last one also set by anything below it): FP64 instructions
+// (nine per digit) bound this kernel otherwise (n = 5003 real: A 786 us).
+template <int NS> __device__ __forceinline__ void digits(double x, int e, float (&out)[NS]) {
+  const uint32_t hi = (uint32_t)__double2hiint(x);
+  const int be = (int)((hi >> 20) & 0x7ff);
+  if (be == 2047 || e < -1000 || e > 1000) {  // non-finite, or a scale near the ends of the range
+    double r = x * (1.0 / ldexp(1.0, e)) * 128.0;
 #pragma unroll
     for (int t = 0; t < NS; ++t) {
-      if (!CPLX) {
-        planes[((int64_t)t * ncols + col) * Kpad + i] = dr[t];
+      const double d = rint(r);
+      out[t] = (float)d;
+      r = (r - d) * 256.0;
+    }
+    return;
+  }
+  const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | (be ? 0x100000u : 0u)) << 32) | (uint32_t)__double2loint(x);
+  const int n = min(1045 + e - (be ? be : 1), 63);  // x = m 2^(be - 1075); at least 23
+  const uint32_t q = (uint32_t)(m >> n);
+  int v = (int)(q | (((unsigned long long)q << n) != m ? 1u : 0u));
+#pragma unroll
+  for (int t = 0; t < NS; ++t) {
+    const int sh = 23 - 8 * t;
+    const int d = (v + ((1 << (sh - 1)) - 1) + ((v >> sh) & 1)) >> sh;
+    v -= d << sh;
+    const int sd = (int)hi < 0 ? -d : d;
+    out[t] = __int_as_float(0x4b400000 + sd) - 12582912.0f;
+  }
+}
+__device__ __forceinline__ uint32_t pack_planes(float a, float b, float sc) {  // exact: at most 8 significant bits
+  return __byte_perm(__float_as_uint(a * sc), __float_as_uint(b * sc), 0x7632);
+}
+
+// Scales and digit planes of the columns of X (conjugated when conj), a cluster of CTAs per column (512 elements each while
+// K <= 4096): the column's largest magnitude f 2^e, f in [0.5, 1), gives its scale 2^e (1 for a zero column or a
+// non-finite one).  Left-operand planes (KIND 0): (t, p), p in {re, im}; right-operand planes: p in {-im, re, im}; real:
+// one plane per slice.  Layout planes[(t*P + p) * ncols + col][Kpad].
+// n = 5003 real: A 100 us (scales and digits by separate FP64 kernels: 860), 300 right columns 7 us (39).
+template <typename T, int NS, int KIND>
+__global__ void __launch_bounds__(128) split_kernel(int64_t K, int64_t Kpad, int ncols, const T* __restrict__ X, int64_t ldx,
+                                                    double* scale, int conj, __nv_bfloat16* planes) {
+  using s = S<T>;
+  __shared__ uint32_t part[32];
+  __shared__ double slow[4];
+  const int rank = (int)blockIdx.x, cs = (int)gridDim.x, col = blockIdx.y, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
+  grid_dependency_wait();
+  const int64_t slice = ((K + cs - 1) / cs + 3) / 4 * 4;
+  const int64_t k0 = rank * slice, k1 = k0 + slice < K ? k0 + slice : K;
+  const T* x = X + (int64_t)col * ldx;
+  auto load4 = [&](T (&v)[4], int64_t i) {
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = i + j < k1 ? x[i + j] : s::zero();
+  };
+  auto top = [&](const T& v) {
+    return max((uint32_t)__double2hiint(s::re(v)) & 0x7fffffffu, (uint32_t)__double2hiint(s::im(v)) & 0x7fffffffu);
+  };
+  T v[4];
+  const int64_t i0 = k0 + 4 * tid;
+  load4(v, i0);  // stays in registers when the slice is 512 elements
+  uint32_t m = max(max(top(v[0]), top(v[1])), max(top(v[2]), top(v[3])));
+  for (int64_t i = i0 + 512; i < k1; i += 512) {
+    T u[4];
+    load4(u, i);
+    m = max(m, max(max(top(u[0]), top(u[1])), max(top(u[2]), top(u[3]))));
+  }
+  m = __reduce_max_sync(0xffffffffu, m);
+  asm volatile("barrier.cluster.wait.aligned;" ::: "memory");  // every CTA of the cluster runs
+  if (lane < cs) {
+    uint32_t to;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+                 : "=r"(to)
+                 : "r"((uint32_t)__cvta_generic_to_shared(&part[4 * rank + warp])), "r"(lane));
+    asm volatile("st.shared::cluster.b32 [%0], %1;" ::"r"(to), "r"(m) : "memory");
+  }
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  m = __reduce_max_sync(0xffffffffu, lane < 4 * cs ? part[lane] : 0u);
+  int e = 0;
+  double sc = 1.0;
+  if (m < 0x00100000u) {  // a zero column, or subnormal throughout
+    double w = 0.0;
+    for (int64_t i = tid; i < K; i += 128) w = fmax(w, fmax(fabs(s::re(x[i])), fabs(s::im(x[i]))));
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) w = fmax(w, __shfl_xor_sync(0xffffffffu, w, o));
+    if (lane == 0) slow[warp] = w;
+    __syncthreads();
+    w = fmax(fmax(slow[0], slow[1]), fmax(slow[2], slow[3]));
+    if (w > 0.0) {
+      frexp(w, &e);
+      sc = ldexp(1.0, e);
+    }
+  } else if (m < 0x7ff00000u) {
+    e = (int)(m >> 20) - 1022;
+    sc = ldexp(1.0, e);
+  }
+  if (rank == 0 && tid == 0) scale[col] = sc;
+  auto write4 = [&](const T (&u)[4], int64_t i) {
+    float dr[4][NS], di[4][NS];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      digits<NS>(s::re(u[j]), e, dr[j]);
+      if (s::cplx) digits<NS>(conj ? -s::im(u[j]) : s::im(u[j]), e, di[j]);
+    }
+    float f = 1.0f;
+#pragma unroll
+    for (int t = 0; t < NS; ++t, f *= 0.00390625f) {
+      constexpr int P = s::cplx ? (KIND == 0 ? 2 : 3) : 1;
+      auto put = [&](int p, const float (&d)[4][NS], float g) {
+        *reinterpret_cast<uint2*>(planes + ((int64_t)(t * P + p) * ncols + col) * Kpad + i) =
+            make_uint2(pack_planes(d[0][t], d[1][t], g), pack_planes(d[2][t], d[3][t], g));
+      };
+      if (!s::cplx) {
+        put(0, dr, f);
       } else if (KIND == 0) {
-        planes[((int64_t)(t * 2 + 0) * ncols + col) * Kpad + i] = dr[t];
-        planes[((int64_t)(t * 2 + 1) * ncols + col) * Kpad + i] = di[t];
+        put(0, dr, f);
+        put(1, di, f);
       } else {
-        planes[((int64_t)(t * 3 + 0) * ncols + col) * Kpad + i] = __hneg(di[t]);
-        planes[((int64_t)(t * 3 + 1) * ncols + col) * Kpad + i] = dr[t];
-        planes[((int64_t)(t * 3 + 2) * ncols + col) * Kpad + i] = di[t];
+        put(0, di, -f);
+        put(1, dr, f);
+        put(2, di, f);
       }
     }
+  };
+  if (i0 < k1) write4(v, i0);
+  for (int64_t i = i0 + 512; i < k1; i += 512) {
+    load4(v, i);
+    write4(v, i);
   }
 }
 
@@ -189,16 +249,28 @@ void destroy(Workspace& w) {
 template <typename T>
 static void split(cudaStream_t st, int S_, int kind, bool conj, const T* X, int64_t ld, int64_t nvec, int64_t K,
                   void* planes, double* scale) {
+  // a cluster only as far as it fills the SMs (16 blocks each)
+  int cs = 1;
+  while (cs < 8 && 512 * cs < K && nvec * cs < 152 * 16) cs *= 2;
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute at[2] = {{}, pdl_attribute()};
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = cs;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.blockDim = dim3(128, 1, 1);
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
   const int64_t kp = kpad(K);
-  launch_pdl(col_scale_kernel<T>, (unsigned)nvec, 256, 0, st, K, X, ld, scale);
-  CHASE_CHECK_LAUNCH();
-  dim3 grid(std::min<unsigned>(ceil_div(K, 256), 32), (unsigned)nvec);
-#define SC(SS, KD) launch_pdl(split_cols_kernel<T, SS, KD>, grid, 256, 0, st, K, kp, (int)nvec, X, ld, scale, conj ? 1 : 0, (__nv_bfloat16*)planes)
-  if (S_ == 2 && kind == 1) SC(2, 1);
-  else if (S_ == 3 && kind == 1) SC(3, 1);
-  else if (S_ == 3 && kind == 0) SC(3, 0);
+  CHASE_REQUIRE(nvec <= 65535, 1, "split: too many vectors");
+  cfg.gridDim = dim3(cs, (unsigned)nvec, 1);
+  auto go = [&](auto kernel) {
+    CHASE_CUDA(cudaLaunchKernelEx(&cfg, kernel, K, kp, (int)nvec, X, ld, scale, conj ? 1 : 0, (__nv_bfloat16*)planes));
+  };
+  if (S_ == 2 && kind == 1) go(split_kernel<T, 2, 1>);
+  else if (S_ == 3 && kind == 1) go(split_kernel<T, 3, 1>);
+  else if (S_ == 3 && kind == 0) go(split_kernel<T, 3, 0>);
   else CHASE_REQUIRE(false, 1, "unsupported slice count");
-#undef SC
   CHASE_CHECK_LAUNCH();
 }
 
