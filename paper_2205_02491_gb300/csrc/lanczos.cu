@@ -3,7 +3,7 @@
 // All runs advance together, two launches per step: the product of A with one vector per run (hemv_kernel, A
 // streamed once per step), and the rest of the step (lanczos_step_kernel, one cluster of CTAs per run): three-term
 // update, one classical Gram-Schmidt reorthogonalisation against the run's basis, normalisation.  The tridiagonal T
-// of each run is diagonalised by implicit QL, and one block computes b_sup = max(theta_max + |beta_last|),
+// of each run is diagonalised by one block per run, and one block computes b_sup = max(theta_max + |beta_last|),
 // mu_1 = min theta_min, theta_max and the density-of-states quantile mu_ne = smallest pooled Ritz value whose
 // cumulative weight (1/runs) sum tau_j^2 reaches ne/n, clamped into (mu_1, b_sup) by 1e-3 of the spectral span.
 #include <cuda_fp16.h>
@@ -673,32 +673,11 @@ __global__ void __launch_bounds__(STEP_THREADS) lanczos_step_kernel(int64_t n, i
 }
 
 // ---------------------------------------------------------------- Ritz values
-// Implicit QL with Wilkinson shifts on the run's tridiagonal T (steps <= 64), one warp per run: eigenvalues, and the
-// first row of the eigenvectors' matrix, which is all the density of states needs (Golub and Welsch 1969).  About
-// 1.7 QL sweeps per eigenvalue of at most `steps` rotations, a serial chain in lane 0; the search for a negligible
-// off-diagonal before each sweep is one step of the whole warp.  Output theta ascending and tau2 = squared first
-// components.  (A two-sided Jacobi over the block took 5.6 ms for 25 steps.)
-__global__ void tridiag_ql_kernel(int steps, const double* alpha, const double* beta, double* theta, double* tau2,
-                                  int* status) {
-  const int r = blockIdx.x, k = steps, lane = threadIdx.x;
-  __shared__ double d[LZ_MAXS], e[LZ_MAXS], z[LZ_MAXS];
-  // scaled by a power of two to norm about 1, so that squares neither overflow nor vanish
-  double m = 0.0;
-  for (int i = lane; i < k; i += 32) {
-    d[i] = alpha[r * LZ_MAXS + i];
-    e[i] = i + 1 < k ? beta[r * LZ_MAXS + i] : 0.0;
-    z[i] = i == 0 ? 1.0 : 0.0;
-    m = fmax(m, fmax(fabs(d[i]), fabs(e[i])));
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
-  int sc = 0;
-  if (m > 0.0 && isfinite(m)) frexp(m, &sc);
-  for (int i = lane; i < k; i += 32) {
-    d[i] = ldexp(d[i], -sc);
-    e[i] = ldexp(e[i], -sc);
-  }
-  __syncwarp();
+// Implicit QL with Wilkinson shifts on a tridiagonal T (diagonal d, off-diagonal e, k <= 64) by one warp: eigenvalues, and
+// z, the first row of the eigenvectors' matrix (Golub and Welsch 1969).  About 1.7 sweeps per eigenvalue of at most k
+// rotations, a serial chain of FP64 operations in lane 0 (0.9 ms for k = 25).
+__device__ __noinline__ void ql_first_row(int k, double* d, double* e, double* z, int* status) {
+  const int lane = threadIdx.x & 31;
   const double eps = 1.1102230246251565e-16;
   for (int l = 0; l < k; ++l) {
     for (int iter = 0;; ++iter) {
@@ -754,8 +733,191 @@ __global__ void tridiag_ql_kernel(int steps, const double* alpha, const double* 
     }
     __syncwarp();
   }
+}
+
+// The same in FP32 with all eigenvectors (columns of Z, ld ldz), the lanes sharing Z's rows.  False: no convergence.
+__device__ __forceinline__ bool ql_fp32(int k, float* d, float* e, float* Z, int ldz) {
+  const int lane = threadIdx.x & 31;
+  const float eps = 5.9604645e-8f;
+  for (int l = 0; l < k; ++l) {
+    for (int iter = 0;; ++iter) {
+      auto small = [&](int i) {
+        return i >= k - 1 || (i >= l && fabsf(e[i]) <= eps * (fabsf(d[i]) + fabsf(d[i + 1]) + 1e-3f));
+      };
+      const unsigned lo = __ballot_sync(0xffffffffu, small(lane));
+      const unsigned hi = __ballot_sync(0xffffffffu, small(lane + 32));
+      const int mm = min(k - 1, lo ? __ffs((int)lo) - 1 : 31 + __ffs((int)hi));
+      if (mm == l) break;
+      if (iter == 60) return false;
+      // every lane makes the same scalars
+      float g = (d[l + 1] - d[l]) / (2.0f * e[l]);
+      const float h = sqrtf(g * g + 1.0f);
+      g = d[mm] - d[l] + e[l] / (g + (g >= 0.0f ? h : -h));
+      float sn = 1.0f, cs = 1.0f, p = 0.0f, di1 = d[mm];
+      float z0 = lane < k ? Z[lane + mm * ldz] : 0.0f, z1 = lane + 32 < k ? Z[lane + 32 + mm * ldz] : 0.0f;
+      int i = mm - 1;
+      for (; i >= l; --i) {
+        const float f = sn * e[i], b = cs * e[i], di = d[i];
+        const float q = fmaf(f, f, g * g);
+        if (!(q > 1e-36f)) return false;  // the rotation is undefined: left to the FP64 version
+        const float ri = rsqrtf(q);
+        const float c0 = lane < k ? Z[lane + i * ldz] : 0.0f, c1 = lane + 32 < k ? Z[lane + 32 + i * ldz] : 0.0f;
+        sn = f * ri;
+        cs = g * ri;
+        g = di1 - p;
+        const float t = fmaf(di - g, sn, 2.0f * cs * b);
+        p = sn * t;
+        if (lane == 0) {
+          e[i + 1] = q * ri;
+          d[i + 1] = g + p;
+        }
+        g = fmaf(cs, t, -b);
+        if (lane < k) Z[lane + (i + 1) * ldz] = fmaf(sn, c0, cs * z0);
+        if (lane + 32 < k) Z[lane + 32 + (i + 1) * ldz] = fmaf(sn, c1, cs * z1);
+        z0 = fmaf(cs, c0, -sn * z0);
+        z1 = fmaf(cs, c1, -sn * z1);
+        di1 = di;
+      }
+      if (lane < k) Z[lane + l * ldz] = z0;
+      if (lane + 32 < k) Z[lane + 32 + l * ldz] = z1;
+      __syncwarp();
+      if (lane == 0) {
+        d[l] -= p;
+        e[l] = g;
+        e[mm] = 0.0f;
+      }
+      __syncwarp();
+    }
+  }
+  return true;
+}
+
+// Eigenvalues theta (ascending) and squared first eigenvector components tau2 of every run's tridiagonal T, one block
+// per run.  An FP64 rotation chain is bound by the latency of its operations (over 100 cycles each), so QL runs in
+// FP32 and its eigenvectors X are corrected in FP64 by products that all threads share (Ogita and Aishima 2018):
+// R = I - X^T X, S = X^T T X, E_ij = (S_ij + l_j R_ij) / (l_j - l_i), X <- X + X E, quadratically convergent.  The step
+// after max |E| <= 1e-8 ends it; a pair of eigenvalues too close for E, or no convergence, leaves T to QL in FP64.
+// k = 25: 125 us, 890 by QL in FP64.  (A two-sided Jacobi over the block took 5.6 ms.)
+constexpr int TRI_THREADS = 256;
+__global__ void __launch_bounds__(TRI_THREADS) tridiag_kernel(int steps, const double* alpha, const double* beta, double* theta,
+                                                              double* tau2, int* status) {
+  const int r = blockIdx.x, k = steps, tid = threadIdx.x, ld = k + 1;
+  extern __shared__ double tri_smem[];
+  double *X = tri_smem, *Y = X + k * ld, *Sm = Y + k * ld, *Rm = Sm + k * ld;  // column-major, ld k + 1
+  __shared__ double d[LZ_MAXS], e[LZ_MAXS], z[LZ_MAXS], lam[LZ_MAXS], red[3][TRI_THREADS / 32];
+  __shared__ float df[LZ_MAXS], ef[LZ_MAXS];
+  __shared__ int sc_sh, ok_sh;
+  // scaled by a power of two to norm about 1, so that squares neither overflow nor vanish
+  if (tid < 32) {
+    double m = 0.0;
+    for (int i = tid; i < k; i += 32) {
+      d[i] = alpha[r * LZ_MAXS + i];
+      e[i] = i + 1 < k ? beta[r * LZ_MAXS + i] : 0.0;
+      z[i] = i == 0 ? 1.0 : 0.0;
+      m = fmax(m, fmax(fabs(d[i]), fabs(e[i])));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
+    int sc = 0;
+    if (m > 0.0 && isfinite(m)) frexp(m, &sc);
+    for (int i = tid; i < k; i += 32) {
+      d[i] = ldexp(d[i], -sc);
+      e[i] = ldexp(e[i], -sc);
+      df[i] = (float)d[i];
+      ef[i] = (float)e[i];
+    }
+    if (tid == 0) sc_sh = sc;
+  }
+  float* Z = reinterpret_cast<float*>(Y);
+  for (int q = tid; q < k * ld; q += TRI_THREADS) Z[q] = q % ld == q / ld ? 1.0f : 0.0f;
+  __syncthreads();
+  if (tid < 32) {
+    const bool ok = ql_fp32(k, df, ef, Z, ld);
+    if (tid == 0) ok_sh = ok;
+  }
+  __syncthreads();
+  for (int q = tid; q < k * ld; q += TRI_THREADS) X[q] = Z[q];
+  __syncthreads();
+  bool ok = ok_sh != 0, last = false;
+  auto block_max = [&](double v, int set) {  // NaN counts as infinity
+    v = v == v ? v : INFINITY;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+    if ((tid & 31) == 0) red[set][tid >> 5] = v;
+    __syncthreads();
+    v = red[set][0];
+    for (int w = 1; w < TRI_THREADS / 32; ++w) v = fmax(v, red[set][w]);
+    return v;
+  };
+  for (int it = 0; ok && !last; ++it) {
+    for (int q = tid; q < k * k; q += TRI_THREADS) {
+      const int j = q / k, i = q - j * k;
+      const double* x = X + j * ld;
+      double v = d[i] * x[i];
+      if (i > 0) v += e[i - 1] * x[i - 1];
+      if (i + 1 < k) v += e[i] * x[i + 1];
+      Y[j * ld + i] = v;
+    }
+    __syncthreads();
+    double off = 0.0, orth = 0.0;
+    for (int q = tid; q < k * k; q += TRI_THREADS) {
+      const int j = q / k, i = q - j * k;
+      if (i > j) continue;  // both are symmetric
+      double sa = 0.0, ra = i == j ? 1.0 : 0.0;
+      for (int p = 0; p < k; ++p) {
+        sa += X[i * ld + p] * Y[j * ld + p];
+        ra -= X[i * ld + p] * X[j * ld + p];
+      }
+      Sm[j * ld + i] = Sm[i * ld + j] = sa;
+      Rm[j * ld + i] = Rm[i * ld + j] = ra;
+      if (i == j) lam[i] = sa / (1.0 - ra);
+      else off = fmax(off, fabs(sa));
+      orth = fmax(orth, fabs(ra));
+    }
+    off = block_max(off, 0);
+    orth = block_max(orth, 1);
+    // eigenvalues closer than this cannot be told apart yet
+    const double close = 8.0 * (off + orth);
+    double big = 0.0, open = 0.0;
+    for (int q = tid; q < k * k; q += TRI_THREADS) {
+      const int j = q / k, i = q - j * k;
+      const double gap = lam[j] - lam[i], rij = Rm[j * ld + i];
+      double ev = 0.5 * rij;
+      if (i != j) {
+        const double c = Sm[j * ld + i] + lam[j] * rij;
+        if (fabs(gap) > close) ev = c / gap;
+        else if (fabs(c) > 1e-17) open = 1.0;  // not an exactly decoupled pair
+      }
+      big = fmax(big, fabs(ev));
+      Y[j * ld + i] = ev;
+    }
+    big = block_max(big, 2);
+    last = __syncthreads_or(open != 0.0) == 0 && big <= 1e-8;
+    ok = big < 0.1 && (last || it < 5);
+    if (!ok) break;
+    for (int q = tid; q < k * k; q += TRI_THREADS) {
+      const int j = q / k, i = q - j * k;
+      double v = X[j * ld + i];
+      for (int p = 0; p < k; ++p) v += X[p * ld + i] * Y[j * ld + p];
+      Sm[j * ld + i] = v;
+    }
+    __syncthreads();
+    double* t = X;
+    X = Sm;
+    Sm = t;
+  }
+  if (ok) {
+    for (int i = tid; i < k; i += TRI_THREADS) {
+      d[i] = lam[i];
+      z[i] = X[i * ld];
+    }
+  } else if (tid < 32) {
+    ql_first_row(k, d, e, z, status);
+  }
+  __syncthreads();
+  const int sc = sc_sh;
   // ascending (stable) order
-  for (int i = lane; i < k; i += 32) {
+  for (int i = tid; i < k; i += TRI_THREADS) {
     const double wi = d[i];
     int rank = 0;
     for (int q = 0; q < k; ++q) rank += (d[q] < wi) || (d[q] == wi && q < i);
@@ -831,11 +993,14 @@ template <typename T> static int step_ctas(int64_t n) {
   return n >= 2048 && big ? STEP_MAXC : 8;
 }
 
-template <typename T> static void hemv_attributes() {
+template <typename T> static void lanczos_attributes() {
   static std::once_flag once;
   static cudaError_t err = cudaSuccess;
   std::call_once(once, []() {
     err = cudaFuncSetAttribute(hemv_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, Hemv<T>::SMEM);
+    if (err == cudaSuccess)
+      err = cudaFuncSetAttribute(tridiag_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 4 * LZ_MAXS * (LZ_MAXS + 1) * (int)sizeof(double));
   });
   CHASE_CUDA(err);
 }
@@ -885,7 +1050,7 @@ void lanczos(cudaStream_t st, const T* A, int64_t n, int64_t lda, int ne, const 
                                   alpha, beta, X, xe));
     CHASE_CHECK_LAUNCH();
   };
-  hemv_attributes<T>();
+  lanczos_attributes<T>();
   step(-1);
   const dim3 g1(ceil_div(n, HEMV_ROWS), nchunk, ceil_div(runs, Frag<T>::RUNS));
   for (int j = 0; j < steps; ++j) {
@@ -893,7 +1058,7 @@ void lanczos(cudaStream_t st, const T* A, int64_t n, int64_t lda, int ne, const 
     CHASE_CHECK_LAUNCH();
     step(j);
   }
-  tridiag_ql_kernel<<<runs, 32, 0, st>>>(steps, alpha, beta, theta, tau2, status);
+  tridiag_kernel<<<runs, TRI_THREADS, 4 * steps * (steps + 1) * (int)sizeof(double), st>>>(steps, alpha, beta, theta, tau2, status);
   CHASE_CHECK_LAUNCH();
   lanczos_bounds_kernel<<<1, 256, 0, st>>>(runs, steps, n, ne, theta, tau2, beta, out4);
   CHASE_CHECK_LAUNCH();

@@ -54,7 +54,7 @@ __device__ __forceinline__ uint32_t pack_planes(float a, float b, float sc) {  /
 // K <= 4096): the column's largest magnitude f 2^e, f in [0.5, 1), gives its scale 2^e (1 for a zero column or a
 // non-finite one).  Left-operand planes (KIND 0): (t, p), p in {re, im}; right-operand planes: p in {-im, re, im}; real:
 // one plane per slice.  Layout planes[(t*P + p) * ncols + col][Kpad].
-// n = 5003 real: A 100 us (scales and digits by separate FP64 kernels: 860), 300 right columns 7 us (39).
+// n = 5003 real: A 88 us (scales and digits by separate FP64 kernels: 860), 300 right columns 14 us (39).
 template <typename T, int NS, int KIND>
 __global__ void __launch_bounds__(128) split_kernel(int64_t K, int64_t Kpad, int ncols, const T* __restrict__ X, int64_t ldx,
                                                     double* scale, int conj, __nv_bfloat16* planes) {
