@@ -10,12 +10,13 @@ from its compact-WY factors.
 A timed step is the paper's fixed-work protocol (one subspace iteration):
 Lanczos bounds, the degree-20 Chebyshev filter of all nev+nex columns, QR,
 Rayleigh-Ritz with the dense eigensolve, residuals, locking, degrees and the
-degree sort, in the FP64 mode (FP64-class split-BF16 tensor-core products).
+degree sort, in the FP64 mode (FP64-class products from residues on the bf16
+tensor cores).
 value = filter TFLOP/s counted as 8 n^2 Matvecs (complex FMA = 8 flops) over
 the filter time.  Full solves to residual 1e-10 in FP64 and mixed mode are
 timed once each after the timed steps (time-to-solution).
 
-The inputs (A: 14.4 GB, its digit planes: 25 GB) are far larger than L2, so no
+The inputs (A: 14.4 GB, its residue planes: 86 GB) are far larger than L2, so no
 explicit L2 flush is needed between steps.
 """
 from __future__ import annotations
@@ -157,21 +158,6 @@ class Clocks:
                 continue
         return {"sm_mhz": statistics.median(sm) if sm else None, "sm_max_mhz": mx, "reasons": sorted(reasons),
                 "samples": len(sm)}
-
-
-# DRAM traffic (ncu dram__bytes_read.sum + dram__bytes_write.sum) of one full-width filter launch of the
-# current kernel, captured at n = 8192 with 1600 columns (`bench.py --hemm-only fp64 --n 8192`, one launch,
-# --clock-control none; profiles/oz_gemm_fp64_complex_n8192.md): 10.046 GB read + 0.235 GB written.  Scaled
-# to the bench's n by (n / 8192)^2: at a fixed column count the launch has n / 128 row blocks, each streaming
-# planes of length n, so both the left- and the right-operand traffic grow as n^2.  Captures stay at n = 8192;
-# set to None when the kernel changes until it is captured again.
-FILTER_TRAFFIC_N8192 = 10.281e9
-
-
-def filter_traffic_bytes(n, ne, slices):
-    if FILTER_TRAFFIC_N8192 is None or ne != 1600 or slices != 7:
-        return None
-    return FILTER_TRAFFIC_N8192 * (n / 8192.0) ** 2
 
 
 def peaks():
@@ -475,18 +461,17 @@ def run_ours(args):
     value = whole_job_tflops(flops_all, filter_ms)
     ms_step = t_ms / args.steps
 
-    # roofline of the dominant kernel: the FP64-class split-product GEMM of the filter.  Work is the
+    # roofline of the dominant kernels: the FP64-class residue product of the filter.  Work is the
     # algorithmic HEMM work of the launches (8 n^2 flops per column and degree step, complex), over the
-    # CUDA-event time of those launches, against the bf16 tensor peak the kernel runs on; the split
-    # products' own bf16 work (digit pairs x the algorithmic work) is reported beside it as the
-    # emulation's efficiency.
+    # CUDA-event time of those launches, against the bf16 tensor peak the kernel runs on; the residue
+    # products' own bf16 work (16 moduli x 3 real products, 12 times the algorithmic work) is reported
+    # beside it as the emulation's efficiency.  DRAM traffic: no capture of this kernel at this size.
     pk = peaks()
-    slices = int(one.opts.oz_slices)
-    pairs = slices * (slices + 1) // 2
+    residue_products = 48
     kern_ms = sum(s["ms_filter_kernel"] for s in stats)
     kern_launches = sum(s["filter_kernel_launches"] for s in stats)
     alg_flops = sum(8.0 * n * n * s["matvecs"] for s in stats)
-    split_flops = pairs * alg_flops
+    split_flops = residue_products / 4 * alg_flops
     achieved = alg_flops / (kern_ms * 1e-3) / 1e12 if kern_ms > 0 else None
     split_tflops = split_flops / (kern_ms * 1e-3) / 1e12 if kern_ms > 0 else None
     peak = pk.get("bf16_tflops_sustained")
@@ -498,17 +483,17 @@ def run_ours(args):
         fp64_units = {"error": repr(ex)[:200]}
     roofline = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s",
                 "frac": (achieved / peak) if (achieved and peak) else None,
-                "traffic": filter_traffic_bytes(n, ne, slices),
+                "traffic": None,
                 "work": "algorithmic: 8 n^2 flops per column and degree step (complex HEMM), "
                         f"{8.0 * n * n * ne:.4g} flops per full-width launch",
-                "algorithmic_bytes_per_launch": 2.0 * 2 * slices * n * n + 2.0 * 3 * slices * ne * n + 3 * 16.0 * n * ne,
-                "kernel": f"oz_gemm_kernel<S={slices},exact levels=5,complex> (bf16 split products, "
-                          f"{pairs} digit pairs per complex product)",
+                "algorithmic_bytes_per_launch": 2.0 * residue_products * (n * n + ne * n + n * ne) + 3 * 16.0 * n * ne,
+                "kernel": f"crt_gemm_kernel + combine_kernel ({residue_products} bf16 residue products per "
+                          "complex product)",
                 "peak_source": "MEASURED_PEAKS.json bf16_tflops_sustained (of measured)",
                 "launch_ms_avg": kern_ms / max(1, kern_launches), "launches": kern_launches,
-                "emulation": {"split_bf16_tflops": split_tflops, "frac": (split_tflops / peak) if (split_tflops and peak)
-                              else None, "digit_pairs": pairs,
-                              "note": "bf16 work of the split products (digit pairs x algorithmic) over the same time"},
+                "emulation": {"residue_bf16_tflops": split_tflops, "frac": (split_tflops / peak) if (split_tflops and peak)
+                              else None, "residue_products": residue_products,
+                              "note": "bf16 work of the residue products over the same time"},
                 "fp64_units": fp64_units}
     one.close()
 

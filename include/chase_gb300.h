@@ -51,8 +51,8 @@ typedef enum { CHASE_R64 = 0, CHASE_C128 = 1 } chase_dtype;
  * QR, Rayleigh-Ritz, the small eigensolve, residuals and Lanczos always run with
  * FP64 accuracy. */
 typedef enum {
-  CHASE_FP64 = 0,       /* FP64-accurate products: split-BF16 tensor-core products
-                           with exact FP32 partial sums, combined in integer/FP64 */
+  CHASE_FP64 = 0,       /* FP64-accurate products: 62-bit integers through residues
+                           modulo 16 moduli on the bf16 tensor cores (exact) */
   CHASE_FP64_NATIVE = 1,/* plain DFMA kernels (reference path; slow on this chip) */
   CHASE_BF16x3 = 2,     /* mixed: 2-slice split-BF16 (3 products) bulk filter, then
                            FP64 sweeps once residuals reach the bulk precision */
@@ -66,9 +66,9 @@ typedef struct {
   int maxiter;         /* outer iterations before CHASE_ERR_NOCONV (default 30) */
   int extra_deg;       /* constant added to the optimised degree (default 2) */
   int nfinal;          /* mixed modes: minimum FP64 sweeps at the end (default 1) */
-  int oz_slices;       /* FP64 mode: BF16 slices per operand, 6 or 7 (default 7) */
-  int native_below_mflop; /* products below this many MFLOP use DFMA kernels; 0: always
-                             split tensor-core products (default 2000) */
+  int oz_slices;       /* 6 or 7 (default 7); accepted, without effect: the FP64 mode has one precision */
+  int native_below_mflop; /* products of QR and Rayleigh-Ritz below this many MFLOP use DFMA kernels; 0: always
+                             tensor-core products; default 2000: the library draws the line (20) */
   int batch_workers;   /* chase_solve_batched: host threads that run the per-problem stages (grouped
                           mode), or problems solved concurrently, each worker with its own stream and
                           workspace sized (n_max, ne_max) (worker-pool mode); default 1, at most 32 */
@@ -119,7 +119,7 @@ void chase_set_wait_limit_ns(uint64_t ns);
  * Runs on its own stream of the current device and returns when it has finished. */
 chase_status chase_measure_fp64_peak(int which, double* tflops_out, double* ms_out);
 
-/* tcgen05 issue-rate probe (not part of Algorithm 1): cycles per MMA of the FP64 split-product kernel's
+/* tcgen05 issue-rate probe (not part of Algorithm 1): cycles per MMA of a seven-slice digit product's
  * per-k-block issue pattern (7 left slices, 28 digit pairs, 2 planes x 2 K-steps: 112 MMAs of M = 128,
  * width n_cols, K = 16, bf16 operands, FP32 accumulators), issued back to back by one thread of one CTA per
  * SM, zero operands.  variant 0: no synchronisation, n_cols in {16, 32, 64, 80, 96, 128, 256}; for n_cols = 80:

@@ -5,7 +5,7 @@
 // Rayleigh-Ritz projection and back-transform, residual norms) and the
 // reference path of the Chebyshev filter product.  On GB300 FP64 runs on the
 // CUDA cores only (about 1.2 TFLOP/s), so the large products of the
-// production path go through the split-BF16 tensor-core kernels instead.
+// production path go through the tensor-core residue products instead.
 #include <algorithm>
 
 #include "common.cuh"

@@ -611,9 +611,9 @@ struct Mod2 {
 // Two pairs may form a cluster: they take neighbouring row tiles of the same columns, and each CTA copies one half (along
 // K) of its right rows for both (multicast), which takes a quarter off the copies' L2 traffic.  A slot is then free
 // when both pairs' MMAs on it are done.
-// What bounds it: the issuing thread, and L2 traffic.  Without any copy, a stage of four MMAs took 720 cycles at any width up to 256
-// columns (512 cycles of math): a barrier check costs it about 200 cycles and the MMA queue is only a few instructions
-// deep.  So a stage holds 128 along K (eight MMAs), and the next stage's barrier is looked at between its halves,
+// What bounds it: the issuing thread, and L2 traffic.  Without any copy, a stage of four MMAs took 720 cycles at any
+// width up to 256 columns (512 cycles of math): a barrier check costs it about 200 cycles and the MMA queue is only a
+// few instructions deep.  So a stage holds 128 along K (eight MMAs), and the next stage's barrier is looked at between its halves,
 // while four MMAs are queued.
 // Register split: 384 threads at 168 (64512 at launch); warps 0-3 give down to 40, warps 4-11 take 232.
 template <int G>

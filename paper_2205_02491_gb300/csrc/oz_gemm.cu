@@ -4,9 +4,8 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 
-#include <mutex>
-
 #include <algorithm>
+#include <mutex>
 
 #include "common.cuh"
 #include "crt.h"
