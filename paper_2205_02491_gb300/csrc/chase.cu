@@ -1623,7 +1623,7 @@ static void solve_batched_grouped(chase_ctx* c, int nprob, const void* const* A,
   so.batch_grouped = 0;
   if ((int)c->slots.size() < nprob) c->slots.resize(nprob, nullptr);
   int64_t need_new = 0;
-  double n2_new = 0.0;
+  std::vector<int> fresh;
   for (int p = 0; p < nprob; ++p) {
     chase_ctx*& sl = c->slots[p];
     const int ne = nev[p] + nex[p];
@@ -1633,15 +1633,25 @@ static void solve_batched_grouped(chase_ctx* c, int nprob, const void* const* A,
     }
     if (!sl) {
       need_new += chase_workspace_bytes(n[p], ne, c->dtype, &so);
-      n2_new += (double)n[p] * (double)n[p];
+      fresh.push_back(p);
     }
   }
-  // memory beyond the new slots' workspaces: half of it goes to their residue planes, in proportion to n^2
-  double extra = 0.0;
+  // Three quarters of the memory beyond the new slots' workspaces go to their residue planes, all of a problem's or
+  // none beyond the least, smallest problems first: a problem whose planes are not all resident converts A in every
+  // product and stays out of the grouped launches (64 problems of up to 8192, shares of half the memory in
+  // proportion to n^2: none had all its planes, 19.9 s for the first step).
+  std::vector<int64_t> extra(nprob, 0);
   if (need_new > 0) {
     size_t freeb = 0, totb = 0;
     CHASE_CUDA(cudaMemGetInfo(&freeb, &totb));
-    extra = std::max(0.0, 0.5 * ((double)freeb - (double)need_new - (double)(64ll << 20)));
+    int64_t left = ((int64_t)freeb - need_new - (64ll << 20)) / 4 * 3;
+    std::stable_sort(fresh.begin(), fresh.end(), [&](int a, int b) { return n[a] < n[b]; });
+    for (int p : fresh) {
+      const int64_t full = crt::plane_bytes(n[p], n[p], CPLX, crt::NMOD);
+      if (full > left) break;
+      extra[p] = full;
+      left -= full;
+    }
   }
   for (int p = 0; p < nprob; ++p) {
     chase_ctx*& sl = c->slots[p];
@@ -1649,8 +1659,7 @@ static void solve_batched_grouped(chase_ctx* c, int nprob, const void* const* A,
     if (!sl) {
       cudaStream_t ws = nullptr;
       CHASE_CUDA(cudaStreamCreateWithFlags(&ws, cudaStreamNonBlocking));
-      chase_status st = create_ctx(&sl, n[p], ne, c->dtype, &so, ws,
-                                   (int64_t)(extra * ((double)n[p] * (double)n[p] / n2_new)));
+      chase_status st = create_ctx(&sl, n[p], ne, c->dtype, &so, ws, extra[p]);
       if (st != CHASE_OK) {
         cudaStreamDestroy(ws);
         sl = nullptr;
