@@ -618,7 +618,7 @@ def run_ours(args):
     if rank == 0:
         line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps,
                 "warmup": args.warmup, "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak",
-                "vs_baseline": None, "dtype": "f64 (FP64-class split-BF16 tensor-core products; QR/RR/eig FP64)",
+                "vs_baseline": None, "dtype": "f64 (FP64-class products through residues on the bf16 tensor cores; QR/RR/eig FP64)",
                 "data": "synthetic (seeded prescribed-spectrum matrices)",
                 "config": workload_config(args, {"parallelism": "replicas" if ws > 1 else "single GPU"}),
                 "clocks": clk, "gpu_launches": launches, "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e,
