@@ -87,8 +87,9 @@ typedef struct {
                           (computed when each pair locked; bounds the returned pairs) */
   int qr_fallbacks;    /* shifted Cholesky-QR fallbacks taken */
   int filter_launches; /* filter product launches */
-  double ms_filter_kernel;      /* CUDA-event time of the FP64 split-product filter kernels alone */
-  int filter_kernel_launches;   /* launches timed in ms_filter_kernel */
+  double ms_filter_kernel;      /* CUDA-event time of the FP64 filter products' kernels; runs of products of less
+                                   than about 100 us are timed as one span, their operands' conversion included */
+  int filter_kernel_launches;   /* products timed in ms_filter_kernel */
   double ms_filter_kernel_lowp; /* same for the mixed-precision bulk filter kernels */
   double ms_backward;           /* time of the last chase_backward */
   int minres_iterations;        /* MINRES iterations of the last chase_backward */

@@ -967,7 +967,7 @@ template <typename T> struct Solver {
     int64_t mv = filter(R.A, R.n, R.lda, Vact, T1act, k, R.m.data(), c->deg, R.b_sup, R.mu_1, R.mu_ne, R.fmode(), true);
     if (oz::available()) {
       int nl = 0;
-      double ms = oz::timing_collect(c->ozw, &nl);
+      double ms = oz::timing_collect(st(), c->ozw, &nl);
       if (R.lowp) {
         S.ms_filter_kernel_lowp += ms;
       } else {

@@ -60,6 +60,8 @@ struct Workspace {
   bool timing = false;
   std::vector<cudaEvent_t> ev;
   int ev_used = 0;
+  bool span_open = false;  // a span of small products has its start recorded in ev[ev_used]
+  int timed = 0;           // products timed
   // A whose exponents and residues (a_src) or digit planes (d_src) are held
   const void* a_src = nullptr;
   int64_t a_n = 0;
@@ -93,9 +95,42 @@ void destroy(Workspace& w);
 // the tuner's choices so far: (size-class key, candidate index) pairs, for reports
 std::vector<std::pair<uint64_t, int>> tuned(const Workspace& w);
 void invalidate(Workspace& w);
-// start recording event pairs around every product kernel; collect returns (ms, launches)
+// start recording event pairs around the product kernels (ProductTimer); collect returns (ms, products)
 void timing_begin(Workspace& w);
-double timing_collect(Workspace& w, int* launches);
+double timing_collect(cudaStream_t st, Workspace& w, int* launches);
+
+// Event pair around one product's kernels (filter roofline), or, for products of less than SPAN_FLOPS of bf16 work (100
+// us), one pair around a whole run of them and what lies between.  Nothing overlaps across an event, and a pair takes
+// about 10 us of a small product's 32: a pair each cost a solve with n = 512 1.6 of 10.6 ms, with n = 3001 1.5 of 52.
+struct ProductTimer {
+  static constexpr double SPAN_FLOPS = 2e11;
+  cudaStream_t st;
+  Workspace& w;
+  bool on = false;
+  ProductTimer(cudaStream_t s, Workspace& ws, double flops) : st(s), w(ws) {
+    if (!w.timing) return;
+    if (flops >= SPAN_FLOPS) close(st, w);
+    if (w.span_open) {
+      ++w.timed;
+    } else if (w.ev_used + 2 <= (int)w.ev.size()) {
+      CHASE_CUDA(cudaEventRecord(w.ev[w.ev_used], st));
+      ++w.timed;
+      if (flops >= SPAN_FLOPS) on = true;
+      else w.span_open = true;
+    }
+  }
+  void stop() {
+    if (on) end(st, w);
+  }
+  static void close(cudaStream_t st, Workspace& w) {
+    if (w.span_open) end(st, w);
+    w.span_open = false;
+  }
+  static void end(cudaStream_t st, Workspace& w) {
+    CHASE_CUDA(cudaEventRecord(w.ev[w.ev_used + 1], st));
+    w.ev_used += 2;
+  }
+};
 int read_flags(cudaStream_t st, Workspace& w);
 // planes of A for the given mode (cached until invalidate)
 template <typename T>

@@ -297,11 +297,13 @@ void timing_begin(Workspace& w) {
     w.ev.resize(256);
     for (auto& e : w.ev) CHASE_CUDA(cudaEventCreate(&e));
   }
-  w.ev_used = 0;
+  w.ev_used = w.timed = 0;
+  w.span_open = false;
   w.timing = true;
 }
 
-double timing_collect(Workspace& w, int* launches) {
+double timing_collect(cudaStream_t st, Workspace& w, int* launches) {
+  ProductTimer::close(st, w);
   double ms = 0.0;
   for (int i = 0; i + 1 < w.ev_used; i += 2) {
     CHASE_CUDA(cudaEventSynchronize(w.ev[i + 1]));
@@ -309,7 +311,7 @@ double timing_collect(Workspace& w, int* launches) {
     CHASE_CUDA(cudaEventElapsedTime(&t, w.ev[i], w.ev[i + 1]));
     ms += t;
   }
-  if (launches) *launches = w.ev_used / 2;
+  if (launches) *launches = w.timed;
   w.ev_used = 0;
   w.timing = false;
   return ms;
@@ -322,21 +324,6 @@ void invalidate(Workspace& w) {
 }
 
 // ---------------------------------------------------------------- FP64-class products
-// event pair around one product's kernels (filter roofline)
-struct ProductTimer {
-  cudaStream_t st;
-  Workspace& w;
-  bool on;
-  ProductTimer(cudaStream_t s, Workspace& ws) : st(s), w(ws), on(ws.timing && ws.ev_used + 2 <= (int)ws.ev.size()) {
-    if (on) CHASE_CUDA(cudaEventRecord(w.ev[w.ev_used], st));
-  }
-  void stop() {
-    if (!on) return;
-    CHASE_CUDA(cudaEventRecord(w.ev[w.ev_used + 1], st));
-    w.ev_used += 2;
-  }
-};
-
 // columns of a product (M rows, inner length K) whose right planes and residues fit the workspace
 static int64_t panel_fit(const Workspace& w, int64_t M, int64_t K) {
   const int64_t by_res = w.residue_bytes / crt::residue_bytes(M, 1, w.complex_);
@@ -370,7 +357,7 @@ static void product(cudaStream_t st, Workspace& w, const void* lpl, const int* l
     } else {
       crt::right_planes<T>(st, &op, 1);
     }
-    ProductTimer t(st, w);
+    ProductTimer t(st, w, 2.0 * crt::NMOD * crt::planes(S<T>::cplx) * (double)M * (double)nc * (double)K);
     for (int m0 = 0; m0 < crt::NMOD; m0 += mods) {
       const int nm = std::min(mods, crt::NMOD - m0);
       lconv(m0, nm);

@@ -457,8 +457,10 @@ void launch_ops(cudaStream_t st, Workspace& w, const ProductOp* ops, int nops, c
                                     Cf::SMEM_BYTES);
   });
   CHASE_CUDA(attr_err);
-  const bool timed = w.timing && w.ev_used + 2 <= (int)w.ev.size();
-  if (timed) CHASE_CUDA(cudaEventRecord(w.ev[w.ev_used], st));
+  double flops = 0.0;
+  for (int q = 0; q < nops; ++q)
+    flops += (CPLX ? 4.0 : 1.0) * S * (S + 1) * (double)ops[q].M * (double)ops[q].N * (double)ops[q].K;
+  ProductTimer timer(st, w, flops);
   if (tune_ev) CHASE_CUDA(cudaEventRecord(tune_ev[0], st));
   launch_pdl(oz_gemm_kernel<S, CPLX, NTT, G>, (unsigned)tiles, NTHREADS, Cf::SMEM_BYTES, st, gp, w.flags);
   CHASE_CHECK_LAUNCH();
@@ -470,10 +472,7 @@ void launch_ops(cudaStream_t st, Workspace& w, const ProductOp* ops, int nops, c
     CHASE_CHECK_LAUNCH();
   }
   if (tune_ev) CHASE_CUDA(cudaEventRecord(tune_ev[1], st));
-  if (timed) {
-    CHASE_CUDA(cudaEventRecord(w.ev[w.ev_used + 1], st));
-    w.ev_used += 2;
-  }
+  timer.stop();
 }
 
 // The launches are instantiated in the oz_inst_*.cu units (compiled in parallel); every other unit sees
