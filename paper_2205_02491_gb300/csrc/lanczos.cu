@@ -760,6 +760,8 @@ __device__ __forceinline__ bool ql_fp32(int k, float* d, float* e, float* Z, int
         const float f = sn * e[i], b = cs * e[i], di = d[i];
         const float q = fmaf(f, f, g * g);
         if (!(q > 1e-36f)) return false;  // the rotation is undefined: left to the FP64 version
+        // every lane has made its reads of the rotation before (and of d[mm], d[l + 1], e[l]) when lane 0 stores over them
+        __syncwarp();
         const float ri = rsqrtf(q);
         const float c0 = lane < k ? Z[lane + i * ldz] : 0.0f, c1 = lane + 32 < k ? Z[lane + 32 + i * ldz] : 0.0f;
         sn = f * ri;
