@@ -474,12 +474,11 @@ template <int G> struct Params {
   CUtensorMap tmA[G];
   CUtensorMap tmB[G];
   int8_t* R[G];
-  int M[G], N[G], K[G], mt[G], nt[G], ldr[G];  // mt: row tiles, in units of `pairs`
+  int M[G], N[G], K[G], mt[G], nt[G], ldr[G];  // mt, nt: row and column tiles
   int nblk[G];                   // 32-column blocks of the product's columns
   int box_b[G];                  // right rows per copy
   int unit_begin[G + 1];
   int nprob, mod0, np;           // np: planes per modulus
-  int pairs;                     // CTA pairs per cluster (1 or 2)
   int stages, stage_bytes;       // ring of the launch (as many stages as its widest right copy leaves room for)
 };
 
@@ -529,15 +528,6 @@ __device__ __forceinline__ void tma_load_pair(uint32_t dst, const CUtensorMap* m
       "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, "
       "%5}], [%2];" ::"r"(dst),
       "l"((unsigned long long)map), "r"(bar), "r"(x), "r"(y), "r"(z)
-      : "memory");
-}
-// the same into every CTA of the mask, each of which signals its own pair's leader (bar lies in an even CTA)
-__device__ __forceinline__ void tma_load_multicast(uint32_t dst, const CUtensorMap* map, uint32_t bar, int x, int y, int z,
-                                                   uint32_t mask) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.tile.mbarrier::complete_tx::bytes.multicast::cluster "
-      "[%0], [%1, {%3, %4, %5}], [%2], %6;" ::"r"(dst),
-      "l"((unsigned long long)map), "r"(bar), "r"(x), "r"(y), "r"(z), "h"((uint16_t)mask)
       : "memory");
 }
 __device__ __forceinline__ void mma_pair(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
@@ -608,9 +598,6 @@ struct Mod2 {
 // accumulator sets (2 x 256 TMEM columns) and the eight reduction warps of each CTA take a finished chunk modulo m
 // into FP32 registers while the next chunk accumulates in the other set.  At a unit's end they write residues
 // (8-bit); the copies and MMAs of the next unit run meanwhile.
-// Two pairs may form a cluster: they take neighbouring row tiles of the same columns, and each CTA copies one half (along
-// K) of its right rows for both (multicast), which takes a quarter off the copies' L2 traffic.  A slot is then free
-// when both pairs' MMAs on it are done.
 // What bounds it: the issuing thread, and L2 traffic.  Without any copy, a stage of four MMAs took 720 cycles at any
 // width up to 256 columns (512 cycles of math): a barrier check costs it about 200 cycles and the MMA queue is only a
 // few instructions deep.  So a stage holds 128 along K (eight MMAs), and the next stage's barrier is looked at between its halves,
@@ -628,17 +615,16 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   uint64_t* drain = acc_empty + 2;
   uint32_t* tmem_slot = (uint32_t*)(drain + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const uint32_t cta = cluster_rank(), rank = cta & 1, pair = cta >> 1, leader = cta & ~1u;
-  const int pairs = gp.pairs;
-  const int cluster = blockIdx.x / (2 * pairs), nclusters = gridDim.x / (2 * pairs);
-  const uint32_t pair_mask = 3u << (2 * pair), all_mask = (1u << (2 * pairs)) - 1;
+  const uint32_t rank = cluster_rank(), leader = 0;
+  constexpr uint32_t both_ctas = 3;
+  const int cluster = blockIdx.x / 2, nclusters = gridDim.x / 2;
   const int total = gp.unit_begin[gp.nprob];
   const int stages = gp.stages, stage_bytes = gp.stage_bytes;
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < MAX_STAGES; ++i) {
       mbar_init(smem_u32(&full[i]), 1);
-      mbar_init(smem_u32(&empty[i]), pairs);
+      mbar_init(smem_u32(&empty[i]), 1);
     }
     for (int i = 0; i < 2; ++i) {
       mbar_init(smem_u32(&acc_full[i]), 1);
@@ -683,7 +669,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         int n0, width;
         tile_cols(gp.nblk[prob], gp.nt[prob], n, n0, width);
         const int box = gp.box_b[prob], K = gp.K[prob];
-        const int y_a = (m * pairs + (int)pair) * TM + (int)rank * 128, y_b = n0 + (int)rank * (width >> 1);
+        const int y_a = m * TM + (int)rank * 128, y_b = n0 + (int)rank * (width >> 1);
         const int z_b = gp.mod0 * gp.np + plane;
         const uint32_t half_bytes = (uint32_t)(A_HALF + box * TK * 2);
         for (int k0 = 0; k0 < K; k0 += SK) {
@@ -696,13 +682,11 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           const uint32_t dst = smem_u32(smem + sl * stage_bytes), bar = cluster_addr(smem_u32(&full[sl]), leader);
           const uint32_t dst_b = dst + 2 * A_HALF, b_half = (uint32_t)(box * TK * 2);
           tma_load_pair(dst, &gp.tmA[prob], bar, k0, y_a, plane);
-          if (pairs == 1) {
-            tma_load_pair(dst_b, &gp.tmB[prob], bar, k0, y_b, z_b);
-            if (two) tma_load_pair(dst_b + b_half, &gp.tmB[prob], bar, k0 + TK, y_b, z_b);
-          } else if (pair == 0 || two) {
-            tma_load_multicast(dst_b + pair * b_half, &gp.tmB[prob], bar, k0 + (int)pair * TK, y_b, z_b, 5u << rank);
+          tma_load_pair(dst_b, &gp.tmB[prob], bar, k0, y_b, z_b);
+          if (two) {
+            tma_load_pair(dst + A_HALF, &gp.tmA[prob], bar, k0 + TK, y_a, plane);
+            tma_load_pair(dst_b + b_half, &gp.tmB[prob], bar, k0 + TK, y_b, z_b);
           }
-          if (two) tma_load_pair(dst + A_HALF, &gp.tmA[prob], bar, k0 + TK, y_a, plane);
           advance();
         }
       }
@@ -770,16 +754,16 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 #pragma unroll
             for (int ks = 0; ks < TK / 16; ++ks) mma_pair(d, ad2 + (uint64_t)(ks * 2), bd2 + (uint64_t)(ks * 2), idesc, 1u);
           }
-          commit_to(slot, all_mask);
+          commit_to(slot, both_ctas);
           if (++in_chunk == CHUNK || k0 + SK >= K) {
-            commit_to(smem_u32(&acc_full[b]), pair_mask);
+            commit_to(smem_u32(&acc_full[b]), both_ctas);
             ++chunk;
             in_chunk = 0;
           }
         }
       }
       // every MMA is done before TMEM is freed
-      commit_to(smem_u32(drain), pair_mask);
+      commit_to(smem_u32(drain), both_ctas);
       const unsigned long long t0 = globaltimer();
       while (!mbar_try(smem_u32(drain), 0) && globaltimer() - t0 < TIMEOUT_NS) {
       }
@@ -838,7 +822,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         }
       }
       if (!ok) break;
-      const int row = (m * pairs + (int)pair) * TM + (int)rank * 128 + q * 32 + lane;
+      const int row = m * TM + (int)rank * 128 + q * 32 + lane;
       if (row < gp.M[prob]) {
         const int N = gp.N[prob], ldr = gp.ldr[prob];
         const int c0 = n0 + half * hc;
@@ -1026,48 +1010,33 @@ void residues(cudaStream_t st, bool by_rows, bool conj, int64_t nvec, int64_t K,
   CHASE_CHECK_LAUNCH();
 }
 
-// clusters of one or two CTA pairs the device keeps resident (0: none)
-template <int G> static int max_clusters(int pairs) {
+// CTA pairs the device keeps resident (0: none)
+template <int G> static int max_pairs() {
   static std::once_flag once;
   static cudaError_t err = cudaSuccess;
-  static int got[2] = {0, 0};
+  static int got = 0;
   std::call_once(once, []() {
     err = cudaFuncSetAttribute(crt_gemm_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
-    for (int p = 1; p <= 2 && err == cudaSuccess; ++p) {
-      cudaLaunchConfig_t cfg{};
-      cudaLaunchAttribute at{};
-      at.id = cudaLaunchAttributeClusterDimension;
-      at.val.clusterDim.x = 2 * p;
-      at.val.clusterDim.y = at.val.clusterDim.z = 1;
-      cfg.gridDim = dim3(2 * p, 1, 1);
-      cfg.blockDim = dim3(NTHREADS, 1, 1);
-      cfg.dynamicSmemBytes = SMEM_BYTES;
-      cfg.attrs = &at;
-      cfg.numAttrs = 1;
-      err = cudaOccupancyMaxActiveClusters(&got[p - 1], crt_gemm_kernel<G>, &cfg);
-    }
+    if (err != cudaSuccess) return;
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = 2;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.gridDim = dim3(2, 1, 1);
+    cfg.blockDim = dim3(NTHREADS, 1, 1);
+    cfg.dynamicSmemBytes = SMEM_BYTES;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    err = cudaOccupancyMaxActiveClusters(&got, crt_gemm_kernel<G>, &cfg);
   });
   CHASE_CUDA(err);
-  return got[pairs - 1];
+  return got;
 }
 
 template <int G> static void launch(cudaStream_t st, const Product* ops, int nops, bool cplx, int mod0, int nmod, int* err) {
   static thread_local Params<G> gp;  // large for G > 1: built in thread-local host memory
   const int np = planes(cplx);
-  // units and rounds over the resident clusters, with one and with two pairs per cluster
-  int64_t u[2] = {0, 0};
-  int64_t cols = 0;
-  for (int p = 0; p < nops; ++p) {
-    const int64_t nt = ceil_div(ceil_div(ops[p].N, 32), TN / 32), mt = ceil_div(ops[p].M, TM);
-    u[0] += mt * nt * np * nmod;
-    u[1] += (mt + 1) / 2 * nt * np * nmod;
-    cols = std::max(cols, std::min<int64_t>(TN, ops[p].N / nt));
-  }
-  const int c1 = std::max(1, max_clusters<G>(1)), c2 = max_clusters<G>(2);
-  // Narrow tiles are bound by the left planes' HBM traffic, which sharing does not lower; else two pairs unless their
-  // last round is emptier by more than the tenth that sharing gains
-  const double r1 = (double)ceil_div(u[0], c1), r2 = c2 > 0 ? (double)ceil_div(u[1], c2) : 1e30;
-  const int pairs = cols >= 128 && r2 <= 1.1 * r1 ? 2 : 1;
   int64_t units = 0;
   int box_max = 0;
   for (int p = 0; p < nops; ++p) {
@@ -1082,7 +1051,7 @@ template <int G> static void launch(cudaStream_t st, const Product* ops, int nop
     gp.N[p] = (int)o.N;
     gp.K[p] = (int)o.K;
     box_max = std::max(box_max, box);
-    gp.mt[p] = (int)ceil_div(ceil_div(o.M, TM), pairs);
+    gp.mt[p] = (int)ceil_div(o.M, TM);
     gp.nt[p] = nt;
     gp.nblk[p] = nblk;
     gp.box_b[p] = box;
@@ -1095,15 +1064,14 @@ template <int G> static void launch(cudaStream_t st, const Product* ops, int nop
   gp.nprob = nops;
   gp.mod0 = mod0;
   gp.np = np;
-  gp.pairs = pairs;
   gp.stage_bytes = 2 * (A_HALF + box_max * TK * 2);
   gp.stages = std::min(MAX_STAGES, SMEM_RING / gp.stage_bytes);
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute at[2] = {{}, pdl_attribute()};
   at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim.x = 2 * pairs;
+  at[0].val.clusterDim.x = 2;
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-  cfg.gridDim = dim3((unsigned)(2 * pairs * std::min<int64_t>(units, pairs == 2 ? c2 : c1)), 1, 1);
+  cfg.gridDim = dim3((unsigned)(2 * std::min<int64_t>(units, std::max(1, max_pairs<G>()))), 1, 1);
   cfg.blockDim = dim3(NTHREADS, 1, 1);
   cfg.dynamicSmemBytes = SMEM_BYTES;
   cfg.stream = st;
