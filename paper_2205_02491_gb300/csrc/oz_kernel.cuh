@@ -176,8 +176,6 @@ __global__ void __maxnreg__(168) oz_gemm_kernel(const __grid_constant__ GroupPar
   uint32_t* tmem_slot = (uint32_t*)(drain + 1);
   volatile int* abort_sh = (volatile int*)(tmem_slot + 1);
 
-  // a CTA of a launch that already hit a wait limit does nothing
-  if (*(volatile int*)err != 0) return;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int num_m = (M + BM - 1) / BM, num_n = (N + Cf::NCOLS - 1) / Cf::NCOLS;
   // K slice of this block (slice-major tile order; one slice unless the product is split along K)
@@ -219,7 +217,10 @@ __global__ void __maxnreg__(168) oz_gemm_kernel(const __grid_constant__ GroupPar
   grid_dependency_wait();
   const uint32_t tmem = *tmem_slot;
 
-  if (warp == 0 && lane == 0) {
+  // a CTA of a launch that already hit a wait limit does nothing: one thread's look at the flag decides for all (another
+  // CTA may set it between two looks), after the wait for the kernel before and with the barriers and TMEM set up
+  if (__syncthreads_or(threadIdx.x == 0 && *(volatile int*)err != 0)) {
+  } else if (warp == 0 && lane == 0) {
     // ------------------------------------------------------------ TMA producer
     int a_iter = 0, b_issued = 0;
     bool ok = true;
