@@ -107,9 +107,10 @@ typedef struct {
 int64_t chase_kernel_launch_count(void);
 
 /* Testing hook (not part of Algorithm 1): wall-clock limit, in nanoseconds, of every grid-barrier wait
- * of the persistent Jacobi sweep kernel of the Rayleigh-Ritz eigensolve, for launches made after the
- * call (process-wide).  0 restores the default of 2 s.  A wait that reaches the limit makes every block
- * of the launch return and the call that launched it return CHASE_ERR_TIMEOUT; the context stays
+ * of the persistent Jacobi sweep kernel of the Rayleigh-Ritz eigensolve and of every wait of the Lanczos
+ * product kernel (which counts a limit below 1000 as run out from the start), for launches made after the
+ * call (process-wide).  0 restores the default of 2 s.  After a wait that reached the limit the blocks of
+ * the launch return and the call that launched it returns CHASE_ERR_TIMEOUT; the context stays
  * usable.  Lets a test make a wait expire without faulting or hanging the GPU. */
 void chase_set_wait_limit_ns(uint64_t ns);
 

@@ -227,7 +227,7 @@ def measure_mma_issue(n_cols: int = 80, variant: int = 0) -> float:
 
 
 def set_wait_limit_ns(ns: int) -> None:
-    """Testing hook: wall-clock limit of the Jacobi sweep kernel's grid-barrier waits (0: default 2 s)."""
+    """Testing hook: wall-clock limit of the waits of the Jacobi sweep and Lanczos product kernels (0: default 2 s)."""
     L.load().chase_set_wait_limit_ns(int(ns))
 
 

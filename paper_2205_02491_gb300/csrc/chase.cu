@@ -918,9 +918,10 @@ template <typename T> struct Solver {
       CHASE_CHECK_LAUNCH();
       t.stop();
     }
-    double hb[6];
-    CHASE_CUDA(cudaMemcpyAsync(hb, c->dwork, 4 * sizeof(double), cudaMemcpyDeviceToHost, st()));
+    double hb[5];
+    CHASE_CUDA(cudaMemcpyAsync(hb, c->dwork, sizeof(hb), cudaMemcpyDeviceToHost, st()));
     CHASE_CUDA(cudaStreamSynchronize(st()));
+    check_lanczos(hb);
     R = Run{};
     R.A = A;
     R.n = n;
@@ -940,8 +941,6 @@ template <typename T> struct Solver {
     R.norm_est = std::max(std::fabs(R.mu_1), std::fabs(theta_max));
     S.norm_est = R.norm_est;
     R.thresh = tol * R.norm_est;
-    CHASE_REQUIRE(std::isfinite(R.b_sup) && std::isfinite(R.mu_1) && std::isfinite(R.mu_ne), CHASE_ERR_NAN,
-                  "non-finite Lanczos bounds");
     copy_cols<T>(st(), n, ne, V0, n, V(), n);
     R.m.assign(ne, deg);
     fill_int_kernel<<<ceil_div(ne, 256), 256, 0, st()>>>(ne, c->deg, deg);
@@ -1435,8 +1434,11 @@ chase_status chase_lanczos(chase_ctx* c, const void* A, int64_t n, int64_t lda, 
   else
     lanczos<double>(c->stream, (const double*)A, n, lda, ne, (const double*)L0, runs, steps, c->dwork,
                     (double*)c->work, c->work_elems, c->dwork + 8);
-  CHASE_CUDA(cudaMemcpyAsync(out_host, c->dwork, 4 * sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+  double hb[5];
+  CHASE_CUDA(cudaMemcpyAsync(hb, c->dwork, sizeof(hb), cudaMemcpyDeviceToHost, c->stream));
   CHASE_CUDA(cudaStreamSynchronize(c->stream));
+  check_lanczos(hb);
+  std::copy(hb, hb + 4, out_host);
   API_END(c)
 }
 

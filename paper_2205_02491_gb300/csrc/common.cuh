@@ -177,8 +177,8 @@ void launch_pdl(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaSt
   CHASE_CUDA(cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...));
 }
 
-// Wall-clock limit of the bounded grid-barrier waits of the Jacobi sweep kernel (nanoseconds).  Two
-// seconds unless a test shortens it through chase_set_wait_limit_ns (0 restores the default).
+// Wall-clock limit (nanoseconds) of the bounded waits of the Jacobi sweep kernel's grid barrier and of the Lanczos product
+// kernel.  Two seconds unless a test shortens it through chase_set_wait_limit_ns (0 restores the default).
 extern std::atomic<unsigned long long> g_wait_limit_ns;
 inline unsigned long long grid_wait_limit_ns() {
   const unsigned long long v = g_wait_limit_ns.load();

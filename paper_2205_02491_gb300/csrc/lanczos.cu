@@ -9,6 +9,7 @@
 #include <cuda_fp16.h>
 
 #include <algorithm>
+#include <cmath>
 #include <mutex>
 
 #include "common.cuh"
@@ -153,7 +154,8 @@ constexpr int NLEV = 8;
 constexpr int H_ACC = 80;                // TMEM columns per accumulator: 72 written
 constexpr int H_A0 = 2 * H_ACC;          // then one operand per producer group
 constexpr int H_ASLOT = 2 * NDIG * 8;    // 14 digit planes of 8 columns
-constexpr unsigned long long H_TIMEOUT_NS = 2000000000ull;
+constexpr unsigned long long H_DRAIN_NS = 2000000000ull;  // limit of the waits for copies and MMAs in flight at the end
+constexpr int LZ_STATUS_QL = 1, LZ_STATUS_WAIT = 2;       // bits of the status word: no QL convergence, a wait ran out
 template <typename T> struct Hemv {
   static constexpr int SLOTS = S<T>::cplx ? 2 : 4;                            // steps of A in flight per thread
   static constexpr int A_BYTES = SLOTS * 2 * HSTEP * 128 * (int)sizeof(T);   // 128 KB
@@ -161,8 +163,8 @@ template <typename T> struct Hemv {
   static constexpr int SMEM = 1024 + H_XSTAGES * X_BYTES + A_BYTES + 256;
 };
 
-// bounded wait: false on timeout or when another role gave up
-__device__ __forceinline__ bool hemv_wait(uint32_t bar, uint32_t parity, volatile int* gave_up) {
+// bounded wait: false after wait_ns or when another role gave up
+__device__ __forceinline__ bool hemv_wait(uint32_t bar, uint32_t parity, volatile int* gave_up, unsigned long long wait_ns) {
   unsigned long long t0 = 0;
   for (uint32_t it = 0;; ++it) {
     if (oz::mbar_try(bar, parity)) return true;
@@ -170,7 +172,7 @@ __device__ __forceinline__ bool hemv_wait(uint32_t bar, uint32_t parity, volatil
       if (*gave_up) return false;
       const unsigned long long t = oz::globaltimer();
       if (t0 == 0) t0 = t;
-      else if (t - t0 > H_TIMEOUT_NS) {
+      else if (t - t0 > wait_ns) {
         *gave_up = 1;
         return false;
       }
@@ -210,7 +212,8 @@ template <typename T>
 __global__ void __launch_bounds__(HEMV_THREADS, 1) hemv_kernel(int64_t n, const T* __restrict__ A, int64_t lda,
                                                                 const unsigned* __restrict__ rmax,
                                                                 const __half* __restrict__ X,
-                                                                const int* __restrict__ xe, int cols, int runs, T* part) {
+                                                                const int* __restrict__ xe, int cols, int runs, T* part,
+                                                                unsigned long long wait_ns, int* status) {
   using s = S<T>;
   using F = Frag<T>;
   using H = Hemv<T>;
@@ -240,7 +243,8 @@ __global__ void __launch_bounds__(HEMV_THREADS, 1) hemv_kernel(int64_t n, const 
       oz::mbar_init(smem_u32(&dempty[i]), 4);
     }
     oz::mbar_init(smem_u32(drain), 1);
-    *gave_up = 0;
+    // a limit below a microsecond, less than any wait for memory takes, has run out before the first one
+    *gave_up = wait_ns < 1000ull;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -272,7 +276,7 @@ __global__ void __launch_bounds__(HEMV_THREADS, 1) hemv_kernel(int64_t n, const 
     bool ok = true;
     for (int k = 0; k < 2 * nblk; ++k) {
       const int b = k & 1;
-      ok = __all_sync(0xffffffffu, hemv_wait(smem_u32(&dfull[b]), (k >> 1) & 1, gave_up));
+      ok = __all_sync(0xffffffffu, hemv_wait(smem_u32(&dfull[b]), (k >> 1) & 1, gave_up, wait_ns));
       if (!ok) break;
       oz::fence_after();
 #pragma unroll
@@ -384,7 +388,7 @@ __global__ void __launch_bounds__(HEMV_THREADS, 1) hemv_kernel(int64_t n, const 
           }
         }
         if (h == 0) {
-          ok = __all_sync(0xffffffffu, hemv_wait(smem_u32(&aempty[g]), (it & 1) ^ 1, gave_up));
+          ok = __all_sync(0xffffffffu, hemv_wait(smem_u32(&aempty[g]), (it & 1) ^ 1, gave_up, wait_ns));
           if (!ok) break;
           oz::fence_after();
         }
@@ -407,15 +411,15 @@ __global__ void __launch_bounds__(HEMV_THREADS, 1) hemv_kernel(int64_t n, const 
       bool ok = true;
       for (int kb = 0; kb < nblk && ok; ++kb) {
         const int st = kb % H_XSTAGES;
-        ok = hemv_wait(smem_u32(&xfull[st]), (kb / H_XSTAGES) & 1, gave_up);
+        ok = hemv_wait(smem_u32(&xfull[st]), (kb / H_XSTAGES) & 1, gave_up, wait_ns);
         if (!ok) break;
         const uint64_t xd = oz::sw128_desc(smem_u32(smem + st * H::X_BYTES));
 #pragma unroll 1
         for (int k = 0; k < HK / HSTEP; ++k) {
           // accumulator: two steps each
           const int g = k & 1, b = k >> 1, it = 2 * kb + (k >> 1);
-          ok = (g != 0 || hemv_wait(smem_u32(&dempty[b]), (kb & 1) ^ 1, gave_up)) &&
-               hemv_wait(smem_u32(&afull[g]), it & 1, gave_up);
+          ok = (g != 0 || hemv_wait(smem_u32(&dempty[b]), (kb & 1) ^ 1, gave_up, wait_ns)) &&
+               hemv_wait(smem_u32(&afull[g]), it & 1, gave_up, wait_ns);
           if (!ok) break;
           oz::fence_after();
 #pragma unroll
@@ -438,7 +442,7 @@ __global__ void __launch_bounds__(HEMV_THREADS, 1) hemv_kernel(int64_t n, const 
       // every MMA is done before TMEM is freed
       oz::mma_commit(smem_u32(drain));
       const unsigned long long t0 = oz::globaltimer();
-      while (!oz::mbar_try(smem_u32(drain), 0) && oz::globaltimer() - t0 < H_TIMEOUT_NS) {
+      while (!oz::mbar_try(smem_u32(drain), 0) && oz::globaltimer() - t0 < H_DRAIN_NS) {
       }
     } else if (warp == 13 && lane == 0) {
       // ------------------------------------------------------------ copies of X
@@ -447,7 +451,7 @@ __global__ void __launch_bounds__(HEMV_THREADS, 1) hemv_kernel(int64_t n, const 
       int issued = 0;
       for (; issued < nblk; ++issued) {
         const int st = issued % H_XSTAGES;
-        if (!hemv_wait(smem_u32(&xempty[st]), ((issued / H_XSTAGES) & 1) ^ 1, gave_up)) break;
+        if (!hemv_wait(smem_u32(&xempty[st]), ((issued / H_XSTAGES) & 1) ^ 1, gave_up, wait_ns)) break;
         oz::mbar_expect_tx(smem_u32(&xfull[st]), H::X_BYTES);
         asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                          smem_u32(smem + st * H::X_BYTES)),
@@ -457,7 +461,7 @@ __global__ void __launch_bounds__(HEMV_THREADS, 1) hemv_kernel(int64_t n, const 
       // the copies in flight land before the CTA exits
       for (int i = issued > H_XSTAGES ? issued - H_XSTAGES : 0; i < issued; ++i) {
         const unsigned long long t0 = oz::globaltimer();
-        while (!oz::mbar_try(smem_u32(&xfull[i % H_XSTAGES]), (i / H_XSTAGES) & 1) && oz::globaltimer() - t0 < H_TIMEOUT_NS) {
+        while (!oz::mbar_try(smem_u32(&xfull[i % H_XSTAGES]), (i / H_XSTAGES) & 1) && oz::globaltimer() - t0 < H_DRAIN_NS) {
         }
       }
     }
@@ -466,6 +470,7 @@ __global__ void __launch_bounds__(HEMV_THREADS, 1) hemv_kernel(int64_t n, const 
   oz::fence_before();
   __syncthreads();
   oz::fence_after();
+  if (threadIdx.x == 0 && *gave_up) atomicOr(status, LZ_STATUS_WAIT);
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
 }
 
@@ -690,7 +695,7 @@ __device__ __noinline__ void ql_first_row(int k, double* d, double* e, double* z
       const int mm = min(k - 1, lo ? __ffs((int)lo) - 1 : 31 + __ffs((int)hi));
       if (mm == l) break;
       if (iter == 60) {
-        if (lane == 0) atomicMax(status, 1);
+        if (lane == 0) atomicOr(status, LZ_STATUS_QL);
         break;
       }
       if (lane == 0) {
@@ -918,27 +923,35 @@ __global__ void __launch_bounds__(TRI_THREADS) tridiag_kernel(int steps, const d
   }
   __syncthreads();
   const int sc = sc_sh;
-  // ascending (stable) order
+  // ascending (stable) order; a T that is not finite has no order and gives NaN throughout
   for (int i = tid; i < k; i += TRI_THREADS) {
     const double wi = d[i];
     int rank = 0;
-    for (int q = 0; q < k; ++q) rank += (d[q] < wi) || (d[q] == wi && q < i);
-    theta[r * LZ_MAXS + rank] = ldexp(wi, sc);
-    tau2[r * LZ_MAXS + rank] = z[i] * z[i];
+    bool bad = false;
+    for (int q = 0; q < k; ++q) {
+      rank += (d[q] < wi) || (d[q] == wi && q < i);
+      bad |= !isfinite(d[q]) || !isfinite(z[q]);
+    }
+    theta[r * LZ_MAXS + (bad ? i : rank)] = bad ? NAN : ldexp(wi, sc);
+    tau2[r * LZ_MAXS + (bad ? i : rank)] = bad ? NAN : z[i] * z[i];
   }
 }
 
 // b_sup, mu_1, mu_ne (DoS quantile), theta_max: the pooled Ritz values ranked in parallel, their weights added in
-// ascending order by one thread.
+// ascending order by one thread.  All four are NaN when any of the values is not finite (fmax and fmin would drop it); the
+// status word follows them.
 __global__ void lanczos_bounds_kernel(int runs, int steps, int64_t n, int ne, const double* theta, const double* tau2,
-                                      const double* beta, double* out4) {
+                                      const double* beta, const int* status, double* out5) {
   __shared__ double th[LZ_MAXR * LZ_MAXS], so[LZ_MAXR * LZ_MAXS], wt[LZ_MAXR * LZ_MAXS];
   const int total = runs * steps;
+  bool bad = false;
   for (int i = threadIdx.x; i < total; i += blockDim.x) {
-    th[i] = theta[(i / steps) * LZ_MAXS + i % steps];
+    const int at = (i / steps) * LZ_MAXS + i % steps;
+    th[i] = theta[at];
     so[i] = wt[i] = 0.0;
+    bad |= !isfinite(th[i]) || !isfinite(tau2[at]) || !isfinite(beta[at]);
   }
-  __syncthreads();
+  bad = __syncthreads_or(bad);
   for (int i = threadIdx.x; i < total; i += blockDim.x) {
     const double t = th[i];
     int rank = 0;
@@ -964,10 +977,11 @@ __global__ void lanczos_bounds_kernel(int runs, int steps, int64_t n, int ne, co
   double span = b_sup - mu1;
   double lo = mu1 + 1e-3 * span, hi = b_sup - 1e-3 * span;
   mu_ne = fmin(fmax(mu_ne, lo), hi);
-  out4[0] = b_sup;
-  out4[1] = mu1;
-  out4[2] = mu_ne;
-  out4[3] = tmax;
+  out5[0] = bad ? NAN : b_sup;
+  out5[1] = bad ? NAN : mu1;
+  out5[2] = bad ? NAN : mu_ne;
+  out5[3] = bad ? NAN : tmax;
+  out5[4] = *status;
 }
 
 // CTAs per run: 16 where the device schedules such clusters and the vectors are long, else 8
@@ -1009,7 +1023,7 @@ template <typename T> static void lanczos_attributes() {
 
 template <typename T>
 void lanczos(cudaStream_t st, const T* A, int64_t n, int64_t lda, int ne, const T* L0, int runs, int steps,
-             double* out4, T* work, int64_t work_elems, double* dwork) {
+             double* out5, T* work, int64_t work_elems, double* dwork) {
   CHASE_REQUIRE(runs >= 1 && runs <= LZ_MAXR, 1, "lanczos: 1 <= runs <= 8");
   CHASE_REQUIRE(steps >= 1 && steps <= LZ_MAXS && steps <= n, 1, "lanczos: 1 <= steps <= min(64, n)");
   const int cols = hemv_cols(n);
@@ -1056,14 +1070,20 @@ void lanczos(cudaStream_t st, const T* A, int64_t n, int64_t lda, int ne, const 
   step(-1);
   const dim3 g1(ceil_div(n, HEMV_ROWS), nchunk, ceil_div(runs, Frag<T>::RUNS));
   for (int j = 0; j < steps; ++j) {
-    launch_pdl(hemv_kernel<T>, g1, HEMV_THREADS, Hemv<T>::SMEM, st, n, A, lda, rmax, X, xe, cols, runs, part);
+    launch_pdl(hemv_kernel<T>, g1, HEMV_THREADS, Hemv<T>::SMEM, st, n, A, lda, rmax, X, xe, cols, runs, part,
+               grid_wait_limit_ns(), status);
     CHASE_CHECK_LAUNCH();
     step(j);
   }
   tridiag_kernel<<<runs, TRI_THREADS, 4 * steps * (steps + 1) * (int)sizeof(double), st>>>(steps, alpha, beta, theta, tau2, status);
   CHASE_CHECK_LAUNCH();
-  lanczos_bounds_kernel<<<1, 256, 0, st>>>(runs, steps, n, ne, theta, tau2, beta, out4);
+  lanczos_bounds_kernel<<<1, 256, 0, st>>>(runs, steps, n, ne, theta, tau2, beta, status, out5);
   CHASE_CHECK_LAUNCH();
+}
+
+void check_lanczos(const double (&out5)[5]) {
+  CHASE_REQUIRE(((int)out5[4] & LZ_STATUS_WAIT) == 0, 8, "a Lanczos product hit its wait limit");
+  for (int i = 0; i < 4; ++i) CHASE_REQUIRE(std::isfinite(out5[i]), 5, "non-finite Lanczos bounds");
 }
 
 template void lanczos<double>(cudaStream_t, const double*, int64_t, int64_t, int, const double*, int, int, double*,
