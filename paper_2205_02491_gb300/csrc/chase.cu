@@ -913,7 +913,8 @@ template <typename T> struct Solver {
     // Lanczos (line 2)
     {
       Timer t(c, 1, &S.ms_lanczos);
-      lanczos<T>(st(), A, n, lda, ne, L0, runs, steps, c->dwork, W(), c->work_elems, c->dwork + 8);
+      lanczos<T>(st(), A, n, lda, ne, L0, runs, steps, c->dwork, W(), c->work_elems, c->dwork + 8,
+                 mode == CHASE_FP64_NATIVE);
       init_bounds_kernel<<<1, 1, 0, st()>>>(c->dwork, c->bounds);
       CHASE_CHECK_LAUNCH();
       t.stop();
@@ -1430,10 +1431,10 @@ chase_status chase_lanczos(chase_ctx* c, const void* A, int64_t n, int64_t lda, 
   CHASE_REQUIRE(runs >= 1 && runs <= 8 && steps >= 1 && steps <= 64 && steps <= n, CHASE_ERR_ARG, "bad runs/steps");
   if (c->dtype == CHASE_C128)
     lanczos<double2>(c->stream, (const double2*)A, n, lda, ne, (const double2*)L0, runs, steps, c->dwork,
-                     (double2*)c->work, c->work_elems, c->dwork + 8);
+                     (double2*)c->work, c->work_elems, c->dwork + 8, false);
   else
     lanczos<double>(c->stream, (const double*)A, n, lda, ne, (const double*)L0, runs, steps, c->dwork,
-                    (double*)c->work, c->work_elems, c->dwork + 8);
+                    (double*)c->work, c->work_elems, c->dwork + 8, false);
   double hb[5];
   CHASE_CUDA(cudaMemcpyAsync(hb, c->dwork, sizeof(hb), cudaMemcpyDeviceToHost, c->stream));
   CHASE_CUDA(cudaStreamSynchronize(c->stream));

@@ -101,12 +101,12 @@ void sort_pairs(cudaStream_t st, int k, double* w, const T* Z, int64_t ldz, T* o
                 int* perm);
 
 // Lanczos bounds (Algorithm 1, line 2).  out5 (device) = {b_sup, mu_1, mu_ne, theta_max, status}; check_lanczos, on a host
-// copy of it, throws for a wait that ran out and for bounds that are not finite.
+// copy of it, throws for a wait that ran out and for bounds that are not finite.  native: FP64 multiply-adds only.
 // work: at least lanczos_work_elems scalars (monotone in n).
 int64_t lanczos_work_elems(int64_t n, int runs, int steps, bool cplx);
 template <typename T>
 void lanczos(cudaStream_t st, const T* A, int64_t n, int64_t lda, int ne, const T* L0, int runs, int steps,
-             double* out5, T* work, int64_t work_elems, double* dwork);
+             double* out5, T* work, int64_t work_elems, double* dwork, bool native);
 void check_lanczos(const double (&out5)[5]);
 
 // Input generator from compact-WY factors.

@@ -1,7 +1,7 @@
 // Lanczos spectral-bound estimation (Algorithm 1, line 2) on the device.
 //
-// All runs advance together, two launches per step: the product of A with one vector per run (hemv_kernel, A
-// streamed once per step), and the rest of the step (lanczos_step_kernel, one cluster of CTAs per run): three-term
+// All runs advance together, two launches per step: the product of A with one vector per run (hemv_kernel, or
+// hemv_dfma_kernel in the native mode; A streamed once per step), and the rest of the step (lanczos_step_kernel, one cluster of CTAs per run): three-term
 // update, one classical Gram-Schmidt reorthogonalisation against the run's basis, normalisation.  The tridiagonal T
 // of each run is diagonalised by one block per run, and one block computes b_sup = max(theta_max + |beta_last|),
 // mu_1 = min theta_min, theta_max and the density-of-states quantile mu_ne = smallest pooled Ritz value whose
@@ -472,6 +472,57 @@ __global__ void __launch_bounds__(HEMV_THREADS, 1) hemv_kernel(int64_t n, const 
   oz::fence_after();
   if (threadIdx.x == 0 && *gave_up) atomicOr(status, LZ_STATUS_WAIT);
   if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem));
+}
+
+// The same by FP64 multiply-adds on the full entries, for the native mode, whose results rest on plain FP64 arithmetic only:
+// R real or complex vectors (X, ld ldx), one row per thread, X staged 128 columns at a time.  The FP64 rate bounds it: complex,
+// n = 8192, 4 runs: 1.8 ms a step.
+constexpr int DFMA_ROWS = 64, DFMA_COLS = 128;
+template <typename T, int R>
+__global__ void __launch_bounds__(DFMA_ROWS) hemv_dfma_kernel(int64_t n, const T* __restrict__ A, int64_t lda,
+                                                               const T* __restrict__ X, int64_t ldx, int cols, T* part) {
+  grid_dependency_wait();
+  using s = S<T>;
+  __shared__ T xs[DFMA_COLS][R];
+  const int64_t i = (int64_t)blockIdx.x * DFMA_ROWS + threadIdx.x;
+  const int64_t jbeg = (int64_t)blockIdx.y * cols, jend = jbeg + cols < n ? jbeg + cols : n;
+  T acc[R];
+#pragma unroll
+  for (int r = 0; r < R; ++r) acc[r] = s::zero();
+  for (int64_t j0 = jbeg; j0 < jend; j0 += DFMA_COLS) {
+    const int nj = (int)(jend - j0 < DFMA_COLS ? jend - j0 : DFMA_COLS);
+    __syncthreads();
+    for (int t = threadIdx.x; t < DFMA_COLS * R; t += DFMA_ROWS)
+      xs[t / R][t % R] = t / R < nj ? X[j0 + t / R + (t % R) * ldx] : s::zero();
+    __syncthreads();
+    if (i >= n) continue;
+    const T* a = A + i + j0 * lda;
+    constexpr int B = 16 / (int)(sizeof(T) / 8);  // loads in flight
+    for (int j = 0; j < nj; j += B) {
+      T v[B];
+#pragma unroll
+      for (int b = 0; b < B; ++b) v[b] = j + b < nj ? a[(j + b) * lda] : s::zero();
+#pragma unroll
+      for (int b = 0; b < B; ++b)
+#pragma unroll
+        for (int r = 0; r < R; ++r) acc[r] = s::fma(v[b], xs[j + b][r], acc[r]);
+    }
+  }
+  if (i >= n) return;
+#pragma unroll
+  for (int r = 0; r < R; ++r) part[((int64_t)blockIdx.y * R + r) * n + i] = acc[r];
+}
+
+template <typename T>
+static void hemv_dfma(cudaStream_t st, int64_t n, const T* A, int64_t lda, const T* X, int64_t ldx, int cols, int runs, T* part) {
+  const dim3 grid(ceil_div(n, DFMA_ROWS), ceil_div(n, cols));
+  switch (runs) {
+#define CASE(R) \
+  case R: launch_pdl(hemv_dfma_kernel<T, R>, grid, DFMA_ROWS, 0, st, n, A, lda, X, ldx, cols, part); break;
+    CASE(1) CASE(2) CASE(3) CASE(4) CASE(5) CASE(6) CASE(7) CASE(8)
+#undef CASE
+  }
+  CHASE_CHECK_LAUNCH();
 }
 
 // Columns per hemv block (a multiple of 64): row blocks times column chunks in full waves of one block per SM, a block
@@ -1023,7 +1074,7 @@ template <typename T> static void lanczos_attributes() {
 
 template <typename T>
 void lanczos(cudaStream_t st, const T* A, int64_t n, int64_t lda, int ne, const T* L0, int runs, int steps,
-             double* out5, T* work, int64_t work_elems, double* dwork) {
+             double* out5, T* work, int64_t work_elems, double* dwork, bool native) {
   CHASE_REQUIRE(runs >= 1 && runs <= LZ_MAXR, 1, "lanczos: 1 <= runs <= 8");
   CHASE_REQUIRE(steps >= 1 && steps <= LZ_MAXS && steps <= n, 1, "lanczos: 1 <= steps <= min(64, n)");
   const int cols = hemv_cols(n);
@@ -1047,8 +1098,10 @@ void lanczos(cudaStream_t st, const T* A, int64_t n, int64_t lda, int ne, const 
   // unused vector columns and rows past n are zero digits
   CHASE_CUDA(cudaMemsetAsync(X, 0, xhalves * sizeof(__half), st));
   CHASE_CUDA(cudaMemsetAsync(rmax, 0, n * sizeof(unsigned), st));
-  row_max_kernel<T><<<dim3(ceil_div(n, 128), ceil_div(n, ROWMAX_COLS)), 128, 0, st>>>(n, A, lda, rmax);
-  CHASE_CHECK_LAUNCH();
+  if (!native) {
+    row_max_kernel<T><<<dim3(ceil_div(n, 128), ceil_div(n, ROWMAX_COLS)), 128, 0, st>>>(n, A, lda, rmax);
+    CHASE_CHECK_LAUNCH();
+  }
 
   cudaLaunchConfig_t cfg{};
   cudaLaunchAttribute at[2] = {{}, pdl_attribute()};
@@ -1070,9 +1123,13 @@ void lanczos(cudaStream_t st, const T* A, int64_t n, int64_t lda, int ne, const 
   step(-1);
   const dim3 g1(ceil_div(n, HEMV_ROWS), nchunk, ceil_div(runs, Frag<T>::RUNS));
   for (int j = 0; j < steps; ++j) {
-    launch_pdl(hemv_kernel<T>, g1, HEMV_THREADS, Hemv<T>::SMEM, st, n, A, lda, rmax, X, xe, cols, runs, part,
-               grid_wait_limit_ns(), status);
-    CHASE_CHECK_LAUNCH();
+    if (native) {
+      hemv_dfma<T>(st, n, A, lda, Vb + (int64_t)j * n, n * steps, cols, runs, part);
+    } else {
+      launch_pdl(hemv_kernel<T>, g1, HEMV_THREADS, Hemv<T>::SMEM, st, n, A, lda, rmax, X, xe, cols, runs, part,
+                 grid_wait_limit_ns(), status);
+      CHASE_CHECK_LAUNCH();
+    }
     step(j);
   }
   tridiag_kernel<<<runs, TRI_THREADS, 4 * steps * (steps + 1) * (int)sizeof(double), st>>>(steps, alpha, beta, theta, tau2, status);
@@ -1087,8 +1144,8 @@ void check_lanczos(const double (&out5)[5]) {
 }
 
 template void lanczos<double>(cudaStream_t, const double*, int64_t, int64_t, int, const double*, int, int, double*,
-                              double*, int64_t, double*);
+                              double*, int64_t, double*, bool);
 template void lanczos<double2>(cudaStream_t, const double2*, int64_t, int64_t, int, const double2*, int, int, double*,
-                               double2*, int64_t, double*);
+                               double2*, int64_t, double*, bool);
 
 }  // namespace chase

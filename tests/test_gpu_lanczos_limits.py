@@ -80,3 +80,23 @@ def test_sweep_wait_limit(pkg):
         pkg.set_wait_limit_ns(0)
     w, _ = s.rayleigh_ritz(A, Q.clone())
     assert np.all(np.isfinite(w))
+
+
+@pytest.mark.parametrize("cplx", [True, False])
+@pytest.mark.parametrize("n,runs", [(63, 1), (129, 3), (700, 4), (1300, 8)])
+def test_native_mode_rests_on_no_tensor_core_product(pkg, cplx, n, runs):
+    """The native mode is the reference for the others: with every wait of the product kernel run out it still solves."""
+    p = G.problem_small(n, 8, 6, complex_=cplx, seed_pid=11)
+    s = pkg.Chase(n, p.ne, complex_=cplx, opts={"lanczos_runs": runs})
+    L0 = G.gaussian(np.random.default_rng(n), (n, runs), cplx)
+    A, V0, L0 = dev(p.dense()), dev(p.V0), dev(L0)
+    ref = s.lanczos(A, p.ne, L0, runs, 25)
+    pkg.set_wait_limit_ns(1)
+    try:
+        w, _ = s.solve(A, p.nev, p.nex, p.tol, p.deg, "fp64_native", V0, L0)
+    finally:
+        pkg.set_wait_limit_ns(0)
+    st = s.stats()
+    assert np.max(np.abs(w.cpu().numpy() - p.lam[:p.nev])) <= 1e-10 * p.norm2()
+    for key in ("b_sup", "mu_1"):
+        assert abs(st[key] - ref[key]) <= 1e-10 * p.norm2(), key
