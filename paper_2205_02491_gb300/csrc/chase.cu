@@ -1177,11 +1177,10 @@ void chase_default_opts(chase_opts* o) {
 static int64_t work_elems_for(int64_t n, int ne, bool cplx, const chase_opts& o) {
   // FP64 Jacobi: ne^2 + 3 ne + 8 scalars; FP32 first pass: 3 ne^2 + 3 ne + 8 half-size scalars
   int64_t jac = 2 * (int64_t)ne * ne + 3 * (int64_t)ne + 16;
-  // the context's own Lanczos settings, and any settings chase_lanczos takes for small n
-  int64_t lz = std::max(lanczos_work_elems(n, o.lanczos_runs, std::min<int>(o.lanczos_steps, (int)n), cplx),
-                        lanczos_work_elems(std::min<int64_t>(n, 4096), 8, 64, cplx));
+  // chase_lanczos takes other runs and steps than the context's, and smaller n, as far as their scalars go
+  int64_t lz = lanczos_quota(n, o.lanczos_runs, std::min<int>(o.lanczos_steps, (int)n));
   int64_t split = 2 * 1024 * 1024;
-  return std::max(std::max(jac, lz), split);
+  return lanczos_context_elems(n, std::max(std::max(jac, lz), split), cplx);
 }
 
 int64_t chase_workspace_bytes(int64_t n_max, int ne_max, chase_dtype dtype, const chase_opts* opts) {

@@ -104,6 +104,10 @@ void sort_pairs(cudaStream_t st, int k, double* w, const T* Z, int64_t ldz, T* o
 // copy of it, throws for a wait that ran out and for bounds that are not finite.  native: FP64 multiply-adds only.
 // work: at least lanczos_work_elems scalars (monotone in n).
 int64_t lanczos_work_elems(int64_t n, int runs, int steps, bool cplx);
+// The scalars a call counts against a context's quota: runs vectors, their bases and n rows per 256 columns.  A work area of
+// lanczos_context_elems(n_max, quota) holds every call of at most that count with n <= n_max.
+inline int64_t lanczos_quota(int64_t n, int runs, int steps) { return runs * n * (steps + 1 + (n + 255) / 256); }
+int64_t lanczos_context_elems(int64_t n_max, int64_t quota, bool cplx);
 template <typename T>
 void lanczos(cudaStream_t st, const T* A, int64_t n, int64_t lda, int ne, const T* L0, int runs, int steps,
              double* out5, T* work, int64_t work_elems, double* dwork, bool native);

@@ -546,11 +546,20 @@ static int hemv_cols(int64_t n) {
 // columns.
 static int64_t hemv_part_rows(int64_t n) { return std::max<int64_t>(608 * HEMV_ROWS, n * (n / 4096 + 1)); }
 
-int64_t lanczos_work_elems(int64_t n, int runs, int steps, bool cplx) {
-  // basis | W | hemv partial sums | vector fragments | row maxima | exponents
+// vector fragments, row maxima, exponents
+static int64_t operand_elems(int64_t n, int runs, bool cplx) {
   const int64_t scal = cplx ? 16 : 8;
-  const int64_t extra = (frag_halves(n, cplx, runs) * 2 + n * 4 + 512 + scal - 1) / scal;
-  return (int64_t)runs * steps * n + runs * n + runs * hemv_part_rows(n) + extra + 16;
+  return (frag_halves(n, cplx, runs) * 2 + n * 4 + 512 + scal - 1) / scal + 16;
+}
+
+int64_t lanczos_work_elems(int64_t n, int runs, int steps, bool cplx) {
+  // basis | W | hemv partial sums | operands
+  return (int64_t)runs * steps * n + runs * n + runs * hemv_part_rows(n) + operand_elems(n, runs, cplx);
+}
+
+int64_t lanczos_context_elems(int64_t n, int64_t quota, bool cplx) {
+  // the partial sums of n below 4464 take more than n rows per 256 columns, by 608 blocks' rows at most
+  return quota + LZ_MAXR * 608ll * HEMV_ROWS + operand_elems(n, LZ_MAXR, cplx);
 }
 
 // ---------------------------------------------------------------- one step of every run

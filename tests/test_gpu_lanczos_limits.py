@@ -100,3 +100,19 @@ def test_native_mode_rests_on_no_tensor_core_product(pkg, cplx, n, runs):
     assert np.max(np.abs(w.cpu().numpy() - p.lam[:p.nev])) <= 1e-10 * p.norm2()
     for key in ("b_sup", "mu_1"):
         assert abs(st[key] - ref[key]) <= 1e-10 * p.norm2(), key
+
+
+@pytest.mark.parametrize("n_max,n,runs,steps", [(16000, 8000, 8, 40), (20000, 20000, 2, 64), (20000, 300, 8, 64)])
+def test_settings_other_than_the_contexts(pkg, n_max, n, runs, steps):
+    """A context made for 4 runs of 25 steps also takes more steps of fewer runs, or more of both at a smaller n."""
+    import torch
+    gen = torch.Generator(device="cuda").manual_seed(n)
+    X = torch.randn((n, n), generator=gen, device="cuda", dtype=torch.float64)
+    A = X.add_(X.mT.clone()).mul_(0.5)
+    L0 = torch.randn((runs, n), generator=gen, device="cuda", dtype=torch.float64)
+    s = pkg.Chase(n_max, 8, complex_=False)
+    out = s.lanczos(A, 8, L0, runs, steps)
+    s.close()
+    s = pkg.Chase(n, 8, complex_=False, opts={"lanczos_runs": runs, "lanczos_steps": steps})
+    assert s.lanczos(A, 8, L0, runs, steps) == out
+    s.close()
