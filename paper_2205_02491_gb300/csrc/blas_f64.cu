@@ -454,12 +454,11 @@ void chol_stack_columns(cudaStream_t st, int k, int jbeg, int jend, T* Sm, int64
 }
 
 // ============================================================== corrections of nearly orthonormal blocks
-// From the Gram matrix Gm = I + E of a block Q: the factor F with Q F closer to orthonormal by the square of E.
-// upper: F = I - striu(E) - diag(E)/2, which keeps the span of every leading set of columns (the QR's factor);
-// else F = I - E/2, the nearest orthonormal block.  dev = max over columns of sum_i |E_ij| (as float bits; NaN stays
+// From the Gram matrix Gm = I + E of a block Q: the factor F = I - striu(E) - diag(E)/2, which takes Q closer to
+// orthonormal by the square of E and keeps the span of every leading set of columns (the QR's factor).  dev = max over columns of sum_i |E_ij| (as float bits; NaN stays
 // largest), an upper bound of ||E||_2 for the caller's decision.
 template <typename T>
-__global__ void __launch_bounds__(128) gram_correction_kernel(int k, int upper, const T* __restrict__ Gm, int64_t ldg, T* F,
+__global__ void __launch_bounds__(128) gram_correction_kernel(int k, const T* __restrict__ Gm, int64_t ldg, T* F,
                                                                int64_t ldf, unsigned* dev) {
   grid_dependency_wait();
   using s = S<T>;
@@ -470,8 +469,8 @@ __global__ void __launch_bounds__(128) gram_correction_kernel(int k, int upper, 
     T e = s::scale(s::add(a, b), 0.5);
     if (i == j) e = s::make(s::re(e) - 1.0, 0.0);
     sum += fabsf((float)s::re(e)) + fabsf((float)s::im(e));
-    T f = (upper && i < j) ? s::scale(e, -1.0) : ((upper && i > j) ? s::zero() : s::scale(e, -0.5));
-    if (i == j) f = s::add(f, s::one());
+    T f = i < j ? s::scale(e, -1.0) : s::zero();
+    if (i == j) f = s::add(s::scale(e, -0.5), s::one());
     F[i + (int64_t)j * ldf] = f;
   }
 #pragma unroll
@@ -486,8 +485,8 @@ __global__ void __launch_bounds__(128) gram_correction_kernel(int k, int upper, 
 }
 
 template <typename T>
-void gram_correction(cudaStream_t st, int k, bool upper, const T* Gm, int64_t ldg, T* F, int64_t ldf, unsigned* dev) {
-  launch_pdl(gram_correction_kernel<T>, k, 128, 0, st, k, upper ? 1 : 0, Gm, ldg, F, ldf, dev);
+void gram_correction(cudaStream_t st, int k, const T* Gm, int64_t ldg, T* F, int64_t ldf, unsigned* dev) {
+  launch_pdl(gram_correction_kernel<T>, k, 128, 0, st, k, Gm, ldg, F, ldf, dev);
   CHASE_CHECK_LAUNCH();
 }
 
@@ -731,7 +730,7 @@ template <typename T> void fill_normal(cudaStream_t st, T* X, int64_t rows, int 
   template void hermitianize<T>(cudaStream_t, int, T*, int64_t);                                                  \
   template void chol_stack_begin<T>(cudaStream_t, int, T*, int64_t);                                             \
   template void chol_stack_columns<T>(cudaStream_t, int, int, int, T*, int64_t, int*, double, int*);             \
-  template void gram_correction<T>(cudaStream_t, int, bool, const T*, int64_t, T*, int64_t, unsigned*);          \
+  template void gram_correction<T>(cudaStream_t, int, const T*, int64_t, T*, int64_t, unsigned*);                \
   template void householder_vec<T>(cudaStream_t, int64_t, T*, T*, double*);                                      \
   template void householder_apply<T>(cudaStream_t, int64_t, const T*, T*, int64_t, int, const double*);            \
   template void reflector_panel<T>(cudaStream_t, int64_t, int, const T*, int64_t, T*, int64_t);                   \

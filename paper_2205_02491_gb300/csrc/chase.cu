@@ -290,10 +290,10 @@ template <typename T> struct Solver {
   }
 
   // Bound of ||G - I||_2 for the Gram matrix in Gb() (ld k); the correction factor goes to Zb() (ld k).
-  double correction(int k, bool upper) {
+  double correction(int k) {
     unsigned* dev = reinterpret_cast<unsigned*>(c->info);
     CHASE_CUDA(cudaMemsetAsync(dev, 0, sizeof(unsigned), st()));
-    gram_correction<T>(st(), k, upper, Gb(), k, Zb(), k, dev);
+    gram_correction<T>(st(), k, Gb(), k, Zb(), k, dev);
     float d = 0.f;
     CHASE_CUDA(cudaMemcpyAsync(&d, dev, sizeof(float), cudaMemcpyDeviceToHost, st()));
     CHASE_CUDA(cudaStreamSynchronize(st()));
@@ -316,7 +316,7 @@ template <typename T> struct Solver {
       double d = -1.0;
       if (factored) {
         gram(Ys, n, n, k, k, CHASE_FP64);
-        d = correction(k, true);
+        d = correction(k);
       }
       const T* F = Zb();
       int64_t ldf = k;
@@ -537,7 +537,7 @@ template <typename T> struct Solver {
       for (int pass = 0; pass < 8; ++pass) {
         project();
         gram(X, ldx, n, k, k, pm);
-        const double d = correction(k, true);
+        const double d = correction(k);
         if (d < CORRECT_MAX) apply_right(X, ldx, n, k, Zb(), k, pm);
         else if (!chol_pass(0.0)) return false;
         if (d <= CORRECT_LAST) return true;
@@ -578,10 +578,10 @@ template <typename T> struct Solver {
   }
 
   // ------------------------------------------------------------ Rayleigh-Ritz eigensolve
-  // Eigenpairs of the Hermitian G = Gb() (k x k): FP32 parallel Jacobi, two first-order refinement
-  // steps in FP64-class products, exact FP64 Jacobi on clusters closer than omega.  Ascending
+  // Eigenpairs of the Hermitian G = Gb() (k x k): FP32 parallel Jacobi, corrections in FP64-class products until they
+  // have converged (eig_mixed.cu), exact FP64 Jacobi on clusters of close eigenvalues.  Ascending
   // eigenvalues to w (device), eigenvectors to Zb().  scratch: 3 k*k scalars.  Returns false when a
-  // step cannot be completed (the caller then uses the FP64 Jacobi solver).
+  // step cannot be completed or the corrections do not converge (the caller then uses the FP64 Jacobi solver).
   // verbose-mode probe: report non-finite entries of a device block
   void dbg_finite(const void* X, int64_t rows, int cols, int64_t ld, size_t esz, const char* what) {
     if (!verbose()) return;
@@ -601,7 +601,6 @@ template <typename T> struct Solver {
     using F = typename Lowp<T>::type;
     T* G = Gb();
     T* Z = Zb();
-    T *X2 = scratch, *Gp = scratch + (size_t)k * k, *X = scratch + 2 * (size_t)k * k;
     F* Gf = (F*)W();
     F* Zf = Gf + (size_t)k * k;
     F* jw = Zf + (size_t)k * k;
@@ -637,72 +636,103 @@ template <typename T> struct Solver {
     c->stats.rr_sweeps += block_sweeps;
     const double scale = std::max(std::fabs(ends[0]), std::fabs(ends[1]));
     if (!(scale > 0.0) || !std::isfinite(scale)) return false;
-    const double omega = 1e-5 * scale;
-    // three first-order corrections: the FP32 pass stops at its rounding floor (up to about 1e-4 relative
-    // off-diagonal norm for large k), which quadratic convergence takes to FP64 level in three steps.  Before each,
-    // Z (I - E/2) with Z^H Z = I + E brings Z back to orthonormality up to E^2: E is the FP32 rounding (1e-5) at
-    // first and the squared correction later, so the last pass leaves rounding level.
-    unsigned* dev = reinterpret_cast<unsigned*>(c->info);
-    CHASE_CUDA(cudaMemsetAsync(dev, 0, sizeof(unsigned), st()));
-    T* Zn = X2;
-    for (int it = 0; it < 4; ++it) {
-      Epi eg;
-      eg.C = Gp;
-      eg.ldc = k;
-      gemm(OP_C, Z, k, OP_N, Z, k, k, k, k, eg, CHASE_FP64);
-      gram_correction<T>(st(), k, false, Gp, k, X, k, dev);
-      Epi ez;
-      ez.C = Zn;
-      ez.ldc = k;
-      gemm(OP_N, Z, k, OP_N, X, k, k, k, k, ez, CHASE_FP64);
-      Epi e1;
-      e1.C = Z;
-      e1.ldc = k;
-      gemm(OP_N, G, k, OP_N, Zn, k, k, k, k, e1, CHASE_FP64);  // G Z (over the block before)
-      Epi e2;
-      e2.C = Gp;
-      e2.ldc = k;
-      gemm(OP_C, Zn, k, OP_N, Z, k, k, k, k, e2, CHASE_FP64);  // G' = Z^H G Z
-      hermitianize<T>(st(), k, Gp, k);
-      dbg_finite(Gp, k, k, k, sizeof(T), "G' in the refinement");
-      if (it == 3) break;
-      eig_correction<T>(st(), k, Gp, k, X, k, omega);
-      Epi e3;
-      e3.C = Z;
-      e3.ldc = k;
-      e3.Y = Zn;
-      e3.ldy = k;
-      e3.gamma = 1.0;
-      gemm(OP_N, Zn, k, OP_N, X, k, k, k, k, e3, CHASE_FP64);  // Z (I + X)
-    }
-    // a block too far from orthonormal for the corrections (or not finite) is left to the FP64 solver
-    float far = 0.f;
-    CHASE_CUDA(cudaMemcpyAsync(&far, dev, sizeof(float), cudaMemcpyDeviceToHost, st()));
-    // eigenvalues: diagonal of G', clusters solved exactly
-    diag_real<T>(st(), k, Gp, k, w);
+    // Z and one of the scratch blocks take turns as the current vectors; the Gram matrix N lies in the other
+    T *Zc = Z, *N = scratch, *Wk = scratch + (size_t)k * k, *Sq = scratch + 2 * (size_t)k * k;
+    unsigned* emax = reinterpret_cast<unsigned*>(c->status_dev + 2);
+    int *cl_dev = c->iwork, *id_dev = c->iwork + k;
     std::vector<double> d(k);
-    CHASE_CUDA(cudaMemcpyAsync(d.data(), w, k * sizeof(double), cudaMemcpyDeviceToHost, st()));
-    CHASE_CUDA(cudaStreamSynchronize(st()));
-    if (!(far < CORRECT_MAX)) return false;
-    std::vector<int> cl;
-    for (int i = 0; i < k;) {
-      int j = i + 1;
-      while (j < k && std::fabs(d[j] - d[j - 1]) <= omega) ++j;
-      if (j - i > 1) {
-        if (j - i > 32) return false;
-        cl.push_back(i);
-        cl.push_back(j - i);
+    std::vector<int> cl, id(k);
+    // Clusters: runs of eigenvalues each within `gap` of the next.  A run of more than `longest` is cut at `narrow`
+    // instead; false when that leaves more than CLUSTER_MAX together.
+    auto clusters = [&](double gap, int longest, double narrow) {
+      CHASE_CUDA(cudaMemcpyAsync(d.data(), w, k * sizeof(double), cudaMemcpyDeviceToHost, st()));
+      CHASE_CUDA(cudaStreamSynchronize(st()));
+      cl.clear();
+      auto run_end = [&](int i, int end, double within) {
+        int j = i + 1;
+        while (j < end && std::fabs(d[j] - d[j - 1]) <= within) ++j;
+        return j;
+      };
+      auto add = [&](int i, int j) {
+        if (j - i > 1) {
+          cl.push_back(i);
+          cl.push_back(j - i);
+        }
+        std::fill(id.begin() + i, id.begin() + j, i);
+        return j - i <= CLUSTER_MAX;
+      };
+      for (int i = 0; i < k;) {
+        const int end = run_end(i, k, gap);
+        if (end - i <= longest) {
+          if (!add(i, end)) return false;
+        } else {
+          for (int a = i; a < end;) {
+            const int b = run_end(a, end, narrow);
+            if (!add(a, b)) return false;
+            a = b;
+          }
+        }
+        i = end;
       }
-      i = j;
+      CHASE_CUDA(cudaMemcpyAsync(id_dev, id.data(), k * sizeof(int), cudaMemcpyHostToDevice, st()));
+      if (!cl.empty()) CHASE_CUDA(cudaMemcpyAsync(cl_dev, cl.data(), cl.size() * sizeof(int), cudaMemcpyHostToDevice, st()));
+      return true;
+    };
+    auto solve_clusters = [&]() {
+      cluster_eig<T>(st(), k, (int)cl.size() / 2, cl_dev, Sq, Wk, Zc, k, w, c->status_dev);
+    };
+    CHASE_CUDA(cudaMemsetAsync(c->status_dev, 0, sizeof(int), st()));
+    // The FP32 pass stops with entries of 1e-7 to 1e-5 of the norm off the diagonal.  Pairs closer than OMEGA are too close
+    // for corrections and end as clusters.  The first correction treats runs of up to WIDE_MAX within OMEGA_WIDE as clusters
+    // too, so that every E is well below 1 and a cluster's own entries do not slow down the others' convergence.
+    // Quadratic from then on: three passes where no gap is near the line, up to six for groups just outside it; E <= 1e-8
+    // leaves rounding level.  Four k x k products a pass (N, G Z, S, Z E).
+    const double OMEGA = 1e-5 * scale, OMEGA_WIDE = 3e-5 * scale;
+    constexpr int WIDE_MAX = 8, MAX_PASSES = 8;
+    bool done = false;
+    for (int it = 0; it < MAX_PASSES && !done; ++it) {
+      Epi en;
+      en.C = N;
+      en.ldc = k;
+      gemm(OP_C, Zc, k, OP_N, Zc, k, k, k, k, en, CHASE_FP64);
+      Epi ew;
+      ew.C = Wk;
+      ew.ldc = k;
+      gemm(OP_N, G, k, OP_N, Zc, k, k, k, k, ew, CHASE_FP64);
+      Epi es;
+      es.C = Sq;
+      es.ldc = k;
+      gemm(OP_C, Zc, k, OP_N, Wk, k, k, k, k, es, CHASE_FP64);
+      dbg_finite(Sq, k, k, k, sizeof(T), "the quotient in the refinement");
+      eig_quotients<T>(st(), k, Sq, N, w, emax);
+      if (it == 0 && !clusters(OMEGA_WIDE, WIDE_MAX, OMEGA)) return false;
+      if (it == 1 && !clusters(OMEGA, k, OMEGA)) return false;
+      eig_correction<T>(st(), k, Sq, N, w, id_dev, Wk, emax);
+      Epi ez;
+      ez.C = N;
+      ez.ldc = k;
+      ez.Y = Zc;
+      ez.ldy = k;
+      ez.gamma = 1.0;
+      gemm(OP_N, Zc, k, OP_N, Wk, k, k, k, k, ez, CHASE_FP64);  // Z (I + E)
+      std::swap(Zc, N);
+      if (it == 0) solve_clusters();
+      if (it < 2) continue;
+      float e = 0.f;
+      CHASE_CUDA(cudaMemcpyAsync(&e, emax, sizeof(float), cudaMemcpyDeviceToHost, st()));
+      CHASE_CUDA(cudaStreamSynchronize(st()));
+      if (!(e < 0.5f)) return false;
+      done = e <= 1e-8f;
     }
-    const int ncl = (int)cl.size() / 2;
-    c->stats.rr_clusters += ncl;
-    if (ncl > 0) {
-      CHASE_CUDA(cudaMemcpyAsync(c->iwork, cl.data(), cl.size() * sizeof(int), cudaMemcpyHostToDevice, st()));
-      CHASE_CUDA(cudaMemsetAsync(c->status_dev, 0, sizeof(int), st()));
-      cluster_eig<T>(st(), k, ncl, c->iwork, Gp, k, Zn, k, w, nullptr, c->status_dev);
+    if (!done) return false;
+    solve_clusters();
+    c->stats.rr_clusters += (int)cl.size() / 2;
+    if (Zc != Z) {
+      sort_pairs<T>(st(), k, w, Zc, k, Z, k, c->dwork + 8, c->iwork + k);
+    } else {
+      sort_pairs<T>(st(), k, w, Zc, k, N, k, c->dwork + 8, c->iwork + k);
+      copy_cols<T>(st(), k, k, N, k, Z, k);
     }
-    sort_pairs<T>(st(), k, w, Zn, k, Z, k, c->dwork + 8, c->iwork + k);
     return true;
   }
 

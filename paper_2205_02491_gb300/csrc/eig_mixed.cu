@@ -1,12 +1,13 @@
 // Helpers of the mixed-precision Rayleigh-Ritz eigensolve (Algorithm 1, line 6).
 //
 // The quotient G is first diagonalised by the parallel Jacobi solver in FP32 (58x
-// the FP64 rate on GB300).  Its eigenvectors Z are then refined in FP64-class
-// arithmetic: with Z orthonormal and G' = Z^H G Z, the first-order correction
-// Z <- Z (I + X), X_pq = G'_pq / (d_q - d_p) for well separated d = diag(G'),
-// converges quadratically (three steps take the FP32 pass, stopped at its rounding floor, to FP64 accuracy).
-// Pairs closer than omega (clusters) are left to an exact FP64 Jacobi on each
-// cluster's block of G', one block per cluster.
+// the FP64 rate on GB300).  Its eigenvectors Z are then refined in FP64-class products (Ogita and Aishima 2018): with
+// N = Z^H Z, S = Z^H G Z, R = I - N and l_p = S_pp / N_pp,
+//   Z <- Z (I + E),  E_pq = (S_pq + l_q R_pq) / (l_q - l_p),
+// converges quadratically.  R's term is what close eigenvalues need: a normalisation Z (I - R / 2) in its place leaves
+// 3/8 R^2 in S, which a gap of 1e-5 amplifies (three eigenvalues 1e-5 apart: residuals up to 1e-3).
+// Pairs of one cluster take E_pq = R_pq / 2, which only keeps them orthonormal, and an exact FP64 Jacobi on the
+// cluster's block of the quotient, one block per cluster.
 #include "common.cuh"
 #include "kernels.h"
 
@@ -29,52 +30,74 @@ template <typename T, typename F> void convert_mat(cudaStream_t st, int k, const
   CHASE_CHECK_LAUNCH();
 }
 
+// l_p = S_pp / N_pp; zeroes the word that receives the largest entry of E
 template <typename T>
-__global__ void correction_kernel(int k, const T* Gp, int64_t ldg, T* X, int64_t ldx, double omega) {
+__global__ void quotients_kernel(int k, const T* S_, const T* N, double* lam, unsigned* emax) {
+  grid_dependency_wait();
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i == 0) *emax = 0u;
+  if (i < k) lam[i] = S<T>::re(S_[i + (int64_t)i * k]) / S<T>::re(N[i + (int64_t)i * k]);
+}
+
+template <typename T>
+void eig_quotients(cudaStream_t st, int k, const T* S_, const T* N, double* lam, unsigned* emax) {
+  launch_pdl(quotients_kernel<T>, ceil_div(k, 128), 128, 0, st, k, S_, N, lam, emax);
+  CHASE_CHECK_LAUNCH();
+}
+
+// id: the columns' clusters.  emax: the bits of the largest |re| + |im| (NaN stays largest).  S and N are Hermitian up to
+// rounding, which a small gap would amplify into a loss of orthonormality: their Hermitian parts are taken.
+template <typename T>
+__global__ void __launch_bounds__(128) correction_kernel(int k, const T* __restrict__ S_, const T* __restrict__ N,
+                                                          const double* __restrict__ lam, const int* __restrict__ id, T* E,
+                                                          unsigned* emax) {
   grid_dependency_wait();
   using s = S<T>;
-  int p = blockIdx.x * blockDim.x + threadIdx.x, q = blockIdx.y;
-  if (p >= k) return;
-  T v = s::zero();
-  if (p != q) {
-    const double dp = s::re(Gp[p + (int64_t)p * ldg]), dq = s::re(Gp[q + (int64_t)q * ldg]);
-    const double gap = dq - dp;
-    if (fabs(gap) > omega) v = s::scale(Gp[p + (int64_t)q * ldg], 1.0 / gap);
+  const int p = blockIdx.x * blockDim.x + threadIdx.x, q = blockIdx.y;
+  unsigned bits = 0u;
+  if (p < k) {
+    const int64_t pq = p + (int64_t)q * k, qp = q + (int64_t)p * k;
+    T r = s::scale(s::add(N[pq], s::conj(N[qp])), -0.5);
+    T v;
+    if (p == q) {
+      v = s::make(0.5 + 0.5 * s::re(r), 0.0);
+    } else if (id[p] == id[q]) {
+      v = s::scale(r, 0.5);
+    } else {
+      const T sv = s::scale(s::add(S_[pq], s::conj(S_[qp])), 0.5);
+      v = s::scale(s::add(sv, s::scale(r, lam[q])), 1.0 / (lam[q] - lam[p]));
+    }
+    E[pq] = v;
+    bits = __float_as_uint(fabsf((float)s::re(v)) + fabsf((float)s::im(v)));
   }
-  X[p + (int64_t)q * ldx] = v;
+  bits = __reduce_max_sync(0xffffffffu, bits);
+  if ((threadIdx.x & 31) == 0) atomicMax(emax, bits);
 }
 
 template <typename T>
-void eig_correction(cudaStream_t st, int k, const T* Gp, int64_t ldg, T* X, int64_t ldx, double omega) {
-  launch_pdl(correction_kernel<T>, dim3(ceil_div(k, 128), k), 128, 0, st, k, Gp, ldg, X, ldx, omega);
+void eig_correction(cudaStream_t st, int k, const T* S_, const T* N, const double* lam, const int* id, T* E, unsigned* emax) {
+  launch_pdl(correction_kernel<T>, dim3(ceil_div(k, 128), k), 128, 0, st, k, S_, N, lam, id, E, emax);
   CHASE_CHECK_LAUNCH();
 }
 
-template <typename T> __global__ void diag_real_kernel(int k, const T* G, int64_t ldg, double* d) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < k) d[i] = S<T>::re(G[i + (int64_t)i * ldg]);
-}
-
-template <typename T> void diag_real(cudaStream_t st, int k, const T* G, int64_t ldg, double* d) {
-  diag_real_kernel<T><<<ceil_div(k, 256), 256, 0, st>>>(k, G, ldg, d);
-  CHASE_CHECK_LAUNCH();
-}
-
-// One CTA per cluster [s, s+c), c <= CMAX: cyclic Jacobi on the block of G', eigenvalues to w[s..s+c),
-// then Z[:, s:s+c] <- Z[:, s:s+c] U in place, row by row.
-constexpr int CMAX = 32;
+// One CTA per cluster [s, s+c), c <= CMAX, after Z <- Z (I + E): the block of the new quotient is S_pq + (l_p + l_q) E_pq up
+// to the square of E (E = R / 2 inside a cluster).  Cyclic Jacobi on it, eigenvalues to w[s..s+c) (l before), then
+// Z[:, s:s+c] <- Z[:, s:s+c] U in place, row by row, both in ascending order.
+constexpr int CMAX = CLUSTER_MAX;
 template <typename T>
-__global__ void cluster_kernel(int k, const int* cl, const T* Gp, int64_t ldg, T* Z, int64_t ldz, double* w,
+__global__ void cluster_kernel(int k, const int* cl, const T* S_, const T* E, T* Z, int64_t ldz, double* w,
                                int* status) {
   using s = S<T>;
   const int start = cl[2 * blockIdx.x], c = cl[2 * blockIdx.x + 1];
   __shared__ T B[CMAX][CMAX + 1];
   __shared__ T U[CMAX][CMAX + 1];
   __shared__ T jpp, jpq, jqp, jqq;
-  __shared__ int cont;
+  __shared__ int cont, rank[CMAX];
   for (int t = threadIdx.x; t < c * c; t += blockDim.x) {
     int i = t % c, j = t / c;
-    B[i][j] = Gp[(start + i) + (int64_t)(start + j) * ldg];
+    const int64_t ij = (start + i) + (int64_t)(start + j) * k, ji = (start + j) + (int64_t)(start + i) * k;
+    const T h = s::scale(s::add(S_[ij], s::conj(S_[ji])), 0.5);
+    B[i][j] = s::add(h, s::scale(E[ij], w[start + i] + w[start + j]));
     U[i][j] = (i == j) ? s::one() : s::zero();
   }
   __syncthreads();
@@ -140,7 +163,14 @@ __global__ void cluster_kernel(int k, const int* cl, const T* Gp, int64_t ldg, T
       }
   }
   if (threadIdx.x == 0 && sweep >= 40) atomicMax(status, 1);
-  for (int i = threadIdx.x; i < c; i += blockDim.x) w[start + i] = s::re(B[i][i]);
+  // ascending (stable) order: the next pass tells clusters by the distance between neighbours
+  for (int i = threadIdx.x; i < c; i += blockDim.x) {
+    const double wi = s::re(B[i][i]);
+    int r = 0;
+    for (int j = 0; j < c; ++j) r += (s::re(B[j][j]) < wi) || (s::re(B[j][j]) == wi && j < i);
+    w[start + r] = wi;
+    rank[i] = r;
+  }
   __syncthreads();
   // Z[:, start:start+c] <- Z[:, start:start+c] U
   for (int r = threadIdx.x; r < k; r += blockDim.x) {
@@ -155,17 +185,16 @@ __global__ void cluster_kernel(int k, const int* cl, const T* Gp, int64_t ldg, T
 #pragma unroll
       for (int m = 0; m < CMAX; ++m)
         if (m < c) acc = s::fma(row[m], U[m][j], acc);
-      Z[r + (int64_t)(start + j) * ldz] = acc;
+      Z[r + (int64_t)(start + rank[j]) * ldz] = acc;
     }
   }
 }
 
 template <typename T>
-void cluster_eig(cudaStream_t st, int k, int nclusters, const int* cl, const T* Gp, int64_t ldg, T* Z, int64_t ldz,
-                 double* w, T* scratch, int* status) {
-  (void)scratch;
+void cluster_eig(cudaStream_t st, int k, int nclusters, const int* cl, const T* S_, const T* E, T* Z, int64_t ldz,
+                 double* w, int* status) {
   if (nclusters <= 0) return;
-  cluster_kernel<T><<<nclusters, 128, 0, st>>>(k, cl, Gp, ldg, Z, ldz, w, status);
+  cluster_kernel<T><<<nclusters, 128, 0, st>>>(k, cl, S_, E, Z, ldz, w, status);
   CHASE_CHECK_LAUNCH();
 }
 
@@ -188,10 +217,9 @@ void sort_pairs(cudaStream_t st, int k, double* w, const T* Z, int64_t ldz, T* o
 }
 
 #define INST(T)                                                                                                  \
-  template void eig_correction<T>(cudaStream_t, int, const T*, int64_t, T*, int64_t, double);                     \
-  template void cluster_eig<T>(cudaStream_t, int, int, const int*, const T*, int64_t, T*, int64_t, double*, T*,   \
-                               int*);                                                                            \
-  template void diag_real<T>(cudaStream_t, int, const T*, int64_t, double*);                                     \
+  template void eig_quotients<T>(cudaStream_t, int, const T*, const T*, double*, unsigned*);                      \
+  template void eig_correction<T>(cudaStream_t, int, const T*, const T*, const double*, const int*, T*, unsigned*); \
+  template void cluster_eig<T>(cudaStream_t, int, int, const int*, const T*, const T*, T*, int64_t, double*, int*); \
   template void sort_pairs<T>(cudaStream_t, int, double*, const T*, int64_t, T*, int64_t, double*, int*);
 INST(double)
 INST(double2)

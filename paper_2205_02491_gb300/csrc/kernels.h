@@ -46,11 +46,11 @@ template <typename T> void chol_stack_begin(cudaStream_t st, int k, T* Sm, int64
 template <typename T>
 void chol_stack_columns(cudaStream_t st, int k, int jbeg, int jend, T* Sm, int64_t lds, int* info, double pivot_floor,
                         int* dep);
-// Correction factor F (k x k) of a nearly orthonormal block with Gram matrix Gm: Q F is orthonormal up to the square of
-// Gm - I; upper: F upper triangular (keeps the QR's spans), else the nearest orthonormal block.  dev (device, zeroed
-// by the caller) receives the bits of a float bound of ||Gm - I||_2 (NaN when not finite).
+// Upper triangular correction factor F (k x k) of a nearly orthonormal block with Gram matrix Gm: Q F is orthonormal up to
+// the square of Gm - I and keeps the QR's spans.  dev (device, zeroed by the caller) receives the bits of a float bound of
+// ||Gm - I||_2 (NaN when not finite).
 template <typename T>
-void gram_correction(cudaStream_t st, int k, bool upper, const T* Gm, int64_t ldg, T* F, int64_t ldf, unsigned* dev);
+void gram_correction(cudaStream_t st, int k, const T* Gm, int64_t ldg, T* F, int64_t ldf, unsigned* dev);
 // Householder QR building blocks (blas_f64.cu): reflector of a column segment (v over x, alpha, real tau),
 // application of one reflector to ncols columns, the panel's reflectors with explicit zeros, the
 // compact-WY factor Tm of a panel from Gv = V^H V, and Q = [I; 0].
@@ -91,11 +91,13 @@ int heev_block_jacobi(cudaStream_t st, int k, F* G, int64_t ldg, double* w, F* Z
 // mixed-precision eigensolve helpers (eig_mixed.cu)
 template <typename T, typename F> void convert_mat(cudaStream_t st, int k, const T* in, int64_t ldi, F* out, int64_t ldo);
 template <typename T>
-void eig_correction(cudaStream_t st, int k, const T* Gp, int64_t ldg, T* X, int64_t ldx, double omega);
+void eig_quotients(cudaStream_t st, int k, const T* S, const T* N, double* lam, unsigned* emax);
 template <typename T>
-void cluster_eig(cudaStream_t st, int k, int nclusters, const int* cl /* start,size pairs (device) */, const T* Gp,
-                 int64_t ldg, T* Z, int64_t ldz, double* w, T* scratch, int* status);
-template <typename T> void diag_real(cudaStream_t st, int k, const T* G, int64_t ldg, double* d);
+void eig_correction(cudaStream_t st, int k, const T* S, const T* N, const double* lam, const int* id, T* E, unsigned* emax);
+constexpr int CLUSTER_MAX = 32;  // columns of a cluster
+template <typename T>
+void cluster_eig(cudaStream_t st, int k, int nclusters, const int* cl /* start,size pairs (device) */, const T* S,
+                 const T* E, T* Z, int64_t ldz, double* w, int* status);
 template <typename T>
 void sort_pairs(cudaStream_t st, int k, double* w, const T* Z, int64_t ldz, T* out, int64_t ldo, double* wtmp,
                 int* perm);
