@@ -229,7 +229,8 @@ __global__ void __launch_bounds__(256) row_exponent_kernel(int64_t nvec, int64_t
 
 // ---------------------------------------------------------------- residue planes
 // round(x 2^(62 - e)) by integer shifts of the mantissa (GB300's FP64 conversions run at 1/64 of the integer
-// rate); |result| <= 2^62 because |x| < 2^e.  Non-finite vectors give arbitrary in-range integers.
+// rate); |result| <= 2^62 because |x| < 2^e, which also keeps any left shift of a finite vector's entries within 64 bits
+// (9 for normal numbers, up to 61 where a whole vector is subnormal).  Non-finite vectors give arbitrary integers.
 __device__ __forceinline__ long long scaled_int(double x, int e) {
   const long long b = __double_as_longlong(x);
   const int be = (int)((b >> 52) & 0x7ff);
@@ -238,7 +239,7 @@ __device__ __forceinline__ long long scaled_int(double x, int e) {
   const int sh = (be != 0 ? be : 1) - 1075 + 62 - e;  // x = m 2^(exponent - 1075)
   long long r;
   if (sh >= 0) {
-    r = m << (sh < 9 ? sh : 9);
+    r = (long long)((unsigned long long)m << (sh < 62 ? sh : 62));
   } else {
     const int rs = sh > -62 ? -sh : 62;
     r = ((m >> (rs - 1)) + 1) >> 1;
