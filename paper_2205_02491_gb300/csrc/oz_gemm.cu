@@ -23,7 +23,7 @@ template <int NS> __device__ __forceinline__ void digits(double x, int e, float 
   const uint32_t hi = (uint32_t)__double2hiint(x);
   const int be = (int)((hi >> 20) & 0x7ff);
   if (be == 2047 || e < -1000 || e > 1000) {  // non-finite, or a scale near the ends of the range
-    double r = x * (1.0 / ldexp(1.0, e)) * 128.0;
+    double r = ldexp(x, 7 - e);  // exact; 1 / 2^e overflows for a subnormal column
 #pragma unroll
     for (int t = 0; t < NS; ++t) {
       const double d = rint(r);

@@ -1,4 +1,5 @@
-"""Products with operands whose entries are all subnormal: scaled without loss by exact powers of two."""
+"""Products with operands whose entries are all subnormal: scaled without loss by exact powers of two, FP64-class and
+mixed."""
 import numpy as np
 import pytest
 
@@ -48,3 +49,16 @@ def test_fp64_product_of_a_subnormal_matrix(pkg, cplx):
     C = host(pkg.Chase(n, k, complex_=cplx).hemm(dev(A), dev(B * 2.0 ** 990), "fp64"))
     ref = exact(A * 2.0 ** 1000, B)
     assert np.all(np.abs(C * 2.0 ** 10 - ref) <= bound(A * 2.0 ** 1000, B, ref))
+
+
+@pytest.mark.parametrize("mode,rel", [("bf16x3", 2.0 ** -13), ("bf16x6", 2.0 ** -20)])
+@pytest.mark.parametrize("n,cplx", [(255, True), (513, False)])
+def test_mixed_product_of_subnormal_columns(pkg, mode, rel, n, cplx):
+    g = np.random.default_rng(n)
+    A = hermitian(g, n, cplx)
+    k = 10
+    B, Bs = small_columns(g, n, k, cplx)
+    C = host(pkg.Chase(n, k, complex_=cplx).hemm(dev(A * 2.0 ** 990), dev(B), mode)) * 2.0 ** 10
+    s = np.max(np.abs(Bs), axis=0)
+    err = np.abs(C / s - A @ (Bs / s))
+    assert np.all(err <= rel * np.linalg.norm(A, axis=1)[:, None] * np.linalg.norm(Bs / s, axis=0)[None, :])
