@@ -137,16 +137,22 @@ void chase_default_opts(chase_opts* opts);
 /* Create a context on the current CUDA device.  Preallocates the whole
  * workspace for problems up to n_max x n_max with nev+nex <= ne_max (the
  * single-GPU form of Eq. GPU_mem plus split-product buffers); returns
- * CHASE_ERR_OOM early if it does not fit.  stream: the cudaStream_t all work of
+ * CHASE_ERR_OOM early if chase_workspace_bytes does not fit.  Beyond that it
+ * takes up to half of the memory left free, for residue planes of A: with all
+ * 16 moduli resident (96 bytes per element of a complex n_max x n_max matrix,
+ * 32 per real one) A is converted once per solve, with fewer once or more per
+ * product, with the same results.  Make allocations that need the room first.  stream: the cudaStream_t all work of
  * the context is enqueued on; NULL is the legacy default stream.  opts may be NULL. */
 chase_status chase_create(chase_ctx** ctx, int64_t n_max, int ne_max, chase_dtype dtype,
                           const chase_opts* opts, void* stream);
 void chase_destroy(chase_ctx* ctx);
 const char* chase_last_error(const chase_ctx* ctx);
 
-/* Device memory the context would allocate for (n_max, ne_max, dtype, mode set),
+/* Device memory a context for (n_max, ne_max, dtype, mode set) needs at least,
  * in bytes; the single-GPU form of Eq. GPU_mem (n^2 term excluded: A is the
- * caller's) plus split-product buffers. */
+ * caller's) plus split-product buffers.  chase_create takes more where it is
+ * free, see there; a grouped batch takes up to three quarters of the memory
+ * its problems' workspaces leave free. */
 int64_t chase_workspace_bytes(int64_t n_max, int ne_max, chase_dtype dtype, const chase_opts* opts);
 
 /* Seeds of the start vectors the library draws when the caller passes none (chase_solve with V0 or L0

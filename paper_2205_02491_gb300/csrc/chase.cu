@@ -1309,6 +1309,7 @@ static chase_status create_ctx(chase_ctx** out, int64_t n_max, int ne_max, chase
       c->workers.push_back(wc);
     }
   } catch (const chase::Error& e) {
+    cudaGetLastError();  // a failed allocation is reported here, not by the next launch
     chase_destroy(c);
     return (chase_status)e.status;
   }

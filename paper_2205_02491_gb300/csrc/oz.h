@@ -90,6 +90,7 @@ bool available();
 int64_t workspace_bytes(int64_t n_max, int ne_max, bool complex_, int a_mods);
 // Moduli of A that `budget` bytes hold, between the fewest and all.
 int a_mods_within(int64_t n_max, bool complex_, int64_t budget);
+// Planes of A for a_mods moduli, or of fewer (the fewest at least) when the allocation fails.
 void create(Workspace& w, int64_t n_max, int ne_max, bool complex_, int a_mods);
 void destroy(Workspace& w);
 // the tuner's choices so far: (size-class key, candidate index) pairs, for reports

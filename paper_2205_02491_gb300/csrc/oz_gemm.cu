@@ -211,10 +211,8 @@ void create(Workspace& w, int64_t n_max, int ne_max, bool complex_, int a_mods) 
   w.ne_max = ne_max;
   w.complex_ = complex_;
   if (!available()) return;
-  w.a_mods = a_mods;
   w.b_bytes = right_bytes(n_max, ne_max, complex_);
   w.residue_bytes = crt::residue_bytes(n_max, panel_cols(n_max, ne_max, complex_), complex_);
-  CHASE_CUDA(cudaMalloc(&w.a_res, crt::plane_bytes(n_max, n_max, complex_, a_mods)));
   CHASE_CUDA(cudaMalloc(&w.l_res, left_bytes(n_max, ne_max, complex_)));
   CHASE_CUDA(cudaMalloc(&w.b_planes, w.b_bytes));
   CHASE_CUDA(cudaMalloc(&w.residue, w.residue_bytes));
@@ -228,6 +226,15 @@ void create(Workspace& w, int64_t n_max, int ne_max, bool complex_, int a_mods) 
   CHASE_CUDA(cudaMemset(w.flags, 0, 16 * sizeof(int)));
   w.partial_elems = PARTIAL_ELEMS;
   CHASE_CUDA(cudaMalloc(&w.partial, (size_t)w.partial_elems * sizeof(double)));
+  // A's planes last, and fewer where the memory that was free when a_mods was chosen has gone to someone else since
+  for (w.a_mods = a_mods;; w.a_mods = std::max(fewest_mods(complex_), w.a_mods / 2)) {
+    const cudaError_t err = cudaMalloc(&w.a_res, crt::plane_bytes(n_max, n_max, complex_, w.a_mods));
+    if (err == cudaSuccess) break;
+    w.a_res = nullptr;
+    cudaGetLastError();
+    CHASE_REQUIRE(err == cudaErrorMemoryAllocation && w.a_mods > fewest_mods(complex_),
+                  err == cudaErrorMemoryAllocation ? 2 : 6, std::string("residue planes: ") + cudaGetErrorString(err));
+  }
   w.ready = true;
 }
 
