@@ -1677,6 +1677,15 @@ static void solve_batched_grouped(chase_ctx* c, int nprob, const void* const* A,
   if (need_new > 0) {
     size_t freeb = 0, totb = 0;
     CHASE_CUDA(cudaMemGetInfo(&freeb, &totb));
+    // what this context and the slots at hand have taken beyond their needs makes room first (grouped launches use the
+    // slots' planes, never this context's)
+    const int64_t want = need_new + (128ll << 20);
+    if ((int64_t)freeb < want) oz::shrink(c->ozw);
+    for (chase_ctx* sl : c->slots) {
+      CHASE_CUDA(cudaMemGetInfo(&freeb, &totb));
+      if (sl && (int64_t)freeb < want) oz::shrink(sl->ozw);
+    }
+    CHASE_CUDA(cudaMemGetInfo(&freeb, &totb));
     int64_t left = ((int64_t)freeb - need_new - (64ll << 20)) / 4 * 3;
     std::stable_sort(fresh.begin(), fresh.end(), [&](int a, int b) { return n[a] < n[b]; });
     for (int p : fresh) {

@@ -92,6 +92,8 @@ int64_t workspace_bytes(int64_t n_max, int ne_max, bool complex_, int a_mods);
 int a_mods_within(int64_t n_max, bool complex_, int64_t budget);
 // Planes of A for a_mods moduli, or of fewer (the fewest at least) when the allocation fails.
 void create(Workspace& w, int64_t n_max, int ne_max, bool complex_, int a_mods);
+// Gives back A's planes beyond the fewest (no call may be using them); the bytes given back.
+int64_t shrink(Workspace& w);
 void destroy(Workspace& w);
 // the tuner's choices so far: (size-class key, candidate index) pairs, for reports
 std::vector<std::pair<uint64_t, int>> tuned(const Workspace& w);

@@ -238,6 +238,19 @@ void create(Workspace& w, int64_t n_max, int ne_max, bool complex_, int a_mods) 
   w.ready = true;
 }
 
+int64_t shrink(Workspace& w) {
+  const int fewest = fewest_mods(w.complex_), had = w.a_mods;
+  if (!w.ready || had <= fewest) return 0;
+  CHASE_CUDA(cudaFree(w.a_res));
+  w.a_res = nullptr;
+  w.ready = false;  // should the allocation fail
+  w.a_mods = fewest;
+  w.a_src = nullptr;
+  CHASE_CUDA(cudaMalloc(&w.a_res, crt::plane_bytes(w.n_max, w.n_max, w.complex_, fewest)));
+  w.ready = true;
+  return crt::plane_bytes(w.n_max, w.n_max, w.complex_, had - fewest);
+}
+
 void destroy(Workspace& w) {
   void* ps[] = {w.a_res,   w.l_res,   w.b_planes, w.residue, w.a_planes, w.a_ex,
                 w.l_ex,    w.b_ex,    w.a_scale,  w.b_scale, w.flags,    w.partial};

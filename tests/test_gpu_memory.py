@@ -56,3 +56,34 @@ def test_contexts_created_together(pkg):
     finally:
         del hold
         torch.cuda.empty_cache()
+
+
+def test_batch_takes_back_what_its_context_holds(pkg):
+    """The batch context holds all of A's planes for its largest size; a batch whose workspaces do not fit beside them
+    takes them back."""
+    import torch
+    from gen import problems as G
+    from tests.helpers import dev
+    probs = [G.problem_small(n, 10, 6, complex_=False, seed_pid=30 + i) for i, n in enumerate((1800, 2100))]
+    n_max, ne = 14000, max(p.ne for p in probs)
+    need = sum(pkg.workspace_bytes(p.n, p.ne, complex_=False) for p in probs)
+    args = lambda: ([dev(p.dense()) for p in probs], [p.nev for p in probs], [p.nex for p in probs], 1e-10, 20, "fp64",  # noqa: E731
+                    [dev(p.V0) for p in probs], [dev(p.L0) for p in probs])
+    a = args()
+    s = pkg.Chase(n_max, ne, complex_=False)
+    torch.cuda.empty_cache()
+    torch.cuda.synchronize()
+    free, _ = torch.cuda.mem_get_info()
+    hold = torch.empty(free - need // 2 - (64 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        w, _ = s.solve_batched(*a)
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    for p, wp in zip(probs, w):
+        assert abs(wp.cpu().numpy() - p.lam[:p.nev]).max() <= 1e-10 * p.norm2()
+    # the context's own planes are the fewest now: same result as any other context's
+    v0, l0 = torch.randn((ne, 2100), dtype=torch.float64, device="cuda"), a[7][1]
+    w1, _ = s.solve(a[0][1], probs[1].nev, probs[1].nex, 1e-10, 20, "fp64", v0, l0)
+    assert abs(w1.cpu().numpy() - probs[1].lam[:probs[1].nev]).max() <= 1e-10 * probs[1].norm2()
+    s.close()
