@@ -141,7 +141,9 @@ void chase_default_opts(chase_opts* opts);
  * takes up to half of the memory left free, for residue planes of A: with all
  * 16 moduli resident (96 bytes per element of a complex n_max x n_max matrix,
  * 32 per real one) A is converted once per solve, with fewer once or more per
- * product, with the same results.  Make allocations that need the room first.  stream: the cudaStream_t all work of
+ * product, with the same results.  A new context or batch that does not fit takes
+ * back what idle contexts of the process hold so; other allocations cannot, and
+ * those that need the room are made first.  stream: the cudaStream_t all work of
  * the context is enqueued on; NULL is the legacy default stream.  opts may be NULL. */
 chase_status chase_create(chase_ctx** ctx, int64_t n_max, int ne_max, chase_dtype dtype,
                           const chase_opts* opts, void* stream);

@@ -34,6 +34,9 @@ std::atomic<unsigned long long> g_wait_limit_ns{0};
 }
 
 struct chase_ctx {
+  // held by every call on the context (by a batch's for its workers and slots too): planes of a context that no call uses
+  // may be taken back by make_room
+  std::recursive_mutex use;
   int device = 0;
   cudaStream_t stream = nullptr;
   bool own_stream = false;
@@ -1136,6 +1139,7 @@ static chase_status fail(chase_ctx* c, int code, const std::string& msg) {
 
 #define API_BEGIN(ctx) \
   if (!(ctx)) return CHASE_ERR_ARG; \
+  std::lock_guard<std::recursive_mutex> in_use((ctx)->use); \
   try {                           \
     CHASE_CUDA(cudaSetDevice((ctx)->device));
 #define API_END(ctx)                                                             \
@@ -1226,6 +1230,24 @@ int64_t chase_workspace_bytes(int64_t n_max, int ne_max, chase_dtype dtype, cons
 
 }  // extern "C"
 
+// Every context of the process.
+static std::mutex g_contexts_mu;
+static std::vector<chase_ctx*> g_contexts;
+
+// Frees device memory until `want` bytes are free, or as much as there is, by shrinking what idle contexts hold beyond
+// their needs: what a new context needs comes before that.
+static void make_room(int device, int64_t want) {
+  std::lock_guard<std::mutex> lock(g_contexts_mu);
+  for (chase_ctx* c : g_contexts) {
+    size_t freeb = 0, totb = 0;
+    CHASE_CUDA(cudaMemGetInfo(&freeb, &totb));
+    if ((int64_t)freeb >= want) return;
+    if (c->device != device) continue;
+    std::unique_lock<std::recursive_mutex> idle(c->use, std::try_to_lock);
+    if (idle.owns_lock()) oz::shrink(c->ozw);
+  }
+}
+
 // extra_bytes: device memory the context may take beyond chase_workspace_bytes to hold A's residue planes for more
 // moduli at a time (< 0: half of what is free after it).  All of them resident save a conversion of A per product.
 static chase_status create_ctx(chase_ctx** out, int64_t n_max, int ne_max, chase_dtype dtype, const chase_opts* opts,
@@ -1258,6 +1280,10 @@ static chase_status create_ctx(chase_ctx** out, int64_t n_max, int ne_max, chase
     CHASE_CUDA(cudaMemGetInfo(&freeb, &totb));
     const int nctx = c->opts.batch_grouped ? 1 : c->opts.batch_workers;
     int64_t need = chase_workspace_bytes(n_max, ne_max, dtype, &c->opts) * (int64_t)nctx;
+    if ((size_t)need + (64ull << 20) > freeb) {
+      make_room(c->device, need + (64ll << 20));
+      CHASE_CUDA(cudaMemGetInfo(&freeb, &totb));
+    }
     if ((size_t)need + (64ull << 20) > freeb) {
       c->err = "workspace of " + std::to_string(need) + " bytes does not fit in free device memory";
       chase_destroy(c);
@@ -1313,6 +1339,10 @@ static chase_status create_ctx(chase_ctx** out, int64_t n_max, int ne_max, chase
     chase_destroy(c);
     return (chase_status)e.status;
   }
+  {
+    std::lock_guard<std::mutex> lock(g_contexts_mu);
+    g_contexts.push_back(c);
+  }
   *out = c;
   return CHASE_OK;
 }
@@ -1326,6 +1356,10 @@ chase_status chase_create(chase_ctx** out, int64_t n_max, int ne_max, chase_dtyp
 
 void chase_destroy(chase_ctx* c) {
   if (!c) return;
+  {
+    std::lock_guard<std::mutex> lock(g_contexts_mu);
+    g_contexts.erase(std::remove(g_contexts.begin(), g_contexts.end(), c), g_contexts.end());
+  }
   for (chase_ctx* w : c->workers) chase_destroy(w);
   c->workers.clear();
   for (chase_ctx* w : c->slots) chase_destroy(w);
@@ -1677,15 +1711,12 @@ static void solve_batched_grouped(chase_ctx* c, int nprob, const void* const* A,
   if (need_new > 0) {
     size_t freeb = 0, totb = 0;
     CHASE_CUDA(cudaMemGetInfo(&freeb, &totb));
-    // what this context and the slots at hand have taken beyond their needs makes room first (grouped launches use the
-    // slots' planes, never this context's)
+    // this context's own planes, which grouped launches never use, and those of slots at hand are among what makes room
     const int64_t want = need_new + (128ll << 20);
-    if ((int64_t)freeb < want) oz::shrink(c->ozw);
-    for (chase_ctx* sl : c->slots) {
+    if ((int64_t)freeb < want) {
+      make_room(c->device, want);
       CHASE_CUDA(cudaMemGetInfo(&freeb, &totb));
-      if (sl && (int64_t)freeb < want) oz::shrink(sl->ozw);
     }
-    CHASE_CUDA(cudaMemGetInfo(&freeb, &totb));
     int64_t left = ((int64_t)freeb - need_new - (64ll << 20)) / 4 * 3;
     std::stable_sort(fresh.begin(), fresh.end(), [&](int a, int b) { return n[a] < n[b]; });
     for (int p : fresh) {
@@ -1710,6 +1741,8 @@ static void solve_batched_grouped(chase_ctx* c, int nprob, const void* const* A,
       sl->own_stream = true;
     }
   }
+  std::vector<std::unique_lock<std::recursive_mutex>> in_use;
+  for (int p = 0; p < nprob; ++p) in_use.emplace_back(c->slots[p]->use);
   // the grouped filter launches run on a stream of their own (measured: giving the problem streams a
   // higher priority only slowed the filter, with no gain in the overlap)
   if (!c->filter_stream) CHASE_CUDA(cudaStreamCreateWithFlags(&c->filter_stream, cudaStreamNonBlocking));
@@ -1945,6 +1978,8 @@ chase_status chase_solve_batched(chase_ctx* c, int nprob, const void* const* A, 
       solve_one_of_batch(c, A[p], n[p], nev[p], nex[p], tol, deg, mode, Vd[p], L0[p], eigvals[p],
                          stats_host ? &stats_host[p] : nullptr);
   } else {
+    std::vector<std::unique_lock<std::recursive_mutex>> in_use;
+    for (chase_ctx* wc : c->workers) in_use.emplace_back(wc->use);
     // inputs the caller enqueued on the context's stream must be complete before the workers'
     // non-blocking streams read them
     CHASE_CUDA(cudaStreamSynchronize(c->stream));

@@ -241,13 +241,21 @@ void create(Workspace& w, int64_t n_max, int ne_max, bool complex_, int a_mods) 
 int64_t shrink(Workspace& w) {
   const int fewest = fewest_mods(w.complex_), had = w.a_mods;
   if (!w.ready || had <= fewest) return 0;
-  CHASE_CUDA(cudaFree(w.a_res));
-  w.a_res = nullptr;
-  w.ready = false;  // should the allocation fail
+  const int64_t bytes = crt::plane_bytes(w.n_max, w.n_max, w.complex_, fewest);
+  void* kept = nullptr;
+  if (cudaMalloc(&kept, bytes) != cudaSuccess) {  // no room beside the old planes
+    cudaGetLastError();
+    CHASE_CUDA(cudaFree(w.a_res));
+    w.a_res = nullptr;
+    w.ready = false;  // should the allocation fail
+    CHASE_CUDA(cudaMalloc(&kept, bytes));
+    w.ready = true;
+  } else {
+    CHASE_CUDA(cudaFree(w.a_res));
+  }
+  w.a_res = kept;
   w.a_mods = fewest;
   w.a_src = nullptr;
-  CHASE_CUDA(cudaMalloc(&w.a_res, crt::plane_bytes(w.n_max, w.n_max, w.complex_, fewest)));
-  w.ready = true;
   return crt::plane_bytes(w.n_max, w.n_max, w.complex_, had - fewest);
 }
 

@@ -87,3 +87,51 @@ def test_batch_takes_back_what_its_context_holds(pkg):
     w1, _ = s.solve(a[0][1], probs[1].nev, probs[1].nex, 1e-10, 20, "fp64", v0, l0)
     assert abs(w1.cpu().numpy() - probs[1].lam[:probs[1].nev]).max() <= 1e-10 * probs[1].norm2()
     s.close()
+
+
+def test_new_contexts_come_before_planes_of_others(pkg):
+    """Three contexts whose needs fit: what the first two hold beyond theirs gives way to the third, also while another
+    thread's calls use one of them; products keep their bits."""
+    import torch
+    n, k = 12000, 48
+    need = pkg.workspace_bytes(n, k, complex_=False)
+    g = torch.Generator(device="cuda").manual_seed(2)
+    X = torch.randn((n, n), generator=g, device="cuda", dtype=torch.float64)
+    A = X.add_(X.mT.clone()).mul_(0.5)
+    B = torch.randn((k, n), generator=g, device="cuda", dtype=torch.float64)
+    first = pkg.Chase(n, k, complex_=False)
+    C = first.hemm(A, B, "fp64")
+    first.close()
+    torch.cuda.empty_cache()
+    torch.cuda.synchronize()
+    free, _ = torch.cuda.mem_get_info()
+    hold = torch.empty(free - 3 * need - (512 << 20), dtype=torch.uint8, device="cuda")
+    made = []
+    try:
+        for _ in range(3):
+            made.append(pkg.Chase(n, k, complex_=False))
+        for s in made:
+            assert torch.equal(s.hemm(A, B, "fp64"), C)
+        made.pop().close()
+        stop, wrong = threading.Event(), []
+
+        def use():
+            while not stop.is_set():
+                if not torch.equal(made[0].hemm(A, B, "fp64"), C):
+                    wrong.append(1)
+
+        t = threading.Thread(target=use)
+        t.start()
+        for _ in range(10):
+            try:
+                pkg.Chase(n, k, complex_=False).close()
+            except pkg.ChaseError as e:  # the context in use kept its planes
+                assert e.status == 2
+        stop.set()
+        t.join()
+        assert not wrong
+    finally:
+        for s in made:
+            s.close()
+        del hold
+        torch.cuda.empty_cache()
