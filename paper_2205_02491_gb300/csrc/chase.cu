@@ -91,6 +91,8 @@ struct chase_ctx {
   cudaStream_t filter_stream = nullptr;  // stream of the grouped filter launches
 };
 
+static void make_room(int device, int64_t want);
+
 namespace {
 
 struct Timer {
@@ -800,7 +802,9 @@ template <typename T> struct Solver {
     // where memory allows (n = 4096, l = 68: 36 MB), else per product
     const size_t lp = crt::plane_bytes(l, n, S<T>::cplx, crt::NMOD), rp = crt::plane_bytes(n, l, S<T>::cplx, crt::NMOD);
     const size_t planes_at = (need + 255) / 256 * 256, with_planes = planes_at + lp + rp + (size_t)(l + n) * sizeof(int);
-    if (c->bwd_bytes < with_planes) {
+    size_t freeb = 0, totb = 0;
+    if (c->bwd_bytes < with_planes) CHASE_CUDA(cudaMemGetInfo(&freeb, &totb));
+    if (c->bwd_bytes < need || (c->bwd_bytes < with_planes && with_planes + (64ull << 20) <= freeb + c->bwd_bytes)) {
       if (c->bwd) CHASE_CUDA(cudaFree(c->bwd));
       c->bwd = nullptr;
       c->bwd_bytes = 0;
@@ -809,6 +813,8 @@ template <typename T> struct Solver {
         cudaGetLastError();
         c->bwd = nullptr;
         got = need;
+        // what the context holds beyond its needs comes after this
+        make_room(c->device, (int64_t)got + (64ll << 20));
         CHASE_CUDA(cudaMalloc(&c->bwd, got));
       }
       c->bwd_bytes = got;
@@ -1234,8 +1240,8 @@ int64_t chase_workspace_bytes(int64_t n_max, int ne_max, chase_dtype dtype, cons
 static std::mutex g_contexts_mu;
 static std::vector<chase_ctx*> g_contexts;
 
-// Frees device memory until `want` bytes are free, or as much as there is, by shrinking what idle contexts hold beyond
-// their needs: what a new context needs comes before that.
+// Frees device memory until `want` bytes are free, or as much as there is, by shrinking what contexts hold beyond their
+// needs: those that are idle, and those that the calling thread's own call holds (whose planes it does not use yet).
 static void make_room(int device, int64_t want) {
   std::lock_guard<std::mutex> lock(g_contexts_mu);
   for (chase_ctx* c : g_contexts) {
@@ -1431,6 +1437,7 @@ chase_status chase_solve(chase_ctx* c, const void* A, int64_t n, int64_t lda, in
       if (c->a_stage) CHASE_CUDA(cudaFree(c->a_stage));
       c->a_stage = nullptr;
       c->a_stage_bytes = 0;
+      make_room(c->device, (int64_t)need + (64ll << 20));
       size_t freeb = 0, totb = 0;
       CHASE_CUDA(cudaMemGetInfo(&freeb, &totb));
       CHASE_REQUIRE(need + (64ull << 20) <= freeb, CHASE_ERR_OOM, "no device memory for a copy of the host A");

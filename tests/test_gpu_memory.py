@@ -1,7 +1,7 @@
-"""Contexts created at the same time: each counts the same free memory, so what they take beyond their needs must give
-way."""
+"""Device memory that is short: what contexts hold beyond their needs gives way to other contexts, batches and calls."""
 import threading
 
+import numpy as np
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -135,3 +135,23 @@ def test_new_contexts_come_before_planes_of_others(pkg):
             s.close()
         del hold
         torch.cuda.empty_cache()
+
+
+def test_copy_of_a_host_matrix_comes_before_planes(pkg):
+    """The device copy of a host A takes the place of planes where there is no other room."""
+    import torch
+    from gen import problems as G
+    p = G.problem_small(5000, 8, 6, complex_=False, seed_pid=40)
+    A, V0, L0 = (torch.from_numpy(np.ascontiguousarray(x.T)) for x in (p.dense(), p.V0, p.L0))
+    s = pkg.Chase(9000, p.ne, complex_=False)
+    torch.cuda.empty_cache()
+    torch.cuda.synchronize()
+    free, _ = torch.cuda.mem_get_info()
+    hold = torch.empty(free - (150 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        w, _ = s.solve(A, p.nev, p.nex, 1e-10, 20, "fp64", V0, L0)
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    assert np.max(np.abs(w.numpy() - p.lam[:p.nev])) <= 1e-10 * p.norm2()
+    s.close()
