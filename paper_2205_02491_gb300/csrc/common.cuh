@@ -198,6 +198,11 @@ __device__ __forceinline__ double fast_rsqrt(double q) {
   return y;
 }
 
+// |a| where its square would underflow: off-diagonal entries within a degenerate group fall far below 1e-150, and a phase
+// a / |a| of the wrong length makes a rotation that is not unitary
+__device__ __forceinline__ double magnitude(double a) { return fabs(a); }
+__device__ __forceinline__ double magnitude(double2 a) { return hypot(a.x, a.y); }
+
 // warp-level FP64 sum
 __device__ inline double warp_sum(double v) {
 #pragma unroll

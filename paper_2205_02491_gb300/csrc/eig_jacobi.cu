@@ -47,7 +47,7 @@ __device__ __forceinline__ void jacobi_params(int k, int kp, int r, int idx, con
     return;
   }
   T g = G[p + (int64_t)q * ldg];
-  double ag = sqrt(s::abs2(g));
+  double ag = magnitude(g);
   if (!(ag > 1e-300)) {
     rot[p] = Rot<T>{q, s::one(), s::zero()};
     rot[q] = Rot<T>{p, s::one(), s::zero()};

@@ -119,8 +119,8 @@ __global__ void cluster_kernel(int k, const int* cl, const T* S_, const T* E, T*
       for (int q = p + 1; q < c; ++q) {
         if (threadIdx.x == 0) {
           T g = B[p][q];
-          double ag = sqrt(s::abs2(g));
-          if (ag == 0.0) {
+          double ag = magnitude(g);
+          if (!(ag > 1e-300)) {
             jpp = s::one();
             jpq = s::zero();
             jqp = s::zero();
