@@ -531,7 +531,7 @@ void generate_wy(cudaStream_t st, T* A, int64_t n, int64_t lda, const double* la
 }
 
 // ============================================================== Householder QR building blocks
-// Reflector of one column segment x (length m): alpha = -ph ||x|| with ph = x0/|x0| (1 for x0 = 0),
+// Reflector of one column segment x (length m): alpha = -ph ||x|| with ph = x0/|x0| (1 below 1e-300),
 // v = x - alpha e1 written over x, H = I - tau v v^H with tau = 2/||v||^2 (0 for x = 0), so H x = alpha e1.
 template <typename T>
 __global__ void __launch_bounds__(1024) householder_vec_kernel(int64_t m, T* x, T* alpha, double* tau) {
@@ -546,9 +546,9 @@ __global__ void __launch_bounds__(1024) householder_vec_kernel(int64_t m, T* x, 
     double t = 0.0;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
     const T x0 = x[0];
-    const double a0 = sqrt(s::abs2(x0));
+    const double a0 = magnitude(x0);
     const double nrm = sqrt(t);
-    const T ph = a0 > 0.0 ? s::scale(x0, 1.0 / a0) : s::one();
+    const T ph = a0 > 1e-300 ? s::scale(x0, 1.0 / a0) : s::one();
     alpha[0] = s::scale(ph, -nrm);
     const T v0 = s::scale(ph, a0 + nrm);
     const double vv = t - a0 * a0 + (a0 + nrm) * (a0 + nrm);

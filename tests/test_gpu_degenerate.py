@@ -1,5 +1,6 @@
 """Phases of numbers whose squares underflow.  The FP64 Jacobi eigensolver on degenerate spectra: entries between equal
-eigenvalues fall far below the square root of the smallest FP64 number while the sweeps go on for the others."""
+eigenvalues fall far below the square root of the smallest FP64 number while the sweeps go on for the others.  Householder
+reflectors: a column whose first entry is that small."""
 import numpy as np
 import pytest
 
@@ -64,3 +65,24 @@ def test_rayleigh_ritz_of_a_degenerate_quotient(pkg, cplx, k):
         assert np.max(np.abs(w - lam)) <= 1e-12, group
         assert torch.linalg.vector_norm(A @ V - V * wt[None, :], dim=0).max().item() <= 1e-12, group
         assert (V.mH @ V - torch.eye(k, dtype=dt, device="cuda")).abs().max().item() <= 1e-12, group
+
+
+@pytest.mark.parametrize("cplx", [True, False])
+@pytest.mark.parametrize("exponent", [-160.0, -160.5, -161.0, -161.5, -305.0])
+def test_householder_qr_with_a_tiny_first_entry(pkg, cplx, exponent):
+    from tests.helpers import dev, host
+    n, k = 400, 24
+    g = np.random.default_rng(7)
+    rand = lambda *shape: g.standard_normal(shape) + (1j * g.standard_normal(shape) if cplx else 0.0)  # noqa: E731
+    X = rand(n, k)
+    X[:, 9] = X[:, 4] + 1e-13 * rand(n)  # numerically dependent: the block goes to the Householder QR
+    X[0] *= 10.0 ** exponent
+    s = pkg.Chase(n, k, complex_=cplx)
+    before = s.stats()["qr_householder"]
+    Xt = dev(X)
+    s.qr(Xt)
+    assert s.stats()["qr_householder"] == before + 1
+    Q = host(Xt)
+    assert np.max(np.abs(np.conj(Q.T) @ Q - np.eye(k))) <= 1e-12
+    R = X - Q @ (np.conj(Q.T) @ X)
+    assert np.max(np.linalg.norm(R, axis=0) / np.linalg.norm(X, axis=0)) <= 1e-10
