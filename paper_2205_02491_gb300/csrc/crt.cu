@@ -1,4 +1,5 @@
-// FP64-class products C = L R on the bf16 tensor cores (tcgen05, TMEM, TMA, CTA pairs) through residues.
+// FP64-class products C = L R on the bf16 tensor cores (tcgen05, TMEM, TMA, CTA pairs) through residues: the modular form of
+// Ozaki's scheme (Ozaki, Uchino and Imamura 2025).
 //
 // Every left row / right column x is scaled by a power of two so that its 2-norm is below 2^62 and rounded to
 // integers X (at most half a unit each).  The integer product then satisfies |C_ij| <= ||X_i|| ||Y_j|| < 2^124
