@@ -1145,8 +1145,8 @@ static chase_status fail(chase_ctx* c, int code, const std::string& msg) {
 
 #define API_BEGIN(ctx) \
   if (!(ctx)) return CHASE_ERR_ARG; \
-  std::lock_guard<std::recursive_mutex> in_use((ctx)->use); \
   try {                           \
+    std::lock_guard<std::recursive_mutex> in_use((ctx)->use); \
     CHASE_CUDA(cudaSetDevice((ctx)->device));
 #define API_END(ctx)                                                             \
   }                                                                              \
@@ -1340,14 +1340,15 @@ static chase_status create_ctx(chase_ctx** out, int64_t n_max, int ne_max, chase
       wc->own_stream = true;
       c->workers.push_back(wc);
     }
+    std::lock_guard<std::mutex> lock(g_contexts_mu);
+    g_contexts.push_back(c);
   } catch (const chase::Error& e) {
     cudaGetLastError();  // a failed allocation is reported here, not by the next launch
     chase_destroy(c);
     return (chase_status)e.status;
-  }
-  {
-    std::lock_guard<std::mutex> lock(g_contexts_mu);
-    g_contexts.push_back(c);
+  } catch (const std::exception&) {
+    chase_destroy(c);
+    return CHASE_ERR_OOM;
   }
   *out = c;
   return CHASE_OK;
