@@ -1236,9 +1236,9 @@ int64_t chase_workspace_bytes(int64_t n_max, int ne_max, chase_dtype dtype, cons
 
 }  // extern "C"
 
-// Every context of the process.
+// Every context of the process (never destroyed: contexts may outlive the library's static objects at exit).
 static std::mutex g_contexts_mu;
-static std::vector<chase_ctx*> g_contexts;
+static std::vector<chase_ctx*>& g_contexts = *new std::vector<chase_ctx*>();
 
 // Frees device memory until `want` bytes are free, or as much as there is, by shrinking what contexts hold beyond their
 // needs: those that are idle, and those that the calling thread's own call holds (whose planes it does not use yet).
